@@ -112,10 +112,10 @@ __device__ __forceinline__ void mandel_of(int al, const double* gr, double* e) {
 // ---------------------------------------------------------------------------
 // K4 (FP32): TMA-pipelined block-packed patch products
 //
-// Persistent CTAs of 128 threads.  Each iteration handles PPI patches whose
+// Persistent CTAs of 64 threads.  Each iteration handles PPI patches (3D: 1, 2D: 32) whose
 // block-packed inverses (see BlockLayout) are streamed into a ring of NSTAGE
 // shared-memory stages by 1D bulk copies (cp.async.bulk, completion counted on
-// an mbarrier), issued by thread 0 NSTAGE iterations ahead.  Thread b of a
+// an mbarrier), issued NSTAGE iterations ahead.  In 3D thread b of a
 // patch owns one 9x9 block S_IJ and forms both S_IJ r_J and S_IJ^T r_I from
 // registers, so each stored entry is read from shared memory exactly once; a
 // fixed-order reduction of the block partials gives y_v = A_v^-1 r|_v.
@@ -261,28 +261,6 @@ __device__ __forceinline__ void block_of(const BlockLayout& BL, int b, int& I, i
   }
 }
 
-template <int DIM, int NST, typename TS = float>
-struct TmaCfg {
-  static constexpr int NP = Sz<DIM>::NP;
-  static constexpr int NB = Sz<DIM>::NB;
-  static constexpr int THREADS = 64;
-  static constexpr int TPP = DIM == 3 ? 64 : 4;        // threads per patch (>= blocks per patch)
-  static constexpr int PPI = THREADS / TPP;            // patches per iteration
-  static constexpr int NSTAGE = NST;
-  static constexpr int STRIDE = block_stride<TS>(NP);  // entries per patch
-  static constexpr int NBR = NP / 9;
-  static constexpr int RPT = (PPI * NP + THREADS - 1) / THREADS;   // r values gathered per thread
-  static constexpr size_t stage_elems = (size_t)PPI * STRIDE;
-  static constexpr size_t stage_bytes = stage_elems * sizeof(TS);
-  // dynamic shared memory: [mbarriers | stages | r | partials]; the barriers need
-  // 8-byte and the bulk-copy destinations 16-byte alignment
-  static constexpr size_t bar_bytes = 128;
-  static constexpr size_t smem_bytes =
-      bar_bytes + NSTAGE * stage_bytes + (size_t)PPI * NP * 4 + (size_t)PPI * NP * NBR * 4;
-  static_assert(NSTAGE * 8 <= bar_bytes, "mbarrier area too small");
-  static_assert((STRIDE * sizeof(TS)) % 16 == 0 && stage_bytes % 16 == 0, "bulk copies need 16-byte alignment");
-};
-
 // Work list of the FP32 star kernels, wl = bit 0 | bit 1: bit 0 clear = the star products
 // of the smoother, set = the local solves on the coarse-cell interiors (the stars of the
 // fine vertices 2K+1 at the coarse-cell centres, which are interior vertices); bit 1 set =
@@ -310,16 +288,6 @@ __device__ __forceinline__ int work_vertex(const Geom& g, int wl, int p, int cou
   vz = DIM == 3 ? 2 * kz + 1 : 0;
   if (split) return (vx - 1) + nix * ((vy - 1) + (DIM == 3 ? niy * (vz - 1) : 0));
   return vx + g.nv[0] * (vy + g.nv[1] * vz);
-}
-
-// r at patch entry i of the vertex (absent nodes give 0)
-template <int DIM>
-__device__ __forceinline__ float patch_r(const Geom& g, const float* __restrict__ r, int vid, int vx, int vy, int vz,
-                                         int i) {
-  constexpr int NB = Sz<DIM>::NB;
-  if (vid < 0) return 0.f;
-  long long nd;
-  return patch_node<DIM>(g, vx, vy, vz, i % NB, nd) ? __ldg(r + (i / NB) * g.N + nd) : 0.f;
 }
 
 // One patch per iteration (3D): the index arithmetic of a thread's entries is split
@@ -379,57 +347,212 @@ __device__ __forceinline__ bool entry_in(const Geom& g, const PatchPos& q, const
   return true;
 }
 
-// (bx, gx: the block's index and the blocks of this instance, see batch.cuh)
+// ---------------------------------------------------------------------------
+// K4 (FP32) in 2D: 32 stars per pair of warps, one star a lane.  A star's 18 x 18 inverse is
+// two diagonal 9x9 blocks and one off-diagonal block, 81 products each way round: the first
+// warp of the pair takes the off-diagonal block (both directions, 81 entries), the second the
+// two diagonal ones (90 entries), so both do 162 FMAs a star from registers; nine values are
+// exchanged through shared memory and each warp writes one component.  What bounds it is
+// instruction issue, so the index arithmetic is done once per star and lane.  The form before,
+// four threads a star with one block each and the partial sums in shared memory, spent about
+// ten times the instructions on indices and reductions: a 128^2 five-level cycle took 1134 us
+// with it and takes 1034 us with this one (same sums, same bits).
+// ---------------------------------------------------------------------------
+template <typename TS>
+struct Star2Exchange {
+  float v[2][2][9][32];   // [parity of the iteration][writer's role][entry][star]
+};
+
+// r on the star of q: comp[c][o], o = ox + 3 oy
+__device__ __forceinline__ void star2_r(const Geom& g, const PatchPos& q, const float* __restrict__ r, float (&r0)[9],
+                                        float (&r1)[9]) {
+#pragma unroll
+  for (int o = 0; o < 9; ++o) {
+    const int ox = o % 3, oy = o / 3;
+    const int i = 2 * q.vx + ox - 1, j = 2 * q.vy + oy - 1;
+    const bool in = q.vid >= 0 && (q.inner || (i > 0 && i < g.nn[0] - 1 && j > 0 && j < g.nn[1] - 1));
+    const int at = q.gbase + (oy - 1) * g.nn[0] + (ox - 1);
+    r0[o] = in ? __ldg(r + at) : 0.f;
+    r1[o] = in ? __ldg(r + (at + (int)g.N)) : 0.f;
+  }
+}
+
+// the role's block products of one star: role 0: a = S_01 r_1, b = S_01^T r_0; role 1: a = S_00 r_0, b = S_11 r_1
+template <bool GLOBAL, typename TS>
+__device__ __forceinline__ void star2_products(const TS* __restrict__ S, int role, const float (&r0)[9],
+                                               const float (&r1)[9], float (&a)[9], float (&b)[9]) {
+  constexpr BlockLayout BL = BlockLayout(18);
+  if (role == 0) {
+    block_product<GLOBAL, TS>(BL, S, 0, false, r0, r1, a, b);
+  } else {
+    float unused[9];
+    block_product<GLOBAL, TS>(BL, S, 1, true, r0, r0, a, unused);
+    block_product<GLOBAL, TS>(BL, S, 2, true, r1, r1, b, unused);
+  }
+}
+
+// y of component `role` (y_c = block (c, 0) part + block (c, 1) part) to the scratch rows or the nodes of out
+__device__ __forceinline__ void star2_store(const Geom& g, const PatchPos& q, int role, const float (&first)[9],
+                                            const float (&second)[9], float* __restrict__ out, int mode) {
+  if (q.vid < 0) return;
+  const int rowlen = 3 * g.nv[0];
+#pragma unroll
+  for (int o = 0; o < 9; ++o) {
+    const int ox = o % 3, oy = o / 3;
+    const float y = first[o] + second[o];
+    if (mode == OUT_SCRATCH) {
+      out[(3 * role + oy) * (g.nv[1] * rowlen) + q.obase + ox] = y;
+    } else {
+      const int i = 2 * q.vx + ox - 1, j = 2 * q.vy + oy - 1;
+      if (q.inner || (i > 0 && i < g.nn[0] - 1 && j > 0 && j < g.nn[1] - 1)) {
+        float* p = out + (q.gbase + (oy - 1) * g.nn[0] + (ox - 1) + role * (int)g.N);
+        *p = mode == OUT_SUBTRACT ? *p - y : y;
+      }
+    }
+  }
+}
+
 template <int DIM, int NST, typename TS = float>
-__device__ __forceinline__ void patch_tma_body(unsigned bx, unsigned gx, const Geom& g, const TS* __restrict__ inv,
-                                               int interior, int count, const float* __restrict__ r,
-                                               float* __restrict__ out, int mode, DevStatus* st, int wait_polls,
-                                               int early_trigger) {
-  using C = TmaCfg<DIM, NST, TS>;
-  constexpr int NP = C::NP, NB = C::NB, PPI = C::PPI, TPP = C::TPP, NSTAGE = C::NSTAGE, NBR = C::NBR;
-  constexpr int RPT = C::RPT, THREADS = C::THREADS;
-  constexpr BlockLayout BL = BlockLayout(NP);
-  constexpr int ISSUER = THREADS - 1;                     // idle in the block phase (b >= NBP)
-  static_assert(ISSUER % TPP >= BlockLayout(NP).nbp, "the issuing thread must not own a block");
+struct TmaCfg {
+  static constexpr int NP = Sz<DIM>::NP;
+  static constexpr int NB = Sz<DIM>::NB;
+  static constexpr int THREADS = 64;
+  static constexpr int TPP = DIM == 3 ? 64 : 2;        // threads per patch (3D: >= blocks per patch)
+  static constexpr int PPI = THREADS / TPP;            // patches per iteration
+  static constexpr int NSTAGE = NST;
+  static constexpr int STRIDE = block_stride<TS>(NP);  // entries per patch
+  static constexpr int NBR = NP / 9;
+  static constexpr int RPT = (PPI * NP + THREADS - 1) / THREADS;   // r values gathered per thread
+  static constexpr size_t stage_elems = (size_t)PPI * STRIDE;
+  static constexpr size_t stage_bytes = stage_elems * sizeof(TS);
+  // dynamic shared memory: [mbarriers | stages | r | partials]; the barriers need
+  // 8-byte and the bulk-copy destinations 16-byte alignment
+  static constexpr size_t bar_bytes = 128;
+  static constexpr size_t work_bytes =                 // 3D: r and the block partials; 2D: the exchange
+      DIM == 3 ? (size_t)PPI * NP * 4 + (size_t)PPI * NP * NBR * 4 : sizeof(Star2Exchange<TS>);
+  static constexpr size_t smem_bytes = bar_bytes + NSTAGE * stage_bytes + work_bytes;
+  static_assert(NSTAGE * 8 <= bar_bytes, "mbarrier area too small");
+  static_assert((STRIDE * sizeof(TS)) % 16 == 0 && stage_bytes % 16 == 0, "bulk copies need 16-byte alignment");
+};
+
+// 2D: the ring's stage holds 32 stars (one copy when the list is contiguous in inv, else one a
+// star), the two warps take the roles of star2_products; the lanes' 16-byte reads of a stage,
+// 172 floats apart, hit all banks.
+template <int NST, typename TS>
+__device__ __forceinline__ void patch_tma2_body(unsigned bx, unsigned gx, const Geom& g, const TS* __restrict__ inv,
+                                                int interior, int count, const float* __restrict__ r,
+                                                float* __restrict__ out, int mode, DevStatus* st, int wait_polls,
+                                                int early_trigger) {
+  using C = TmaCfg<2, NST, TS>;
+  constexpr int PPI = C::PPI, NSTAGE = C::NSTAGE;
+  static_assert(PPI == 32, "one star a lane");
   extern __shared__ __align__(128) unsigned char smraw[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(smraw);
   TS* stages = reinterpret_cast<TS*>(smraw + C::bar_bytes);
-  float* rs = reinterpret_cast<float*>(smraw + C::bar_bytes + NSTAGE * C::stage_bytes);   // [PPI][NP]
-  float* part = rs + PPI * NP;                            // [PPI][NP][NBR]
+  auto& sm = *reinterpret_cast<Star2Exchange<TS>*>(smraw + C::bar_bytes + NSTAGE * C::stage_bytes);
+  __shared__ int s_fail;
+  const int tid = threadIdx.x, lane = tid & 31, role = tid >> 5;
+  const int ngroups = (count + PPI - 1) / PPI;
+  // one warp issues a stage's copies: the star products' list is contiguous (one copy), the
+  // interior solves' stars are every second vertex (a copy a lane)
+  auto issue = [&](int grp, int stage) {
+    const int p = grp * PPI + lane;
+    int vx, vy, vz;
+    const int vid = work_vertex<2>(g, interior, p, count, vx, vy, vz);
+    const int have = count - grp * PPI < PPI ? count - grp * PPI : PPI;
+    TS* dst = stages + stage * C::stage_elems;
+    if (lane == 0) tma::mbar_expect_tx(&bars[stage], (uint32_t)(have * C::STRIDE * sizeof(TS)));
+    __syncwarp();
+    if (!(interior & 1)) {
+      if (lane == 0)
+        tma::bulk_load(dst, inv + (long long)vid * C::STRIDE, (uint32_t)(have * C::STRIDE * sizeof(TS)), &bars[stage]);
+    } else if (vid >= 0) {
+      tma::bulk_load(dst + (size_t)lane * C::STRIDE, inv + (long long)vid * C::STRIDE, C::STRIDE * sizeof(TS),
+                     &bars[stage]);
+    }
+  };
+  if (tid == 32) {
+    s_fail = 0;
+    for (int i = 0; i < NSTAGE; ++i) tma::mbar_init(&bars[i], 1);
+    tma::fence_init();
+  }
+  __syncthreads();
+  if (role == 1)
+    for (int i = 0; i < NSTAGE; ++i)
+      if ((int)(bx + i * gx) < ngroups) issue(bx + i * gx, i);
+  pdl_wait();
+  if (early_trigger) pdl_trigger();   // as in the 3D form below
+  PatchPos q = patch_pos<2>(g, interior, bx * PPI + lane, count);
+  float r0[9], r1[9];
+  star2_r(g, q, r, r0, r1);
+  int it = 0;
+  for (int grp = bx; grp < ngroups; grp += gx, ++it) {
+    const int stage = it % NSTAGE;
+    if (!tma::mbar_wait(&bars[stage], (uint32_t)((it / NSTAGE) & 1), wait_polls)) {
+      report(st, 7 /* ALS_ETIMEOUT */, grp);
+      s_fail = 1;
+    }
+    float a[9], b[9], got[9];
+    star2_products<false, TS>(stages + stage * C::stage_elems + (size_t)lane * C::STRIDE, role, r0, r1, a, b);
+    auto& ex = sm.v[it & 1];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) ex[role][k][lane] = role == 0 ? b[k] : a[k];
+    // the next group's r: in flight over the exchange
+    const PatchPos qn = patch_pos<2>(g, interior, (grp + gx) * PPI + lane, count);
+    star2_r(g, qn, r, r0, r1);
+    __syncthreads();                        // the exchange is complete, the stage is consumed
+    if (s_fail) break;
+    if (role == 1 && (int)(grp + NSTAGE * gx) < ngroups) {
+      tma::fence_async();
+      issue(grp + NSTAGE * gx, stage);
+    }
+#pragma unroll
+    for (int k = 0; k < 9; ++k) got[k] = ex[1 - role][k][lane];
+    if (role == 0) star2_store(g, q, 0, got, a, out, mode);
+    else star2_store(g, q, 1, got, b, out, mode);
+    q = qn;
+  }
+  if (!early_trigger) pdl_trigger();
+  if (s_fail && tid == 32) {
+    // drain, as in the 3D form below
+    int k = it;
+    for (int grp = bx + it * gx; grp < ngroups && k < it + NSTAGE; grp += gx, ++k)
+      tma::mbar_wait(&bars[k % NSTAGE], (uint32_t)((k / NSTAGE) & 1));
+  }
+}
+
+// (bx, gx: the block's index and the blocks of this instance, see batch.cuh)
+template <int NST, typename TS>
+__device__ __forceinline__ void patch_tma3_body(unsigned bx, unsigned gx, const Geom& g, const TS* __restrict__ inv,
+                                               int interior, int count, const float* __restrict__ r,
+                                               float* __restrict__ out, int mode, DevStatus* st, int wait_polls,
+                                               int early_trigger) {
+  constexpr int DIM = 3;
+  using C = TmaCfg<DIM, NST, TS>;
+  constexpr int NP = C::NP, NSTAGE = C::NSTAGE, NBR = C::NBR;
+  constexpr int RPT = C::RPT, THREADS = C::THREADS;
+  constexpr BlockLayout BL = BlockLayout(NP);
+  constexpr int ISSUER = THREADS - 1;                     // idle in the block phase (b >= NBP)
+  static_assert(C::PPI == 1 && ISSUER >= BlockLayout(NP).nbp, "the issuing thread must not own a block");
+  extern __shared__ __align__(128) unsigned char smraw[];
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smraw);
+  TS* stages = reinterpret_cast<TS*>(smraw + C::bar_bytes);
+  float* rs = reinterpret_cast<float*>(smraw + C::bar_bytes + NSTAGE * C::stage_bytes);   // [NP]
+  float* part = rs + NP;                                  // [NP][NBR]
   __shared__ int s_fail;
   const int tid = threadIdx.x;
-  const int ngroups = (count + PPI - 1) / PPI;
+  const int ngroups = count;   // one star an iteration
 
-  auto issue = [&](int grp, int stage) {   // one bulk copy per patch of the group
-    uint32_t bytes = 0;
-    int vids[PPI];
-    for (int ps = 0; ps < PPI; ++ps) {
-      int vx, vy, vz;
-      vids[ps] = work_vertex<DIM>(g, interior, grp * PPI + ps, count, vx, vy, vz);
-      if (vids[ps] >= 0) bytes += C::STRIDE * sizeof(TS);
-    }
-    tma::mbar_expect_tx(&bars[stage], bytes);
-    for (int ps = 0; ps < PPI; ++ps)
-      if (vids[ps] >= 0)
-        tma::bulk_load(stages + stage * C::stage_elems + (size_t)ps * C::STRIDE,
-                       inv + (long long)vids[ps] * C::STRIDE, C::STRIDE * sizeof(TS), &bars[stage]);
+  auto issue = [&](int grp, int stage) {   // one bulk copy: the star's block-packed inverse
+    int vx, vy, vz;
+    const int vid = work_vertex<DIM>(g, interior, grp, count, vx, vy, vz);
+    tma::mbar_expect_tx(&bars[stage], C::STRIDE * sizeof(TS));
+    tma::bulk_load(stages + stage * C::stage_elems, inv + (long long)vid * C::STRIDE, C::STRIDE * sizeof(TS),
+                   &bars[stage]);
   };
-  auto gather = [&](int grp, float (&v)[RPT]) {
-#pragma unroll
-    for (int k = 0; k < RPT; ++k) {
-      const int e = tid + k * THREADS;
-      v[k] = 0.f;
-      if (e < PPI * NP && grp < ngroups) {
-        int vx, vy, vz;
-        const int vid = work_vertex<DIM>(g, interior, grp * PPI + e / NP, count, vx, vy, vz);
-        v[k] = patch_r<DIM>(g, r, vid, vx, vy, vz, e % NP);
-      }
-    }
-  };
-  // PPI == 1: the thread's entries all belong to the iteration's one patch
   EntryConst ec[RPT];
 #pragma unroll
-  for (int k = 0; k < RPT; ++k) ec[k] = entry_const<DIM>(g, tid + k * THREADS, PPI * NP);
+  for (int k = 0; k < RPT; ++k) ec[k] = entry_const<DIM>(g, tid + k * THREADS, NP);
   auto gather1 = [&](const PatchPos& q, float (&v)[RPT]) {
 #pragma unroll
     for (int k = 0; k < RPT; ++k) {
@@ -456,15 +579,9 @@ __device__ __forceinline__ void patch_tma_body(unsigned bx, unsigned gx, const G
   // kernel writes) may start now and run beside this one
   if (early_trigger) pdl_trigger();
   float rpre[RPT];
-  PatchPos qcur{}, qnext{};
-  if constexpr (PPI == 1) {
-    qnext = patch_pos<DIM>(g, interior, bx, count);
-    gather1(qnext, rpre);
-  } else {
-    gather(bx, rpre);
-  }
-
-  const int ps = tid / TPP, b = tid % TPP;
+  PatchPos qcur{}, qnext = patch_pos<DIM>(g, interior, bx, count);
+  gather1(qnext, rpre);
+  const int b = tid;
   int I = 0, J = 0;
   bool diag = false;
   if (b < BL.nbp) block_of(BL, b, I, J, diag);
@@ -475,36 +592,31 @@ __device__ __forceinline__ void patch_tma_body(unsigned bx, unsigned gx, const G
 #pragma unroll
     for (int k = 0; k < RPT; ++k) {
       const int e = tid + k * THREADS;
-      if (e < PPI * NP) rs[e] = rpre[k];
+      if (e < NP) rs[e] = rpre[k];
     }
     // next group's r: in flight while this one is computed
-    if constexpr (PPI == 1) {
-      qcur = qnext;
-      qnext = patch_pos<DIM>(g, interior, grp + gx, count);
-      gather1(qnext, rpre);
-    } else {
-      gather(grp + gx, rpre);
-    }
+    qcur = qnext;
+    qnext = patch_pos<DIM>(g, interior, grp + gx, count);
+    gather1(qnext, rpre);
     if (!tma::mbar_wait(&bars[stage], parity, wait_polls)) {
       if (tid == ISSUER) { report(st, 7 /* ALS_ETIMEOUT */, grp); s_fail = 1; }
     }
     __syncthreads();                        // (A) r and the stage are visible
     if (s_fail) break;
     if (b < BL.nbp) {
-      const TS* S = stages + stage * C::stage_elems + (size_t)ps * C::STRIDE;
+      const TS* S = stages + stage * C::stage_elems;
       float rI[9], rJ[9], yI[9], yJ[9];
 #pragma unroll
       for (int k = 0; k < 9; ++k) {
-        rI[k] = rs[ps * NP + 9 * I + k];
-        rJ[k] = rs[ps * NP + 9 * J + k];
+        rI[k] = rs[9 * I + k];
+        rJ[k] = rs[9 * J + k];
       }
       block_product<false, TS>(BL, S, b, diag, rI, rJ, yI, yJ);
-      float* pp = part + ps * NP * NBR;
 #pragma unroll
-      for (int k = 0; k < 9; ++k) pp[(9 * I + k) * NBR + J] = yI[k];
+      for (int k = 0; k < 9; ++k) part[(9 * I + k) * NBR + J] = yI[k];
       if (!diag) {
 #pragma unroll
-        for (int k = 0; k < 9; ++k) pp[(9 * J + k) * NBR + I] = yJ[k];
+        for (int k = 0; k < 9; ++k) part[(9 * J + k) * NBR + I] = yJ[k];
       }
     }
     __syncthreads();                        // (B) the stage is consumed, the partials are complete
@@ -516,39 +628,18 @@ __device__ __forceinline__ void patch_tma_body(unsigned bx, unsigned gx, const G
       }
     }
     // y_i = sum_J partial(i, J), fixed order
-    if constexpr (PPI == 1) {
 #pragma unroll
-      for (int k = 0; k < RPT; ++k) {
-        if (!ec[k].ok || qcur.vid < 0) continue;
-        const int i = tid + k * THREADS;
-        float acc = 0.f;
+    for (int k = 0; k < RPT; ++k) {
+      if (!ec[k].ok || qcur.vid < 0) continue;
+      const int i = tid + k * THREADS;
+      float acc = 0.f;
 #pragma unroll
-        for (int jb = 0; jb < NBR; ++jb) acc += part[i * NBR + jb];
-        if (mode == OUT_SCRATCH) {
-          out[qcur.obase + ec[k].ooff] = acc;
-        } else if (entry_in<DIM>(g, qcur, ec[k])) {
-          float* o = out + (qcur.gbase + ec[k].goff);
-          *o = mode == OUT_SUBTRACT ? *o - acc : acc;
-        }
-      }
-    } else {
-      for (int e = tid; e < PPI * NP; e += THREADS) {
-        const int p = e / NP, i = e % NP;
-        int vx, vy, vz;
-        const int v = work_vertex<DIM>(g, interior, grp * PPI + p, count, vx, vy, vz);
-        if (v < 0) continue;
-        float acc = 0.f;
-#pragma unroll
-        for (int jb = 0; jb < NBR; ++jb) acc += part[(p * NP + i) * NBR + jb];
-        if (mode == OUT_SCRATCH) {
-          out[patch_out_index<DIM>(g, vx, vy, vz, i)] = acc;
-        } else {
-          long long nd;
-          if (patch_node<DIM>(g, vx, vy, vz, i % NB, nd)) {
-            float* o = out + (i / NB) * g.N + nd;
-            *o = mode == OUT_SUBTRACT ? *o - acc : acc;
-          }
-        }
+      for (int jb = 0; jb < NBR; ++jb) acc += part[i * NBR + jb];
+      if (mode == OUT_SCRATCH) {
+        out[qcur.obase + ec[k].ooff] = acc;
+      } else if (entry_in<DIM>(g, qcur, ec[k])) {
+        float* o = out + (qcur.gbase + ec[k].goff);
+        *o = mode == OUT_SUBTRACT ? *o - acc : acc;
       }
     }
     // no third barrier: r is read only between (A) and (B) of an iteration and
@@ -566,6 +657,17 @@ __device__ __forceinline__ void patch_tma_body(unsigned bx, unsigned gx, const G
 }
 
 template <int DIM, int NST, typename TS = float>
+__device__ __forceinline__ void patch_tma_body(unsigned bx, unsigned gx, const Geom& g, const TS* __restrict__ inv,
+                                               int interior, int count, const float* __restrict__ r,
+                                               float* __restrict__ out, int mode, DevStatus* st, int wait_polls,
+                                               int early_trigger) {
+  if constexpr (DIM == 2)
+    patch_tma2_body<NST, TS>(bx, gx, g, inv, interior, count, r, out, mode, st, wait_polls, early_trigger);
+  else
+    patch_tma3_body<NST, TS>(bx, gx, g, inv, interior, count, r, out, mode, st, wait_polls, early_trigger);
+}
+
+template <int DIM, int NST, typename TS = float>
 __global__ void __launch_bounds__(64) k_patch_tma(Geom g, const TS* __restrict__ inv, int interior, int count,
                                                   const float* __restrict__ r, float* __restrict__ out, int mode,
                                                   DevStatus* st, int wait_polls, int early_trigger) {
@@ -574,85 +676,126 @@ __global__ void __launch_bounds__(64) k_patch_tma(Geom g, const TS* __restrict__
 }
 
 // ---------------------------------------------------------------------------
-// K4 (FP32), direct variant: each thread streams its 9x9 block of the
-// block-packed inverse straight from global memory with coalesced 16-byte
-// loads (thread b of a patch reads consecutive words), gathers its r_I, r_J
-// itself, and the block partials are reduced through double-buffered shared
-// memory: one barrier per iteration, 2 (3D) or 32 (2D) patches per 128-thread CTA.
+// K4 (FP32), direct variant: the inverses are read straight from global memory.  3D: one
+// thread per 9x9 block of the block-packed inverse (64 threads a star, coalesced 16-byte
+// loads), r of the CTA's stars staged in shared memory with the index arithmetic split as in
+// the TMA form (EntryConst, PatchPos), the block partials reduced through shared memory.
+// 2D: a lane per star, see above; stars are 688 bytes apart, so the lanes' 16-byte loads are
+// not coalesced and each line is fetched from L1 several times.
 // ---------------------------------------------------------------------------
 template <int DIM, typename TS = float>
 struct DirCfg {
   static constexpr int NP = Sz<DIM>::NP;
   static constexpr int THREADS = 128;
-  static constexpr int TPP = DIM == 3 ? 64 : 4;
+  static constexpr int TPP = DIM == 3 ? 64 : 2;
   static constexpr int PPC = THREADS / TPP;
   static constexpr int NBR = NP / 9;
   static constexpr int STRIDE = block_stride<TS>(NP);
+  static constexpr int RPT = 2;                      // 3D: entries per thread (81 over 64)
+  struct Smem3 {
+    float rs[PPC][NP];                               // r and block partials
+    float part[PPC][NP][NBR];
+  };
+  struct Smem2 {
+    Star2Exchange<TS> ex[THREADS / 64];
+  };
+  using Smem = typename std::conditional<DIM == 3, Smem3, Smem2>::type;
 };
 
-// r at entry 9*IB + k (k < 9) of the patch of vertex (vx, vy, vz)
-template <int DIM>
-__device__ __forceinline__ void gather9(const Geom& g, const float* __restrict__ r, int vx, int vy, int vz, int IB,
-                                        float (&out)[9]) {
-  constexpr int NB = Sz<DIM>::NB;
-#pragma unroll
-  for (int k = 0; k < 9; ++k) {
-    const int i = 9 * IB + k;
-    long long nd;
-    out[k] = patch_node<DIM>(g, vx, vy, vz, i % NB, nd) ? __ldg(r + (i / NB) * g.N + nd) : 0.f;
-  }
+// barrier of one 64-thread group of the CTA
+__device__ __forceinline__ void pair_sync(int group) {
+  asm volatile("bar.sync %0, 64;" ::"r"(1 + group) : "memory");
 }
 
 template <int DIM, typename TS = float>
 __device__ __forceinline__ void patch_direct_body(unsigned bx, unsigned gx, const Geom& g, const TS* __restrict__ inv,
                                                   int interior, int count, const float* __restrict__ r,
-                                                  float* __restrict__ out, int mode) {
+                                                  float* __restrict__ out, int mode,
+                                                  typename DirCfg<DIM, TS>::Smem& sm) {
   using C = DirCfg<DIM, TS>;
-  constexpr int NP = C::NP, NB = Sz<DIM>::NB, PPC = C::PPC, TPP = C::TPP, NBR = C::NBR;
-  constexpr BlockLayout BL = BlockLayout(NP);
-  __shared__ float part[2][PPC][NP][NBR];
-  const int tid = threadIdx.x, ps = tid / TPP, b = tid % TPP;
-  const int ngroups = (count + PPC - 1) / PPC;
-  int buf = 0;
-  int I = 0, J = 0;
-  bool diag = false;
-  if (b < BL.nbp) block_of(BL, b, I, J, diag);
+  const int tid = threadIdx.x, group = tid >> 6;
   pdl_wait();
-  for (int grp = bx; grp < ngroups; grp += gx, buf ^= 1) {
-    if (b < BL.nbp) {
-      int vx, vy, vz;
-      const int v = work_vertex<DIM>(g, interior, grp * PPC + ps, count, vx, vy, vz);
-      if (v >= 0) {
-        float rI[9], rJ[9], yI[9], yJ[9];
-        gather9<DIM>(g, r, vx, vy, vz, I, rI);
-        gather9<DIM>(g, r, vx, vy, vz, J, rJ);
-        block_product<true, TS>(BL, inv + (long long)v * C::STRIDE, b, diag, rI, rJ, yI, yJ);
+  if constexpr (DIM == 2) {
+    // the 64-thread groups of the grid walk the groups of 32 stars, a block's groups far apart
+    const int lane = tid & 31, role = (tid >> 5) & 1;
+    const int ngroups = (count + 31) / 32;
+    int it = 0;
+    for (int grp = bx + group * gx; grp < ngroups; grp += gx * (C::THREADS / 64), ++it) {
+      const PatchPos q = patch_pos<2>(g, interior, grp * 32 + lane, count);
+      float r0[9], r1[9], a[9], b[9], got[9];
+      star2_r(g, q, r, r0, r1);
+      if (q.vid >= 0) star2_products<true, TS>(inv + (long long)q.vid * C::STRIDE, role, r0, r1, a, b);
+      auto& ex = sm.ex[group].v[it & 1];
+      if (q.vid >= 0) {
 #pragma unroll
-        for (int k = 0; k < 9; ++k) part[buf][ps][9 * I + k][J] = yI[k];
+        for (int k = 0; k < 9; ++k) ex[role][k][lane] = role == 0 ? b[k] : a[k];
+      }
+      pair_sync(group);
+#pragma unroll
+      for (int k = 0; k < 9; ++k) got[k] = ex[1 - role][k][lane];
+      if (role == 0) star2_store(g, q, 0, got, a, out, mode);
+      else star2_store(g, q, 1, got, b, out, mode);
+    }
+  } else {
+    constexpr int NP = C::NP, PPC = C::PPC, TPP = C::TPP, NBR = C::NBR;
+    constexpr BlockLayout BL = BlockLayout(NP);
+    const int ps = tid / TPP, b = tid % TPP;
+    const int ngroups = (count + PPC - 1) / PPC;
+    int I = 0, J = 0;
+    bool diag = false;
+    if (b < BL.nbp) block_of(BL, b, I, J, diag);
+    EntryConst ec[C::RPT];
+#pragma unroll
+    for (int k = 0; k < C::RPT; ++k) ec[k] = entry_const<DIM>(g, b + k * TPP, NP);
+    auto gather = [&](const PatchPos& q, float (&v)[C::RPT]) {
+#pragma unroll
+      for (int k = 0; k < C::RPT; ++k) {
+        v[k] = 0.f;
+        if (ec[k].ok && q.vid >= 0 && entry_in<DIM>(g, q, ec[k])) v[k] = __ldg(r + (q.gbase + ec[k].goff));
+      }
+    };
+    float rn[C::RPT];
+    PatchPos q = patch_pos<DIM>(g, interior, bx * PPC + ps, count);
+    gather(q, rn);
+    // (r is read between the two barriers and rewritten after the second; the partials are
+    // read after the second and rewritten after the next iteration's first)
+    for (int grp = bx; grp < ngroups; grp += gx) {
+#pragma unroll
+      for (int k = 0; k < C::RPT; ++k)
+        if (ec[k].ok) sm.rs[ps][b + k * TPP] = rn[k];
+      pair_sync(group);
+      const PatchPos qn = patch_pos<DIM>(g, interior, (grp + gx) * PPC + ps, count);
+      if (b < BL.nbp && q.vid >= 0) {
+        float rI[9], rJ[9], yI[9], yJ[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+          rI[k] = sm.rs[ps][9 * I + k];
+          rJ[k] = sm.rs[ps][9 * J + k];
+        }
+        block_product<true, TS>(BL, inv + (long long)q.vid * C::STRIDE, b, diag, rI, rJ, yI, yJ);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) sm.part[ps][9 * I + k][J] = yI[k];
         if (!diag) {
 #pragma unroll
-          for (int k = 0; k < 9; ++k) part[buf][ps][9 * J + k][I] = yJ[k];
+          for (int k = 0; k < 9; ++k) sm.part[ps][9 * J + k][I] = yJ[k];
         }
       }
-    }
-    __syncthreads();
-    for (int e = tid; e < PPC * NP; e += C::THREADS) {
-      const int p = e / NP, i = e % NP;
-      int vx, vy, vz;
-      const int v = work_vertex<DIM>(g, interior, grp * PPC + p, count, vx, vy, vz);
-      if (v < 0) continue;
-      float acc = 0.f;
+      gather(qn, rn);                       // the next star's r, in flight over the reduction
+      pair_sync(group);
 #pragma unroll
-      for (int jb = 0; jb < NBR; ++jb) acc += part[buf][p][i][jb];
-      if (mode == OUT_SCRATCH) {
-        out[patch_out_index<DIM>(g, vx, vy, vz, i)] = acc;
-      } else {
-        long long nd;
-        if (patch_node<DIM>(g, vx, vy, vz, i % NB, nd)) {
-          float* o = out + (i / NB) * g.N + nd;
+      for (int k = 0; k < C::RPT; ++k) {
+        if (!ec[k].ok || q.vid < 0) continue;
+        float acc = 0.f;
+#pragma unroll
+        for (int jb = 0; jb < NBR; ++jb) acc += sm.part[ps][b + k * TPP][jb];
+        if (mode == OUT_SCRATCH) {
+          out[q.obase + ec[k].ooff] = acc;
+        } else if (entry_in<DIM>(g, q, ec[k])) {
+          float* o = out + (q.gbase + ec[k].goff);
           *o = mode == OUT_SUBTRACT ? *o - acc : acc;
         }
       }
+      q = qn;
     }
   }
 }
@@ -661,7 +804,8 @@ template <int DIM, typename TS = float>
 __global__ void __launch_bounds__(128) k_patch_direct(Geom g, const TS* __restrict__ inv, int interior, int count,
                                                       const float* __restrict__ r, float* __restrict__ out,
                                                       int mode) {
-  patch_direct_body<DIM, TS>(blockIdx.x, gridDim.x, g, inv, interior, count, r, out, mode);
+  __shared__ typename DirCfg<DIM, TS>::Smem sm;
+  patch_direct_body<DIM, TS>(blockIdx.x, gridDim.x, g, inv, interior, count, r, out, mode, sm);
 }
 
 template <int DIM>
@@ -1270,8 +1414,13 @@ __global__ void __launch_bounds__(128) k_patch_direct_b(const __grid_constant__ 
   const int i = batch_slot(tb, blockIdx.x);
   const PatchArgs& a = tb.a[i];
   const unsigned bx = blockIdx.x - tb.start[i], gx = tb.start[i + 1] - tb.start[i];
-  if (a.g.dim == 3) patch_direct_body<3>(bx, gx, a.g, a.inv, a.wl, a.count, a.r, a.out, a.mode);
-  else patch_direct_body<2>(bx, gx, a.g, a.inv, a.wl, a.count, a.r, a.out, a.mode);
+  if (a.g.dim == 3) {
+    __shared__ DirCfg<3>::Smem sm;
+    patch_direct_body<3>(bx, gx, a.g, a.inv, a.wl, a.count, a.r, a.out, a.mode, sm);
+  } else {
+    __shared__ DirCfg<2>::Smem sm;
+    patch_direct_body<2>(bx, gx, a.g, a.inv, a.wl, a.count, a.r, a.out, a.mode, sm);
+  }
 }
 __global__ void __launch_bounds__(256) k_patch_bnd_b(const __grid_constant__ BatchTab<PatchArgs> tb) {
   const int i = batch_slot(tb, blockIdx.x);
