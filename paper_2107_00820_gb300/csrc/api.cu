@@ -66,7 +66,6 @@ struct Prof {
 // fused smoother, doubles in the per-operation one
 struct SmallLayout : GmresLayout {
   explicit SmallLayout(int steps) : GmresLayout(steps) {}
-  GmresDev dev(double* base) const { return GmresDev{base, s}; }
 };
 
 }  // namespace
@@ -295,14 +294,12 @@ void smooth_fused(als_ctx* c, MGWork& w, int l, bool x_is_zero, void* t) {
   const long long len = Lv.g.N * c->dim;
   const cudaStream_t s = c->stream;
   const int steps = std::max(1, c->opt.sweeps);
-  SmallLayout sl(steps);
-  double* sm = w.small[l];
-  const GmresDev st = sl.dev(sm);
+  const GmresDev st = gmres_dev(Lv, w.small[l], steps, w.partial, x_is_zero);
   void* V0 = w.V[l];
   if (x_is_zero) {
-    gm_start(prec, len, w.b[l], V0, w.partial, st, s);                   // V0 = b
+    gm_start(prec, len, w.b[l], V0, st, s);                              // V0 = b
   } else {
-    ApplyEpi e{w.b[l], -1.0, 0, nullptr, 0, nullptr, 1, st, w.partial};
+    ApplyEpi e{w.b[l], -1.0, 0, nullptr, 0, 1, st};
     op_apply_epi(Lv, prec, c->gamma, w.x[l], V0, e, s);                  // V0 = b - A x
   }
   for (int j = 0; j < steps; ++j) {
@@ -311,19 +308,18 @@ void smooth_fused(als_ctx* c, MGWork& w, int l, bool x_is_zero, void* t) {
     void* Zj = vptr(w.Z[l], w.es, (long long)j * len);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (l == c->L - 1) prof_events(c, t_prof_counter, e0, e1);
-    ApplyEpi e{nullptr, 1.0, j + 1, w.V[l], len, vptr(sm, w.es, sl.H + (long long)j * sl.ldh), 0, st, w.partial};
+    ApplyEpi e{nullptr, 1.0, j + 1, w.V[l], len, 0, st};
     if (fuse_patch_gather(c, prec)) {
-      // patch products only; the cell kernel sums them per node into Z_j (= D^-1 v_j / h_j)
+      // patch products only; the cell kernel sums them per node into Z_j = D^-1 V_j
       patch_products(Lv, Vj, w.scratch[l], s, e0, e1);
       e.pout = w.scratch[l];
-      e.pden = vptr(sm, w.es, sl.hn + j);
     } else {
-      patch_smooth(Lv, prec, Vj, Zj, w.scratch[l], s, e0, e1, vptr(sm, w.es, sl.hn + j));  // Z_j = D^-1 v_j
+      patch_smooth(Lv, prec, Vj, Zj, w.scratch[l], s, e0, e1);            // Z_j = D^-1 V_j
     }
     cudaEvent_t a0 = nullptr, a1 = nullptr;
     if (l == c->L - 1) prof_events(c, t_prof_counter, a0, a1, 1);
-    op_apply_epi(Lv, prec, c->gamma, Zj, Vn, e, s, a0, a1);            // A Z_j, H[0..j][j]
-    gm_orth(prec, len, j, w.V[l], len, w.partial, st, s);                 // V_{j+1}, Givens step j
+    op_apply_epi(Lv, prec, c->gamma, Zj, Vn, e, s, a0, a1);            // A Z_j and its dots
+    gm_orth(prec, len, j, w.V[l], len, st, s);                            // V_{j+1}, H[0..j][j]
   }
   gm_update(prec, len, steps, w.Z[l], w.V[l], len, st, w.x[l], x_is_zero ? 1 : 0, t, s);
 }
@@ -1740,7 +1736,6 @@ void merged_smooth(MergedCycle& M, int l, bool x_is_zero, bool residual, cudaStr
   const std::vector<als_ctx*> S = at_level(M, l);
   if (S.empty()) return;
   const int steps = std::max(1, S[0]->opt.sweeps);
-  SmallLayout sl(steps);
   std::vector<BGmres> g;
   std::vector<BApply> ap;
   for (als_ctx* c : S) {
@@ -1752,14 +1747,13 @@ void merged_smooth(MergedCycle& M, int l, bool x_is_zero, bool residual, cudaStr
     it.Z = w.Z[l];
     it.V = w.V[l];
     it.ld = len;
-    it.partial = w.partial;
-    it.st = sl.dev(w.small[l]);
+    it.st = gmres_dev(c->lev[l], w.small[l], steps, w.partial, x_is_zero);
     it.x = w.x[l];
     it.x_zero = x_is_zero ? 1 : 0;
     it.t = residual ? w.t[l] : nullptr;
     g.push_back(it);
     ap.push_back(BApply{&c->lev[l], c->gamma, w.x[l], w.V[l],
-                        ApplyEpi{w.b[l], -1.0, 0, nullptr, 0, nullptr, 1, it.st, w.partial}});
+                        ApplyEpi{w.b[l], -1.0, 0, nullptr, 0, 1, it.st}});
   }
   if (x_is_zero) batch_gm_start(g, s);     // V0 = b
   else batch_apply_epi(ap, s);             // V0 = b - A x
@@ -1773,15 +1767,12 @@ void merged_smooth(MergedCycle& M, int l, bool x_is_zero, bool residual, cudaStr
       void* Vj = vptr(w.V[l], w.es, (long long)j * len);
       void* Vn = vptr(w.V[l], w.es, (long long)(j + 1) * len);
       void* Zj = vptr(w.Z[l], w.es, (long long)j * len);
-      const void* den = vptr(w.small[l], w.es, sl.hn + j);
-      prod.push_back(BPatch{&c->lev[l], Vj, w.scratch[l], nullptr, nullptr});
-      ApplyEpi e{nullptr, 1.0, j + 1, w.V[l], len, vptr(w.small[l], w.es, sl.H + (long long)j * sl.ldh), 0, g[i].st,
-                 w.partial};
+      prod.push_back(BPatch{&c->lev[l], Vj, w.scratch[l], nullptr});
+      ApplyEpi e{nullptr, 1.0, j + 1, w.V[l], len, 0, g[i].st};
       if (fuse_patch_gather(c, PREC_F32)) {
         e.pout = w.scratch[l];
-        e.pden = den;
       } else {
-        gath.push_back(BPatch{&c->lev[l], nullptr, w.scratch[l], den, Zj});
+        gath.push_back(BPatch{&c->lev[l], nullptr, w.scratch[l], Zj});
       }
       az.push_back(BApply{&c->lev[l], c->gamma, Zj, Vn, e});
       g[i].j = j;
@@ -1802,7 +1793,7 @@ void merged_restrict(MergedCycle& M, int l, cudaStream_t s) {
   const bool robust = S[0]->opt.transfer == ALS_TRANSFER_ROBUST;
   for (als_ctx* c : S) {
     MGWork& w = c->w32;
-    isv.push_back(BPatch{&c->lev[l], w.t[l], w.t2[l], nullptr, nullptr});
+    isv.push_back(BPatch{&c->lev[l], w.t[l], w.t2[l], nullptr});
     ap.push_back(BApply{&c->lev[l], c->gamma, w.t2[l], w.t3[l], ApplyEpi{}});
     tr.push_back(BTransfer{&c->lev[l - 1], &c->lev[l], w.t[l], w.b[l - 1], robust ? w.t3[l] : nullptr});
   }
@@ -1823,7 +1814,7 @@ void merged_prolong(MergedCycle& M, int l, cudaStream_t s) {
     MGWork& w = c->w32;
     tr.push_back(BTransfer{&c->lev[l - 1], &c->lev[l], w.x[l - 1], w.t[l], w.x[l]});
     ap.push_back(BApply{&c->lev[l], c->gamma, w.t[l], w.t3[l], ApplyEpi{}});
-    isv.push_back(BPatch{&c->lev[l], w.t3[l], w.x[l], nullptr, nullptr});
+    isv.push_back(BPatch{&c->lev[l], w.t3[l], w.x[l], nullptr});
   }
   batch_prolong(tr, s);                              // t = P_H x_{l-1}, x += t
   if (robust) {
@@ -1865,8 +1856,8 @@ void merged_tune(MergedCycle& M, cudaStream_t s) {
     for (als_ctx* c : at_level(M, l)) {
       MGWork& w = c->w32;
       vec_zero(PREC_F32, c->lev[l].g.N * c->dim, w.V[l], s);
-      prod.push_back(BPatch{&c->lev[l], w.V[l], w.scratch[l], nullptr, nullptr});
-      isv.push_back(BPatch{&c->lev[l], w.V[l], w.t2[l], nullptr, nullptr});
+      prod.push_back(BPatch{&c->lev[l], w.V[l], w.scratch[l], nullptr});
+      isv.push_back(BPatch{&c->lev[l], w.V[l], w.t2[l], nullptr});
     }
     for (int kind = 0; kind < 2; ++kind) {
       float best = 1e30f;

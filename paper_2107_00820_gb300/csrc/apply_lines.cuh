@@ -58,22 +58,21 @@ __device__ __forceinline__ int ofs_xy(int m, int c, int x, int y, int z) { retur
 __device__ __forceinline__ int ofs_yz(int m, int c, int x, int y, int z) { return m * 81 + c * 9 + 3 * x + y + 27 * z; }
 __device__ __forceinline__ int ofs_pt(int m, int c, int x, int y, int z) { return m * 81 + c * 27 + 3 * x + 9 * y + z; }
 
-// Input of the apply taken straight from the star-patch outputs (ZP): x = z = (sum of the
-// <= 2^d patch outputs containing each node) / den, summed in the fixed order of the patch
+// Input of the apply taken straight from the star-patch outputs (ZP): x = z = the sum of the
+// <= 2^d patch outputs containing each node, summed in the fixed order of the patch
 // gather (z tap, y tap, then the x pair), 0 at Dirichlet nodes; z is also stored, each node
 // by the one cell that owns it (the cell with the node's lower corner, the last cell for the
 // upper boundary nodes), so the separate gather launch is not needed.
 template <typename T>
 struct PatchIn {
   const T* out;   // patch outputs in the row layout (patch_out_index)
-  const T* den;   // the GMRES column norm h_j (device scalar)
   T* z;           // z written here
 };
 
 // z at the three nodes 2cx + a of the x-line (component c, y node nj, z node nk); 0 on Dirichlet rows
 template <typename T>
-__device__ __forceinline__ void patch_line(const Geom& g, const PatchIn<T>& pin, T inv_den, int c, int cx, int nj,
-                                           int nk, T (&u)[3]) {
+__device__ __forceinline__ void patch_line(const Geom& g, const PatchIn<T>& pin, int c, int cx, int nj, int nk,
+                                           T (&u)[3]) {
   u[0] = u[1] = u[2] = T(0);
   if (nj == 0 || nj == g.nn[1] - 1 || nk == 0 || nk == g.nn[2] - 1) return;
   // taps per axis: odd node 2v+1 -> vertices v (offset 2), v+1 (offset 0); even node 2v -> v (offset 1)
@@ -100,7 +99,7 @@ __device__ __forceinline__ void patch_line(const Geom& g, const PatchIn<T>& pin,
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const int ni = 2 * cx + a;
-    u[a] = (ni == 0 || ni == g.nn[0] - 1) ? T(0) : acc[a] * inv_den;
+    u[a] = (ni == 0 || ni == g.nn[0] - 1) ? T(0) : acc[a];
   }
 }
 
@@ -177,8 +176,7 @@ __device__ __forceinline__ void apply_lines_body(unsigned bx, const Geom& g, con
         const int nj = 2 * cy + b1, nk = 2 * cz + b2;
         const long long row = (long long)c * g.N + (long long)(unsigned)(g.nn[0] * (nj + g.nn[1] * nk));
         if constexpr (ZP) {
-          const T dn = pin.den[0];
-          patch_line<T>(g, pin, dn != T(0) ? T(1) / dn : T(0), c, cx, nj, nk, u);
+          patch_line<T>(g, pin, c, cx, nj, nk, u);
           // the owned nodes of the line: lower corner, or the last cell for the upper boundary
           if ((b1 < 2 || cy == g.n[1] - 1) && (b2 < 2 || cz == g.n[2] - 1)) {
 #pragma unroll

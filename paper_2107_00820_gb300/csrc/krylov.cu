@@ -200,23 +200,18 @@ void vec_scale_dev(int prec, long long n, const double* num, const double* den, 
 // ---------------------------------------------------------------------------
 // GMRES(s) smoother steps with an unnormalised stored basis (see GmresDev)
 // ---------------------------------------------------------------------------
-// Each thread handles PER entries spaced RED_THREADS apart, with all loads of
-// its entries issued before any arithmetic; the grid then has about n / (256 PER)
-// blocks, which keeps the ticket counter of the single-launch reduction cold
-// (same-address atomics serialise: several thousand blocks cost microseconds).
+// Each thread handles GM_PER entries spaced RED_THREADS apart, with all loads of
+// its entries issued before any arithmetic; the grid then has about n / 1024
+// blocks, which keeps the partials that every consumer block adds few.
 // Column loops are unrolled to KMAXB with predicates.  In FP32 the arithmetic
 // and all sums run in float, and so does the small GMRES bookkeeping (the state
 // array holds elements of the smoother's precision).
-constexpr int GM_PER = 4;
 
-// V0 = b, |b|^2 -> gmres_start
+// V0 = b, |b|^2 partials
 // (bx, nb: the block's index and the blocks of this reduction, see batch.cuh)
 template <typename T>
 __device__ __forceinline__ void gm_start_body(unsigned bx, unsigned nb, unsigned n, const T* __restrict__ b,
-                                              T* __restrict__ V0, double* __restrict__ partial, GmresDev sd) {
-  __shared__ T nrm2_s[1];
-  const GmresView<T> st = gmres_view<T>(sd);
-  T* rows = reinterpret_cast<T*>(partial + 1);
+                                              T* __restrict__ V0, const GmresDev& sd) {
   const unsigned base = bx * (RED_THREADS * GM_PER) + threadIdx.x;
   pdl_wait();
   T v[GM_PER];
@@ -233,53 +228,90 @@ __device__ __forceinline__ void gm_start_body(unsigned bx, unsigned nb, unsigned
     acc[0] += v[q] * v[q];
   }
   pdl_trigger();
-  block_partials<T, T>(acc, 1, rows + bx);
-  if (last_block(partial, nb)) {
-    finish_sums_n<T>(partial, 1, nrm2_s, nullptr, (int)nb);
-    if (threadIdx.x == 0) gmres_start(st, nrm2_s[0]);
-  }
+  store_partials<T>(sd, 1, 1, acc, bx, nb);
 }
 template <typename T>
 __global__ void __launch_bounds__(RED_THREADS) k_gm_start(unsigned n, const T* __restrict__ b, T* __restrict__ V0,
-                                                          double* __restrict__ partial, GmresDev sd) {
-  gm_start_body<T>(blockIdx.x, gridDim.x, n, b, V0, partial, sd);
+                                                          GmresDev sd) {
+  gm_start_body<T>(blockIdx.x, gridDim.x, n, b, V0, sd);
 }
 
-// Gram-Schmidt update of the new column w = V_{j+1} against columns 0..j with the
-// coefficients H[0..j][j] / hn[i], then |w|^2 -> gmres_step(j)
+// Gram-Schmidt step j: w = column j+1 holds A Z_j with Z_j = D^-1 (column j) unscaled, so
+// A D^-1 v_j = w / hn[j];  H[i][j] = (V_i . w) / (hn[i] hn[j]),
+// V_{j+1} = w / hn[j] - sum_i V_i H[i][j] / hn[i], and the partials of |V_{j+1}|^2.
+// Every block adds the partials of the dots (and of |V_j|^2, before the wait: the kernel that
+// wrote them is three launches back) for itself.  The last block is an extra one: it does the
+// one-thread bookkeeping of step j - 1 while the others work.
 template <typename T>
 __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned n, int j, const T* __restrict__ V,
-                                             long long ld, double* __restrict__ partial, GmresDev sd) {
+                                             long long ld, const GmresDev& sd) {
+  __shared__ T sh[RED_THREADS / 32][KMAXB];
   __shared__ T coef[KMAXB];
-  __shared__ T nrm2_s[1];
+  __shared__ T nrm2;
   const GmresView<T> st = gmres_view<T>(sd);
-  T* rows = reinterpret_cast<T*>(partial + 1);
-  T* w = const_cast<T*>(V) + (long long)(j + 1) * ld;
+  T acc[KMAXB];
+  const bool extra = bx == nb - 1;
   const unsigned base = bx * (RED_THREADS * GM_PER) + threadIdx.x;
+  T* w = const_cast<T*>(V) + (long long)(j + 1) * ld;
   T a[GM_PER];
   T vc[GM_PER][KMAXB];
-  // columns 0..j come from earlier kernels of the chain (complete before this launch
-  // began): read through L2 before the wait; column j+1 and H come from the predecessor
+  T hni = T(0);
+  // columns 0..j, hn and the norm partials come from earlier kernels of the chain (complete
+  // before this launch began): read through L2 before the wait; column j+1 and the dots come
+  // from the predecessor
+  if (!extra) {
 #pragma unroll
-  for (int q = 0; q < GM_PER; ++q) {
-    const unsigned i = base + q * RED_THREADS;
+    for (int q = 0; q < GM_PER; ++q) {
+      const unsigned i = base + q * RED_THREADS;
 #pragma unroll
-    for (int c = 0; c < KMAXB; ++c) vc[q][c] = (i < n && c <= j) ? __ldcg(V + (long long)c * ld + i) : T(0);
+      for (int c = 0; c < KMAXB; ++c) vc[q][c] = (i < n && c <= j) ? __ldcg(V + (long long)c * ld + i) : T(0);
+    }
+    if ((int)threadIdx.x < j) hni = __ldcg(st.hn + threadIdx.x);
   }
+  sum_rows<T>(norm_rows<T>(sd, j), norm_count(sd, j, n), 1, acc);
+  {
+    const T v = block_total<T>(acc, 1, sh);
+    if (threadIdx.x == 0) nrm2 = v;
+  }
+  __syncthreads();
+  if (extra) {
+    if (threadIdx.x == 0) {
+      if (j == 0) gmres_start(st, nrm2);
+      else gmres_step(st, j - 1, nrm2);
+    }
+    return;
+  }
+  const T hnj = sqrt(fmax(nrm2, T(0)));
+  const T inv = hnj != T(0) ? T(1) / hnj : T(0);
+  if ((int)threadIdx.x == j) hni = hnj;
   pdl_wait();
-  const T* hcol = st.H + (long long)j * st.ldh;
-  if ((int)threadIdx.x <= j)
-    coef[threadIdx.x] = st.hn[threadIdx.x] != T(0) ? hcol[threadIdx.x] / st.hn[threadIdx.x] : T(0);
 #pragma unroll
   for (int q = 0; q < GM_PER; ++q) {
     const unsigned i = base + q * RED_THREADS;
     a[q] = i < n ? w[i] : T(0);
   }
+  sum_rows<T>(dot_rows<T>(sd), sd.nbd, j + 1, acc);
+  {
+    const T v = block_total<T>(acc, j + 1, sh);
+    if ((int)threadIdx.x <= j) {
+      T h = T(0), c = T(0);
+      if (hni != T(0)) {
+        h = (v / hni) * inv;
+        c = h / hni;
+      }
+      coef[threadIdx.x] = c;
+      if (bx == 0) {
+        st.H[(long long)j * st.ldh + threadIdx.x] = h;
+        if ((int)threadIdx.x == j) st.hn[j] = hnj;
+      }
+    }
+  }
   __syncthreads();
-  T acc[KMAXB] = {T(0)};
+  acc[0] = T(0);
 #pragma unroll
   for (int q = 0; q < GM_PER; ++q) {
     const unsigned i = base + q * RED_THREADS;
+    a[q] *= inv;
 #pragma unroll
     for (int c = 0; c < KMAXB; ++c)
       if (c <= j) a[q] -= vc[q][c] * coef[c];
@@ -287,35 +319,32 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
     acc[0] += a[q] * a[q];
   }
   pdl_trigger();
-  block_partials<T, T>(acc, 1, rows + bx);
-  if (last_block(partial, nb)) {
-    finish_sums_n<T>(partial, 1, nrm2_s, nullptr, (int)nb);
-    if (threadIdx.x == 0) {
-      gmres_step(st, j, nrm2_s[0]);
-      if (j == st.m - 2) gmres_coeffs(st, j + 1);   // last step: the update's coefficients, once
-    }
-  }
+  const T v = block_total<T>(acc, 1, sh);
+  if (threadIdx.x == 0) norm_rows<T>(sd, j + 1)[bx] = v;
 }
 template <typename T>
 __global__ void __launch_bounds__(RED_THREADS) k_gm_orth(unsigned n, int j, const T* __restrict__ V, long long ld,
-                                                         double* __restrict__ partial, GmresDev sd) {
-  gm_orth_body<T>(blockIdx.x, gridDim.x, n, j, V, ld, partial, sd);
+                                                         GmresDev sd) {
+  gm_orth_body<T>(blockIdx.x, gridDim.x, n, j, V, ld, sd);
 }
 
-// x = (x_zero ? 0 : x) + sum_j Z_j y_j with y = R^-1 g, and, if t != NULL, the
+// x = (x_zero ? 0 : x) + sum_j Z_j y_j / hn[j] with y = R^-1 g, and, if t != NULL, the
 // GMRES residual  t = r0 - A Z y = sum_i u_i v_i,  u = Q^T (g[k] e_k)  from the
-// Arnoldi relation (Q = product of the Givens rotations), no operator apply.  y and
-// u were formed once by the last block of the last k_gm_orth (gmres_coeffs).
+// Arnoldi relation (Q = product of the Givens rotations), no operator apply.  Every block
+// finishes the last Givens step and forms y and u for itself, on a copy of the state.
 template <typename T>
 __device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, int k, const T* __restrict__ Z,
-                                               const T* __restrict__ V, long long ld, GmresDev sd,
+                                               const T* __restrict__ V, long long ld, const GmresDev& sd,
                                                T* __restrict__ x, int x_zero, T* __restrict__ t) {
+  __shared__ T sh[RED_THREADS / 32][KMAXB];
+  __shared__ T state[GmresLayout(KMAXB).total];
   __shared__ T y[KMAXB], u[KMAXB + 1];
-  const GmresView<T> st = gmres_view<T>(sd);
+  static_assert(GmresLayout(KMAXB).total <= RED_THREADS, "one state entry a thread");
+  const GmresView<T> st = gmres_view<T>(GmresDev{state, k});
   const unsigned base = bx * (RED_THREADS * GM_PER) + threadIdx.x;
   // Z, x and V_0..V_{k-1} come from earlier kernels of the chain (complete before this
-  // launch began): read through L2 before the wait; V_k and the coefficients come
-  // from the predecessor (the last Gram-Schmidt step)
+  // launch began): read through L2 before the wait; V_k, its norm and the last column of H
+  // come from the predecessor (the last Gram-Schmidt step)
   T zc[GM_PER][KMAXB], xa[GM_PER];
 #pragma unroll
   for (int q = 0; q < GM_PER; ++q) {
@@ -325,9 +354,21 @@ __device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, int k, c
     xa[q] = (i < n && !x_zero) ? __ldcg(x + i) : T(0);
   }
   pdl_wait();
-  // coefficients from the last k_gm_orth of the cycle (gmres_coeffs), cast to T
-  if ((int)threadIdx.x < k) y[threadIdx.x] = st.yu[threadIdx.x];
-  else if ((int)threadIdx.x <= 2 * k && t) u[threadIdx.x - k] = st.yu[threadIdx.x];
+  if ((int)threadIdx.x < GmresLayout(k).total) state[threadIdx.x] = __ldcg(static_cast<const T*>(sd.base) + threadIdx.x);
+  T acc[KMAXB];
+  sum_rows<T>(norm_rows<T>(sd, k), norm_count(sd, k, n), 1, acc);
+  const T nrm2 = block_total<T>(acc, 1, sh);   // (its barrier also publishes the state)
+  if (threadIdx.x == 0) {
+    gmres_step(st, k - 1, nrm2);
+    gmres_coeffs(st, k);
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < k) {
+    const T hn = st.hn[threadIdx.x];
+    y[threadIdx.x] = hn != T(0) ? st.yu[threadIdx.x] / hn : T(0);
+  } else if ((int)threadIdx.x <= 2 * k) {
+    u[threadIdx.x - k] = st.yu[threadIdx.x];
+  }
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < GM_PER; ++q) {
@@ -362,34 +403,35 @@ __global__ void __launch_bounds__(RED_THREADS) k_gm_update(unsigned n, int k, co
   gm_update_body<T>(blockIdx.x, n, k, Z, V, ld, sd, x, x_zero, t);
 }
 
-static unsigned full_grid(long long n) {
-  return (unsigned)((n + RED_THREADS * GM_PER - 1) / (RED_THREADS * GM_PER));
+GmresDev gmres_dev(const LevelDev& L, void* state, int steps, double* partial, bool x_is_zero) {
+  const long long n = L.g.N * L.g.dim;
+  const int nbd = apply_epi_blocks(L), nbv = gm_blocks(n);
+  return GmresDev{state, steps, partial + 1, nbd, x_is_zero ? nbv : nbd, nbd * KMAXB, nbd > nbv ? nbd : nbv};
 }
 
-void gm_start(int prec, long long n, const void* b, void* V0, double* partial, const GmresDev& st, cudaStream_t s) {
+void gm_start(int prec, long long n, const void* b, void* V0, const GmresDev& st, cudaStream_t s) {
   if (prec == PREC_F64)
-    launch_pdl(k_gm_start<double>, full_grid(n), RED_THREADS, 0, s, (unsigned)n, (const double*)b, (double*)V0, partial, st);
+    launch_pdl(k_gm_start<double>, gm_blocks(n), RED_THREADS, 0, s, (unsigned)n, (const double*)b, (double*)V0, st);
   else
-    launch_pdl(k_gm_start<float>, full_grid(n), RED_THREADS, 0, s, (unsigned)n, (const float*)b, (float*)V0, partial, st);
+    launch_pdl(k_gm_start<float>, gm_blocks(n), RED_THREADS, 0, s, (unsigned)n, (const float*)b, (float*)V0, st);
   count_launch(1);
 }
 
-void gm_orth(int prec, long long n, int j, const void* V, long long ld, double* partial, const GmresDev& st,
-             cudaStream_t s) {
+void gm_orth(int prec, long long n, int j, const void* V, long long ld, const GmresDev& st, cudaStream_t s) {
   if (prec == PREC_F64)
-    launch_pdl(k_gm_orth<double>, full_grid(n), RED_THREADS, 0, s, (unsigned)n, j, (const double*)V, ld, partial, st);
+    launch_pdl(k_gm_orth<double>, gm_blocks(n) + 1, RED_THREADS, 0, s, (unsigned)n, j, (const double*)V, ld, st);
   else
-    launch_pdl(k_gm_orth<float>, full_grid(n), RED_THREADS, 0, s, (unsigned)n, j, (const float*)V, ld, partial, st);
+    launch_pdl(k_gm_orth<float>, gm_blocks(n) + 1, RED_THREADS, 0, s, (unsigned)n, j, (const float*)V, ld, st);
   count_launch(1);
 }
 
 void gm_update(int prec, long long n, int k, const void* Z, const void* V, long long ld, const GmresDev& st,
                void* x, int x_zero, void* t, cudaStream_t s) {
   if (prec == PREC_F64)
-    launch_pdl(k_gm_update<double>, full_grid(n), RED_THREADS, 0, s, (unsigned)n, k, (const double*)Z, (const double*)V, ld,
+    launch_pdl(k_gm_update<double>, gm_blocks(n), RED_THREADS, 0, s, (unsigned)n, k, (const double*)Z, (const double*)V, ld,
                                                                st, (double*)x, x_zero, (double*)t);
   else
-    launch_pdl(k_gm_update<float>, full_grid(n), RED_THREADS, 0, s, (unsigned)n, k, (const float*)Z, (const float*)V, ld,
+    launch_pdl(k_gm_update<float>, gm_blocks(n), RED_THREADS, 0, s, (unsigned)n, k, (const float*)Z, (const float*)V, ld,
                                                               st, (float*)x, x_zero, (float*)t);
   count_launch(1);
 }
@@ -404,7 +446,6 @@ struct GmArgs {
   const float* Z;
   float* V;
   long long ld;
-  double* partial;
   GmresDev st;
   float* x;
   int x_zero;
@@ -414,12 +455,12 @@ struct GmArgs {
 __global__ void __launch_bounds__(RED_THREADS) k_gm_start_b(const __grid_constant__ BatchTab<GmArgs> tb) {
   const int i = batch_slot(tb, blockIdx.x);
   const GmArgs& a = tb.a[i];
-  gm_start_body<float>(blockIdx.x - tb.start[i], tb.start[i + 1] - tb.start[i], a.n, a.b, a.V, a.partial, a.st);
+  gm_start_body<float>(blockIdx.x - tb.start[i], tb.start[i + 1] - tb.start[i], a.n, a.b, a.V, a.st);
 }
 __global__ void __launch_bounds__(RED_THREADS) k_gm_orth_b(const __grid_constant__ BatchTab<GmArgs> tb) {
   const int i = batch_slot(tb, blockIdx.x);
   const GmArgs& a = tb.a[i];
-  gm_orth_body<float>(blockIdx.x - tb.start[i], tb.start[i + 1] - tb.start[i], a.n, a.j, a.V, a.ld, a.partial, a.st);
+  gm_orth_body<float>(blockIdx.x - tb.start[i], tb.start[i + 1] - tb.start[i], a.n, a.j, a.V, a.ld, a.st);
 }
 __global__ void __launch_bounds__(RED_THREADS) k_gm_update_b(const __grid_constant__ BatchTab<GmArgs> tb) {
   const int i = batch_slot(tb, blockIdx.x);
@@ -442,21 +483,20 @@ __global__ void __launch_bounds__(256) k_zero_b(const __grid_constant__ BatchTab
   pdl_trigger();
 }
 
-static int batch_gm(void (*k)(BatchTab<GmArgs>), const std::vector<BGmres>& items, cudaStream_t s) {
+static int batch_gm(void (*k)(BatchTab<GmArgs>), const std::vector<BGmres>& items, int extra, cudaStream_t s) {
   std::vector<GmArgs> a;
   std::vector<unsigned> nb;
   for (const BGmres& it : items) {
-    a.push_back(GmArgs{(unsigned)it.n, it.j, (const float*)it.b, (const float*)it.Z, (float*)it.V, it.ld, it.partial,
-                       it.st, (float*)it.x, it.x_zero, (float*)it.t});
-    nb.push_back(full_grid(it.n));
+    a.push_back(GmArgs{(unsigned)it.n, it.j, (const float*)it.b, (const float*)it.Z, (float*)it.V, it.ld, it.st, (float*)it.x, it.x_zero, (float*)it.t});
+    nb.push_back(gm_blocks(it.n) + extra);
   }
   const int n = launch_batch(k, a, nb, RED_THREADS, 0, s);
   count_launch(n);
   return n;
 }
-int batch_gm_start(const std::vector<BGmres>& items, cudaStream_t s) { return batch_gm(k_gm_start_b, items, s); }
-int batch_gm_orth(const std::vector<BGmres>& items, cudaStream_t s) { return batch_gm(k_gm_orth_b, items, s); }
-int batch_gm_update(const std::vector<BGmres>& items, cudaStream_t s) { return batch_gm(k_gm_update_b, items, s); }
+int batch_gm_start(const std::vector<BGmres>& items, cudaStream_t s) { return batch_gm(k_gm_start_b, items, 0, s); }
+int batch_gm_orth(const std::vector<BGmres>& items, cudaStream_t s) { return batch_gm(k_gm_orth_b, items, 1, s); }
+int batch_gm_update(const std::vector<BGmres>& items, cudaStream_t s) { return batch_gm(k_gm_update_b, items, 0, s); }
 
 int batch_zero(const std::vector<BZero>& items, cudaStream_t s) {
   std::vector<ZeroArgs> a;
@@ -470,9 +510,10 @@ int batch_zero(const std::vector<BZero>& items, cudaStream_t s) {
   return n;
 }
 
-// workspace of the smoother's fused reductions: one partial row of KMAXB per block
+// workspace of the smoother's fused reductions: KMAXB + 2 rows of one value per block (the
+// gathers have at most 0.4 n / 256 + 1 blocks: four nodes a thread, rows of at least five nodes)
 size_t gmres_partial_doubles(long long n) {
-  return (size_t)((n + RED_THREADS - 1) / RED_THREADS) * KMAXB + 1;   // covers every grid used
+  return (size_t)((n + 511) / 512 + 1) * (KMAXB + 2) + 1;
 }
 
 // ---------------------------------------------------------------------------

@@ -71,28 +71,25 @@ void op_apply(const LevelDev& L, int prec, int mode, double gamma, const void* x
               const void* p_in, void* p_out, cudaStream_t s);
 // A_gamma apply (viscous + AL) fused with the reduction that consumes y:
 //   y = b + sigma A x (b NULL: y = sigma A x);
-//   start = 0: out[j] = (V_j . y) / hn[j] for j < k (k <= KMAXB; Arnoldi dots)
-//   start = 1: |y|^2 starts the GMRES cycle st
-// out and the GMRES state hold elements of the apply's precision.
+//   start = 0: block partials of the Arnoldi dots V_j . y, j < k (k <= KMAXB)
+//   start = 1: block partials of |y|^2, which starts the GMRES cycle st
 struct ApplyEpi {
   const void* b;
   double sigma;
   int k;
   const void* V;
   long long ld;
-  void* out;
   int start;
   GmresDev st;
-  double* partial;
   // FP32, 3D: when pout is set, the apply's input x is not read but formed from the
-  // star-patch outputs pout (row layout) divided by the device scalar pden, and stored
-  // into x (the patch gather fused into the cell kernel)
+  // star-patch outputs pout (row layout) and stored into x (the patch gather fused into
+  // the cell kernel)
   const void* pout = nullptr;
-  const void* pden = nullptr;
 };
 // e0/e1 (optional) are recorded immediately before and after the cell kernel
 void op_apply_epi(const LevelDev& L, int prec, double gamma, const void* x, void* y, const ApplyEpi& e,
                   cudaStream_t s, cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr);
+int apply_epi_blocks(const LevelDev& L);   // blocks of its reduction
 void op_load_vector(const LevelDev& L, const double* f_qp, double* F, cudaStream_t s);
 void op_apply_multi(const LevelDev& L, double gamma, const double* X, double* Y, int nvec,
                     long long stride, cudaStream_t s);
@@ -109,9 +106,8 @@ int block_stride_bf16(int np);
 // the setup calls it, and so does the loading of caller-supplied FP64 inverses
 void patch_derive32(const LevelDev& L, cudaStream_t s);
 // e0/e1 (optional) are recorded immediately before and after the patch kernel
-// den (optional device scalar of precision prec): z = D^-1 r / den (0 where den == 0)
 void patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, cudaStream_t s,
-                  cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr, const void* den = nullptr);
+                  cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr);
 size_t patch_scratch_bytes(const LevelDev& L, int prec);
 // FP32: the star-patch products y_v = A_v^-1 r|_v into the scratch rows only (their
 // node sums are formed by the consumer, see ApplyEpi::pout)
@@ -129,6 +125,14 @@ void patch_interior_solve(const LevelDev& fine, int prec, const void* in, void* 
 // operator.cu, patches.cu, transfer.cu and coarse.cu call these when L.k == 3, and they
 // pass 3D levels on to qk3.cu's qk3_* functions of the same arguments
 void qk_tables();
+// entries per thread and blocks of the order-3 gathers with a reduction: one entry a thread
+// (latency) until the grid fills the GPU four times over, then kEpiPer
+constexpr int kEpiPer = 4;
+inline int qk_epi_per(const LevelDev& L) { return L.g.N * L.g.dim > 608LL * RED_THREADS ? kEpiPer : 1; }
+inline int qk_epi_blocks(const LevelDev& L) {
+  const long long per = (long long)RED_THREADS * qk_epi_per(L);
+  return (int)((L.g.N * L.g.dim + per - 1) / per);
+}
 void qk_apply(const LevelDev& L, int prec, int mode, double gamma, const void* x, void* y, const void* p_in, void* p_out,
               cudaStream_t s);
 void qk_load_vector(const LevelDev& L, const double* f_qp, double* F, cudaStream_t s);
@@ -145,8 +149,7 @@ void qk_patch_setup(const LevelDev& L, double gamma, DevStatus* st, cudaStream_t
 // inv32 formed from inv64
 size_t qk_star32_floats(int dim);
 void qk_derive32(const LevelDev& L, cudaStream_t s);
-void qk_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, const void* den,
-                     cudaStream_t s);
+void qk_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, cudaStream_t s);
 void qk_interior_solve(const LevelDev& fine, int prec, const void* in, void* out, int subtract, cudaStream_t s);
 void qk_prolong(const LevelDev& coarse, const LevelDev& fine, int prec, const void* xc, void* xf, cudaStream_t s,
                 void* xadd);
@@ -171,8 +174,7 @@ size_t qk3_star32_floats();
 void qk3_derive32(const LevelDev& L, cudaStream_t s);
 // df64: the elimination in double-float arithmetic (the assembly stays FP64)
 void qk3_patch_setup(const LevelDev& L, double gamma, DevStatus* st, cudaStream_t s, int df64);
-void qk3_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, const void* den,
-                      cudaStream_t s);
+void qk3_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, cudaStream_t s);
 void qk3_interior_solve(const LevelDev& fine, int prec, const void* in, void* out, int subtract, cudaStream_t s);
 void qk3_prolong(const LevelDev& coarse, const LevelDev& fine, int prec, const void* xc, void* xf, cudaStream_t s,
                  void* xadd);
@@ -215,9 +217,10 @@ void vec_multiaxpy_norm(int prec, long long n, int k, const void* V, long long l
 // orthogonalise column j+1 and take the Givens step j; x (+)= Z y and, if t, the
 // GMRES residual t = r0 - A Z y from the Arnoldi relation.  s <= KMAXB.
 size_t gmres_partial_doubles(long long n);   // workspace of op_apply_epi and gm_* for n entries
-void gm_start(int prec, long long n, const void* b, void* V0, double* partial, const GmresDev& st, cudaStream_t s);
-void gm_orth(int prec, long long n, int j, const void* V, long long ld, double* partial, const GmresDev& st,
-             cudaStream_t s);
+// a smoothing's state on level L: state array, partials (workspace above), from x = 0 or not
+GmresDev gmres_dev(const LevelDev& L, void* state, int steps, double* partial, bool x_is_zero);
+void gm_start(int prec, long long n, const void* b, void* V0, const GmresDev& st, cudaStream_t s);
+void gm_orth(int prec, long long n, int j, const void* V, long long ld, const GmresDev& st, cudaStream_t s);
 void gm_update(int prec, long long n, int k, const void* Z, const void* V, long long ld, const GmresDev& st,
                void* x, int x_zero, void* t, cudaStream_t s);
 size_t multidot_partial_doubles(int k);
@@ -240,7 +243,6 @@ struct BPatch {            // star products of the smoother (r -> scratch rows),
   const LevelDev* L;       // solves on the coarse-cell interiors (r = in, out)
   const void* r;
   void* out;
-  const void* den;         // the gather's divisor (batch_patch_gather), may be NULL
   void* z;                 // the gather's output (batch_patch_gather)
 };
 // variant: the patch-kernel variant of patch_autotune (0 = TMA ring, 2 stages; 1 = 3 stages;
@@ -264,7 +266,6 @@ struct BGmres {            // gm_start (b, V), gm_orth (V, j), gm_update (Z, V, 
   void* V;
   long long ld;
   int j;
-  double* partial;
   GmresDev st;
   void* x;
   int x_zero;

@@ -525,19 +525,14 @@ static unsigned gather_threads(const Geom& g) {
 }
 
 // Gather fused with the reduction that consumes the result:
-//   y = b + sigma A x (b NULL: y = sigma A x);  out[j] = (V_j . y) / hn[j], j < k;
-//   start: |y|^2 starts a GMRES cycle.  Fixed grid and order: reproducible.
+//   y = b + sigma A x (b NULL: y = sigma A x);  block partials of V_j . y, j < k, or, start,
+//   of |y|^2.  Fixed grid and order: reproducible.
 // All sums run in T (in FP32 the GMRES state is float too, see GmresView).
 template <typename T, int DIM>
 __device__ __forceinline__ void gather_epi_body(unsigned bx, unsigned nb, const Geom& g, const T* __restrict__ ebuf,
                                                 const T* __restrict__ x, T* __restrict__ y, const T* __restrict__ b,
                                                 double sigma, int k, const T* __restrict__ V, long long ld,
-                                                T* __restrict__ out, int start, GmresDev sd,
-                                                double* __restrict__ partial) {
-  __shared__ T nrm2_s[1];
-  const GmresView<T> st = gmres_view<T>(sd);
-  T* rows = reinterpret_cast<T*>(partial + 1);
-  const int kk = start ? 1 : k;
+                                                int start, const GmresDev& sd) {
   T acc[KMAXB];
 #pragma unroll
   for (int j = 0; j < KMAXB; ++j) acc[j] = T(0);
@@ -573,24 +568,15 @@ __device__ __forceinline__ void gather_epi_body(unsigned bx, unsigned nb, const 
     }
   }
   pdl_trigger();
-  block_partials<T, T>(acc, kk, rows + (long long)bx * kk);
-  if (last_block(partial, nb)) {
-    if (start) {
-      finish_sums_n<T>(partial, 1, nrm2_s, nullptr, (int)nb);
-      if (threadIdx.x == 0) gmres_start(st, nrm2_s[0]);
-    } else {
-      finish_sums_n<T>(partial, k, out, st.hn, (int)nb);
-    }
-  }
+  store_partials<T>(sd, start, k, acc, bx, nb);
 }
 template <typename T, int DIM>
 __global__ void __launch_bounds__(RED_THREADS) k_gather_epi(Geom g, const T* __restrict__ ebuf,
                                                             const T* __restrict__ x, T* __restrict__ y,
                                                             const T* __restrict__ b, double sigma, int k,
-                                                            const T* __restrict__ V, long long ld,
-                                                            T* __restrict__ out, int start, GmresDev sd,
-                                                            double* __restrict__ partial) {
-  gather_epi_body<T, DIM>(blockIdx.x, gridDim.x, g, ebuf, x, y, b, sigma, k, V, ld, out, start, sd, partial);
+                                                            const T* __restrict__ V, long long ld, int start,
+                                                            GmresDev sd) {
+  gather_epi_body<T, DIM>(blockIdx.x, gridDim.x, g, ebuf, x, y, b, sigma, k, V, ld, start, sd);
 }
 
 #include "apply_lines.cuh"
@@ -732,7 +718,7 @@ static void launch_apply_epi(const LevelDev& L, double gamma, const void* x, voi
     if (e.pout) {   // x = z formed from the patch outputs; z stored on the way
       launch_cells<T, DIM, TENSOR, OP_VISC | OP_AL, true, true>(
           grid, s, g, col, cell_const<T>(g, gamma), nullptr, (T*)y, coef, nullptr, nullptr, 0, (T*)L.ebuf, winv,
-          PatchIn<T>{(const T*)e.pout, (const T*)e.pden, (T*)x});
+          PatchIn<T>{(const T*)e.pout, (T*)x});
       fused = true;
     }
   }
@@ -740,10 +726,13 @@ static void launch_apply_epi(const LevelDev& L, double gamma, const void* x, voi
     launch_cells<T, DIM, TENSOR, OP_VISC | OP_AL, true>(grid, s, g, col, cell_const<T>(g, gamma), (const T*)x, (T*)y,
                                                          coef, nullptr, nullptr, 0, (T*)L.ebuf, winv);
   if (e1) cudaEventRecordWithFlags(e1, s, cudaEventRecordExternal);
-  launch_pdl(k_gather_epi<T, DIM>, (gather_threads(g) + RED_THREADS - 1) / RED_THREADS, RED_THREADS, 0, s, g,
-             (const T*)L.ebuf, (const T*)x, (T*)y, (const T*)e.b, e.sigma, e.k, (const T*)e.V, e.ld, (T*)e.out,
-             e.start, e.st, e.partial);
+  launch_pdl(k_gather_epi<T, DIM>, apply_epi_blocks(L), RED_THREADS, 0, s, g, (const T*)L.ebuf, (const T*)x, (T*)y,
+             (const T*)e.b, e.sigma, e.k, (const T*)e.V, e.ld, e.start, e.st);
   count_launch(2);
+}
+
+int apply_epi_blocks(const LevelDev& L) {
+  return L.k == 3 ? qk_epi_blocks(L) : (int)((gather_threads(L.g) + RED_THREADS - 1) / RED_THREADS);
 }
 
 void op_apply_epi(const LevelDev& L, int prec, double gamma, const void* x, void* y, const ApplyEpi& e,
@@ -811,20 +800,16 @@ struct GatherArgs {
   int k, start, keep_bnd;
   const float* V;
   long long ld;
-  float* out;
   GmresDev st;
-  double* partial;
 };
 __global__ void __launch_bounds__(RED_THREADS) k_gather_epi_b(const __grid_constant__ BatchTab<GatherArgs> tb) {
   const int i = batch_slot(tb, blockIdx.x);
   const GatherArgs& a = tb.a[i];
   const unsigned bx = blockIdx.x - tb.start[i], nb = tb.start[i + 1] - tb.start[i];
   if (a.g.dim == 3)
-    gather_epi_body<float, 3>(bx, nb, a.g, a.ebuf, a.x, a.y, a.b, a.sigma, a.k, a.V, a.ld, a.out, a.start, a.st,
-                              a.partial);
+    gather_epi_body<float, 3>(bx, nb, a.g, a.ebuf, a.x, a.y, a.b, a.sigma, a.k, a.V, a.ld, a.start, a.st);
   else
-    gather_epi_body<float, 2>(bx, nb, a.g, a.ebuf, a.x, a.y, a.b, a.sigma, a.k, a.V, a.ld, a.out, a.start, a.st,
-                              a.partial);
+    gather_epi_body<float, 2>(bx, nb, a.g, a.ebuf, a.x, a.y, a.b, a.sigma, a.k, a.V, a.ld, a.start, a.st);
 }
 __global__ void __launch_bounds__(256) k_gather_cells_b(const __grid_constant__ BatchTab<GatherArgs> tb) {
   const int i = batch_slot(tb, blockIdx.x);
@@ -845,7 +830,7 @@ static CellArgs cell_args(const BApply& it, bool zp) {
   a.coef = L.coef32;
   a.ebuf = (float*)L.ebuf;
   a.winv = L.winv32;
-  if (zp) a.pin = PatchIn<float>{(const float*)it.e.pout, (const float*)it.e.pden, (float*)it.x};
+  if (zp) a.pin = PatchIn<float>{(const float*)it.e.pout, (float*)it.x};
   return a;
 }
 static unsigned cell_blocks(const Geom& g) {
@@ -879,9 +864,8 @@ int batch_apply_epi(const std::vector<BApply>& items, cudaStream_t s) {
   for (const BApply& it : items) {
     const LevelDev& L = *it.L;
     a.push_back(GatherArgs{L.g, (const float*)L.ebuf, (const float*)it.x, (float*)it.y, (const float*)it.e.b,
-                           it.e.sigma, it.e.k, it.e.start, 1, (const float*)it.e.V, it.e.ld, (float*)it.e.out,
-                           it.e.st, it.e.partial});
-    nb.push_back((gather_threads(L.g) + RED_THREADS - 1) / RED_THREADS);
+                           it.e.sigma, it.e.k, it.e.start, 1, (const float*)it.e.V, it.e.ld, it.e.st});
+    nb.push_back(apply_epi_blocks(L));
   }
   n += launch_batch(k_gather_epi_b, a, nb, RED_THREADS, 0, s);
   count_launch(n);

@@ -1175,16 +1175,11 @@ __global__ void __launch_bounds__(256) k_patch_apply(Geom g, const TF* __restric
 // stars contain each node (row layout, patch_out_index): per (y, z) tap pair the
 // chunk x = 4j .. 4j+3 reads the six contiguous columns 6j+1 .. 6j+6 (node 4j:
 // first; 4j+1: second and third; 4j+2: fourth; 4j+3: fifth and sixth).  Fixed
-// order; Dirichlet nodes get 0; divided by den[0] when den is given.
+// order; Dirichlet nodes get 0.
 template <typename TV, int DIM>
 __device__ __forceinline__ void patch_gather_body(unsigned bx, const Geom& g, const TV* __restrict__ out,
-                                                  TV* __restrict__ z, const TV* __restrict__ den) {
-  __shared__ TV inv_den;
+                                                  TV* __restrict__ z) {
   pdl_wait();
-  if (den) {                        // one division per block, not per entry
-    if (threadIdx.x == 0) inv_den = den[0] != TV(0) ? TV(1) / den[0] : TV(0);
-    __syncthreads();
-  }
   RowChunk rc;
   if (!row_chunk(g, DIM, bx * blockDim.x + threadIdx.x, rc)) return;
   const int nn0 = g.nn[0];
@@ -1231,15 +1226,13 @@ __device__ __forceinline__ void patch_gather_body(unsigned bx, const Geom& g, co
     const int xi = GX * rc.j + q;
     if (xi >= nn0) break;
     TV vq = (row_bnd || xi == 0 || xi == nn0 - 1) ? TV(0) : acc[q];
-    if (den) vq *= inv_den;
     z[rc.t0 + q] = vq;
   }
 }
 
 template <typename TV, int DIM>
-__global__ void k_patch_gather(Geom g, const TV* __restrict__ out, TV* __restrict__ z,
-                               const TV* __restrict__ den) {
-  patch_gather_body<TV, DIM>(blockIdx.x, g, out, z, den);
+__global__ void k_patch_gather(Geom g, const TV* __restrict__ out, TV* __restrict__ z) {
+  patch_gather_body<TV, DIM>(blockIdx.x, g, out, z);
 }
 
 static unsigned row_gather_blocks(const Geom& g, int dim) {
@@ -1253,15 +1246,14 @@ size_t patch_scratch_bytes(const LevelDev& L, int prec) {
 
 template <typename TF, typename TV, int DIM>
 static void smooth_impl(const LevelDev& L, const TF* inv, const void* r, void* z, void* scratch, cudaStream_t s,
-                        cudaEvent_t e0, cudaEvent_t e1, const void* den) {
+                        cudaEvent_t e0, cudaEvent_t e1) {
   const long long warps = L.g.nverts;
   const unsigned blocks = (unsigned)std::min<long long>((warps + 7) / 8, 152LL * 16);
   // External records become event-record nodes when the stream is being captured
   if (e0) cudaEventRecordWithFlags(e0, s, cudaEventRecordExternal);
   launch_pdl(k_patch_apply<TF, TV, DIM>, blocks, 256, 0, s, L.g, inv, L.pstride, (const TV*)r, (TV*)scratch);
   if (e1) cudaEventRecordWithFlags(e1, s, cudaEventRecordExternal);
-  launch_pdl(k_patch_gather<TV, DIM>, row_gather_blocks(L.g, DIM), 256, 0, s, L.g, (const TV*)scratch, (TV*)z,
-             (const TV*)den);
+  launch_pdl(k_patch_gather<TV, DIM>, row_gather_blocks(L.g, DIM), 256, 0, s, L.g, (const TV*)scratch, (TV*)z);
   count_launch(2);
 }
 
@@ -1279,10 +1271,10 @@ static void star_products(int v, const LevelDev& L, const float* r, float* scrat
 
 template <int DIM>
 static void smooth_tma(const LevelDev& L, const void* r, void* z, void* scratch, cudaStream_t s, cudaEvent_t e0,
-                       cudaEvent_t e1, const void* den) {
+                       cudaEvent_t e1) {
   star_products<DIM>(patch_variant(L), L, (const float*)r, (float*)scratch, s, e0, e1);
   launch_pdl(k_patch_gather<float, DIM>, row_gather_blocks(L.g, DIM), 256, 0, s, L.g, (const float*)scratch,
-             (float*)z, (const float*)den);
+             (float*)z);
   count_launch(1);
 }
 
@@ -1293,19 +1285,19 @@ void patch_products(const LevelDev& L, const void* r, void* scratch, cudaStream_
 }
 
 void patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, cudaStream_t s,
-                  cudaEvent_t e0, cudaEvent_t e1, const void* den) {
+                  cudaEvent_t e0, cudaEvent_t e1) {
   if (L.k == 3) {
     if (e0) cudaEventRecordWithFlags(e0, s, cudaEventRecordExternal);
-    qk_patch_smooth(L, prec, r, z, scratch, den, s);
+    qk_patch_smooth(L, prec, r, z, scratch, s);
     if (e1) cudaEventRecordWithFlags(e1, s, cudaEventRecordExternal);
     return;
   }
   if (prec == PREC_F64) {
-    if (L.g.dim == 2) smooth_impl<double, double, 2>(L, L.inv64, r, z, scratch, s, e0, e1, den);
-    else smooth_impl<double, double, 3>(L, L.inv64, r, z, scratch, s, e0, e1, den);
+    if (L.g.dim == 2) smooth_impl<double, double, 2>(L, L.inv64, r, z, scratch, s, e0, e1);
+    else smooth_impl<double, double, 3>(L, L.inv64, r, z, scratch, s, e0, e1);
   } else {
-    if (L.g.dim == 2) smooth_tma<2>(L, r, z, scratch, s, e0, e1, den);
-    else smooth_tma<3>(L, r, z, scratch, s, e0, e1, den);
+    if (L.g.dim == 2) smooth_tma<2>(L, r, z, scratch, s, e0, e1);
+    else smooth_tma<3>(L, r, z, scratch, s, e0, e1);
   }
 }
 
@@ -1398,8 +1390,6 @@ struct PatchArgs {
   const int* bvid;
   const long long* boff;
   long long nb;
-  // gather
-  const float* den;
 };
 
 template <int NST>
@@ -1433,8 +1423,8 @@ __global__ void __launch_bounds__(256) k_patch_gather_b(const __grid_constant__ 
   const int i = batch_slot(tb, blockIdx.x);
   const PatchArgs& a = tb.a[i];
   const unsigned bx = blockIdx.x - tb.start[i];
-  if (a.g.dim == 3) patch_gather_body<float, 3>(bx, a.g, a.r, a.out, a.den);
-  else patch_gather_body<float, 2>(bx, a.g, a.r, a.out, a.den);
+  if (a.g.dim == 3) patch_gather_body<float, 3>(bx, a.g, a.r, a.out);
+  else patch_gather_body<float, 2>(bx, a.g, a.r, a.out);
 }
 
 template <int NST>
@@ -1549,7 +1539,6 @@ int batch_patch_gather(const std::vector<BPatch>& items, cudaStream_t s) {
     x.g = it.L->g;
     x.r = (const float*)it.out;   // the scratch rows of the star products
     x.out = (float*)it.z;
-    x.den = (const float*)it.den;
     a.push_back(x);
     nb.push_back(row_gather_blocks(it.L->g, it.L->g.dim));
   }

@@ -19,6 +19,7 @@
 #include "cell.cuh"
 #include "krylov.h"
 #include "level.h"
+#include "pdl.cuh"
 #include "qk_tables.h"
 
 namespace als {
@@ -234,74 +235,86 @@ __device__ __forceinline__ int cells_of(int i, int n, int (&c)[2], int (&a)[2]) 
   return m;
 }
 
+// the cells containing lattice index i along an axis of n cells, two taps in a fixed order:
+// (c - 1, local K) where i is the cell corner between c - 1 and c, then (c, i - K c)
+struct CellTaps {
+  int c[2], a[2];
+  bool ok[2];
+  __device__ __forceinline__ CellTaps(int i, int n) {
+    const int c0 = i / K, r = i - K * c0;
+    c[0] = c0 - 1; a[0] = K; ok[0] = r == 0 && c0 > 0;
+    c[1] = c0; a[1] = r; ok[1] = c0 < n;
+  }
+};
+
 // y(node) = sum of the staged cell outputs of the cells containing it, fixed order;
-// keep_bnd: y = x at Dirichlet nodes; raw: no Dirichlet treatment
+// keep_bnd: y = x at Dirichlet nodes; raw: no Dirichlet treatment.  32-bit indices (the
+// per-cell outputs stay below 2^31 entries) and predicated taps, so that all loads issue at once.
 template <typename T>
 __device__ __forceinline__ T qk_gather_value(const Geom& g, const T* __restrict__ ebuf, const T* __restrict__ x,
-                                             long long t, int keep_bnd, int raw) {
-  const int comp = (int)(t / g.N);
-  const long long nd = t - comp * g.N;
-  const int i = (int)(nd % g.nn[0]), j = (int)(nd / g.nn[0]);
+                                             unsigned t, int keep_bnd, int raw) {
+  const unsigned N = (unsigned)g.N, nx = (unsigned)g.nn[0];
+  const int comp = (int)(t / N);
+  const unsigned nd = t - comp * N;
+  const int j = (int)(nd / nx), i = (int)(nd - j * nx);
   const bool bnd = i == 0 || i == g.nn[0] - 1 || j == 0 || j == g.nn[1] - 1;
   if (bnd && !raw) return keep_bnd ? x[t] : T(0);
-  int cxs[2], axs[2], cys[2], ays[2];
-  const int mx = cells_of(i, g.n[0], cxs, axs), my = cells_of(j, g.n[1], cys, ays);
-  T acc = T(0);
-  for (int b = 0; b < my; ++b)
-    for (int a = 0; a < mx; ++a) {
-      const long long cell = (long long)cxs[a] + (long long)g.n[0] * cys[b];
-      acc += ebuf[(cell * 2 + comp) * NB + axs[a] + N1 * ays[b]];
+  const CellTaps tx(i, g.n[0]), ty(j, g.n[1]);
+  T v[2][2];
+#pragma unroll
+  for (int b = 0; b < 2; ++b)
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      const int cell = tx.c[a] + g.n[0] * ty.c[b];
+      v[b][a] = tx.ok[a] && ty.ok[b] ? ebuf[(cell * 2 + comp) * NB + tx.a[a] + N1 * ty.a[b]] : T(0);
     }
-  return acc;
+  return ((v[0][0] + v[0][1]) + v[1][0]) + v[1][1];
 }
 
 template <typename T>
 __global__ void k_qk_gather(Geom g, const T* __restrict__ ebuf, const T* __restrict__ x, T* __restrict__ y, int keep_bnd,
                             int raw) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 2 * g.N) return;
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= 2u * (unsigned)g.N) return;
   y[t] = qk_gather_value<T>(g, ebuf, x, t, keep_bnd, raw);
 }
 
 // The gather fused with the reduction that consumes its result, as for order 2 (the
 // GMRES smoother's Arnoldi step): y = b + sigma A x (b NULL: sigma A x; Dirichlet rows of
-// A x are x, the identity);  start = 0: out[j] = (V_j . y) / hn[j], j < k;  start = 1:
-// |y|^2 starts the GMRES cycle.  Block partials in a fixed order: reproducible.
-template <typename T>
+// A x are x, the identity);  block partials of V_j . y, j < k, or, start = 1, of |y|^2.
+// PER entries a thread, 256 apart: large levels take kEpiPer, which keeps the partials that
+// every block of the Gram-Schmidt kernel adds at about a thousand.
+template <typename T, int PER>
 __global__ void __launch_bounds__(RED_THREADS) k_qk_gather_epi(Geom g, const T* __restrict__ ebuf,
                                                                const T* __restrict__ x, T* __restrict__ y,
                                                                const T* __restrict__ b, double sigma, int k,
-                                                               const T* __restrict__ V, long long ld,
-                                                               T* __restrict__ out, int start, GmresDev sd,
-                                                               double* __restrict__ partial) {
-  __shared__ T nrm2_s[1];
-  const GmresView<T> st = gmres_view<T>(sd);
-  T* rows = reinterpret_cast<T*>(partial + 1);
-  const int kk = start ? 1 : k;
+                                                               const T* __restrict__ V, long long ld, int start,
+                                                               GmresDev sd) {
   T acc[KMAXB];
 #pragma unroll
   for (int jj = 0; jj < KMAXB; ++jj) acc[jj] = T(0);
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < 2 * g.N) {
-    const T v = (b ? b[t] : T(0)) + (T)sigma * qk_gather_value<T>(g, ebuf, x, t, 1, 0);
-    y[t] = v;
+  const unsigned n = 2 * (unsigned)g.N, t0 = blockIdx.x * (RED_THREADS * PER) + threadIdx.x;
+  pdl_wait();
+  T v[PER];
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const unsigned t = t0 + q * RED_THREADS;
+    v[q] = t < n ? (b ? b[t] : T(0)) + (T)sigma * qk_gather_value<T>(g, ebuf, x, t, 1, 0) : T(0);
+  }
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const unsigned t = t0 + q * RED_THREADS;
+    if (t < n) y[t] = v[q];
     if (start) {
-      acc[0] = v * v;
+      acc[0] += v[q] * v[q];
     } else {
 #pragma unroll
       for (int jj = 0; jj < KMAXB; ++jj)
-        if (jj < k) acc[jj] = V[(long long)jj * ld + t] * v;
+        if (jj < k && t < n) acc[jj] += __ldcg(V + (long long)jj * ld + t) * v[q];
     }
   }
-  block_partials<T, T>(acc, kk, rows + (long long)blockIdx.x * kk);
-  if (last_block(partial)) {
-    if (start) {
-      finish_sums<T>(partial, 1, nrm2_s);
-      if (threadIdx.x == 0) gmres_start(st, nrm2_s[0]);
-    } else {
-      finish_sums<T>(partial, k, out, st.hn);
-    }
-  }
+  pdl_trigger();
+  store_partials<T>(sd, start, k, acc, blockIdx.x, gridDim.x);
 }
 
 template <typename T, int MODE>
@@ -732,28 +745,45 @@ __global__ void k_qk_wrap32(long long nverts, int pstride, const double* __restr
   inv32[e] = val;
 }
 
-// z(node) = sum over the stars containing the node (vertices v with |i - 3v| <= 2 per
-// axis), fixed order; 0 at Dirichlet nodes; divided by den[0] when den is given
+// the vertices whose stars contain lattice index i (|i - 3v| <= 2), two taps: v0 = i / 3, then
+// v0 + 1 unless i = 3 v0; o: offset index in the star, 0 .. S1 - 1
+struct StarTaps {
+  int v[2], o[2];
+  bool two;
+  __device__ __forceinline__ explicit StarTaps(int i) {
+    const int v0 = i / K, r = i - K * v0;
+    v[0] = v0; o[0] = r + K - 1;
+    v[1] = v0 + 1; o[1] = r - 1;
+    two = r != 0;
+  }
+};
+
+// z(node) = sum over the stars containing the node, fixed order; 0 at Dirichlet nodes
 template <typename T>
-__global__ void k_qk_star_gather(Geom g, const T* __restrict__ sc, T* __restrict__ z, const T* __restrict__ den) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 2 * g.N) return;
-  const int comp = (int)(t / g.N);
-  const long long nd = t - comp * g.N;
-  const int i = (int)(nd % g.nn[0]), j = (int)(nd / g.nn[0]);
-  if (i == 0 || i == g.nn[0] - 1 || j == 0 || j == g.nn[1] - 1) { z[t] = T(0); return; }
-  int vxs[2], oxs[2], vys[2], oys[2], mx = 0, my = 0;
-  { const int v0 = i / K, r = i - K * v0; vxs[mx] = v0; oxs[mx++] = r; if (r != 0) { vxs[mx] = v0 + 1; oxs[mx++] = r - K; } }
-  { const int v0 = j / K, r = j - K * v0; vys[my] = v0; oys[my++] = r; if (r != 0) { vys[my] = v0 + 1; oys[my++] = r - K; } }
-  T acc = T(0);
-  for (int b = 0; b < my; ++b)
-    for (int a = 0; a < mx; ++a) {
-      const long long v = (long long)vxs[a] + (long long)(g.n[0] + 1) * vys[b];
-      const int e = comp * S1 * S1 + (oxs[a] + K - 1) + S1 * (oys[b] + K - 1);
-      acc += sc[v * NS + e];
+__global__ void k_qk_star_gather(Geom g, const T* __restrict__ sc, T* __restrict__ z) {
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x, N = (unsigned)g.N, nx = (unsigned)g.nn[0];
+  pdl_wait();
+  if (t < 2u * N) {
+    const int comp = (int)(t / N);
+    const unsigned nd = t - comp * N;
+    const int j = (int)(nd / nx), i = (int)(nd - j * nx);
+    T acc = T(0);
+    if (!(i == 0 || i == g.nn[0] - 1 || j == 0 || j == g.nn[1] - 1)) {
+      const StarTaps tx(i), ty(j);
+      T v[2][2];
+#pragma unroll
+      for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+          const bool ok = (a == 0 || tx.two) && (b == 0 || ty.two);
+          const int vid = tx.v[a] + (g.n[0] + 1) * ty.v[b];
+          v[b][a] = ok ? sc[vid * NS + comp * S1 * S1 + tx.o[a] + S1 * ty.o[b]] : T(0);
+        }
+      acc = ((v[0][0] + v[0][1]) + v[1][0]) + v[1][1];
     }
-  if (den) acc = den[0] != T(0) ? acc / den[0] : T(0);
-  z[t] = acc;
+    z[t] = acc;
+  }
+  pdl_trigger();
 }
 
 // ---------------------------------------------------------------------------
@@ -856,9 +886,9 @@ static void apply_epi_t(const LevelDev& L, double gamma, const void* x, void* y,
   qk::k_qk_cells<T, OP_VISC | OP_AL><<<(unsigned)((L.g.ncells + 7) / 8), 256, 0, s>>>(
       L.g, qk::cell_scal<T>(L.g, gamma), (const T*)x, mu, winv, nullptr, nullptr, (T*)L.ebuf);
   if (e1) cudaEventRecordWithFlags(e1, s, cudaEventRecordExternal);
-  qk::k_qk_gather_epi<T><<<(unsigned)((2 * L.g.N + RED_THREADS - 1) / RED_THREADS), RED_THREADS, 0, s>>>(
-      L.g, (const T*)L.ebuf, (const T*)x, (T*)y, (const T*)e.b, e.sigma, e.k, (const T*)e.V, e.ld, (T*)e.out, e.start,
-      e.st, e.partial);
+  const auto kernel = qk_epi_per(L) == 1 ? qk::k_qk_gather_epi<T, 1> : qk::k_qk_gather_epi<T, kEpiPer>;
+  launch_pdl(kernel, qk_epi_blocks(L), RED_THREADS, 0, s, L.g, (const T*)L.ebuf, (const T*)x, (T*)y, (const T*)e.b,
+             e.sigma, e.k, (const T*)e.V, e.ld, e.start, e.st);
   count_launch(2);
 }
 
@@ -902,19 +932,18 @@ void qk_patch_setup(const LevelDev& L, double gamma, DevStatus* st, cudaStream_t
   count_launch(1);
 }
 
-void qk_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, const void* den,
-                     cudaStream_t s) {
-  if (L.g.dim == 3) return qk3_patch_smooth(L, prec, r, z, scratch, den, s);
+void qk_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, cudaStream_t s) {
+  if (L.g.dim == 3) return qk3_patch_smooth(L, prec, r, z, scratch, s);
   const unsigned b2 = (unsigned)((2 * L.g.N + 255) / 256);
   constexpr int W64 = qk::star_warps<double>(), W32 = qk::star_warps<float>();
   if (prec == PREC_F64) {
     qk::k_qk_star_apply<double><<<(unsigned)((L.g.nverts + W64 - 1) / W64), 32 * W64, 0, s>>>(
         L.g, L.inv64, L.pstride, 0, 0, (const double*)r, (double*)scratch);
-    qk::k_qk_star_gather<double><<<b2, 256, 0, s>>>(L.g, (const double*)scratch, (double*)z, (const double*)den);
+    launch_pdl(qk::k_qk_star_gather<double>, b2, 256, 0, s, L.g, (const double*)scratch, (double*)z);
   } else {
     qk::k_qk_star_apply_w<<<qk::star_w_blocks(L.g.nverts), 256, 0, s>>>(L.g, L.inv32, 0, 0, (const float*)r,
                                                                       (float*)scratch);
-    qk::k_qk_star_gather<float><<<b2, 256, 0, s>>>(L.g, (const float*)scratch, (float*)z, (const float*)den);
+    launch_pdl(qk::k_qk_star_gather<float>, b2, 256, 0, s, L.g, (const float*)scratch, (float*)z);
   }
   count_launch(2);
 }

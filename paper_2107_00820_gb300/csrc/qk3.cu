@@ -29,6 +29,7 @@
 #include "df64.cuh"
 #include "krylov.h"
 #include "level.h"
+#include "pdl.cuh"
 #include "qk_tables.h"
 
 namespace als {
@@ -317,84 +318,97 @@ __global__ void __launch_bounds__(64 * CPB) k_qk3_cells(Geom g, CellScal<T> cs, 
   }
 }
 
-// the cells (and local index) containing lattice index i along an axis of n cells
-__device__ __forceinline__ int cells_of(int i, int n, int (&c)[2], int (&a)[2]) {
-  int m = 0;
-  const int c0 = i / K, r = i - K * c0;
-  if (r == 0 && c0 > 0) { c[m] = c0 - 1; a[m] = K; ++m; }
-  if (c0 < n) { c[m] = c0; a[m] = r; ++m; }
-  return m;
+// the cells containing lattice index i along an axis of n cells, two taps in a fixed order:
+// (c - 1, local K) where i is the cell corner between c - 1 and c, then (c, i - K c)
+struct CellTaps {
+  int c[2], a[2];
+  bool ok[2];
+  __device__ __forceinline__ CellTaps(int i, int n) {
+    const int c0 = i / K, r = i - K * c0;
+    c[0] = c0 - 1; a[0] = K; ok[0] = r == 0 && c0 > 0;
+    c[1] = c0; a[1] = r; ok[1] = c0 < n;
+  }
+};
+
+// component and lattice coordinates of vector entry t (32-bit: entries stay below 2^31)
+__device__ __forceinline__ void entry_coords(const Geom& g, unsigned t, int& comp, int& i, int& j, int& k) {
+  const unsigned N = (unsigned)g.N, nx = (unsigned)g.nn[0], ny = (unsigned)g.nn[1];
+  comp = (int)(t / N);
+  const unsigned nd = t - comp * N, r = nd / nx;
+  i = (int)(nd - r * nx);
+  k = (int)(r / ny);
+  j = (int)(r - k * ny);
 }
 
 // y(node) = sum of the staged cell outputs of the (up to 8) cells containing it, fixed
-// order; keep_bnd: y = x at Dirichlet nodes; raw: no Dirichlet treatment
+// order; keep_bnd: y = x at Dirichlet nodes; raw: no Dirichlet treatment.  Predicated taps, so
+// that all loads issue at once.
 template <typename T>
 __device__ __forceinline__ T gather_value(const Geom& g, const T* __restrict__ ebuf, const T* __restrict__ x,
-                                          long long t, int keep_bnd, int raw) {
-  const int comp = (int)(t / g.N);
-  const long long nd = t - comp * g.N;
-  const int i = (int)(nd % g.nn[0]);
-  const long long r = nd / g.nn[0];
-  const int j = (int)(r % g.nn[1]), k = (int)(r / g.nn[1]);
+                                          unsigned t, int keep_bnd, int raw) {
+  int comp, i, j, k;
+  entry_coords(g, t, comp, i, j, k);
   if (bnd_node(g, i, j, k) && !raw) return keep_bnd ? x[t] : T(0);
-  int cxs[2], axs[2], cys[2], ays[2], czs[2], azs[2];
-  const int mx = cells_of(i, g.n[0], cxs, axs), my = cells_of(j, g.n[1], cys, ays), mz = cells_of(k, g.n[2], czs, azs);
-  T acc = T(0);
-  for (int c = 0; c < mz; ++c)
-    for (int b = 0; b < my; ++b)
-      for (int a = 0; a < mx; ++a) {
-        const long long cell = (long long)cxs[a] + (long long)g.n[0] * ((long long)cys[b] + (long long)g.n[1] * czs[c]);
-        acc += ebuf[(cell * 3 + comp) * NB + axs[a] + N1 * ays[b] + N1 * N1 * azs[c]];
-      }
+  const CellTaps tx(i, g.n[0]), ty(j, g.n[1]), tz(k, g.n[2]);
+  T v[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int a = q & 1, b = (q >> 1) & 1, c = q >> 2;
+    const int cell = tx.c[a] + g.n[0] * (ty.c[b] + g.n[1] * tz.c[c]);
+    v[q] = tx.ok[a] && ty.ok[b] && tz.ok[c]
+               ? ebuf[(cell * 3 + comp) * NB + tx.a[a] + N1 * ty.a[b] + N1 * N1 * tz.a[c]]
+               : T(0);
+  }
+  T acc = v[0];
+#pragma unroll
+  for (int q = 1; q < 8; ++q) acc += v[q];
   return acc;
 }
 
 template <typename T>
 __global__ void k_qk3_gather(Geom g, const T* __restrict__ ebuf, const T* __restrict__ x, T* __restrict__ y,
                              int keep_bnd, int raw) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 3 * g.N) return;
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= 3u * (unsigned)g.N) return;
   y[t] = gather_value<T>(g, ebuf, x, t, keep_bnd, raw);
 }
 
-// the gather fused with the GMRES smoother's Arnoldi reduction (as for the other
-// discretisations): y = b + sigma A x; start = 0: out[j] = (V_j . y) / hn[j], j < k;
-// start = 1: |y|^2 starts the GMRES cycle.  Block partials in a fixed order.
-template <typename T>
+// The gather fused with the reduction that consumes its result, as for order 2 (the
+// GMRES smoother's Arnoldi step): y = b + sigma A x (b NULL: sigma A x; Dirichlet rows of
+// A x are x, the identity);  block partials of V_j . y, j < k, or, start = 1, of |y|^2.
+// PER entries a thread, 256 apart: large levels take kEpiPer, which keeps the partials that
+// every block of the Gram-Schmidt kernel adds at about a thousand.
+template <typename T, int PER>
 __global__ void __launch_bounds__(RED_THREADS) k_qk3_gather_epi(Geom g, const T* __restrict__ ebuf,
-                                                                const T* __restrict__ x, T* __restrict__ y,
-                                                                const T* __restrict__ b, double sigma, int k,
-                                                                const T* __restrict__ V, long long ld,
-                                                                T* __restrict__ out, int start, GmresDev sd,
-                                                                double* __restrict__ partial) {
-  __shared__ T nrm2_s[1];
-  const GmresView<T> st = gmres_view<T>(sd);
-  T* rows = reinterpret_cast<T*>(partial + 1);
-  const int kk = start ? 1 : k;
+                                                               const T* __restrict__ x, T* __restrict__ y,
+                                                               const T* __restrict__ b, double sigma, int k,
+                                                               const T* __restrict__ V, long long ld, int start,
+                                                               GmresDev sd) {
   T acc[KMAXB];
 #pragma unroll
   for (int jj = 0; jj < KMAXB; ++jj) acc[jj] = T(0);
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < 3 * g.N) {
-    const T v = (b ? b[t] : T(0)) + (T)sigma * gather_value<T>(g, ebuf, x, t, 1, 0);
-    y[t] = v;
+  const unsigned n = 3 * (unsigned)g.N, t0 = blockIdx.x * (RED_THREADS * PER) + threadIdx.x;
+  pdl_wait();
+  T v[PER];
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const unsigned t = t0 + q * RED_THREADS;
+    v[q] = t < n ? (b ? b[t] : T(0)) + (T)sigma * gather_value<T>(g, ebuf, x, t, 1, 0) : T(0);
+  }
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const unsigned t = t0 + q * RED_THREADS;
+    if (t < n) y[t] = v[q];
     if (start) {
-      acc[0] = v * v;
+      acc[0] += v[q] * v[q];
     } else {
 #pragma unroll
       for (int jj = 0; jj < KMAXB; ++jj)
-        if (jj < k) acc[jj] = V[(long long)jj * ld + t] * v;
+        if (jj < k && t < n) acc[jj] += __ldcg(V + (long long)jj * ld + t) * v[q];
     }
   }
-  block_partials<T, T>(acc, kk, rows + (long long)blockIdx.x * kk);
-  if (last_block(partial)) {
-    if (start) {
-      finish_sums<T>(partial, 1, nrm2_s);
-      if (threadIdx.x == 0) gmres_start(st, nrm2_s[0]);
-    } else {
-      finish_sums<T>(partial, k, out, st.hn);
-    }
-  }
+  pdl_trigger();
+  store_partials<T>(sd, start, k, acc, blockIdx.x, gridDim.x);
 }
 
 template <typename T, int MODE>
@@ -438,9 +452,9 @@ static void apply_epi_t(const LevelDev& L, double gamma, const void* x, void* y,
   k_qk3_cells<T, OP_VISC | OP_AL><<<(unsigned)((L.g.ncells + CPB - 1) / CPB), 64 * CPB, 0, s>>>(
       L.g, cell_scal<T>(L.g, gamma), (const T*)x, mu, winv, nullptr, nullptr, (T*)L.ebuf);
   if (e1) cudaEventRecordWithFlags(e1, s, cudaEventRecordExternal);
-  k_qk3_gather_epi<T><<<(unsigned)((3 * L.g.N + RED_THREADS - 1) / RED_THREADS), RED_THREADS, 0, s>>>(
-      L.g, (const T*)L.ebuf, (const T*)x, (T*)y, (const T*)e.b, e.sigma, e.k, (const T*)e.V, e.ld, (T*)e.out, e.start,
-      e.st, e.partial);
+  const auto kernel = qk_epi_per(L) == 1 ? k_qk3_gather_epi<T, 1> : k_qk3_gather_epi<T, kEpiPer>;
+  launch_pdl(kernel, qk_epi_blocks(L), RED_THREADS, 0, s, L.g, (const T*)L.ebuf, (const T*)x, (T*)y, (const T*)e.b,
+             e.sigma, e.k, (const T*)e.V, e.ld, e.start, e.st);
   count_launch(2);
 }
 
@@ -1020,36 +1034,45 @@ __global__ void k_qk3_wrap32(long long nverts, int pstride, const double* __rest
   inv32[e] = val;
 }
 
-// z(node) = sum over the (up to 8) stars containing the node (vertices v with
-// |i - 3v| <= 2 per axis), fixed order; 0 at Dirichlet nodes; divided by den[0] when given
-template <typename T>
-__global__ void k_qk3_star_gather(Geom g, const T* __restrict__ sc, T* __restrict__ z, const T* __restrict__ den) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 3 * g.N) return;
-  const int comp = (int)(t / g.N);
-  const long long nd = t - comp * g.N;
-  const int i = (int)(nd % g.nn[0]);
-  const long long rr = nd / g.nn[0];
-  const int j = (int)(rr % g.nn[1]), k = (int)(rr / g.nn[1]);
-  if (bnd_node(g, i, j, k)) { z[t] = T(0); return; }
-  int vs[3][2], os[3][2], m[3];
-  const int ijk[3] = {i, j, k};
-  for (int a = 0; a < 3; ++a) {
-    const int v0 = ijk[a] / K, r = ijk[a] - K * v0;
-    m[a] = 0;
-    vs[a][m[a]] = v0; os[a][m[a]++] = r;
-    if (r != 0) { vs[a][m[a]] = v0 + 1; os[a][m[a]++] = r - K; }
+// the vertices whose stars contain lattice index i (|i - 3v| <= 2), two taps: v0 = i / 3, then
+// v0 + 1 unless i = 3 v0; o: offset index in the star, 0 .. S1 - 1
+struct StarTaps {
+  int v[2], o[2];
+  bool two;
+  __device__ __forceinline__ explicit StarTaps(int i) {
+    const int v0 = i / K, r = i - K * v0;
+    v[0] = v0; o[0] = r + K - 1;
+    v[1] = v0 + 1; o[1] = r - 1;
+    two = r != 0;
   }
-  T acc = T(0);
-  for (int c = 0; c < m[2]; ++c)
-    for (int b = 0; b < m[1]; ++b)
-      for (int a = 0; a < m[0]; ++a) {
-        const long long v = (long long)vs[0][a] + (long long)g.nv[0] * ((long long)vs[1][b] + (long long)g.nv[1] * vs[2][c]);
-        const int e = comp * SN + (os[0][a] + K - 1) + S1 * (os[1][b] + K - 1) + S1 * S1 * (os[2][c] + K - 1);
-        acc += sc[v * NS + e];
+};
+
+// z(node) = sum over the (up to 8) stars containing the node, fixed order; 0 at Dirichlet nodes
+template <typename T>
+__global__ void k_qk3_star_gather(Geom g, const T* __restrict__ sc, T* __restrict__ z) {
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_wait();
+  if (t < 3u * (unsigned)g.N) {
+    int comp, i, j, k;
+    entry_coords(g, t, comp, i, j, k);
+    T acc = T(0);
+    if (!bnd_node(g, i, j, k)) {
+      const StarTaps tx(i), ty(j), tz(k);
+      T v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int a = q & 1, b = (q >> 1) & 1, c = q >> 2;
+        const bool ok = (a == 0 || tx.two) && (b == 0 || ty.two) && (c == 0 || tz.two);
+        const int vid = tx.v[a] + g.nv[0] * (ty.v[b] + g.nv[1] * tz.v[c]);
+        v[q] = ok ? sc[vid * NS + comp * SN + tx.o[a] + S1 * ty.o[b] + S1 * S1 * tz.o[c]] : T(0);
       }
-  if (den) acc = den[0] != T(0) ? acc / den[0] : T(0);
-  z[t] = acc;
+      acc = v[0];
+#pragma unroll
+      for (int q = 1; q < 8; ++q) acc += v[q];
+    }
+    z[t] = acc;
+  }
+  pdl_trigger();
 }
 
 // ---------------------------------------------------------------------------
@@ -1253,14 +1276,13 @@ void qk3_patch_setup(const LevelDev& L, double gamma, DevStatus* st, cudaStream_
   }
 }
 
-void qk3_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, const void* den,
-                      cudaStream_t s) {
+void qk3_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, cudaStream_t s) {
   const unsigned b3 = (unsigned)((3 * L.g.N + 255) / 256);
   const unsigned nv = (unsigned)L.g.nverts;
   if (prec == PREC_F64) {
     qk3::k_qk3_star_apply<double><<<nv, qk3::STAR_THREADS, 0, s>>>(L.g, L.inv64, L.pstride, 0, 0, (const double*)r,
                                                                    (double*)scratch);
-    qk3::k_qk3_star_gather<double><<<b3, 256, 0, s>>>(L.g, (const double*)scratch, (double*)z, (const double*)den);
+    launch_pdl(qk3::k_qk3_star_gather<double>, b3, 256, 0, s, L.g, (const double*)scratch, (double*)z);
   } else {
     if (L.inv16)
       qk3::k_qk3_star_apply_w<__nv_bfloat16><<<nv, qk3::STAR_THREADS, 0, s>>>(
@@ -1268,7 +1290,7 @@ void qk3_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void*
     else
       qk3::k_qk3_star_apply_w<float><<<nv, qk3::STAR_THREADS, 0, s>>>(L.g, L.inv32, 0, 0, (const float*)r,
                                                                       (float*)scratch);
-    qk3::k_qk3_star_gather<float><<<b3, 256, 0, s>>>(L.g, (const float*)scratch, (float*)z, (const float*)den);
+    launch_pdl(qk3::k_qk3_star_gather<float>, b3, 256, 0, s, L.g, (const float*)scratch, (float*)z);
   }
   count_launch(2);
 }

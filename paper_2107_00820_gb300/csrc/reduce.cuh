@@ -97,11 +97,49 @@ __device__ __forceinline__ void finish_sums(double* ws, int k, R* out, const R* 
   finish_sums_n<R>(ws, k, out, div, (int)gridDim.x);
 }
 
+// Sum of kk <= KMAXB columns over a block, returned to thread j < kk (others: 0): warp shuffles
+// with the columns interleaved, one shared pass.  The caller puts a barrier between the
+// return and the next use of sh.
+template <typename T>
+__device__ __forceinline__ T block_total(const T (&acc)[KMAXB], int kk, T (&sh)[RED_THREADS / 32][KMAXB]) {
+  T v[KMAXB];
+#pragma unroll
+  for (int j = 0; j < KMAXB; ++j) v[j] = acc[j];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int j = 0; j < KMAXB; ++j)
+      if (j < kk) v[j] += __shfl_down_sync(0xffffffffu, v[j], o);
+  if ((threadIdx.x & 31) == 0)
+#pragma unroll
+    for (int j = 0; j < KMAXB; ++j)
+      if (j < kk) sh[threadIdx.x >> 5][j] = v[j];
+  __syncthreads();
+  T t = T(0);
+  if ((int)threadIdx.x < kk)
+#pragma unroll
+    for (int i = 0; i < RED_THREADS / 32; ++i) t += sh[i][threadIdx.x];
+  return t;
+}
+
+// acc[j] += the thread's share (blocks tid, tid + 256, ..) of column j of nb block partials
+template <typename T>
+__device__ __forceinline__ void sum_rows(const T* __restrict__ rows, int nb, int k, T (&acc)[KMAXB]) {
+#pragma unroll
+  for (int j = 0; j < KMAXB; ++j) acc[j] = T(0);
+#pragma unroll 4
+  for (int b = threadIdx.x; b < nb; b += RED_THREADS) {
+#pragma unroll
+    for (int j = 0; j < KMAXB; ++j)
+      if (j < k) acc[j] += __ldcg(rows + j * nb + b);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // GMRES(s) state on the device, in the smoother's precision T (column-major
 // Hessenberg H, leading dim ldh).  The Krylov basis is stored unnormalised:
 // column i holds hn[i] * v_i, where v_i is the orthonormal Arnoldi vector, and
-// every consumer divides by hn[i].  Layout of the state array, in elements of T:
+// Z_i = D^-1 (column i) likewise; their consumers divide by hn[i].  Layout of the state array, in elements of T:
 // H [ldh s] | cs [s] | sn [s] | g [s+1] | y [s] | res | beta | nrm2 | hn [s+1] | yu [2s+1].
 // ---------------------------------------------------------------------------
 struct GmresLayout {
@@ -112,11 +150,44 @@ struct GmresLayout {
         res(y + steps), beta(res + 1), nrm2(beta + 1), hn(nrm2 + 1), yu(hn + steps + 1), total(yu + 2 * steps + 1) {}
 };
 
-// host-side handle: the state array (elements of the smoother's precision) and s
+// host-side handle: the state array (elements of the smoother's precision), s, and the block
+// partials of the reductions.  A reduction kernel only writes its partials, [column][block];
+// every block of the kernel that needs the sums adds them for itself, in one fixed order.
+// (A last-block finish, with its fence, ticket, second fence, reload and one-thread
+// bookkeeping, cost 1 to 2 us at the end of each of the two reductions of a step: a third of a
+// small level's time.)  The dots of a gather: nbd blocks at rows.  |column j|^2: at
+// rows + noff + (j & 1) nstride, written while the other area is still being read; nb0 blocks
+// for column 0 (gather or copy), ceil(n / 1024) for the others.
 struct GmresDev {
   void* base;
   int s;
+  void* rows;
+  int nbd, nb0, noff, nstride;
 };
+
+template <typename T>
+__host__ __device__ __forceinline__ T* dot_rows(const GmresDev& d) { return static_cast<T*>(d.rows); }
+template <typename T>
+__host__ __device__ __forceinline__ T* norm_rows(const GmresDev& d, int j) {
+  return static_cast<T*>(d.rows) + d.noff + (j & 1) * d.nstride;
+}
+constexpr int GM_PER = 4;   // entries per thread of the smoother's vector kernels
+__host__ __device__ __forceinline__ int gm_blocks(long long n) {
+  return (int)((n + RED_THREADS * GM_PER - 1) / (RED_THREADS * GM_PER));
+}
+__host__ __device__ __forceinline__ int norm_count(const GmresDev& d, int j, long long n) {
+  return j == 0 ? d.nb0 : gm_blocks(n);
+}
+
+// the block partials of a gather: |y|^2 of column 0 (start) or the k dots (every thread calls)
+template <typename T>
+__device__ __forceinline__ void store_partials(const GmresDev& d, int start, int k, const T (&acc)[KMAXB], unsigned bx,
+                                               unsigned nb) {
+  __shared__ T sh[RED_THREADS / 32][KMAXB];
+  const int kk = start ? 1 : k;
+  const T v = block_total<T>(acc, kk, sh);
+  if ((int)threadIdx.x < kk) (start ? norm_rows<T>(d, 0) : dot_rows<T>(d))[threadIdx.x * nb + bx] = v;
+}
 
 template <typename T>
 struct GmresView {
@@ -150,27 +221,37 @@ __device__ __forceinline__ void gmres_start(const GmresView<T>& st, T nrm2) {
 }
 
 // step k (k < KMAXB): H[k+1][k] = |w|, hn[k+1] = |w|, then the rotations of
-// column k; all operands are loaded first so the chain runs in registers (one thread)
+// column k; all operands are loaded first and every index is a compile-time one (loops
+// unrolled to KMAXB, predicated), so the chain runs in registers (one thread).  With runtime
+// loop bounds the arrays lived in local memory, and this chain, on the serial tail of every
+// Gram-Schmidt step, took about three times as long.
 template <typename T>
 __device__ __forceinline__ void gmres_step(const GmresView<T>& st, int k, T nrm2) {
   T* hg = st.H + (long long)k * st.ldh;
-  T h[KMAXB + 1], cs[KMAXB], sn[KMAXB];
-  for (int i = 0; i <= k; ++i) h[i] = hg[i];
-  for (int i = 0; i < k; ++i) { cs[i] = st.cs[i]; sn[i] = st.sn[i]; }
+  T h[KMAXB], cs[KMAXB], sn[KMAXB];
+#pragma unroll
+  for (int i = 0; i < KMAXB; ++i) {
+    h[i] = i <= k ? hg[i] : T(0);
+    cs[i] = i < k ? st.cs[i] : T(1);
+    sn[i] = i < k ? st.sn[i] : T(0);
+  }
   const T gk = st.g[k];
   const T hk1 = sqrt(fmax(nrm2, T(0)));
-  h[k + 1] = hk1;
-  for (int i = 0; i < k; ++i) {
-    const T a = h[i], b = h[i + 1];
-    h[i] = cs[i] * a + sn[i] * b;
-    h[i + 1] = -sn[i] * a + cs[i] * b;
-  }
-  const T a = h[k], b = h[k + 1];
+  T a = h[0];                       // the entry the next rotation starts from
+#pragma unroll
+  for (int i = 0; i < KMAXB - 1; ++i)
+    if (i < k) {
+      const T b = h[i + 1];
+      h[i] = cs[i] * a + sn[i] * b;
+      a = -sn[i] * a + cs[i] * b;
+    }
+  const T b = hk1;
   const T r = hypot(a, b);
   T c = T(1), sv = T(0);
   if (r > T(0)) { c = a / r; sv = b / r; }
-  h[k] = r;
-  for (int i = 0; i <= k; ++i) hg[i] = h[i];
+#pragma unroll
+  for (int i = 0; i < KMAXB; ++i)
+    if (i <= k) hg[i] = i == k ? r : h[i];
   hg[k + 1] = T(0);
   st.hn[k + 1] = hk1;
   st.cs[k] = c; st.sn[k] = sv;
@@ -185,28 +266,34 @@ __device__ __forceinline__ void gmres_step(const GmresView<T>& st, int k, T nrm2
 // sum_i u_i (stored column i) by the Arnoldi relation.  Stored in st.yu.
 template <typename T>
 __device__ __forceinline__ void gmres_coeffs(const GmresView<T>& st, int k) {
-  T Hs[KMAXB][KMAXB], gs[KMAXB + 1], cs[KMAXB], sn[KMAXB], hn[KMAXB + 1];
-  for (int c = 0; c < k; ++c) {
-    for (int r = 0; r <= c; ++r) Hs[r][c] = st.H[(long long)c * st.ldh + r];
-    cs[c] = st.cs[c]; sn[c] = st.sn[c];
+  // (the stores come last: they may alias the state, and would hold the loads back)
+  T ys[KMAXB], us[KMAXB];
+#pragma unroll
+  for (int i = KMAXB - 1; i >= 0; --i) {
+    if (i >= k) continue;
+    T a = st.g[i];
+#pragma unroll
+    for (int c = 0; c < KMAXB; ++c)
+      if (c > i && c < k) a -= st.H[(long long)c * st.ldh + i] * ys[c];
+    const T d = st.H[(long long)i * st.ldh + i];
+    ys[i] = d != T(0) ? a / d : T(0);
   }
-  for (int c = 0; c <= k; ++c) { gs[c] = st.g[c]; hn[c] = st.hn[c]; }
-  T ys[KMAXB];
-  for (int i = k - 1; i >= 0; --i) {
-    T a = gs[i];
-    for (int c = i + 1; c < k; ++c) a -= Hs[i][c] * ys[c];
-    ys[i] = Hs[i][i] != T(0) ? a / Hs[i][i] : T(0);
-    st.yu[i] = ys[i];
+  T b = st.g[k];                    // u_(i+1) before rotation i is undone (u_0..u_i are still 0)
+#pragma unroll
+  for (int i = KMAXB - 1; i >= 0; --i) {
+    if (i >= k) continue;
+    const T hn = st.hn[i + 1];
+    us[i] = hn != T(0) ? (st.cs[i] * b) / hn : T(0);
+    b = -(st.sn[i] * b);
   }
-  T us[KMAXB + 1];
-  for (int i = 0; i < k; ++i) us[i] = T(0);
-  us[k] = gs[k];
-  for (int i = k - 1; i >= 0; --i) {
-    const T a = us[i], b = us[i + 1];
-    us[i] = cs[i] * a - sn[i] * b;
-    us[i + 1] = sn[i] * a + cs[i] * b;
-  }
-  for (int i = 0; i <= k; ++i) st.yu[k + i] = hn[i] != T(0) ? us[i] / hn[i] : T(0);
+  const T h0 = st.hn[0];
+#pragma unroll
+  for (int i = 0; i < KMAXB; ++i)
+    if (i < k) {
+      st.yu[i] = ys[i];
+      st.yu[k + i + 1] = us[i];
+    }
+  st.yu[k] = h0 != T(0) ? b / h0 : T(0);
 }
 
 }  // namespace als
