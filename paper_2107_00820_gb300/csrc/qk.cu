@@ -226,15 +226,6 @@ __global__ void __launch_bounds__(256) k_qk_cells(Geom g, CellScal<T> cs, const 
   }
 }
 
-// the cells (and local index) containing lattice index i along an axis of n cells
-__device__ __forceinline__ int cells_of(int i, int n, int (&c)[2], int (&a)[2]) {
-  int m = 0;
-  const int c0 = i / K, r = i - K * c0;
-  if (r == 0 && c0 > 0) { c[m] = c0 - 1; a[m] = K; ++m; }
-  if (c0 < n) { c[m] = c0; a[m] = r; ++m; }
-  return m;
-}
-
 // the cells containing lattice index i along an axis of n cells, two taps in a fixed order:
 // (c - 1, local K) where i is the cell corner between c - 1 and c, then (c, i - K c)
 struct CellTaps {
@@ -824,36 +815,53 @@ __global__ void k_qk_prolong(Geom gc, Geom gf, const T* __restrict__ xc, T* __re
 }
 
 // rc = P_H^T (rf - sub): coarse node J gathers the fine nodes owned by the coarse cells that
-// contain it, weighted by its basis function there
+// contain it, weighted by its basis function there.  The 7 x 4 weights are staged in shared
+// memory (per-lane indices serialise in constant memory) and each cell's 7 x 7 taps are
+// predicated instead of skipped, so that their loads are in flight together.
 template <typename T>
-__global__ void k_qk_restrict(Geom gc, Geom gf, const T* __restrict__ rf, const T* __restrict__ sub, T* __restrict__ rc) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 2 * gc.N) return;
-  const int comp = (int)(t / gc.N);
-  const long long nd = t - comp * gc.N;
-  const int I = (int)(nd % gc.nn[0]), J = (int)(nd / gc.nn[0]);
-  if (I == 0 || I == gc.nn[0] - 1 || J == 0 || J == gc.nn[1] - 1) { rc[t] = T(0); return; }
-  int cxs[2], axs[2], cys[2], ays[2];
-  const int mx = cells_of(I, gc.n[0], cxs, axs), my = cells_of(J, gc.n[1], cys, ays);
+__global__ void __launch_bounds__(256) k_qk_restrict(Geom gc, Geom gf, const T* __restrict__ rf,
+                                                     const T* __restrict__ sub, T* __restrict__ rc) {
+  __shared__ T W[2 * K + 1][N1];
+  for (int e = threadIdx.x; e < (2 * K + 1) * N1; e += blockDim.x) W[e / N1][e % N1] = Tab<T>::pw(e / N1, e % N1);
+  __syncthreads();
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x, N = (unsigned)gc.N, nx = (unsigned)gc.nn[0];
+  if (t >= 2u * N) return;
+  const int comp = (int)(t / N);
+  const unsigned nd = t - comp * N;
+  const int J = (int)(nd / nx), I = (int)(nd - J * nx);
   T acc = T(0);
-  for (int b = 0; b < my; ++b)
-    for (int a = 0; a < mx; ++a)
-      for (int fy = 0; fy <= 2 * K; ++fy) {
-        const int j = 2 * K * cys[b] + fy;
-        if (fy == 2 * K && cys[b] != gc.n[1] - 1) continue;   // owned by the next coarse cell
-        if (j == 0 || j == gf.nn[1] - 1) continue;
-        const T wy = Tab<T>::pw(fy, ays[b]);
-        if (wy == T(0)) continue;
-        for (int fx = 0; fx <= 2 * K; ++fx) {
-          const int i = 2 * K * cxs[a] + fx;
-          if (fx == 2 * K && cxs[a] != gc.n[0] - 1) continue;
-          if (i == 0 || i == gf.nn[0] - 1) continue;
-          const T wx = Tab<T>::pw(fx, axs[a]);
-          if (wx == T(0)) continue;
-          const long long fn = comp * gf.N + i + (long long)gf.nn[0] * j;
-          acc += wx * wy * (sub ? rf[fn] - sub[fn] : rf[fn]);
+  if (!(I == 0 || I == gc.nn[0] - 1 || J == 0 || J == gc.nn[1] - 1)) {
+    const CellTaps tx(I, gc.n[0]), ty(J, gc.n[1]);
+    const T* rfc = rf + comp * (int)gf.N;
+    const T* sbc = sub ? sub + comp * (int)gf.N : nullptr;
+#pragma unroll 1
+    for (int b = 0; b < 2; ++b)
+#pragma unroll 1
+      for (int a = 0; a < 2; ++a) {
+        if (!((a ? tx.ok[1] : tx.ok[0]) && (b ? ty.ok[1] : ty.ok[0]))) continue;
+        const int cx = a ? tx.c[1] : tx.c[0], ax = a ? tx.a[1] : tx.a[0];
+        const int cy = b ? ty.c[1] : ty.c[0], ay = b ? ty.a[1] : ty.a[0];
+        T v[2 * K + 1][2 * K + 1];
+#pragma unroll
+        for (int fy = 0; fy <= 2 * K; ++fy)
+#pragma unroll
+          for (int fx = 0; fx <= 2 * K; ++fx) {
+            const int i = 2 * K * cx + fx, j = 2 * K * cy + fy;
+            // the last fine node of a cell belongs to the next coarse cell; Dirichlet nodes give 0
+            const bool ok = (fx < 2 * K || cx == gc.n[0] - 1) && (fy < 2 * K || cy == gc.n[1] - 1) && i > 0 &&
+                            i < gf.nn[0] - 1 && j > 0 && j < gf.nn[1] - 1;
+            const int fn = i + gf.nn[0] * j;
+            v[fy][fx] = ok ? (sbc ? rfc[fn] - sbc[fn] : rfc[fn]) : T(0);
+          }
+#pragma unroll
+        for (int fy = 0; fy <= 2 * K; ++fy) {
+          T row = T(0);
+#pragma unroll
+          for (int fx = 0; fx <= 2 * K; ++fx) row += W[fx][ax] * v[fy][fx];
+          acc += W[fy][ay] * row;
         }
       }
+  }
   rc[t] = acc;
 }
 
