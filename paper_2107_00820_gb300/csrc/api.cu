@@ -277,15 +277,15 @@ bool fused_gmres(const als_ctx* c) {
   return c->opt.smoother == ALS_SMOOTH_GMRES && std::max(1, c->opt.sweeps) <= KMAXB;
 }
 
-// FP32 3D cycles form Z_j inside the operator's cell kernel from the patch outputs
+// Order-2 cycles form Z_j inside the operator's cell kernel from the patch outputs
 // (one launch less per Arnoldi step); ALS_FUSE_GATHER=0 keeps the separate gather
-bool fuse_patch_gather(const als_ctx* c, int prec) {
+bool fuse_patch_gather(const als_ctx* c) {
   static int v = -1;
   if (v < 0) {
     const char* e = getenv("ALS_FUSE_GATHER");
     v = (e && e[0] == '0') ? 0 : 1;
   }
-  return v == 1 && prec == PREC_F32 && c->dim == 3 && c->k == 2;
+  return v == 1 && c->k == 2;
 }
 
 void smooth_fused(als_ctx* c, MGWork& w, int l, bool x_is_zero, void* t) {
@@ -309,9 +309,9 @@ void smooth_fused(als_ctx* c, MGWork& w, int l, bool x_is_zero, void* t) {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (l == c->L - 1) prof_events(c, t_prof_counter, e0, e1);
     ApplyEpi e{nullptr, 1.0, j + 1, w.V[l], len, 0, st};
-    if (fuse_patch_gather(c, prec)) {
+    if (fuse_patch_gather(c)) {
       // patch products only; the cell kernel sums them per node into Z_j = D^-1 V_j
-      patch_products(Lv, Vj, w.scratch[l], s, e0, e1);
+      patch_products(Lv, prec, Vj, w.scratch[l], s, e0, e1);
       e.pout = w.scratch[l];
     } else {
       patch_smooth(Lv, prec, Vj, Zj, w.scratch[l], s, e0, e1);            // Z_j = D^-1 V_j
@@ -1769,7 +1769,7 @@ void merged_smooth(MergedCycle& M, int l, bool x_is_zero, bool residual, cudaStr
       void* Zj = vptr(w.Z[l], w.es, (long long)j * len);
       prod.push_back(BPatch{&c->lev[l], Vj, w.scratch[l], nullptr});
       ApplyEpi e{nullptr, 1.0, j + 1, w.V[l], len, 0, g[i].st};
-      if (fuse_patch_gather(c, PREC_F32)) {
+      if (fuse_patch_gather(c)) {
         e.pout = w.scratch[l];
       } else {
         gath.push_back(BPatch{&c->lev[l], nullptr, w.scratch[l], Zj});

@@ -81,7 +81,7 @@ struct ApplyEpi {
   long long ld;
   int start;
   GmresDev st;
-  // FP32, 3D: when pout is set, the apply's input x is not read but formed from the
+  // when pout is set (order 2), the apply's input x is not read but formed from the
   // star-patch outputs pout (row layout) and stored into x (the patch gather fused into
   // the cell kernel)
   const void* pout = nullptr;
@@ -109,10 +109,10 @@ void patch_derive32(const LevelDev& L, cudaStream_t s);
 void patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, cudaStream_t s,
                   cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr);
 size_t patch_scratch_bytes(const LevelDev& L, int prec);
-// FP32: the star-patch products y_v = A_v^-1 r|_v into the scratch rows only (their
+// the star-patch products y_v = A_v^-1 r|_v into the scratch rows only (their
 // node sums are formed by the consumer, see ApplyEpi::pout)
-void patch_products(const LevelDev& L, const void* r, void* scratch, cudaStream_t s, cudaEvent_t e0 = nullptr,
-                    cudaEvent_t e1 = nullptr);
+void patch_products(const LevelDev& L, int prec, const void* r, void* scratch, cudaStream_t s,
+                    cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr);
 // times the FP32 patch-kernel variants on this level and keeps the fastest (ms_out[3], optional)
 int patch_autotune(LevelDev& L, const void* r, void* scratch, cudaStream_t s, float* ms_out = nullptr);
 // local solves on the coarse-cell interiors (stars of the fine vertices at the

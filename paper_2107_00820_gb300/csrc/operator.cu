@@ -93,336 +93,6 @@ __device__ __forceinline__ bool colour_cell(const Colour& col, long long t, int&
   return true;
 }
 
-// One warp evaluates one cell (3D: 27 lanes = 27 nodes = 27 Gauss points) or
-// three cells (2D: 9 lanes each).  The three 1D contractions of the sum
-// factorisation run lane-parallel through shared memory, the divergence
-// moments are a warp (3D) or lane-group (2D) reduction, and the isotropic AL /
-// pressure part of the stress is formed at every point before the transposed
-// contractions take the fluxes back to the nodes.
-template <typename T, int DIM, bool TENSOR, int MODE, bool STAGED>
-__device__ __forceinline__ void apply_body(unsigned bx, const Geom& g, const Colour& col, const CellConst<T>& cc,
-                                           const T* __restrict__ x, T* __restrict__ y, const T* __restrict__ coef,
-                                           const T* __restrict__ p_in, T* __restrict__ p_out, long long vstride,
-                                           T* __restrict__ ebuf, const T* __restrict__ winv) {
-  constexpr int NB = Sz<DIM>::NB, NPR = Sz<DIM>::NPR;
-  constexpr int CPW = DIM == 2 ? 3 : 1;        // cells per warp
-  constexpr int NCQ = TENSOR ? Sz<DIM>::NC : 1;
-  constexpr bool RAW = (MODE & OP_RAW) != 0;
-  constexpr bool VISC = (MODE & OP_VISC) != 0;
-  constexpr bool NEED_U = (MODE & (OP_VISC | OP_AL | OP_B)) != 0;
-  constexpr bool NEED_FLUX = (MODE & (OP_VISC | OP_AL | OP_BT)) != 0;
-  __shared__ T sh[8][2][9][27];
-  x += blockIdx.y * vstride;
-  y += blockIdx.y * vstride;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int grp = lane / NB < CPW ? lane / NB : 0;
-  const bool lane_ok = lane < CPW * NB;
-  const int l = lane_ok ? lane - grp * NB : 0;
-  const int base = grp * NB;
-  T (*SA)[27] = sh[w][0];
-  T (*SB)[27] = sh[w][1];
-  const long long t = ((long long)bx * (blockDim.x >> 5) + w) * CPW + grp;
-  int cx = 0, cy = 0, cz = 0;
-  const bool act = lane_ok && colour_cell(col, t, cx, cy, cz);
-  const long long cell = (long long)(unsigned)(cx + g.n[0] * (cy + g.n[1] * cz));
-  const int i0 = l % 3, i1 = (l / 3) % 3, i2 = DIM == 3 ? l / 9 : 0;
-  const int ni = 2 * cx + i0, nj = 2 * cy + i1, nk = DIM == 3 ? 2 * cz + i2 : 0;
-  const long long nd = (long long)(unsigned)(ni + g.nn[0] * (nj + g.nn[1] * nk));
-  const bool bnd = on_boundary(g, ni, nj, nk);
-
-  T grad[DIM][DIM];
-#pragma unroll
-  for (int c = 0; c < DIM; ++c)
-#pragma unroll
-    for (int k = 0; k < DIM; ++k) grad[c][k] = T(0);
-  pdl_wait();
-
-  if constexpr (NEED_U) {
-    // stage 1: nodal values (Dirichlet columns masked unless RAW)
-#pragma unroll
-    for (int c = 0; c < DIM; ++c) {
-      const T v = (act && (RAW || !bnd)) ? x[c * g.N + nd] : T(0);
-      if (lane_ok) SA[c][base + l] = v;
-    }
-    __syncwarp();
-    if constexpr (DIM == 3) {
-      // stage 2 (x): lane = (qx, ay, az): B_x u, D_x u
-      if (lane_ok) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          T t0 = T(0), t1 = T(0);
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            const T v = SA[c][a + 3 * i1 + 9 * i2];
-            t0 += Ref<T>::B(i0, a) * v;
-            t1 += Ref<T>::D(i0, a) * v;
-          }
-          SB[c][l] = t0;
-          SB[3 + c][l] = t1;
-        }
-      }
-      __syncwarp();
-      // stage 3 (y): lane = (qx, qy, az): B_x B_y u, B_x D_y u, D_x B_y u
-      if (lane_ok) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          T a0 = T(0), a1 = T(0), a2 = T(0);
-#pragma unroll
-          for (int b = 0; b < 3; ++b) {
-            const T v0 = SB[c][i0 + 3 * b + 9 * i2], v1 = SB[3 + c][i0 + 3 * b + 9 * i2];
-            a0 += Ref<T>::B(i1, b) * v0;
-            a1 += Ref<T>::D(i1, b) * v0;
-            a2 += Ref<T>::B(i1, b) * v1;
-          }
-          SA[c][l] = a0;
-          SA[3 + c][l] = a1;
-          SA[6 + c][l] = a2;
-        }
-      }
-      __syncwarp();
-      // stage 4 (z): lane = (qx, qy, qz): the gradient at this point
-      if (lane_ok) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          T gx = T(0), gy = T(0), gz = T(0);
-#pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            const int idx = i0 + 3 * i1 + 9 * k;
-            gx += Ref<T>::B(i2, k) * SA[6 + c][idx];
-            gy += Ref<T>::B(i2, k) * SA[3 + c][idx];
-            gz += Ref<T>::D(i2, k) * SA[c][idx];
-          }
-          grad[c][0] = gx * cc.s[0];
-          grad[c][1] = gy * cc.s[1];
-          grad[c][2] = gz * cc.s[2];
-        }
-      }
-    } else {
-      // stage 2 (x): lane = (qx, ay): B_x u, D_x u
-      if (lane_ok) {
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          T t0 = T(0), t1 = T(0);
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            const T v = SA[c][base + a + 3 * i1];
-            t0 += Ref<T>::B(i0, a) * v;
-            t1 += Ref<T>::D(i0, a) * v;
-          }
-          SB[c][base + l] = t0;
-          SB[2 + c][base + l] = t1;
-        }
-      }
-      __syncwarp();
-      // stage 3 (y): lane = (qx, qy)
-      if (lane_ok) {
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          T gx = T(0), gy = T(0);
-#pragma unroll
-          for (int b = 0; b < 3; ++b) {
-            gx += Ref<T>::B(i1, b) * SB[2 + c][base + i0 + 3 * b];
-            gy += Ref<T>::D(i1, b) * SB[c][base + i0 + 3 * b];
-          }
-          grad[c][0] = gx * cc.s[0];
-          grad[c][1] = gy * cc.s[1];
-        }
-      }
-    }
-  }
-
-  // point weight, pressure basis at this point
-  const T wq = cc.wdet * Ref<T>::W(i0) * Ref<T>::W(i1) * (DIM == 3 ? Ref<T>::W(i2) : T(1));
-  T psi[NPR];
-  psi[0] = T(1);
-  psi[1] = Ref<T>::G(i0);
-  psi[2] = Ref<T>::G(i1);
-  if constexpr (DIM == 3) psi[3] = Ref<T>::G(i2);
-
-  // divergence moments m_p = (psi_p, div u)_K
-  T m[NPR];
-#pragma unroll
-  for (int p = 0; p < NPR; ++p) m[p] = T(0);
-  if constexpr ((MODE & (OP_AL | OP_B)) != 0) {
-    T dv = T(0);
-#pragma unroll
-    for (int c = 0; c < DIM; ++c) dv += grad[c][c];
-    dv = lane_ok ? wq * dv : T(0);
-    if constexpr (DIM == 3) {
-#pragma unroll
-      for (int p = 0; p < NPR; ++p) {
-        T v = dv * psi[p];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        m[p] = v;
-      }
-    } else {
-      __syncwarp();
-      if (lane_ok) {
-#pragma unroll
-        for (int p = 0; p < NPR; ++p) SB[p][base + l] = dv * psi[p];
-      }
-      __syncwarp();
-#pragma unroll
-      for (int p = 0; p < NPR; ++p) {
-        T v = T(0);
-#pragma unroll
-        for (int q = 0; q < 9; ++q) v += SB[p][base + q];
-        m[p] = v;
-      }
-    }
-    if constexpr ((MODE & OP_B) != 0) {
-      if (act && l < NPR) p_out[cell * NPR + l] = -m[l];
-    }
-  }
-  if constexpr (NEED_FLUX) {
-  // isotropic part of the stress: gamma Pi div u - p_h
-  T pi[NPR];
-#pragma unroll
-  for (int p = 0; p < NPR; ++p) {
-    pi[p] = T(0);
-    if constexpr ((MODE & OP_AL) != 0) {
-      if (winv) {   // W = M_p(1/mu): per-cell (d+1)^2 block of W^-1
-        T acc = T(0);
-        if (act) {
-#pragma unroll
-          for (int q = 0; q < NPR; ++q) acc += winv[(cell * NPR + p) * NPR + q] * m[q];
-        }
-        pi[p] += cc.gamma * acc;
-      } else {      // W = M_p = |K| diag(1, 1/3, ..)
-        pi[p] += cc.gamma * m[p] * (p == 0 ? cc.inv_m0 : cc.inv_m1);
-      }
-    }
-    if constexpr ((MODE & OP_BT) != 0) pi[p] -= act ? p_in[cell * NPR + p] : T(0);
-  }
-  T iso = T(0);
-#pragma unroll
-  for (int p = 0; p < NPR; ++p) iso += pi[p] * psi[p];
-  T sg[DIM][DIM];
-  if constexpr (VISC) {
-    if (act) stress<T, DIM, TENSOR>(coef + (cell * NB + l) * NCQ, grad, iso, sg);
-    else {
-#pragma unroll
-      for (int c = 0; c < DIM; ++c)
-#pragma unroll
-        for (int k = 0; k < DIM; ++k) sg[c][k] = T(0);
-    }
-  } else {
-#pragma unroll
-    for (int c = 0; c < DIM; ++c)
-#pragma unroll
-      for (int k = 0; k < DIM; ++k) sg[c][k] = (c == k) ? iso : T(0);
-  }
-  __syncwarp();
-  // fluxes F[c][k] = |J| w_q sigma_ck (2/h_k)
-  if (lane_ok) {
-#pragma unroll
-    for (int c = 0; c < DIM; ++c)
-#pragma unroll
-      for (int k = 0; k < DIM; ++k) SA[DIM * c + k][base + l] = wq * sg[c][k] * cc.s[k];
-  }
-  __syncwarp();
-  T yl[DIM];
-  if constexpr (DIM == 3) {
-    // stage 5 (z^T): lane = (qx, qy, az)
-    if (lane_ok) {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        T ge = T(0), gb = T(0), ga = T(0);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          const int idx = i0 + 3 * i1 + 9 * q;
-          ge += Ref<T>::B(q, i2) * SA[3 * c + 0][idx];
-          gb += Ref<T>::B(q, i2) * SA[3 * c + 1][idx];
-          ga += Ref<T>::D(q, i2) * SA[3 * c + 2][idx];
-        }
-        SB[c][l] = ge;
-        SB[3 + c][l] = gb;
-        SB[6 + c][l] = ga;
-      }
-    }
-    __syncwarp();
-    // stage 6 (y^T): lane = (qx, ay, az)
-    if (lane_ok) {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        T p0 = T(0), p1 = T(0);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          const int idx = i0 + 3 * q + 9 * i2;
-          p0 += Ref<T>::B(q, i1) * SB[6 + c][idx] + Ref<T>::D(q, i1) * SB[3 + c][idx];
-          p1 += Ref<T>::B(q, i1) * SB[c][idx];
-        }
-        SA[c][l] = p0;
-        SA[3 + c][l] = p1;
-      }
-    }
-    __syncwarp();
-    // stage 7 (x^T): lane = (ax, ay, az)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      T v = T(0);
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const int idx = q + 3 * i1 + 9 * i2;
-        v += Ref<T>::B(q, i0) * SA[c][idx] + Ref<T>::D(q, i0) * SA[3 + c][idx];
-      }
-      yl[c] = v;
-    }
-  } else {
-    // stage 5 (y^T): lane = (qx, ay)
-    if (lane_ok) {
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        T p0 = T(0), p1 = T(0);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          const int idx = base + i0 + 3 * q;
-          p0 += Ref<T>::D(q, i1) * SA[2 * c + 1][idx];
-          p1 += Ref<T>::B(q, i1) * SA[2 * c + 0][idx];
-        }
-        SB[c][base + l] = p0;
-        SB[2 + c][base + l] = p1;
-      }
-    }
-    __syncwarp();
-    // stage 6 (x^T): lane = (ax, ay)
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      T v = T(0);
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const int idx = base + q + 3 * i1;
-        v += Ref<T>::B(q, i0) * SB[c][idx] + Ref<T>::D(q, i0) * SB[2 + c][idx];
-      }
-      yl[c] = v;
-    }
-  }
-  if constexpr (STAGED) {
-    // staged outputs in the row layout (stage_row), summed per node by the gather in a fixed order
-    if (act) {
-#pragma unroll
-      for (int c = 0; c < DIM; ++c)
-        ebuf[(long long)stage_row(g, c, i1, i2, cy, cz) * (3 * g.n[0]) + 3 * cx + i0] = yl[c];
-    }
-  } else {
-    if (act && (RAW || !bnd)) {
-#pragma unroll
-      for (int c = 0; c < DIM; ++c) y[c * g.N + nd] += yl[c];
-    }
-  }
-  }  // NEED_FLUX
-  pdl_trigger();
-}
-template <typename T, int DIM, bool TENSOR, int MODE, bool STAGED>
-__global__ void __launch_bounds__(256) k_apply(Geom g, Colour col, CellConst<T> cc, const T* __restrict__ x,
-                                               T* __restrict__ y, const T* __restrict__ coef,
-                                               const T* __restrict__ p_in, T* __restrict__ p_out,
-                                               long long vstride, T* __restrict__ ebuf,
-                                               const T* __restrict__ winv) {
-  apply_body<T, DIM, TENSOR, MODE, STAGED>(blockIdx.x, g, col, cc, x, y, coef, p_in, p_out, vstride, ebuf, winv);
-}
-
 // y_D = x_D (identity rows) when keep_bnd, else 0; interior rows zeroed.
 template <typename T>
 __global__ void k_init_out(Geom g, const T* __restrict__ x, T* __restrict__ y, int keep_bnd, long long vstride) {
@@ -580,19 +250,38 @@ __global__ void __launch_bounds__(RED_THREADS) k_gather_epi(Geom g, const T* __r
 }
 
 #include "apply_lines.cuh"
+#include "apply_cells.cuh"
 
-// one launch of the cell kernel: the line form in 3D, the point form in 2D
-// (ZP, 3D staged only: the input comes from the star-patch outputs, see PatchIn)
+// Which form a 3D scalar apply takes.  Measured (apply_agamma call on n^3 cells, us, line form
+// against register form): FP32 16^3 32.4 / 32.7, 20^3 35.0 / 33.8, 24^3 40.0 / 35.8, 32^3
+// 54.8 / 42.3; FP64 12^3 59.3 / 71.3, 14^3 74.8 / 71.3, 16^3 90.3 / 72.0, 20^3 136 / 99 (a warp's
+// FP64 instruction takes 64 cycles of its scheduler's pipe, so the register form's longer chain
+// is a floor of about 40 us until its warps outnumber the schedulers).
+static bool cells_in_registers(const Geom& g, bool fp64) { return g.ncells >= (fp64 ? 2500 : 5000); }
+
+// the cell kernel of one apply: 2D two lanes per cell; 3D the line form, or, where a whole apply
+// is staged (STAGED; all cells, one vector), the register form on large levels
+// (ZP, staged only: the input comes from the star-patch outputs, see PatchIn)
 template <typename T, int DIM, bool TENSOR, int MODE, bool STAGED, bool ZP = false>
-static void launch_cells(dim3 grid, cudaStream_t s, const Geom& g, const Colour& col, const CellConst<T>& cc,
+static void launch_cells(int nvec, cudaStream_t s, const Geom& g, const Colour& col, const CellConst<T>& cc,
                          const T* x, T* y, const T* coef, const T* p_in, T* p_out, long long vstride, T* ebuf,
                          const T* winv, PatchIn<T> pin = PatchIn<T>{}) {
-  if constexpr (DIM == 3)
-    launch_pdl(k_apply_lines<T, TENSOR, MODE, STAGED, ZP>, grid, 256, 0, s, g, col, cc, x, y, coef, p_in, p_out,
-               vstride, ebuf, winv, pin);
-  else
-    launch_pdl(k_apply<T, DIM, TENSOR, MODE, STAGED>, grid, 256, 0, s, g, col, cc, x, y, coef, p_in, p_out, vstride,
-               ebuf, winv);
+  if constexpr (DIM == 3) {
+    if constexpr (STAGED && !TENSOR) {
+      if (cells_in_registers(g, sizeof(T) == 8)) {
+        using C = Cells3<T, MODE>;
+        launch_pdl(k_apply_cells3<T, MODE, ZP>, (unsigned)((g.ncells + C::CELLS - 1) / C::CELLS), C::THREADS, 0, s, g,
+                   cc, x, coef, p_in, p_out, ebuf, winv, pin);
+        return;
+      }
+    }
+    launch_pdl(k_apply_lines<T, TENSOR, MODE, STAGED, ZP>, dim3((unsigned)((col.count + 7) / 8), nvec), 256, 0, s, g,
+               col, cc, x, y, coef, p_in, p_out, vstride, ebuf, winv, pin);
+  } else {
+    launch_pdl(k_apply_cells2<T, TENSOR, MODE, STAGED, ZP>,
+               dim3((unsigned)((col.count + C2_CELLS - 1) / C2_CELLS), nvec), C2_THREADS, 0, s, g, col, cc, x, y,
+               coef, p_in, p_out, vstride, ebuf, winv, pin);
+  }
 }
 
 template <typename T, int DIM, bool TENSOR, int MODE>
@@ -600,7 +289,6 @@ static void launch_apply(const LevelDev& L, double gamma, const void* x, void* y
                          void* p_out, int nvec, long long vstride, cudaStream_t s) {
   const Geom& g = L.g;
   constexpr bool NEED_FLUX = (MODE & (OP_VISC | OP_AL | OP_BT)) != 0;
-  constexpr int CPB = 8 * (DIM == 2 ? 3 : 1);   // cells per 256-thread block
   const T* coef = nullptr;
   const T* winv = nullptr;
   if constexpr (std::is_same<T, double>::value) { coef = L.coef64; winv = L.winv64; }
@@ -609,7 +297,7 @@ static void launch_apply(const LevelDev& L, double gamma, const void* x, void* y
   if (nvec == 1 && L.ebuf) {
     // one launch over all cells into the per-cell buffer, one gather launch per node
     const Colour col = all_cells(g);
-    launch_cells<T, DIM, TENSOR, MODE, true>(dim3((unsigned)((col.count + CPB - 1) / CPB)), s, g, col,
+    launch_cells<T, DIM, TENSOR, MODE, true>(1, s, g, col,
                                              cell_const<T>(g, gamma), (const T*)x, (T*)y, coef, (const T*)p_in,
                                              (T*)p_out, 0, (T*)L.ebuf, winv);
     if (NEED_FLUX) {
@@ -631,8 +319,7 @@ static void launch_apply(const LevelDev& L, double gamma, const void* x, void* y
     const int ncol = NEED_FLUX ? (1 << DIM) : 1;   // B u alone is cell-local: one launch
     for (int colour = 0; colour < ncol; ++colour) {
       const Colour col = NEED_FLUX ? make_colour(g, colour) : all_cells(g);
-      dim3 grid((unsigned)((col.count + CPB - 1) / CPB), nv);
-      launch_cells<T, DIM, TENSOR, MODE, false>(grid, s, g, col, cell_const<T>(g, gamma), xv, yv, coef,
+      launch_cells<T, DIM, TENSOR, MODE, false>(nv, s, g, col, cell_const<T>(g, gamma), xv, yv, coef,
                                                 (const T*)p_in, (T*)p_out, vstride, nullptr, winv);
     }
     count_launch((NEED_FLUX ? 1 : 0) + ncol);
@@ -704,7 +391,6 @@ template <typename T, int DIM, bool TENSOR>
 static void launch_apply_epi(const LevelDev& L, double gamma, const void* x, void* y, const ApplyEpi& e,
                              cudaStream_t s, cudaEvent_t e0, cudaEvent_t e1) {
   const Geom& g = L.g;
-  constexpr int CPB = 8 * (DIM == 2 ? 3 : 1);
   const T* coef = nullptr;
   const T* winv = nullptr;
   if constexpr (std::is_same<T, double>::value) { coef = L.coef64; winv = L.winv64; }
@@ -712,18 +398,12 @@ static void launch_apply_epi(const LevelDev& L, double gamma, const void* x, voi
   const Colour col = all_cells(g);
   // External records become event-record nodes when the stream is being captured
   if (e0) cudaEventRecordWithFlags(e0, s, cudaEventRecordExternal);
-  const dim3 grid((unsigned)((col.count + CPB - 1) / CPB));
-  bool fused = false;
-  if constexpr (DIM == 3 && std::is_same<T, float>::value) {
-    if (e.pout) {   // x = z formed from the patch outputs; z stored on the way
-      launch_cells<T, DIM, TENSOR, OP_VISC | OP_AL, true, true>(
-          grid, s, g, col, cell_const<T>(g, gamma), nullptr, (T*)y, coef, nullptr, nullptr, 0, (T*)L.ebuf, winv,
-          PatchIn<T>{(const T*)e.pout, (T*)x});
-      fused = true;
-    }
-  }
-  if (!fused)
-    launch_cells<T, DIM, TENSOR, OP_VISC | OP_AL, true>(grid, s, g, col, cell_const<T>(g, gamma), (const T*)x, (T*)y,
+  if (e.pout)   // x = z formed from the patch outputs; z stored on the way
+    launch_cells<T, DIM, TENSOR, OP_VISC | OP_AL, true, true>(
+        1, s, g, col, cell_const<T>(g, gamma), nullptr, (T*)y, coef, nullptr, nullptr, 0, (T*)L.ebuf, winv,
+        PatchIn<T>{(const T*)e.pout, (T*)x});
+  else
+    launch_cells<T, DIM, TENSOR, OP_VISC | OP_AL, true>(1, s, g, col, cell_const<T>(g, gamma), (const T*)x, (T*)y,
                                                          coef, nullptr, nullptr, 0, (T*)L.ebuf, winv);
   if (e1) cudaEventRecordWithFlags(e1, s, cudaEventRecordExternal);
   launch_pdl(k_gather_epi<T, DIM>, apply_epi_blocks(L), RED_THREADS, 0, s, g, (const T*)L.ebuf, (const T*)x, (T*)y,
@@ -762,7 +442,7 @@ void op_apply_epi(const LevelDev& L, int prec, double gamma, const void* x, void
 
 // ---------------------------------------------------------------------------
 // merged launches (batch.cuh): FP32, scalar viscosity, 2D and 3D instances in one launch
-// (the line form for 3D items, the point form for 2D items, as for a single instance)
+// (each item in the form its single-instance apply takes)
 // ---------------------------------------------------------------------------
 struct CellArgs {
   Geom g;
@@ -775,19 +455,30 @@ struct CellArgs {
   const float* winv;
   PatchIn<float> pin;
 };
-// ZP: 3D items form x from their star-patch outputs (PatchIn), as op_apply_epi does with
-// ApplyEpi::pout; 2D items never do
+// ZP: x is formed from the star-patch outputs (PatchIn), as op_apply_epi does with ApplyEpi::pout.
+// Three kernels, for 2D items, 3D items in the line form and 3D items in the register form
 template <int MODE, bool ZP>
-__global__ void __launch_bounds__(256) k_cells_b(const __grid_constant__ BatchTab<CellArgs> tb) {
+__global__ void __launch_bounds__(C2_THREADS) k_cells2_b(const __grid_constant__ BatchTab<CellArgs> tb) {
   const int i = batch_slot(tb, blockIdx.x);
   const CellArgs& a = tb.a[i];
-  const unsigned bx = blockIdx.x - tb.start[i];
-  if (a.g.dim == 3)
-    apply_lines_body<float, false, MODE, true, ZP>(bx, a.g, a.col, a.cc, a.x, a.y, a.coef, nullptr, nullptr, 0,
-                                                   a.ebuf, a.winv, a.pin);
-  else
-    apply_body<float, 2, false, MODE, true>(bx, a.g, a.col, a.cc, a.x, a.y, a.coef, nullptr, nullptr, 0, a.ebuf,
-                                            a.winv);
+  apply_cells2_body<float, false, MODE, true, ZP>((blockIdx.x - tb.start[i]) * (C2_THREADS / 32) + threadIdx.x / 32,
+                                                  a.g, a.col, a.cc, a.x, a.y, a.coef, nullptr, nullptr, 0, a.ebuf, a.winv, a.pin);
+}
+template <int MODE, bool ZP>
+__global__ void __launch_bounds__(256) k_lines_b(const __grid_constant__ BatchTab<CellArgs> tb) {
+  const int i = batch_slot(tb, blockIdx.x);
+  const CellArgs& a = tb.a[i];
+  apply_lines_body<float, false, MODE, true, ZP>(blockIdx.x - tb.start[i], a.g, a.col, a.cc, a.x, a.y, a.coef, nullptr,
+                                                 nullptr, 0, a.ebuf, a.winv, a.pin);
+}
+template <int MODE, bool ZP>
+__global__ void __launch_bounds__(Cells3<float, MODE>::THREADS, Cells3<float, MODE>::BLOCKS)
+    k_cells3_b(const __grid_constant__ BatchTab<CellArgs> tb) {
+  __shared__ typename Cells3<float, MODE>::Smem sm;
+  const int i = batch_slot(tb, blockIdx.x);
+  const CellArgs& a = tb.a[i];
+  apply_cells3_body<float, MODE, ZP>(blockIdx.x - tb.start[i], a.g, a.cc, a.x, a.coef, nullptr, nullptr, a.ebuf,
+                                     a.winv, a.pin, sm);
 }
 
 struct GatherArgs {
@@ -833,32 +524,31 @@ static CellArgs cell_args(const BApply& it, bool zp) {
   if (zp) a.pin = PatchIn<float>{(const float*)it.e.pout, (float*)it.x};
   return a;
 }
-static unsigned cell_blocks(const Geom& g) {
-  const long long cpb = g.dim == 2 ? 24 : 8;
-  return (unsigned)((g.ncells + cpb - 1) / cpb);
-}
-
-// the cell kernels of every item: 3D items with star-patch input (e.pout) in the ZP
-// kernel together with the 2D items, the other 3D items in the plain kernel
-template <int MODE>
-static int batch_cells(const std::vector<BApply>& items, bool use_pout, cudaStream_t s) {
-  std::vector<CellArgs> zp, plain;
-  std::vector<unsigned> nzp, nplain;
-  bool any_zp = false;
-  for (const BApply& it : items) any_zp |= use_pout && it.L->g.dim == 3 && it.e.pout;
+// the cell kernels of every item (all of them with star-patch input, or none), one launch per
+// kernel that some item takes
+template <int MODE, bool ZP>
+static int batch_cells(const std::vector<BApply>& items, cudaStream_t s) {
+  std::vector<CellArgs> a[3];
+  std::vector<unsigned> nb[3];
+  using C3 = Cells3<float, MODE>;
+  const int per[3] = {C2_CELLS, 8, C3::CELLS};
   for (const BApply& it : items) {
-    const bool z3 = use_pout && it.L->g.dim == 3 && it.e.pout;
-    if (z3 || (any_zp && it.L->g.dim == 2)) { zp.push_back(cell_args(it, z3)); nzp.push_back(cell_blocks(it.L->g)); }
-    else { plain.push_back(cell_args(it, false)); nplain.push_back(cell_blocks(it.L->g)); }
+    const Geom& g = it.L->g;
+    const int k = g.dim == 2 ? 0 : (cells_in_registers(g, false) ? 2 : 1);
+    a[k].push_back(cell_args(it, ZP));
+    nb[k].push_back((unsigned)((g.ncells + per[k] - 1) / per[k]));
   }
   int n = 0;
-  if (!zp.empty()) n += launch_batch(k_cells_b<MODE, true>, zp, nzp, 256, 0, s);
-  if (!plain.empty()) n += launch_batch(k_cells_b<MODE, false>, plain, nplain, 256, 0, s);
+  if (!a[0].empty()) n += launch_batch(k_cells2_b<MODE, ZP>, a[0], nb[0], C2_THREADS, 0, s);
+  if (!a[1].empty()) n += launch_batch(k_lines_b<MODE, ZP>, a[1], nb[1], 256, 0, s);
+  if (!a[2].empty())
+    n += launch_batch(k_cells3_b<MODE, ZP>, a[2], nb[2], C3::THREADS, 0, s);
   return n;
 }
 
 int batch_apply_epi(const std::vector<BApply>& items, cudaStream_t s) {
-  int n = batch_cells<OP_VISC | OP_AL>(items, true, s);
+  const bool zp = !items.empty() && items[0].e.pout;   // a smoothing's items agree
+  int n = zp ? batch_cells<OP_VISC | OP_AL, true>(items, s) : batch_cells<OP_VISC | OP_AL, false>(items, s);
   std::vector<GatherArgs> a;
   std::vector<unsigned> nb;
   for (const BApply& it : items) {
@@ -873,7 +563,7 @@ int batch_apply_epi(const std::vector<BApply>& items, cudaStream_t s) {
 }
 
 int batch_apply_al(const std::vector<BApply>& items, cudaStream_t s) {
-  int n = batch_cells<OP_AL>(items, false, s);
+  int n = batch_cells<OP_AL, false>(items, s);
   std::vector<GatherArgs> a;
   std::vector<unsigned> nb;
   for (const BApply& it : items) {

@@ -1244,17 +1244,15 @@ size_t patch_scratch_bytes(const LevelDev& L, int prec) {
   return (size_t)L.g.nverts * L.np * (prec == PREC_F64 ? sizeof(double) : sizeof(float));
 }
 
-template <typename TF, typename TV, int DIM>
-static void smooth_impl(const LevelDev& L, const TF* inv, const void* r, void* z, void* scratch, cudaStream_t s,
-                        cudaEvent_t e0, cudaEvent_t e1) {
-  const long long warps = L.g.nverts;
-  const unsigned blocks = (unsigned)std::min<long long>((warps + 7) / 8, 152LL * 16);
+template <int DIM>
+static void star_products64(const LevelDev& L, const double* r, double* scratch, cudaStream_t s, cudaEvent_t e0,
+                            cudaEvent_t e1) {
+  const unsigned blocks = (unsigned)std::min<long long>((L.g.nverts + 7) / 8, 152LL * 16);
   // External records become event-record nodes when the stream is being captured
   if (e0) cudaEventRecordWithFlags(e0, s, cudaEventRecordExternal);
-  launch_pdl(k_patch_apply<TF, TV, DIM>, blocks, 256, 0, s, L.g, inv, L.pstride, (const TV*)r, (TV*)scratch);
+  launch_pdl(k_patch_apply<double, double, DIM>, blocks, 256, 0, s, L.g, L.inv64, L.pstride, r, scratch);
   if (e1) cudaEventRecordWithFlags(e1, s, cudaEventRecordExternal);
-  launch_pdl(k_patch_gather<TV, DIM>, row_gather_blocks(L.g, DIM), 256, 0, s, L.g, (const TV*)scratch, (TV*)z);
-  count_launch(2);
+  count_launch(1);
 }
 
 // All star products y_v = A_v^-1 r|_v of a level into the scratch rows (FP32) with kernel
@@ -1269,19 +1267,21 @@ static void star_products(int v, const LevelDev& L, const float* r, float* scrat
   if (L.split) launch_patch_bnd<DIM>(L, r, scratch, s);
 }
 
-template <int DIM>
-static void smooth_tma(const LevelDev& L, const void* r, void* z, void* scratch, cudaStream_t s, cudaEvent_t e0,
-                       cudaEvent_t e1) {
-  star_products<DIM>(patch_variant(L), L, (const float*)r, (float*)scratch, s, e0, e1);
-  launch_pdl(k_patch_gather<float, DIM>, row_gather_blocks(L.g, DIM), 256, 0, s, L.g, (const float*)scratch,
-             (float*)z);
-  count_launch(1);
+void patch_products(const LevelDev& L, int prec, const void* r, void* scratch, cudaStream_t s, cudaEvent_t e0,
+                    cudaEvent_t e1) {
+  if (prec == PREC_F64) {
+    if (L.g.dim == 2) star_products64<2>(L, (const double*)r, (double*)scratch, s, e0, e1);
+    else star_products64<3>(L, (const double*)r, (double*)scratch, s, e0, e1);
+  } else {
+    if (L.g.dim == 2) star_products<2>(patch_variant(L), L, (const float*)r, (float*)scratch, s, e0, e1);
+    else star_products<3>(patch_variant(L), L, (const float*)r, (float*)scratch, s, e0, e1);
+  }
 }
 
-void patch_products(const LevelDev& L, const void* r, void* scratch, cudaStream_t s, cudaEvent_t e0,
-                    cudaEvent_t e1) {
-  if (L.g.dim == 2) star_products<2>(patch_variant(L), L, (const float*)r, (float*)scratch, s, e0, e1);
-  else star_products<3>(patch_variant(L), L, (const float*)r, (float*)scratch, s, e0, e1);
+template <typename T, int DIM>
+static void launch_patch_gather(const LevelDev& L, const void* scratch, void* z, cudaStream_t s) {
+  launch_pdl(k_patch_gather<T, DIM>, row_gather_blocks(L.g, DIM), 256, 0, s, L.g, (const T*)scratch, (T*)z);
+  count_launch(1);
 }
 
 void patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, cudaStream_t s,
@@ -1292,12 +1292,13 @@ void patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scr
     if (e1) cudaEventRecordWithFlags(e1, s, cudaEventRecordExternal);
     return;
   }
+  patch_products(L, prec, r, scratch, s, e0, e1);
   if (prec == PREC_F64) {
-    if (L.g.dim == 2) smooth_impl<double, double, 2>(L, L.inv64, r, z, scratch, s, e0, e1);
-    else smooth_impl<double, double, 3>(L, L.inv64, r, z, scratch, s, e0, e1);
+    if (L.g.dim == 2) launch_patch_gather<double, 2>(L, scratch, z, s);
+    else launch_patch_gather<double, 3>(L, scratch, z, s);
   } else {
-    if (L.g.dim == 2) smooth_tma<2>(L, r, z, scratch, s, e0, e1);
-    else smooth_tma<3>(L, r, z, scratch, s, e0, e1);
+    if (L.g.dim == 2) launch_patch_gather<float, 2>(L, scratch, z, s);
+    else launch_patch_gather<float, 3>(L, scratch, z, s);
   }
 }
 
