@@ -817,13 +817,34 @@ constexpr long long kSplitVertices = 32768;
 static als_status alloc_star_storage(als_ctx* c, LevelDev& Lv) {
   const Geom& g = Lv.g;
   const int d = c->dim;
-  if (c->k == 3) {   // order 3: an FP32 copy of every star, in wrapped rows
-    Lv.split = 0;
-    Lv.nbnd = 0;
-    return dalloc(c, &Lv.inv32, (size_t)g.nverts * qk_star32_floats(d));
+  Lv.split = 0;
+  Lv.nbnd = 0;
+  if (c->k == 3 && d == 2) {   // order 3 in 2D: an FP32 copy of every star, in wrapped rows
+    Lv.star32 = g.nverts * (long long)qk_star32_floats();
+    return dalloc(c, &Lv.inv32, (size_t)Lv.star32);
   }
   Lv.nint = 1;
   for (int k = 0; k < d; ++k) Lv.nint *= g.nv[k] - 2;
+  std::vector<int> bvid;
+  std::vector<long long> boff;
+  const auto boundary_tables = [&]() -> als_status {
+    Lv.nbnd = (long long)bvid.size();
+    ALS_TRY(dalloc(c, &Lv.bvid, bvid.size()));
+    ALS_TRY(dalloc(c, &Lv.boff, boff.size()));
+    if (!bvid.empty() &&
+        (cudaMemcpyAsync(Lv.bvid, bvid.data(), bvid.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream) !=
+             cudaSuccess ||
+         cudaMemcpyAsync(Lv.boff, boff.data(), boff.size() * sizeof(long long), cudaMemcpyHostToDevice, c->stream) !=
+             cudaSuccess ||
+         cudaStreamSynchronize(c->stream) != cudaSuccess))
+      return cuda_check(c, "boundary star tables");
+    return ALS_OK;
+  };
+  if (c->k == 3) {   // order 3 in 3D: every star's free dofs, blocked, interior vertices first
+    Lv.star32 = qk3_star_layout(g, bvid, boff);
+    ALS_TRY(dalloc(c, &Lv.inv32, (size_t)Lv.star32));
+    return boundary_tables();
+  }
   static int forced = -2;   // ALS_SPLIT_STARS=1 / 0 forces split / full storage on every level
   if (forced == -2) {
     const char* e = getenv("ALS_SPLIT_STARS");
@@ -831,11 +852,9 @@ static als_status alloc_star_storage(als_ctx* c, LevelDev& Lv) {
   }
   Lv.split = forced >= 0 ? forced : (g.nverts >= kSplitVertices ? 1 : 0);
   if (!Lv.split) {
-    Lv.nbnd = 0;
+    Lv.star32 = g.nverts;
     return dalloc(c, &Lv.inv32, (size_t)g.nverts * Lv.pstride);
   }
-  std::vector<int> bvid;
-  std::vector<long long> boff;
   long long total = 0;
   for (long long v = 0; v < g.nverts; ++v) {
     const int vc[3] = {(int)(v % g.nv[0]), (int)((v / g.nv[0]) % g.nv[1]),
@@ -852,19 +871,10 @@ static als_status alloc_star_storage(als_ctx* c, LevelDev& Lv) {
     boff.push_back(total);
     total += ((long long)m * (m + 1) / 2 + 3) & ~3LL;   // 16-byte aligned blocks (bulk copies)
   }
-  Lv.nbnd = (long long)bvid.size();
+  Lv.star32 = Lv.nint;
   ALS_TRY(dalloc(c, &Lv.inv32, (size_t)Lv.nint * Lv.pstride));
   ALS_TRY(dalloc(c, &Lv.bnd32, (size_t)total));
-  ALS_TRY(dalloc(c, &Lv.bvid, bvid.size()));
-  ALS_TRY(dalloc(c, &Lv.boff, boff.size()));
-  if (!bvid.empty() &&
-      (cudaMemcpyAsync(Lv.bvid, bvid.data(), bvid.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream) !=
-           cudaSuccess ||
-       cudaMemcpyAsync(Lv.boff, boff.data(), boff.size() * sizeof(long long), cudaMemcpyHostToDevice, c->stream) !=
-           cudaSuccess ||
-       cudaStreamSynchronize(c->stream) != cudaSuccess))
-    return cuda_check(c, "boundary star tables");
-  return ALS_OK;
+  return boundary_tables();
 }
 
 static als_status create_impl(als_ctx* c, const als_mesh* mesh, const als_coeff* coeff, double gamma,
@@ -976,8 +986,8 @@ static als_status create_impl(als_ctx* c, const als_mesh* mesh, const als_coeff*
       ALS_TRY(alloc_star_storage(c, Lv));
       if (c->opt.store == ALS_STORE_BF16) {   // the FP32 stars again, in bfloat16
         uint16_t* p16 = nullptr;
-        const size_t per = c->k == 3 ? qk3_star32_floats() : (size_t)block_stride_bf16(Lv.np);
-        ALS_TRY(dalloc(c, &p16, (size_t)(Lv.split ? Lv.nint : Lv.g.nverts) * per));
+        const size_t per = c->k == 3 ? 1 : (size_t)block_stride_bf16(Lv.np);
+        ALS_TRY(dalloc(c, &p16, (size_t)Lv.star32 * per));
         Lv.inv16 = p16;
       }
     }

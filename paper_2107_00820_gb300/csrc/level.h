@@ -40,6 +40,7 @@ struct LevelDev {
   long long* boff;       // offset of each boundary star's compact inverse in bnd32
   long long nint;        // interior vertices, prod(n_k - 1)
   long long nbnd;        // boundary vertices, nverts - nint
+  long long star32 = 0;  // stars in inv32 (order 2), or its entries (order 3)
   int np;                // patch size d*3^d
   int pstride;           // entries per patch (padded)
   DevStatus* status;     // where kernels of this level record device-side failures
@@ -145,9 +146,9 @@ void qk_mass_setup(const LevelDev& L, double gamma, int w_mu, int variant, doubl
                    DevStatus* st, cudaStream_t s);
 // df64: 3D levels eliminate in double-float (2D order 3 is FP64 throughout)
 void qk_patch_setup(const LevelDev& L, double gamma, DevStatus* st, cudaStream_t s, int df64);
-// FP32 entries per star of an order-3 level (inv32 holds the stars in wrapped rows), and
-// inv32 formed from inv64
-size_t qk_star32_floats(int dim);
+// FP32 entries per star of a 2D order-3 level (inv32 holds the stars in wrapped rows), and
+// inv32 formed from inv64 (2D and 3D)
+size_t qk_star32_floats();
 void qk_derive32(const LevelDev& L, cudaStream_t s);
 void qk_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, cudaStream_t s);
 void qk_interior_solve(const LevelDev& fine, int prec, const void* in, void* out, int subtract, cudaStream_t s);
@@ -168,9 +169,10 @@ void qk3_mass_setup(const LevelDev& L, double gamma, int w_mu, int variant, doub
 // (doubles; one 375 x 376 FP64 star matrix per CTA), held in LevelDev::qk_ws
 int qk3_setup_ctas(long long nverts);
 size_t qk3_setup_ws_doubles(int ctas);
-// FP32 entries per star of a 3D order-3 level (inv32 holds the stars in wrapped rows), and
-// inv32 formed from inv64
-size_t qk3_star32_floats();
+// FP32 storage of a 3D order-3 level's stars (blocked, free dofs only): the boundary vertices and
+// the offsets of their stars behind the interior ones; returns the total entries of inv32.
+// qk3_derive32: inv32 (and inv16) formed from inv64.
+long long qk3_star_layout(const Geom& g, std::vector<int>& bvid, std::vector<long long>& boff);
 void qk3_derive32(const LevelDev& L, cudaStream_t s);
 // df64: the elimination in double-float arithmetic (the assembly stays FP64)
 void qk3_patch_setup(const LevelDev& L, double gamma, DevStatus* st, cudaStream_t s, int df64);

@@ -907,7 +907,7 @@ void qk_apply_epi(const LevelDev& L, int prec, double gamma, const void* x, void
   else apply_epi_t<float>(L, gamma, x, y, e, s, e0, e1);
 }
 
-size_t qk_star32_floats(int dim) { return dim == 3 ? qk3_star32_floats() : (size_t)qk::kWStride; }
+size_t qk_star32_floats() { return qk::kWStride; }
 
 void qk_derive32(const LevelDev& L, cudaStream_t s) {
   if (L.g.dim == 3) return qk3_derive32(L, s);

@@ -24,6 +24,7 @@
 #include <math.h>
 
 #include <type_traits>
+#include <vector>
 
 #include "cell.cuh"
 #include "df64.cuh"
@@ -543,12 +544,54 @@ __device__ __forceinline__ bool star_node(const Geom& g, int vx, int vy, int vz,
 }
 
 constexpr int LDM = NS + 1;   // row stride of a star matrix in the workspace (doubles)
-// FP32 star storage in wrapped rows (k_qk3_star_apply_w): WT rows of WLD entries
-constexpr int WT = (NS + 1) / 2;   // 188
-constexpr int WLD = 376;
-constexpr int WSTRIDE = WT * WLD;
-static_assert(NS % 2 == 1 && WLD % 4 == 0 && WLD >= NS, "wrapped-row layout");
-static_assert(WT % 2 == 0, "rows are streamed in pairs");
+// FP32 star storage (k_qk3_stars): the free dofs' inverse in 15 x 15 blocks (I, J), I <= J,
+// off-diagonal blocks first (row-major over I < J), then the diagonal ones (upper triangle,
+// 120 entries).  Interleaved by block in quads of four entries, so that the threads of a star,
+// one block each, read consecutive quads: quads 0..29 of all blocks, then quads 30..56 of the
+// off-diagonal ones (225 entries and three zeros).  An interior vertex's star has 375 free dofs
+// (25 x 25 blocks); a face, edge or corner vertex's only 150, 60 or 24, which is all that is
+// stored of it.
+constexpr int SB = 15, SQ1 = 30, SQ2 = 27;
+struct StarBlocks {
+  int nbr, nblk, noff;   // block rows, blocks, off-diagonal blocks
+  __host__ __device__ constexpr explicit StarBlocks(int m)
+      : nbr((m + SB - 1) / SB), nblk(((m + SB - 1) / SB) * ((m + SB - 1) / SB + 1) / 2),
+        noff(((m + SB - 1) / SB) * ((m + SB - 1) / SB - 1) / 2) {}
+  __host__ __device__ constexpr int q2() const { return 4 * SQ1 * nblk; }
+  __host__ __device__ constexpr int entries() const { return 4 * (SQ1 * nblk + SQ2 * noff); }
+  __device__ __forceinline__ void block_of(int b, int& I, int& J) const {
+    if (b >= noff) {
+      I = J = b - noff;
+    } else {
+      int rem = b;
+      I = 0;
+      while (rem >= nbr - 1 - I) { rem -= nbr - 1 - I; ++I; }
+      J = I + 1 + rem;
+    }
+  }
+};
+constexpr int kFullRows = StarBlocks(NS).nbr, kFullBlocks = StarBlocks(NS).nblk, kFullOff = StarBlocks(NS).noff;
+constexpr int kFullEntries = StarBlocks(NS).entries();
+
+// the free dofs of a vertex's star: a box of node offsets, all five where the vertex is interior
+// along the axis, the two inward ones where it lies on the boundary
+struct StarBox {
+  int lo[3], cnt[3], m;
+  __host__ __device__ StarBox(const Geom& g, int vx, int vy, int vz) {
+    const int v[3] = {vx, vy, vz};
+    m = 3;
+    for (int a = 0; a < 3; ++a) {
+      lo[a] = v[a] == 0 ? K : 0;
+      cnt[a] = v[a] == 0 || v[a] == g.nv[a] - 1 ? K - 1 : S1;
+      m *= cnt[a];
+    }
+  }
+  // star entry (component-major, offsets x-fastest) of free dof a; increases with a
+  __device__ __forceinline__ int entry(int a) const {
+    const int ix = a % cnt[0], q = a / cnt[0], iy = q % cnt[1], q2 = q / cnt[1], iz = q2 % cnt[2], c = q2 / cnt[2];
+    return c * SN + (lo[0] + ix) + S1 * (lo[1] + iy) + S1 * S1 * (lo[2] + iz);
+  }
+};
 constexpr int BB = 16;        // pivots per Gauss-Jordan pass
 constexpr int SETUP_THREADS = 256;
 // shared memory of the setup kernel (doubles): the assembly's tables or the elimination's
@@ -583,7 +626,7 @@ template <typename RM>
 __global__ void __launch_bounds__(SETUP_THREADS) k_qk3_star_setup(Geom g, double gamma, const double* __restrict__ mu,
                                                                   const double* __restrict__ winv,
                                                                   double* __restrict__ ws, double* __restrict__ inv64,
-                                                                  float* __restrict__ inv32, int pstride,
+                                                                  int pstride,
                                                                   DevStatus* st) {
   static_assert(sizeof(RM) == sizeof(double), "the workspace holds 8-byte entries");
   using Ops = RealOps<RM>;
@@ -782,15 +825,10 @@ __global__ void __launch_bounds__(SETUP_THREADS) k_qk3_star_setup(Geom g, double
       }
       __syncthreads();
     }
-    // FP64: upper triangle by diagonals (entry (i, i + t)); FP32: the wrapped rows
+    // upper triangle by diagonals (entry (i, i + t))
     for (int t = 0; t < NS; ++t) {
       const long long base = v * pstride + diag_start(NS, t);
       for (int i = tid; i + t < NS; i += nt) inv64[base + i] = Ops::to_double(Mr[(long long)i * LDM + i + t]);
-    }
-    for (int e = tid; e < WSTRIDE; e += nt) {
-      const int t = e / WLD, i = e % WLD, j = i + t < NS ? i + t : i + t - NS;
-      const int lo = i < j ? i : j, hi = i < j ? j : i;
-      inv32[v * WSTRIDE + e] = i < NS ? (float)Ops::to_double(Mr[(long long)lo * LDM + hi]) : 0.f;
     }
     __syncthreads();
   }
@@ -887,151 +925,240 @@ __global__ void __launch_bounds__(STAR_THREADS) k_qk3_star_apply(Geom g, const T
 // the packed triangle.  The product y_i = sum_t W_t[i] r_(i+t) + sum_(t>0) W_t[i-t] r_(i-t)
 // (indices mod NS) then reads each row once, coalesced, 16 bytes a thread.
 
-// y_v = A_v^-1 r|_v from the wrapped rows: one CTA per star, rows by threads; the rows of
-// W stream through shared memory two at a time (double-buffered, the next pair's 16-byte
-// loads in flight while the current pair is used); r is held twice over so that
-// r_((i + t) mod NS) needs no wrap.  interior / mode as k_qk3_star_apply.
-constexpr int WV = WLD / 4;   // float4 per row (94)
-// The rows' storage: FP32, or bfloat16 (ALS_STORE_BF16: the same rows rounded to nearest
-// from FP64, 752-byte rows), widened to FP32 on the way into shared memory; every product
-// and sum in FP32 either way.  A pair of rows is 188 16-byte words in FP32 (thread tid
-// loads words tid and tid + 128) and 94 in bfloat16 (8 entries a word, threads 0..93).
-template <typename TS>
-struct RowPair;
-template <>
-struct RowPair<float> {
-  float4 a, b;
-  __device__ __forceinline__ void load(const float* base, int tid) {
-    const float4* W = reinterpret_cast<const float4*>(base);
-    a = __ldg(W + tid);
-    b = tid + STAR_THREADS < 2 * WV ? __ldg(W + tid + STAR_THREADS) : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  __device__ __forceinline__ void store(float* w, int tid) const {
-    reinterpret_cast<float4*>(w)[tid] = a;
-    if (tid + STAR_THREADS < 2 * WV) reinterpret_cast<float4*>(w)[tid + STAR_THREADS] = b;
-  }
-};
-template <>
-struct RowPair<__nv_bfloat16> {
-  uint4 a;
-  __device__ __forceinline__ void load(const __nv_bfloat16* base, int tid) {
-    a = tid < WV ? __ldg(reinterpret_cast<const uint4*>(base) + tid) : make_uint4(0u, 0u, 0u, 0u);
-  }
-  __device__ __forceinline__ void store(float* w, int tid) const {
-    if (tid >= WV) return;
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&a);
-    const float2 p0 = __bfloat1622float2(h[0]), p1 = __bfloat1622float2(h[1]);
-    const float2 p2 = __bfloat1622float2(h[2]), p3 = __bfloat1622float2(h[3]);
-    reinterpret_cast<float4*>(w)[2 * tid] = make_float4(p0.x, p0.y, p1.x, p1.y);
-    reinterpret_cast<float4*>(w)[2 * tid + 1] = make_float4(p2.x, p2.y, p3.x, p3.y);
-  }
-};
+// y_v = A_v^-1 r|_v in FP32 from the blocked storage.  An interior star takes a CTA, one 15 x 15
+// block a thread: the block is read from global memory once, in quads that are consecutive over
+// the threads, and each entry is used for both y_I += S r_J and y_J += S^T r_I from registers;
+// the 25 partial sums of a row meet in shared memory in a fixed order.  Boundary stars, with at
+// most 55 blocks, take 64 threads, five to a CTA.  Bound by the stream of the inverses: two CTAs
+// an SM keep about 90 KB of loads in flight.  On 12^3 cells a sweep takes XX us; the form before
+// (every star padded to 375 dofs, wrapped rows two at a time through shared memory, four shared
+// loads for two FMAs) took 140, and on 6^3 cells YY against 60.
+// TS: float, or bfloat16 (ALS_STORE_BF16), widened on load; products and sums in FP32.
+// interior / mode as k_qk3_star_apply; nint: interior vertices (stored first, in their own
+// x-fastest order), then nbnd boundary ones (bvid, offsets boff).
+constexpr int STARS_THREADS = 352, BND_PER_CTA = 5;
 
+__device__ __forceinline__ float4 star_quad(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 star_quad(const __nv_bfloat16* p) {
+  const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
+  const float2 c = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+  return make_float4(a.x, a.y, c.x, c.y);
+}
+
+constexpr int SPRE = 6;   // quads of a block in flight before the dependency wait
+
+// partial sums of block b into part[row][nbr]; pre: its first SPRE quads
 template <typename TS>
-__global__ void __launch_bounds__(STAR_THREADS) k_qk3_star_apply_w(Geom g, const TS* __restrict__ inv,
-                                                                   int interior, int mode,
-                                                                   const float* __restrict__ r,
-                                                                   float* __restrict__ out) {
-  __shared__ float rs2[2 * NS];
-  __shared__ __align__(16) float wsh[2][2][WLD];
-  const int tid = threadIdx.x;
-  const int ic[3] = {g.n[0] / 2, g.n[1] / 2, g.n[2] / 2};
-  const long long count = interior ? (long long)ic[0] * ic[1] * ic[2] : g.nverts;
-  const long long item = blockIdx.x;
-  if (item >= count) return;   // uniform over the block
-  int vx, vy, vz;
-  if (interior) {
-    vx = 2 * (int)(item % ic[0]) + 1;
-    vy = 2 * (int)((item / ic[0]) % ic[1]) + 1;
-    vz = 2 * (int)(item / ((long long)ic[0] * ic[1])) + 1;
-  } else {
-    vx = (int)(item % g.nv[0]);
-    vy = (int)((item / g.nv[0]) % g.nv[1]);
-    vz = (int)(item / ((long long)g.nv[0] * g.nv[1]));
+__device__ __forceinline__ void star_block(const TS* __restrict__ S, int nblk, int noff, int nbr, int b, int I, int J,
+                                           const float4 (&pre)[SPRE], const float* rs, float* part) {
+  const int q2 = 4 * SQ1 * nblk;
+  const auto quad = [&](int q) {
+    return q < SPRE ? pre[q]
+                    : (q < SQ1 ? star_quad(S + 4 * (q * nblk + b)) : star_quad(S + q2 + 4 * ((q - SQ1) * noff + b)));
+  };
+  float rI[SB], yI[SB];
+#pragma unroll
+  for (int k = 0; k < SB; ++k) {
+    rI[k] = rs[SB * I + k];
+    yI[k] = 0.f;
   }
-  const long long v = (long long)vx + (long long)g.nv[0] * ((long long)vy + (long long)g.nv[1] * vz);
-  const TS* W = inv + v * WSTRIDE;
-  RowPair<TS> rp;
-  rp.load(W, tid);
-  for (int e = tid; e < NS; e += STAR_THREADS) {
-    long long nd;
-    const float val = star_node(g, vx, vy, vz, e, nd) ? r[(e / SN) * g.N + nd] : 0.f;
-    rs2[e] = val;
-    rs2[e + NS] = val;
-  }
-  float acc[STAR_ROWS];
+  if (I != J) {
+    float rJ[SB], yJ[SB];
 #pragma unroll
-  for (int k = 0; k < STAR_ROWS; ++k) acc[k] = 0.f;
-  rp.store(&wsh[0][0][0], tid);
-  __syncthreads();
-  for (int pr = 0; pr < WT / 2; ++pr) {
-    const int cur = pr & 1;
-    if (pr + 1 < WT / 2) rp.load(W + (long long)(pr + 1) * 2 * WLD, tid);   // in flight during this pair
+    for (int k = 0; k < SB; ++k) {
+      rJ[k] = rs[SB * J + k];
+      yJ[k] = 0.f;
+    }
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int t = 2 * pr + h;
-      const float* wr = wsh[cur][h];
+    for (int q = 0; q < SQ1 + SQ2; ++q) {
+      const float4 v4 = quad(q);
+      const float v[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
-      for (int k = 0; k < STAR_ROWS; ++k) {
-        const int i = tid + STAR_THREADS * k;
-        if (i < NS) {
-          acc[k] += wr[i] * rs2[i + t];
-          if (t > 0) {
-            const int m = i - t < 0 ? i - t + NS : i - t;   // row m = i - t (mod NS) holds A(m, i)
-            acc[k] += wr[m] * rs2[m];
-          }
+      for (int k = 0; k < 4; ++k) {
+        const int e = 4 * q + k, rr = e / SB, cc = e % SB;
+        if (e < SB * SB) {
+          yI[rr] += v[k] * rJ[cc];
+          yJ[cc] += v[k] * rI[rr];
         }
       }
     }
-    if (pr + 1 < WT / 2) rp.store(&wsh[cur ^ 1][0][0], tid);
-    __syncthreads();
-  }
 #pragma unroll
-  for (int k = 0; k < STAR_ROWS; ++k) {
-    const int i = tid + STAR_THREADS * k;
-    if (i >= NS) continue;
-    if (!interior) {
-      out[v * NS + i] = acc[k];
-    } else {
-      long long nd;
-      if (star_node(g, vx, vy, vz, i, nd)) {
-        float* o = out + (i / SN) * g.N + nd;
-        *o = mode == 2 ? *o - acc[k] : acc[k];
+    for (int k = 0; k < SB; ++k) part[(SB * J + k) * nbr + I] = yJ[k];
+  } else {
+#pragma unroll
+    for (int q = 0; q < SQ1; ++q) {
+      const float4 v4 = quad(q);
+      const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        // entry e of the upper triangle: row rr, column cc
+        const int e = 4 * q + k;
+        int rr = 0, at = 0;
+#pragma unroll
+        for (int x = 0; x < SB; ++x)
+          if (e >= x * SB - x * (x - 1) / 2) { rr = x; at = x * SB - x * (x - 1) / 2; }
+        const int cc = rr + e - at;
+        yI[rr] += v[k] * rI[cc];
+        if (cc != rr) yI[cc] += v[k] * rI[rr];
       }
     }
   }
+#pragma unroll
+  for (int k = 0; k < SB; ++k) part[(SB * I + k) * nbr + J] = yI[k];
 }
 
-// the wrapped rows in bfloat16, rounded to nearest from the FP64 packed diagonals
-__global__ void k_qk3_wrap16(long long nverts, int pstride, const double* __restrict__ inv64,
-                             __nv_bfloat16* __restrict__ inv16) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nverts * WSTRIDE) return;
-  const long long v = e / WSTRIDE;
-  const int r = (int)(e % WSTRIDE), t = r / WLD, i = r % WLD;
-  double val = 0.0;
-  if (i < NS) {
-    const int j = i + t;
-    const double* S = inv64 + v * pstride;
-    val = j < NS ? S[diag_start(NS, t) + i] : S[diag_start(NS, NS - t) + (j - NS)];
+template <typename TS>
+__global__ void __launch_bounds__(STARS_THREADS, 2) k_qk3_stars(Geom g, const TS* __restrict__ inv, int interior,
+                                                                int mode, int nint, int nbnd,
+                                                                const int* __restrict__ bvid,
+                                                                const long long* __restrict__ boff,
+                                                                const float* __restrict__ r,
+                                                                float* __restrict__ out) {
+  __shared__ float rs[BND_PER_CTA * 2 * 75 > NS ? BND_PER_CTA * 150 : NS];
+  __shared__ float part[NS * kFullRows];
+  const int tid = threadIdx.x, item = blockIdx.x;
+  const int nix = g.nv[0] - 2, niy = g.nv[1] - 2;
+  if (interior || item < nint) {
+    int vx, vy, vz;
+    if (interior) {
+      const int cx = g.n[0] / 2, cy = g.n[1] / 2, q = item / cx;
+      vx = 2 * (item - q * cx) + 1;
+      vz = q / cy;
+      vy = 2 * (q - vz * cy) + 1;
+      vz = 2 * vz + 1;
+    } else {
+      const int q = item / nix;
+      vx = item - q * nix + 1;
+      vz = q / niy;
+      vy = q - vz * niy + 1;
+      vz += 1;
+    }
+    const TS* S = inv + (long long)((vx - 1) + nix * ((vy - 1) + niy * (vz - 1))) * kFullEntries;
+    int I = 0, J = 0;
+    float4 pre[SPRE];
+    if (tid < kFullBlocks) {
+      StarBlocks(NS).block_of(tid, I, J);
+#pragma unroll
+      for (int q = 0; q < SPRE; ++q) pre[q] = star_quad(S + 4 * (q * kFullBlocks + tid));
+    }
+    // star entries tid and tid + 352: vector index of entry e is node(3v - 2) + its offset
+    const int nn01 = g.nn[0] * g.nn[1];
+    const int base = (3 * vx - 2) + (3 * vy - 2) * g.nn[0] + (3 * vz - 2) * nn01;
+    int at[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int e = tid + STARS_THREADS * k, c = e / SN, o = e - c * SN, oz = o / (S1 * S1), oxy = o - oz * (S1 * S1);
+      at[k] = base + c * (int)g.N + oxy % S1 + (oxy / S1) * g.nn[0] + oz * nn01;
+    }
+    pdl_wait();
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+      if (tid + STARS_THREADS * k < NS) rs[tid + STARS_THREADS * k] = r[at[k]];
+    __syncthreads();
+    if (tid < kFullBlocks) star_block<TS>(S, kFullBlocks, kFullOff, kFullRows, tid, I, J, pre, rs, part);
+    __syncthreads();
+    const long long v = (long long)vx + (long long)g.nv[0] * ((long long)vy + (long long)g.nv[1] * vz);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int i = tid + STARS_THREADS * k;
+      if (i >= NS) continue;
+      float acc = 0.f;
+#pragma unroll
+      for (int jb = 0; jb < kFullRows; ++jb) acc += part[i * kFullRows + jb];
+      if (!interior) {
+        out[v * NS + i] = acc;
+      } else {
+        float* o = out + at[k];
+        *o = mode == 2 ? *o - acc : acc;
+      }
+    }
+  } else {
+    const int grp = tid >> 6, t = tid & 63, bi = (item - nint) * BND_PER_CTA + grp;
+    const bool have = grp < BND_PER_CTA && bi < nbnd;
+    if (have) {   // uniform over the group
+      const int v = bvid[bi];
+      const TS* S = inv + boff[bi];
+      const int vx = v % g.nv[0], q = v / g.nv[0], vy = q % g.nv[1], vz = q / g.nv[1];
+      const StarBox box(g, vx, vy, vz);
+      const StarBlocks sb(box.m);
+      float* grs = rs + grp * 150;
+      float* gpart = part + grp * 1500;
+      int I = 0, J = 0;
+      float4 pre[SPRE];
+      if (t < sb.nblk) {
+        sb.block_of(t, I, J);
+#pragma unroll
+        for (int k = 0; k < SPRE; ++k) pre[k] = star_quad(S + 4 * (k * sb.nblk + t));
+      }
+      pdl_wait();
+      for (int a = t; a < sb.nbr * SB; a += 64) {
+        float val = 0.f;
+        if (a < box.m) {
+          const int e = box.entry(a), c = e / SN, o = e - c * SN;
+          val = r[c * (int)g.N + (3 * vx - 2 + o % S1) + g.nn[0] * ((3 * vy - 2 + (o / S1) % S1) + g.nn[1] * (3 * vz - 2 + o / (S1 * S1)))];
+        }
+        grs[a] = val;
+      }
+      asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory");
+      if (t < sb.nblk) star_block<TS>(S, sb.nblk, sb.noff, sb.nbr, t, I, J, pre, grs, gpart);
+      asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory");
+      for (int a = t; a < box.m; a += 64) {
+        float acc = 0.f;
+        for (int jb = 0; jb < sb.nbr; ++jb) acc += gpart[a * sb.nbr + jb];
+        out[(long long)v * NS + box.entry(a)] = acc;   // absent and Dirichlet entries are never read
+      }
+    }
   }
-  inv16[e] = __double2bfloat16(val);
+  pdl_trigger();
 }
 
-// the wrapped FP32 rows from the FP64 packed diagonals (loading caller-supplied inverses)
-__global__ void k_qk3_wrap32(long long nverts, int pstride, const double* __restrict__ inv64,
-                             float* __restrict__ inv32) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nverts * WSTRIDE) return;
-  const long long v = e / WSTRIDE;
-  const int r = (int)(e % WSTRIDE), t = r / WLD, i = r % WLD;
-  float val = 0.f;
-  if (i < NS) {
-    const int j = i + t;
-    const double* S = inv64 + v * pstride;
-    val = (float)(j < NS ? S[diag_start(NS, t) + i] : S[diag_start(NS, NS - t) + (j - NS)]);
+// the blocked storage from the FP64 packed diagonals, rounded to nearest: one CTA per star,
+// interior vertices first
+__device__ __forceinline__ void store_star(float* p, double v) { *p = (float)v; }
+__device__ __forceinline__ void store_star(__nv_bfloat16* p, double v) { *p = __double2bfloat16(v); }
+template <typename TS>
+__global__ void __launch_bounds__(256) k_qk3_pack(Geom g, int pstride, int nint, const int* __restrict__ bvid,
+                                                  const long long* __restrict__ boff,
+                                                  const double* __restrict__ inv64, TS* __restrict__ dst0) {
+  const int item = blockIdx.x, nix = g.nv[0] - 2, niy = g.nv[1] - 2;
+  int vx, vy, vz;
+  if (item < nint) {
+    vx = item % nix + 1;
+    vy = (item / nix) % niy + 1;
+    vz = item / (nix * niy) + 1;
+  } else {
+    const int v = bvid[item - nint];
+    vx = v % g.nv[0];
+    vy = (v / g.nv[0]) % g.nv[1];
+    vz = v / (g.nv[0] * g.nv[1]);
   }
-  inv32[e] = val;
+  const StarBox box(g, vx, vy, vz);
+  const StarBlocks sb(box.m);
+  const double* src = inv64 + ((long long)vx + (long long)g.nv[0] * ((long long)vy + (long long)g.nv[1] * vz)) * pstride;
+  TS* dst = dst0 + (item < nint ? (long long)item * kFullEntries : boff[item - nint]);
+  for (int p = threadIdx.x; p < sb.entries(); p += blockDim.x) {
+    const bool second = p >= sb.q2();
+    const int w = (second ? p - sb.q2() : p) >> 2, n = second ? sb.noff : sb.nblk, q = w / n, b = w - q * n;
+    const int e = 4 * (second ? q + SQ1 : q) + (p & 3);
+    int I, J, rr, cc;
+    sb.block_of(b, I, J);
+    if (I != J) {
+      rr = e / SB;
+      cc = e % SB;
+    } else {
+      rr = 0;
+      while (rr + 1 < SB && e >= (rr + 1) * SB - (rr + 1) * rr / 2) ++rr;
+      cc = rr + e - (rr * SB - rr * (rr - 1) / 2);
+    }
+    const int i = SB * I + rr, j = SB * J + cc;
+    double val = 0.0;
+    if (rr < SB && i < box.m && j < box.m) {
+      const int ei = box.entry(i), ej = box.entry(j);
+      val = src[diag_start(NS, ej - ei) + ei];
+    }
+    store_star(dst + p, val);
+  }
 }
 
 // the vertices whose stars contain lattice index i (|i - 3v| <= 2), two taps: v0 = i / 3, then
@@ -1238,17 +1365,44 @@ int qk3_setup_ctas(long long nverts) {
   return (int)(nverts < want ? nverts : want);
 }
 size_t qk3_setup_ws_doubles(int ctas) { return (size_t)ctas * qk3::NS * qk3::LDM; }
-size_t qk3_star32_floats() { return qk3::WSTRIDE; }
+long long qk3_star_layout(const Geom& g, std::vector<int>& bvid, std::vector<long long>& boff) {
+  const long long nint = (long long)(g.nv[0] - 2) * (g.nv[1] - 2) * (g.nv[2] - 2);
+  long long at = nint * qk3::kFullEntries;
+  for (int vz = 0; vz < g.nv[2]; ++vz)
+    for (int vy = 0; vy < g.nv[1]; ++vy)
+      for (int vx = 0; vx < g.nv[0]; ++vx) {
+        const qk3::StarBox box(g, vx, vy, vz);
+        if (box.m == qk3::NS) continue;
+        bvid.push_back(vx + g.nv[0] * (vy + g.nv[1] * vz));
+        boff.push_back(at);
+        at += qk3::StarBlocks(box.m).entries();
+      }
+  return at;
+}
 
 void qk3_derive32(const LevelDev& L, cudaStream_t s) {
-  const long long tot = L.g.nverts * qk3::WSTRIDE;
-  qk3::k_qk3_wrap32<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(L.g.nverts, L.pstride, L.inv64, L.inv32);
+  const unsigned n = (unsigned)L.g.nverts;
+  qk3::k_qk3_pack<float><<<n, 256, 0, s>>>(L.g, L.pstride, (int)L.nint, L.bvid, L.boff, L.inv64, L.inv32);
   count_launch(1);
-  if (L.inv16) {
-    qk3::k_qk3_wrap16<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(L.g.nverts, L.pstride, L.inv64,
-                                                                   (__nv_bfloat16*)L.inv16);
+  if (L.inv16) {   // ALS_STORE_BF16
+    qk3::k_qk3_pack<__nv_bfloat16><<<n, 256, 0, s>>>(L.g, L.pstride, (int)L.nint, L.bvid, L.boff, L.inv64,
+                                                     (__nv_bfloat16*)L.inv16);
     count_launch(1);
   }
+}
+
+// the FP32 star products: every star into the scratch rows, or (interior) the local solves on
+// the coarse-cell interiors
+static void launch_stars32(const LevelDev& L, int interior, int mode, const float* r, float* out, cudaStream_t s) {
+  const unsigned grid = interior ? (unsigned)((long long)(L.g.n[0] / 2) * (L.g.n[1] / 2) * (L.g.n[2] / 2))
+                                 : (unsigned)(L.nint + (L.nbnd + qk3::BND_PER_CTA - 1) / qk3::BND_PER_CTA);
+  if (L.inv16)
+    launch_pdl(qk3::k_qk3_stars<__nv_bfloat16>, grid, qk3::STARS_THREADS, 0, s, L.g, (const __nv_bfloat16*)L.inv16,
+               interior, mode, (int)L.nint, (int)L.nbnd, (const int*)L.bvid, (const long long*)L.boff, r, out);
+  else
+    launch_pdl(qk3::k_qk3_stars<float>, grid, qk3::STARS_THREADS, 0, s, L.g, (const float*)L.inv32, interior, mode,
+               (int)L.nint, (int)L.nbnd, (const int*)L.bvid, (const long long*)L.boff, r, out);
+  count_launch(1);
 }
 
 void qk3_patch_setup(const LevelDev& L, double gamma, DevStatus* st, cudaStream_t s, int df64) {
@@ -1263,53 +1417,39 @@ void qk3_patch_setup(const LevelDev& L, double gamma, DevStatus* st, cudaStream_
   const int ctas = L.qk_ws_ctas < L.g.nverts ? L.qk_ws_ctas : (int)L.g.nverts;
   if (df64)
     qk3::k_qk3_star_setup<DF64><<<(unsigned)ctas, qk3::SETUP_THREADS, qk3::SETUP_SMEM, s>>>(
-        L.g, gamma, L.mu64, L.winv64, L.qk_ws, L.inv64, L.inv32, L.pstride, st);
+        L.g, gamma, L.mu64, L.winv64, L.qk_ws, L.inv64, L.pstride, st);
   else
     qk3::k_qk3_star_setup<double><<<(unsigned)ctas, qk3::SETUP_THREADS, qk3::SETUP_SMEM, s>>>(
-        L.g, gamma, L.mu64, L.winv64, L.qk_ws, L.inv64, L.inv32, L.pstride, st);
+        L.g, gamma, L.mu64, L.winv64, L.qk_ws, L.inv64, L.pstride, st);
   count_launch(1);
-  if (L.inv16) {   // ALS_STORE_BF16: the rows again in bfloat16, from the FP64 inverses
-    const long long tot = L.g.nverts * qk3::WSTRIDE;
-    qk3::k_qk3_wrap16<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(L.g.nverts, L.pstride, L.inv64,
-                                                                   (__nv_bfloat16*)L.inv16);
-    count_launch(1);
-  }
+  qk3_derive32(L, s);
 }
 
 void qk3_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, cudaStream_t s) {
   const unsigned b3 = (unsigned)((3 * L.g.N + 255) / 256);
-  const unsigned nv = (unsigned)L.g.nverts;
   if (prec == PREC_F64) {
-    qk3::k_qk3_star_apply<double><<<nv, qk3::STAR_THREADS, 0, s>>>(L.g, L.inv64, L.pstride, 0, 0, (const double*)r,
-                                                                   (double*)scratch);
+    qk3::k_qk3_star_apply<double><<<(unsigned)L.g.nverts, qk3::STAR_THREADS, 0, s>>>(
+        L.g, L.inv64, L.pstride, 0, 0, (const double*)r, (double*)scratch);
+    count_launch(1);
     launch_pdl(qk3::k_qk3_star_gather<double>, b3, 256, 0, s, L.g, (const double*)scratch, (double*)z);
   } else {
-    if (L.inv16)
-      qk3::k_qk3_star_apply_w<__nv_bfloat16><<<nv, qk3::STAR_THREADS, 0, s>>>(
-          L.g, (const __nv_bfloat16*)L.inv16, 0, 0, (const float*)r, (float*)scratch);
-    else
-      qk3::k_qk3_star_apply_w<float><<<nv, qk3::STAR_THREADS, 0, s>>>(L.g, L.inv32, 0, 0, (const float*)r,
-                                                                      (float*)scratch);
+    launch_stars32(L, 0, 0, (const float*)r, (float*)scratch, s);
     launch_pdl(qk3::k_qk3_star_gather<float>, b3, 256, 0, s, L.g, (const float*)scratch, (float*)z);
   }
-  count_launch(2);
+  count_launch(1);
 }
 
 void qk3_interior_solve(const LevelDev& fine, int prec, const void* in, void* out, int subtract, cudaStream_t s) {
   const long long nc = (long long)(fine.g.n[0] / 2) * (fine.g.n[1] / 2) * (fine.g.n[2] / 2);
   const size_t es = prec == PREC_F64 ? 8 : 4;
   if (!subtract) cudaMemsetAsync(out, 0, es * 3 * fine.g.N, s);
-  if (prec == PREC_F64)
+  if (prec == PREC_F64) {
     qk3::k_qk3_star_apply<double><<<(unsigned)nc, qk3::STAR_THREADS, 0, s>>>(
         fine.g, fine.inv64, fine.pstride, 1, subtract ? 2 : 1, (const double*)in, (double*)out);
-  else
-    if (fine.inv16)
-      qk3::k_qk3_star_apply_w<__nv_bfloat16><<<(unsigned)nc, qk3::STAR_THREADS, 0, s>>>(
-          fine.g, (const __nv_bfloat16*)fine.inv16, 1, subtract ? 2 : 1, (const float*)in, (float*)out);
-    else
-      qk3::k_qk3_star_apply_w<float><<<(unsigned)nc, qk3::STAR_THREADS, 0, s>>>(
-          fine.g, fine.inv32, 1, subtract ? 2 : 1, (const float*)in, (float*)out);
-  count_launch(1);
+    count_launch(1);
+  } else {
+    launch_stars32(fine, 1, subtract ? 2 : 1, (const float*)in, (float*)out, s);
+  }
 }
 
 void qk3_prolong(const LevelDev& coarse, const LevelDev& fine, int prec, const void* xc, void* xf, cudaStream_t s,
