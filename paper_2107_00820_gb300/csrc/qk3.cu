@@ -32,6 +32,7 @@
 #include "level.h"
 #include "pdl.cuh"
 #include "qk_tables.h"
+#include "tma.cuh"
 
 namespace als {
 namespace qk3 {
@@ -925,191 +926,310 @@ __global__ void __launch_bounds__(STAR_THREADS) k_qk3_star_apply(Geom g, const T
 // the packed triangle.  The product y_i = sum_t W_t[i] r_(i+t) + sum_(t>0) W_t[i-t] r_(i-t)
 // (indices mod NS) then reads each row once, coalesced, 16 bytes a thread.
 
-// y_v = A_v^-1 r|_v in FP32 from the blocked storage.  An interior star takes a CTA, one 15 x 15
-// block a thread: the block is read from global memory once, in quads that are consecutive over
-// the threads, and each entry is used for both y_I += S r_J and y_J += S^T r_I from registers;
-// the 25 partial sums of a row meet in shared memory in a fixed order.  Boundary stars, with at
-// most 55 blocks, take 64 threads, five to a CTA.  Bound by the stream of the inverses: two CTAs
-// an SM keep about 90 KB of loads in flight.  On 12^3 cells a sweep takes XX us; the form before
-// (every star padded to 375 dofs, wrapped rows two at a time through shared memory, four shared
-// loads for two FMAs) took 140, and on 6^3 cells YY against 60.
-// TS: float, or bfloat16 (ALS_STORE_BF16), widened on load; products and sums in FP32.
-// interior / mode as k_qk3_star_apply; nint: interior vertices (stored first, in their own
-// x-fastest order), then nbnd boundary ones (bvid, offsets boff).
-constexpr int STARS_THREADS = 352, BND_PER_CTA = 5;
+// y_v = A_v^-1 r|_v in FP32 from the blocked storage; every entry of a block is used for both
+// y_I += S r_J and y_J += S^T r_I from registers, the partial sums of a row (one per block
+// column) meet in shared memory and are added in a fixed order.  TS: float, or bfloat16
+// (ALS_STORE_BF16), widened on load; products and sums in FP32.
+//
+// Interior stars (285 KB each in FP32) are bound by their stream from memory: one persistent CTA
+// an SM, whose producer warp keeps a ring of bulk copies (three quads of every block a stage in
+// FP32) ahead of eleven consumer warps, one block a thread, across the stars' boundaries.
+// The launch takes 70 us on 12^3 cells (381 MB, 5.4 TB/s) and 18 on 6^3 (one star an SM); with
+// the same blocks loaded straight into registers, a CTA per star, it took 97 and 19, and before
+// that, with every star padded to 375 dofs and wrapped rows staged two at a time (four shared
+// loads for two FMAs), 140 and 60; six ring stages instead of nine give 74.
+// Boundary stars, at most 55 blocks: 64 threads each, in a launch of their own beside it.
+//
+// Waits on the ring are bounded (wait_polls); on expiry the kernel records ALS_ETIMEOUT, stops
+// storing, waits (at the default limit) for the copies in flight and returns.
+constexpr int STARS_WARPS = 11, STARS_THREADS = 32 * (STARS_WARPS + 1);
 
-__device__ __forceinline__ float4 star_quad(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 star_quad(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ float4 star_quad(const __nv_bfloat16* p) {
-  const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+  const uint2 u = *reinterpret_cast<const uint2*>(p);
   const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
   const float2 c = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
   return make_float4(a.x, a.y, c.x, c.y);
 }
 
-constexpr int SPRE = 6;   // quads of a block in flight before the dependency wait
-
-// partial sums of block b into part[row][nbr]; pre: its first SPRE quads
-template <typename TS>
-__device__ __forceinline__ void star_block(const TS* __restrict__ S, int nblk, int noff, int nbr, int b, int I, int J,
-                                           const float4 (&pre)[SPRE], const float* rs, float* part) {
-  const int q2 = 4 * SQ1 * nblk;
-  const auto quad = [&](int q) {
-    return q < SPRE ? pre[q]
-                    : (q < SQ1 ? star_quad(S + 4 * (q * nblk + b)) : star_quad(S + q2 + 4 * ((q - SQ1) * noff + b)));
-  };
-  float rI[SB], yI[SB];
+// the products of quad q (compile-time after unrolling) of an off-diagonal block
+__device__ __forceinline__ void quad_off(int q, float4 v4, const float (&rI)[SB], const float (&rJ)[SB],
+                                         float (&yI)[SB], float (&yJ)[SB]) {
+  const float v[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
-  for (int k = 0; k < SB; ++k) {
-    rI[k] = rs[SB * I + k];
-    yI[k] = 0.f;
-  }
-  if (I != J) {
-    float rJ[SB], yJ[SB];
-#pragma unroll
-    for (int k = 0; k < SB; ++k) {
-      rJ[k] = rs[SB * J + k];
-      yJ[k] = 0.f;
-    }
-#pragma unroll
-    for (int q = 0; q < SQ1 + SQ2; ++q) {
-      const float4 v4 = quad(q);
-      const float v[4] = {v4.x, v4.y, v4.z, v4.w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int e = 4 * q + k, rr = e / SB, cc = e % SB;
-        if (e < SB * SB) {
-          yI[rr] += v[k] * rJ[cc];
-          yJ[cc] += v[k] * rI[rr];
-        }
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < SB; ++k) part[(SB * J + k) * nbr + I] = yJ[k];
-  } else {
-#pragma unroll
-    for (int q = 0; q < SQ1; ++q) {
-      const float4 v4 = quad(q);
-      const float v[4] = {v4.x, v4.y, v4.z, v4.w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        // entry e of the upper triangle: row rr, column cc
-        const int e = 4 * q + k;
-        int rr = 0, at = 0;
-#pragma unroll
-        for (int x = 0; x < SB; ++x)
-          if (e >= x * SB - x * (x - 1) / 2) { rr = x; at = x * SB - x * (x - 1) / 2; }
-        const int cc = rr + e - at;
-        yI[rr] += v[k] * rI[cc];
-        if (cc != rr) yI[cc] += v[k] * rI[rr];
-      }
+  for (int k = 0; k < 4; ++k) {
+    const int e = 4 * q + k, rr = e / SB, cc = e % SB;
+    if (e < SB * SB) {
+      yI[rr] += v[k] * rJ[cc];
+      yJ[cc] += v[k] * rI[rr];
     }
   }
+}
+// of a diagonal block: entries of the upper triangle
+__device__ __forceinline__ void quad_diag(int q, float4 v4, const float (&rI)[SB], float (&yI)[SB]) {
+  const float v[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
-  for (int k = 0; k < SB; ++k) part[(SB * I + k) * nbr + J] = yI[k];
+  for (int k = 0; k < 4; ++k) {
+    const int e = 4 * q + k;
+    int rr = 0, at = 0;
+#pragma unroll
+    for (int x = 0; x < SB; ++x)
+      if (e >= x * SB - x * (x - 1) / 2) { rr = x; at = x * SB - x * (x - 1) / 2; }
+    const int cc = rr + e - at;
+    yI[rr] += v[k] * rI[cc];
+    if (cc != rr) yI[cc] += v[k] * rI[rr];
+  }
 }
 
 template <typename TS>
-__global__ void __launch_bounds__(STARS_THREADS, 2) k_qk3_stars(Geom g, const TS* __restrict__ inv, int interior,
-                                                                int mode, int nint, int nbnd,
-                                                                const int* __restrict__ bvid,
-                                                                const long long* __restrict__ boff,
-                                                                const float* __restrict__ r,
-                                                                float* __restrict__ out) {
-  __shared__ float rs[BND_PER_CTA * 2 * 75 > NS ? BND_PER_CTA * 150 : NS];
-  __shared__ float part[NS * kFullRows];
-  const int tid = threadIdx.x, item = blockIdx.x;
+struct StarRing {
+  static constexpr int CQ = sizeof(TS) == 4 ? 3 : 6;              // quads per stage
+  static constexpr int NA = SQ1 / CQ, NBS = (SQ2 + CQ - 1) / CQ;  // stages of the two parts of a star
+  static constexpr int STAGES = 9;
+  static constexpr int STAGE_ENTRIES = 4 * CQ * kFullBlocks;
+  static constexpr size_t STAGE_BYTES = (size_t)STAGE_ENTRIES * sizeof(TS);
+  static constexpr size_t BAR_BYTES = 256;
+  static constexpr size_t SMEM = BAR_BYTES + STAGES * STAGE_BYTES + (NS + 1 + NS * kFullRows) * sizeof(float);
+  static_assert(NA + NBS > STAGES && SQ1 % CQ == 0 && 2 * STAGES * 8 <= (int)BAR_BYTES, "ring layout");
+  static_assert(STAGE_BYTES % 16 == 0 && (4 * 3 * kFullOff * sizeof(TS)) % 16 == 0 &&
+                    (kFullEntries * sizeof(TS)) % 16 == 0 && (4 * SQ1 * kFullBlocks * sizeof(TS)) % 16 == 0,
+                "bulk copies need 16-byte alignment");
+};
+
+// vertex of interior item `item` (interior: the fine vertex at a coarse cell's centre) and its
+// index among the interior vertices
+__device__ __forceinline__ long long star_item(const Geom& g, int interior, int item, int& vx, int& vy, int& vz) {
   const int nix = g.nv[0] - 2, niy = g.nv[1] - 2;
-  if (interior || item < nint) {
-    int vx, vy, vz;
-    if (interior) {
-      const int cx = g.n[0] / 2, cy = g.n[1] / 2, q = item / cx;
-      vx = 2 * (item - q * cx) + 1;
-      vz = q / cy;
-      vy = 2 * (q - vz * cy) + 1;
-      vz = 2 * vz + 1;
-    } else {
-      const int q = item / nix;
-      vx = item - q * nix + 1;
-      vz = q / niy;
-      vy = q - vz * niy + 1;
-      vz += 1;
+  if (interior) {
+    const int cx = g.n[0] / 2, cy = g.n[1] / 2, q = item / cx;
+    vx = 2 * (item - q * cx) + 1;
+    vz = q / cy;
+    vy = 2 * (q - vz * cy) + 1;
+    vz = 2 * vz + 1;
+  } else {
+    const int q = item / nix;
+    vx = item - q * nix + 1;
+    vz = q / niy;
+    vy = q - vz * niy + 1;
+    vz += 1;
+  }
+  return (vx - 1) + nix * ((vy - 1) + (long long)niy * (vz - 1));
+}
+
+template <typename TS>
+__global__ void __launch_bounds__(STARS_THREADS, 1) k_qk3_stars(Geom g, const TS* __restrict__ inv, int interior,
+                                                                int mode, int count, const float* __restrict__ r,
+                                                                float* __restrict__ out, DevStatus* st,
+                                                                int wait_polls, int early_trigger) {
+  using C = StarRing<TS>;
+  extern __shared__ __align__(128) unsigned char smraw[];
+  uint64_t* full = reinterpret_cast<uint64_t*>(smraw);
+  uint64_t* empty = full + C::STAGES;
+  TS* ring = reinterpret_cast<TS*>(smraw + C::BAR_BYTES);
+  float* rs = reinterpret_cast<float*>(smraw + C::BAR_BYTES + C::STAGES * C::STAGE_BYTES);
+  float* part = rs + NS + 1;
+  __shared__ int s_fail;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  if (tid == 0) {
+    s_fail = 0;
+    for (int i = 0; i < C::STAGES; ++i) {
+      tma::mbar_init(&full[i], 1);
+      tma::mbar_init(&empty[i], STARS_WARPS);
     }
-    const TS* S = inv + (long long)((vx - 1) + nix * ((vy - 1) + niy * (vz - 1))) * kFullEntries;
-    int I = 0, J = 0;
-    float4 pre[SPRE];
-    if (tid < kFullBlocks) {
-      StarBlocks(NS).block_of(tid, I, J);
-#pragma unroll
-      for (int q = 0; q < SPRE; ++q) pre[q] = star_quad(S + 4 * (q * kFullBlocks + tid));
-    }
-    // star entries tid and tid + 352: vector index of entry e is node(3v - 2) + its offset
-    const int nn01 = g.nn[0] * g.nn[1];
-    const int base = (3 * vx - 2) + (3 * vy - 2) * g.nn[0] + (3 * vz - 2) * nn01;
-    int at[2];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int e = tid + STARS_THREADS * k, c = e / SN, o = e - c * SN, oz = o / (S1 * S1), oxy = o - oz * (S1 * S1);
-      at[k] = base + c * (int)g.N + oxy % S1 + (oxy / S1) * g.nn[0] + oz * nn01;
-    }
-    pdl_wait();
-#pragma unroll
-    for (int k = 0; k < 2; ++k)
-      if (tid + STARS_THREADS * k < NS) rs[tid + STARS_THREADS * k] = r[at[k]];
-    __syncthreads();
-    if (tid < kFullBlocks) star_block<TS>(S, kFullBlocks, kFullOff, kFullRows, tid, I, J, pre, rs, part);
-    __syncthreads();
-    const long long v = (long long)vx + (long long)g.nv[0] * ((long long)vy + (long long)g.nv[1] * vz);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int i = tid + STARS_THREADS * k;
-      if (i >= NS) continue;
-      float acc = 0.f;
-#pragma unroll
-      for (int jb = 0; jb < kFullRows; ++jb) acc += part[i * kFullRows + jb];
-      if (!interior) {
-        out[v * NS + i] = acc;
-      } else {
-        float* o = out + at[k];
-        *o = mode == 2 ? *o - acc : acc;
+    tma::fence_init();
+  }
+  __syncthreads();
+  if (warp == STARS_WARPS) {
+    // producer: the inverses are written by the setup only, so it fills the ring before the
+    // dependency wait (a star has more stages than the ring); a stage is refilled once all consumer warps have released it
+    if ((tid & 31) == 0) {
+      int k = 0;   // stages issued
+      for (int item = blockIdx.x; item < count; item += gridDim.x) {
+        int vx, vy, vz;
+        const TS* S = inv + star_item(g, interior, item, vx, vy, vz) * kFullEntries;
+        for (int c = 0; c < C::NA + C::NBS; ++c, ++k) {
+          const int s = k % C::STAGES;
+          if (k == C::STAGES) {   // the ring is full of copies on their way
+            pdl_wait();
+            if (early_trigger) pdl_trigger();
+          }
+          if (k >= C::STAGES && !tma::mbar_wait(&empty[s], (uint32_t)((k / C::STAGES - 1) & 1))) {
+            report(st, 7 /* ALS_ETIMEOUT */, item);
+            *(volatile int*)&s_fail = 1;
+          }
+          if (*(volatile int*)&s_fail) break;
+          const bool a = c < C::NA;
+          const int q = a ? c * C::CQ : (c - C::NA) * C::CQ;
+          const int nq = a ? C::CQ : (SQ2 - q < C::CQ ? SQ2 - q : C::CQ);
+          const uint32_t bytes = (uint32_t)(4 * nq * (a ? kFullBlocks : kFullOff) * sizeof(TS));
+          const TS* src = S + (a ? 4 * q * kFullBlocks : 4 * SQ1 * kFullBlocks + 4 * q * kFullOff);
+          tma::mbar_expect_tx(&full[s], bytes);
+          tma::bulk_load(ring + s * C::STAGE_ENTRIES, src, bytes, &full[s]);
+        }
+        if (*(volatile int*)&s_fail) break;
       }
+      // after a failure: no copy may be in flight when the CTA exits
+      for (int m = k > C::STAGES ? k - C::STAGES : 0; m < k; ++m)
+        tma::mbar_wait(&full[m % C::STAGES], (uint32_t)((m / C::STAGES) & 1));
     }
   } else {
-    const int grp = tid >> 6, t = tid & 63, bi = (item - nint) * BND_PER_CTA + grp;
-    const bool have = grp < BND_PER_CTA && bi < nbnd;
-    if (have) {   // uniform over the group
-      const int v = bvid[bi];
-      const TS* S = inv + boff[bi];
-      const int vx = v % g.nv[0], q = v / g.nv[0], vy = q % g.nv[1], vz = q / g.nv[1];
-      const StarBox box(g, vx, vy, vz);
-      const StarBlocks sb(box.m);
-      float* grs = rs + grp * 150;
-      float* gpart = part + grp * 1500;
-      int I = 0, J = 0;
-      float4 pre[SPRE];
-      if (t < sb.nblk) {
-        sb.block_of(t, I, J);
+    int I = 0, J = 0;
+    const int b = tid;
+    const bool mine = b < kFullBlocks, off = b < kFullOff;
+    if (mine) StarBlocks(NS).block_of(b, I, J);
+    const int nn01 = g.nn[0] * g.nn[1];
+    int eo[2];   // offsets of star entries tid and tid + 352 from node 3v - 2
 #pragma unroll
-        for (int k = 0; k < SPRE; ++k) pre[k] = star_quad(S + 4 * (k * sb.nblk + t));
+    for (int k = 0; k < 2; ++k) {
+      const int e = tid + 32 * STARS_WARPS * k, c = e / SN, o = e - c * SN, oz = o / (S1 * S1), oxy = o - oz * (S1 * S1);
+      eo[k] = c * (int)g.N + oxy % S1 + (oxy / S1) * g.nn[0] + oz * nn01;
+    }
+    const auto base_of = [&](int item, int& vx, int& vy, int& vz) {
+      star_item(g, interior, item, vx, vy, vz);
+      return (3 * vx - 2) + (3 * vy - 2) * g.nn[0] + (3 * vz - 2) * nn01;
+    };
+    pdl_wait();
+    // early_trigger: the boundary-star kernel, which needs nothing this one writes, may start
+    if (early_trigger) pdl_trigger();
+    int vx, vy, vz, base = 0;
+    float rn[2] = {0.f, 0.f};
+    if ((int)blockIdx.x < count) {
+      base = base_of(blockIdx.x, vx, vy, vz);
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        if (tid + 32 * STARS_WARPS * k < NS) rn[k] = r[base + eo[k]];
+    }
+    int k = 0;   // stages consumed
+    for (int item = blockIdx.x; item < count; item += gridDim.x) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+        if (tid + 32 * STARS_WARPS * q < NS) rs[tid + 32 * STARS_WARPS * q] = rn[q];
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * STARS_WARPS) : "memory");
+      const long long v = (long long)vx + (long long)g.nv[0] * ((long long)vy + (long long)g.nv[1] * vz);
+      const int here = base;
+      if (item + (int)gridDim.x < count) {   // the next star's r, in flight over this one
+        base = base_of(item + gridDim.x, vx, vy, vz);
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+          if (tid + 32 * STARS_WARPS * q < NS) rn[q] = r[base + eo[q]];
       }
-      pdl_wait();
-      for (int a = t; a < sb.nbr * SB; a += 64) {
-        float val = 0.f;
-        if (a < box.m) {
-          const int e = box.entry(a), c = e / SN, o = e - c * SN;
-          val = r[c * (int)g.N + (3 * vx - 2 + o % S1) + g.nn[0] * ((3 * vy - 2 + (o / S1) % S1) + g.nn[1] * (3 * vz - 2 + o / (S1 * S1)))];
+      float rI[SB], rJ[SB], yI[SB], yJ[SB];
+#pragma unroll
+      for (int q = 0; q < SB; ++q) {
+        rI[q] = mine ? rs[SB * I + q] : 0.f;
+        rJ[q] = mine ? rs[SB * J + q] : 0.f;
+        yI[q] = yJ[q] = 0.f;
+      }
+#pragma unroll
+      for (int c = 0; c < C::NA + C::NBS; ++c, ++k) {
+        const int s = k % C::STAGES;
+        if (!*(volatile int*)&s_fail && !tma::mbar_wait(&full[s], (uint32_t)((k / C::STAGES) & 1), wait_polls)) {
+          report(st, 7 /* ALS_ETIMEOUT */, item);
+          *(volatile int*)&s_fail = 1;
         }
-        grs[a] = val;
+        const TS* W = ring + s * C::STAGE_ENTRIES;
+#pragma unroll
+        for (int q = 0; q < C::CQ; ++q) {
+          if (c < C::NA) {
+            const int qq = c * C::CQ + q;
+            if (off) quad_off(qq, star_quad(W + 4 * (q * kFullBlocks + b)), rI, rJ, yI, yJ);
+            else if (mine) quad_diag(qq, star_quad(W + 4 * (q * kFullBlocks + b)), rI, yI);
+          } else if (SQ1 + (c - C::NA) * C::CQ + q < SQ1 + SQ2) {
+            if (off) quad_off(SQ1 + (c - C::NA) * C::CQ + q, star_quad(W + 4 * (q * kFullOff + b)), rI, rJ, yI, yJ);
+          }
+        }
+        __syncwarp();
+        if ((tid & 31) == 0) tma::mbar_arrive(&empty[s]);
       }
-      asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory");
-      if (t < sb.nblk) star_block<TS>(S, sb.nblk, sb.noff, sb.nbr, t, I, J, pre, grs, gpart);
-      asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory");
-      for (int a = t; a < box.m; a += 64) {
+      if (mine) {
+#pragma unroll
+        for (int q = 0; q < SB; ++q) part[(SB * I + q) * kFullRows + J] = yI[q];
+        if (off) {
+#pragma unroll
+          for (int q = 0; q < SB; ++q) part[(SB * J + q) * kFullRows + I] = yJ[q];
+        }
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * STARS_WARPS) : "memory");
+      if (*(volatile int*)&s_fail) break;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int i = tid + 32 * STARS_WARPS * q;
+        if (i >= NS) continue;
         float acc = 0.f;
-        for (int jb = 0; jb < sb.nbr; ++jb) acc += gpart[a * sb.nbr + jb];
-        out[(long long)v * NS + box.entry(a)] = acc;   // absent and Dirichlet entries are never read
+#pragma unroll
+        for (int jb = 0; jb < kFullRows; ++jb) acc += part[i * kFullRows + jb];
+        if (!interior) {
+          out[v * NS + i] = acc;
+        } else {
+          float* o = out + here + eo[q];
+          *o = mode == 2 ? *o - acc : acc;
+        }
       }
     }
+    if (!early_trigger) pdl_trigger();
   }
+}
+
+// the boundary stars: one star per 64-thread CTA; runs beside the interior-star kernel, which
+// lets it start once its own dependency wait has returned, and waits for it only at its end
+template <typename TS>
+__global__ void __launch_bounds__(64) k_qk3_stars_bnd(Geom g, const TS* __restrict__ inv, const int* __restrict__ bvid,
+                                                      const long long* __restrict__ boff,
+                                                      const float* __restrict__ r, float* __restrict__ out) {
+  constexpr int MMAX = 150, RMAX = MMAX / SB;
+  __shared__ float rs[MMAX];
+  __shared__ float part[MMAX * RMAX];
+  const int t = threadIdx.x, v = __ldg(bvid + blockIdx.x);
+  const TS* S = inv + __ldg(boff + blockIdx.x);
+  const int vx = v % g.nv[0], q0 = v / g.nv[0], vy = q0 % g.nv[1], vz = q0 / g.nv[1];
+  const StarBox box(g, vx, vy, vz);
+  const StarBlocks sb(box.m);
+  for (int a = t; a < sb.nbr * SB; a += 64) {
+    float val = 0.f;
+    if (a < box.m) {
+      const int e = box.entry(a), c = e / SN, o = e - c * SN;
+      val = __ldcg(r + (c * (int)g.N + (3 * vx - 2 + o % S1) +
+                        g.nn[0] * ((3 * vy - 2 + (o / S1) % S1) + g.nn[1] * (3 * vz - 2 + o / (S1 * S1)))));
+    }
+    rs[a] = val;
+  }
+  __syncthreads();
+  if (t < sb.nblk) {
+    int I, J;
+    sb.block_of(t, I, J);
+    float rI[SB], yI[SB];
+#pragma unroll
+    for (int k = 0; k < SB; ++k) {
+      rI[k] = rs[SB * I + k];
+      yI[k] = 0.f;
+    }
+    if (I != J) {
+      float rJ[SB], yJ[SB];
+#pragma unroll
+      for (int k = 0; k < SB; ++k) {
+        rJ[k] = rs[SB * J + k];
+        yJ[k] = 0.f;
+      }
+#pragma unroll
+      for (int q = 0; q < SQ1; ++q) quad_off(q, star_quad(S + 4 * (q * sb.nblk + t)), rI, rJ, yI, yJ);
+#pragma unroll
+      for (int q = 0; q < SQ2; ++q) quad_off(SQ1 + q, star_quad(S + sb.q2() + 4 * (q * sb.noff + t)), rI, rJ, yI, yJ);
+#pragma unroll
+      for (int k = 0; k < SB; ++k) part[(SB * J + k) * sb.nbr + I] = yJ[k];
+    } else {
+#pragma unroll
+      for (int q = 0; q < SQ1; ++q) quad_diag(q, star_quad(S + 4 * (q * sb.nblk + t)), rI, yI);
+    }
+#pragma unroll
+    for (int k = 0; k < SB; ++k) part[(SB * I + k) * sb.nbr + J] = yI[k];
+  }
+  __syncthreads();
+  for (int a = t; a < box.m; a += 64) {
+    float acc = 0.f;
+    for (int jb = 0; jb < sb.nbr; ++jb) acc += part[a * sb.nbr + jb];
+    out[(long long)v * NS + box.entry(a)] = acc;   // absent and Dirichlet entries are never read
+  }
+  pdl_wait();
   pdl_trigger();
 }
 
@@ -1391,21 +1511,30 @@ void qk3_derive32(const LevelDev& L, cudaStream_t s) {
   }
 }
 
+template <typename TS>
+static void launch_stars_t(const LevelDev& L, const TS* inv, int interior, int mode, const float* r, float* out,
+                           cudaStream_t s) {
+  const int count = interior ? (L.g.n[0] / 2) * (L.g.n[1] / 2) * (L.g.n[2] / 2) : (int)L.nint;
+  const int bnd = interior ? 0 : (int)L.nbnd;
+  launch_pdl(qk3::k_qk3_stars<TS>, (unsigned)(count < 152 ? count : 152), qk3::STARS_THREADS, qk3::StarRing<TS>::SMEM,
+             s, L.g, inv, interior, mode, count, r, out, L.status, L.wait_polls, bnd > 0 ? 1 : 0);
+  if (bnd > 0)
+    launch_pdl(qk3::k_qk3_stars_bnd<TS>, (unsigned)bnd, 64, 0, s, L.g, inv, (const int*)L.bvid,
+               (const long long*)L.boff, r, out);
+  count_launch(bnd > 0 ? 2 : 1);
+}
 // the FP32 star products: every star into the scratch rows, or (interior) the local solves on
 // the coarse-cell interiors
 static void launch_stars32(const LevelDev& L, int interior, int mode, const float* r, float* out, cudaStream_t s) {
-  const unsigned grid = interior ? (unsigned)((long long)(L.g.n[0] / 2) * (L.g.n[1] / 2) * (L.g.n[2] / 2))
-                                 : (unsigned)(L.nint + (L.nbnd + qk3::BND_PER_CTA - 1) / qk3::BND_PER_CTA);
-  if (L.inv16)
-    launch_pdl(qk3::k_qk3_stars<__nv_bfloat16>, grid, qk3::STARS_THREADS, 0, s, L.g, (const __nv_bfloat16*)L.inv16,
-               interior, mode, (int)L.nint, (int)L.nbnd, (const int*)L.bvid, (const long long*)L.boff, r, out);
-  else
-    launch_pdl(qk3::k_qk3_stars<float>, grid, qk3::STARS_THREADS, 0, s, L.g, (const float*)L.inv32, interior, mode,
-               (int)L.nint, (int)L.nbnd, (const int*)L.bvid, (const long long*)L.boff, r, out);
-  count_launch(1);
+  if (L.inv16) launch_stars_t(L, (const __nv_bfloat16*)L.inv16, interior, mode, r, out, s);
+  else launch_stars_t(L, (const float*)L.inv32, interior, mode, r, out, s);
 }
 
 void qk3_patch_setup(const LevelDev& L, double gamma, DevStatus* st, cudaStream_t s, int df64) {
+  cudaFuncSetAttribute(qk3::k_qk3_stars<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)qk3::StarRing<float>::SMEM);
+  cudaFuncSetAttribute(qk3::k_qk3_stars<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)qk3::StarRing<__nv_bfloat16>::SMEM);
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(qk3::k_qk3_star_setup<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
