@@ -1072,63 +1072,157 @@ size_t setup_tab_bytes(int dim) {
 }
 
 // ---------------------------------------------------------------------------
-// K4: y_v = A_v^-1 r|_v, one warp per patch; rows by lanes, diagonals in order
+// K4 (FP64): y_v = A_v^-1 r|_v from the inverses packed by diagonals
 // ---------------------------------------------------------------------------
-// y = A r for a symmetric A packed by diagonals, one warp, rows by lanes, over the
-// wrapped diagonals t = 0 .. NP-1: row i takes the entry (i, (i + t) mod NP), which is
-// entry i of diagonal t while i + t < NP and entry i + t - NP of diagonal NP - t after
-// (the symmetric partner), so every (i, j) is used exactly once and every lane of a row
-// chunk does useful work at every t (NP^2 products for NP^2 lane-FMAs, where a pass over
-// the NP diagonals in both directions would issue 2 NP^2 with half the lanes idle; the FP64
-// pipe is this kernel's bound).  Both segments of a wrapped diagonal are contiguous, so the
-// loads stay coalesced.
-template <typename TF, typename TV, int DIM>
-__device__ __forceinline__ void patch_gemv(const TF* __restrict__ S, const TV* rs, int lane, TV (&acc)[(Sz<DIM>::NP + 31) / 32]) {
-  constexpr int NP = Sz<DIM>::NP, R = (NP + 31) / 32;
-#pragma unroll
-  for (int k = 0; k < R; ++k) acc[k] = TV(0);
-#pragma unroll 3
-  for (int t = 0; t < NP; ++t) {
-    const TF* du = S + diag_start(NP, t);                                 // (i, i + t), i < NP - t
-    const TF* dl = S + (t > 0 ? diag_start(NP, NP - t) - (NP - t) : 0);  // (i + t - NP, i), i >= NP - t
-#pragma unroll
-    for (int k = 0; k < R; ++k) {
-      const int i = lane + 32 * k;
-      if (i < NP) {
-        const int j = i + t;
-        const bool up = j < NP;
-        acc[k] += (TV)(up ? du[i] : dl[i]) * rs[up ? j : j - NP];
-      }
+// Bound by the FP64 pipe: a warp's instruction takes 64 cycles of its scheduler, 19 of the SM
+// when all four are busy, whatever lanes are active, so what counts is the number of warp
+// instructions.  Interior stars: the rows of all stars are laid over the lanes one after another
+// (row R of the launch is row R mod NP of star R / NP), so that every lane works, and a thread
+// forms one row over the wrapped diagonals t = 0 .. NP-1: entry (i, (i + t) mod NP) is entry i of
+// diagonal t while i + t < NP and entry i + t - NP of diagonal NP - t after (the symmetric
+// partner); consecutive rows read consecutive entries.  r of the block's stars is held twice
+// over in shared memory, so that no index wraps.  Boundary stars: a warp each, the free rows
+// times the free columns alone (27, 9 or 3 of 81 in 3D).  730 k warp products on 16^3 cells; a
+// warp per star, rows in three chunks of 32 and the identity rows of the boundary stars included,
+// took 1.19 M.  One FP64 cycle, three levels: 2070 us on 16^3 cells against 2711, 883 on 40 x 72
+// against 917.
+template <int DIM>
+struct Star64 {
+  static constexpr int NP = Sz<DIM>::NP, THREADS = 256, U = 9;   // U diagonals in flight (NP = 9 x 9 or 2 x 9)
+  static constexpr int SPAN = (THREADS + NP - 2) / NP + 1;       // stars that a block's rows touch
+};
+
+// boundary vertex b of the level: the planes of the last axis' ends first, then the rims between
+template <int DIM>
+__device__ __forceinline__ void boundary_vertex(const Geom& g, int b, int& vx, int& vy, int& vz) {
+  const int nx = g.nv[0], ny = g.nv[1];
+  vz = 0;
+  if (DIM == 3) {
+    const int plane = nx * ny, rim = 2 * nx + 2 * (ny - 2);
+    if (b < 2 * plane) {
+      vz = b < plane ? 0 : g.nv[2] - 1;
+      b -= b < plane ? 0 : plane;
+      vy = b / nx;
+      vx = b - vy * nx;
+      return;
     }
+    b -= 2 * plane;
+    vz = b / rim + 1;
+    b -= (vz - 1) * rim;
+  }
+  if (b < 2 * nx) {
+    vy = b < nx ? 0 : ny - 1;
+    vx = b < nx ? b : b - nx;
+  } else {
+    b -= 2 * nx;
+    vy = (b >> 1) + 1;
+    vx = (b & 1) ? nx - 1 : 0;
   }
 }
 
-template <typename TF, typename TV, int DIM>
-__global__ void __launch_bounds__(256) k_patch_apply(Geom g, const TF* __restrict__ inv, int pstride,
-                                                     const TV* __restrict__ r, TV* __restrict__ out) {
-  constexpr int NP = Sz<DIM>::NP, NB = Sz<DIM>::NB, R = (NP + 31) / 32;
-  __shared__ TV rsh[8][NP];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
-  pdl_wait();
-  for (long long v = (long long)blockIdx.x * (blockDim.x >> 5) + w; v < g.nverts; v += nwarps) {
-    int vx, vy, vz;
-    vertex_coords<DIM>(g, v, vx, vy, vz);
-    for (int i = lane; i < NP; i += 32) {
-      long long nd;
-      const bool ok = patch_node<DIM>(g, vx, vy, vz, i % NB, nd);
-      rsh[w][i] = ok ? r[(i / NB) * g.N + nd] : TV(0);
-    }
-    __syncwarp();
-    TV acc[R];
-    patch_gemv<TF, TV, DIM>(inv + v * pstride, rsh[w], lane, acc);
+// interior = 0: all star products into the scratch rows (entries of absent and Dirichlet nodes
+// are not written; nothing reads them), blocks from nbi on take the boundary stars;  1: the local
+// solves on the coarse-cell interiors, out (-)= at their nodes
+template <int DIM>
+__global__ void __launch_bounds__(256) k_star64(Geom g, const double* __restrict__ inv, int pstride, int interior,
+                                                int count, int nbi, int nbnd, const double* __restrict__ r,
+                                                double* __restrict__ out, int mode) {
+  using C = Star64<DIM>;
+  constexpr int NP = C::NP, NB = Sz<DIM>::NB, U = C::U;
+  __shared__ double r2[C::SPAN][2 * NP];
+  const int tid = threadIdx.x;
+  if ((int)blockIdx.x < nbi) {
+    const int R0 = blockIdx.x * C::THREADS, p0 = R0 / NP, p = (R0 + tid) / NP, i = R0 + tid - p * NP;
+    const bool act = p < count;
+    // the interior stars' list is that of split storage (wl bit 1), the inverses are every vertex's
+    int vx = 0, vy = 0, vz = 0;
+    work_vertex<DIM>(g, interior | 2, act ? p : 0, count, vx, vy, vz);
+    const double* S = inv + (long long)(vx + g.nv[0] * (vy + g.nv[1] * vz)) * pstride + i;
+    // diagonal t: entry i (or i - NP + NP - t of the partner diagonal)
+    auto entry = [&](int t) {
+      return __ldg(S + (i + t < NP ? diag_start(NP, t) : diag_start(NP, NP - t) - (NP - t)));
+    };
+    double cur[U];
 #pragma unroll
-    for (int k = 0; k < R; ++k) {
-      const int i = lane + 32 * k;
-      if (i < NP) out[patch_out_index<DIM>(g, vx, vy, vz, i)] = acc[k];
+    for (int u = 0; u < U; ++u) cur[u] = entry(u);
+    pdl_wait();
+    for (int e = tid; e < C::SPAN * NP; e += C::THREADS) {
+      const int s = e / NP, k = e - s * NP;
+      if (p0 + s < count) {
+        int wx, wy, wz;
+        work_vertex<DIM>(g, interior | 2, p0 + s, count, wx, wy, wz);
+        long long nd = 0;
+        patch_node<DIM>(g, wx, wy, wz, k % NB, nd);   // always inside
+        r2[s][k] = r2[s][k + NP] = r[(k / NB) * g.N + nd];
+      }
     }
-    __syncwarp();
+    __syncthreads();
+    const double* rr = &r2[p - p0][i];
+    double acc = 0.0;
+#pragma unroll
+    for (int t0 = 0; t0 < NP; t0 += U) {
+      double nxt[U];
+      if (t0 + U < NP) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) nxt[u] = entry(t0 + U + u);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) acc += cur[u] * rr[t0 + u];
+#pragma unroll
+      for (int u = 0; u < U; ++u) cur[u] = nxt[u];
+    }
+    if (act) {
+      if (!interior) {
+        out[patch_out_index<DIM>(g, vx, vy, vz, i)] = acc;
+      } else {
+        long long nd = 0;
+        patch_node<DIM>(g, vx, vy, vz, i % NB, nd);
+        double* o = out + (i / NB) * g.N + nd;
+        *o = mode == OUT_SUBTRACT ? *o - acc : acc;
+      }
+    }
+  } else {
+    constexpr int MMAX = DIM == 3 ? 27 : 6;
+    __shared__ double rb[8][MMAX];
+    __shared__ int eb[8][MMAX];
+    const int lane = tid & 31, w = tid >> 5, b = (blockIdx.x - nbi) * 8 + w;
+    if (b < nbnd) {
+      int vx, vy, vz;
+      boundary_vertex<DIM>(g, b, vx, vy, vz);
+      const StarAxes<DIM> ax(g, vx, vy, vz);
+      const double* S = inv + (long long)(vx + g.nv[0] * (vy + g.nv[1] * vz)) * pstride;
+      const int i = lane < ax.m ? ax.entry(lane) : 0;
+      pdl_wait();
+      if (lane < ax.m) {
+        long long nd = 0;
+        patch_node<DIM>(g, vx, vy, vz, i % NB, nd);   // a free node
+        rb[w][lane] = r[(i / NB) * g.N + nd];
+        eb[w][lane] = i;
+      }
+      __syncwarp();
+      double acc = 0.0;
+#pragma unroll 3
+      for (int c = 0; c < ax.m; ++c) {
+        const int j = eb[w][c], lo = i < j ? i : j, t = i < j ? j - i : i - j;
+        acc += __ldg(S + diag_start(NP, t) + lo) * rb[w][c];
+      }
+      if (lane < ax.m) out[patch_out_index<DIM>(g, vx, vy, vz, i)] = acc;
+    }
   }
+  pdl_trigger();
+}
+
+template <int DIM>
+static void launch_star64(const LevelDev& L, int interior, const double* r, double* out, int mode, cudaStream_t s) {
+  const Geom& g = L.g;
+  const long long nint = (long long)(g.nv[0] - 2) * (g.nv[1] - 2) * (DIM == 3 ? g.nv[2] - 2 : 1);
+  const long long count =
+      interior ? (long long)(g.n[0] / 2) * (g.n[1] / 2) * (DIM == 3 ? g.n[2] / 2 : 1) : nint;
+  const long long nbnd = interior ? 0 : g.nverts - nint;
+  const int nbi = (int)((count * Star64<DIM>::NP + Star64<DIM>::THREADS - 1) / Star64<DIM>::THREADS);
+  launch_pdl(k_star64<DIM>, (unsigned)(nbi + (nbnd + 7) / 8), Star64<DIM>::THREADS, 0, s, g, (const double*)L.inv64,
+             L.pstride, interior, (int)count, nbi, (int)nbnd, r, out, mode);
+  count_launch(1);
 }
 
 // z on GX consecutive nodes of a node row = sum of the outputs of the patches whose
@@ -1207,12 +1301,10 @@ size_t patch_scratch_bytes(const LevelDev& L, int prec) {
 template <int DIM>
 static void star_products64(const LevelDev& L, const double* r, double* scratch, cudaStream_t s, cudaEvent_t e0,
                             cudaEvent_t e1) {
-  const unsigned blocks = (unsigned)std::min<long long>((L.g.nverts + 7) / 8, 152LL * 16);
   // External records become event-record nodes when the stream is being captured
   if (e0) cudaEventRecordWithFlags(e0, s, cudaEventRecordExternal);
-  launch_pdl(k_patch_apply<double, double, DIM>, blocks, 256, 0, s, L.g, L.inv64, L.pstride, r, scratch);
+  launch_star64<DIM>(L, 0, r, scratch, OUT_SCRATCH, s);
   if (e1) cudaEventRecordWithFlags(e1, s, cudaEventRecordExternal);
-  count_launch(1);
 }
 
 // All star products y_v = A_v^-1 r|_v of a level into the scratch rows (FP32) with kernel
@@ -1266,64 +1358,19 @@ void patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scr
 // local solves on coarse-cell interiors (robust transfer, Eq. (Ptilde)):
 // coarse cell K <-> fine vertex 2K+1, whose star is exactly int(K)
 // ---------------------------------------------------------------------------
-template <typename TF, typename TV, int DIM>
-__global__ void __launch_bounds__(256) k_interior_solve(Geom g, const TF* __restrict__ inv, int pstride,
-                                                        const TV* __restrict__ in, TV* __restrict__ out,
-                                                        int subtract) {
-  constexpr int NP = Sz<DIM>::NP, NB = Sz<DIM>::NB, R = (NP + 31) / 32;
-  __shared__ TV rsh[8][NP];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int ncx = g.n[0] / 2, ncy = g.n[1] / 2, ncz = DIM == 3 ? g.n[2] / 2 : 1;
-  const long long ncoarse = (long long)ncx * ncy * ncz;
-  const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
-  pdl_wait();
-  for (long long K = (long long)blockIdx.x * (blockDim.x >> 5) + w; K < ncoarse; K += nwarps) {
-    const int kx = (int)(K % ncx), ky = (int)((K / ncx) % ncy), kz = DIM == 3 ? (int)(K / ((long long)ncx * ncy)) : 0;
-    const int vx = 2 * kx + 1, vy = 2 * ky + 1, vz = DIM == 3 ? 2 * kz + 1 : 0;
-    const long long v = (long long)vx + (long long)g.nv[0] * ((long long)vy + (long long)g.nv[1] * vz);
-    for (int i = lane; i < NP; i += 32) {
-      long long nd;
-      patch_node<DIM>(g, vx, vy, vz, i % NB, nd);  // always interior
-      rsh[w][i] = in[(i / NB) * g.N + nd];
-    }
-    __syncwarp();
-    TV acc[R];
-    patch_gemv<TF, TV, DIM>(inv + v * pstride, rsh[w], lane, acc);
-#pragma unroll
-    for (int k = 0; k < R; ++k) {
-      const int i = lane + 32 * k;
-      if (i < NP) {
-        long long nd;
-        patch_node<DIM>(g, vx, vy, vz, i % NB, nd);
-        TV* o = out + (i / NB) * g.N + nd;
-        *o = subtract ? *o - acc[k] : acc[k];
-      }
-    }
-    __syncwarp();
-  }
-}
-
-template <typename TF, typename TV, int DIM>
-static void interior_impl(const LevelDev& L, const TF* inv, const void* in, void* out, int subtract, cudaStream_t s) {
-  long long nc = (long long)(L.g.n[0] / 2) * (L.g.n[1] / 2) * (DIM == 3 ? L.g.n[2] / 2 : 1);
-  if (!subtract) cudaMemsetAsync(out, 0, sizeof(TV) * L.g.N * DIM, s);
-  const unsigned blocks = (unsigned)std::min<long long>((nc + 7) / 8, 152LL * 16);
-  launch_pdl(k_interior_solve<TF, TV, DIM>, blocks, 256, 0, s, L.g, inv, L.pstride, (const TV*)in, (TV*)out, subtract);
-  count_launch(1);
-}
-
 void patch_interior_solve(const LevelDev& fine, int prec, const void* in, void* out, int subtract, cudaStream_t s) {
   if (fine.k == 3) {
     qk_interior_solve(fine, prec, in, out, subtract, s);
     return;
   }
+  const int md = subtract ? OUT_SUBTRACT : OUT_WRITE;
   if (prec == PREC_F64) {
-    if (fine.g.dim == 2) interior_impl<double, double, 2>(fine, fine.inv64, in, out, subtract, s);
-    else interior_impl<double, double, 3>(fine, fine.inv64, in, out, subtract, s);
+    if (!subtract) cudaMemsetAsync(out, 0, sizeof(double) * fine.g.N * fine.g.dim, s);
+    if (fine.g.dim == 2) launch_star64<2>(fine, 1, (const double*)in, (double*)out, md, s);
+    else launch_star64<3>(fine, 1, (const double*)in, (double*)out, md, s);
   } else {
     const long long nc = (long long)(fine.g.n[0] / 2) * (fine.g.n[1] / 2) * (fine.g.dim == 3 ? fine.g.n[2] / 2 : 1);
     if (!subtract) cudaMemsetAsync(out, 0, sizeof(float) * fine.g.N * fine.g.dim, s);
-    const int md = subtract ? OUT_SUBTRACT : OUT_WRITE;
     const int v = patch_variant(fine);
     if (fine.g.dim == 2) launch_patch_variant<2>(v, fine, 1, nc, (const float*)in, (float*)out, md, fine.status, s);
     else launch_patch_variant<3>(v, fine, 1, nc, (const float*)in, (float*)out, md, fine.status, s);
