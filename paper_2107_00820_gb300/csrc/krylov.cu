@@ -237,8 +237,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_gm_start(unsigned n, const T* _
 }
 
 // Gram-Schmidt step j: w = column j+1 holds A Z_j with Z_j = D^-1 (column j) unscaled, so
-// A D^-1 v_j = w / hn[j];  H[i][j] = (V_i . w) / (hn[i] hn[j]),
-// V_{j+1} = w / hn[j] - sum_i V_i H[i][j] / hn[i], and the partials of |V_{j+1}|^2.
+// A D^-1 v_j = w / hn_j;  H[i][j] = (V_i . w) / (hn_i hn_j),
+// V_{j+1} = w / hn_j - sum_i V_i H[i][j] / hn_i, and the partials of |V_{j+1}|^2.
 // Every block adds the partials of the dots (and of |V_j|^2, before the wait: the kernel that
 // wrote them is three launches back) for itself.  The last block is an extra one: it does the
 // one-thread bookkeeping of step j - 1 while the others work.
@@ -255,8 +255,8 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
   T* w = const_cast<T*>(V) + (long long)(j + 1) * ld;
   T a[GM_PER];
   T vc[GM_PER][KMAXB];
-  T hni = T(0);
-  // columns 0..j, hn and the norm partials come from earlier kernels of the chain (complete
+  T rhni = T(0);
+  // columns 0..j, rhn and the norm partials come from earlier kernels of the chain (complete
   // before this launch began): read through L2 before the wait; column j+1 and the dots come
   // from the predecessor
   if (!extra) {
@@ -266,7 +266,7 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
 #pragma unroll
       for (int c = 0; c < KMAXB; ++c) vc[q][c] = (i < n && c <= j) ? __ldcg(V + (long long)c * ld + i) : T(0);
     }
-    if ((int)threadIdx.x < j) hni = __ldcg(st.hn + threadIdx.x);
+    if ((int)threadIdx.x < j) rhni = __ldcg(st.rhn + threadIdx.x);
   }
   sum_rows<T>(norm_rows<T>(sd, j), norm_count(sd, j, n), 1, acc);
   {
@@ -281,9 +281,8 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
     }
     return;
   }
-  const T hnj = sqrt(fmax(nrm2, T(0)));
-  const T inv = hnj != T(0) ? T(1) / hnj : T(0);
-  if ((int)threadIdx.x == j) hni = hnj;
+  const T inv = recip_or_zero<T>(sqrt(fmax(nrm2, T(0))));
+  if ((int)threadIdx.x == j) rhni = inv;
   pdl_wait();
 #pragma unroll
   for (int q = 0; q < GM_PER; ++q) {
@@ -294,15 +293,11 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
   {
     const T v = block_total<T>(acc, j + 1, sh);
     if ((int)threadIdx.x <= j) {
-      T h = T(0), c = T(0);
-      if (hni != T(0)) {
-        h = (v / hni) * inv;
-        c = h / hni;
-      }
-      coef[threadIdx.x] = c;
+      const T h = v * rhni * inv;
+      coef[threadIdx.x] = h * rhni;
       if (bx == 0) {
         st.H[(long long)j * st.ldh + threadIdx.x] = h;
-        if ((int)threadIdx.x == j) st.hn[j] = hnj;
+        if ((int)threadIdx.x == j) st.rhn[j] = inv;
       }
     }
   }
@@ -328,7 +323,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_gm_orth(unsigned n, int j, cons
   gm_orth_body<T>(blockIdx.x, gridDim.x, n, j, V, ld, sd);
 }
 
-// x = (x_zero ? 0 : x) + sum_j Z_j y_j / hn[j] with y = R^-1 g, and, if t != NULL, the
+// x = (x_zero ? 0 : x) + sum_j Z_j y_j / hn_j with y = R^-1 g, and, if t != NULL, the
 // GMRES residual  t = r0 - A Z y = sum_i u_i v_i,  u = Q^T (g[k] e_k)  from the
 // Arnoldi relation (Q = product of the Givens rotations), no operator apply.  Every block
 // finishes the last Givens step and forms y and u for itself, on a copy of the state.
@@ -339,6 +334,7 @@ __device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, int k, c
   __shared__ T sh[RED_THREADS / 32][KMAXB];
   __shared__ T state[GmresLayout(KMAXB).total];
   __shared__ T y[KMAXB], u[KMAXB + 1];
+  __shared__ T nrm2;
   static_assert(GmresLayout(KMAXB).total <= RED_THREADS, "one state entry a thread");
   const GmresView<T> st = gmres_view<T>(GmresDev{state, k});
   const unsigned base = bx * (RED_THREADS * GM_PER) + threadIdx.x;
@@ -357,17 +353,13 @@ __device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, int k, c
   if ((int)threadIdx.x < GmresLayout(k).total) state[threadIdx.x] = __ldcg(static_cast<const T*>(sd.base) + threadIdx.x);
   T acc[KMAXB];
   sum_rows<T>(norm_rows<T>(sd, k), norm_count(sd, k, n), 1, acc);
-  const T nrm2 = block_total<T>(acc, 1, sh);   // (its barrier also publishes the state)
-  if (threadIdx.x == 0) {
-    gmres_step(st, k - 1, nrm2);
-    gmres_coeffs(st, k);
-  }
+  const T tot = block_total<T>(acc, 1, sh);   // (its barrier also publishes the state)
+  if (threadIdx.x == 0) nrm2 = tot;
   __syncthreads();
-  if ((int)threadIdx.x < k) {
-    const T hn = st.hn[threadIdx.x];
-    y[threadIdx.x] = hn != T(0) ? st.yu[threadIdx.x] / hn : T(0);
-  } else if ((int)threadIdx.x <= 2 * k) {
-    u[threadIdx.x - k] = st.yu[threadIdx.x];
+  if (threadIdx.x < 64) {   // y and u in a warp each
+    const int what = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const T v = gmres_finish<T>(st, nrm2, what);
+    if (lane < k + what) (what ? u : y)[lane] = v;
   }
   __syncthreads();
 #pragma unroll

@@ -97,28 +97,47 @@ __device__ __forceinline__ void finish_sums(double* ws, int k, R* out, const R* 
   finish_sums_n<R>(ws, k, out, div, (int)gridDim.x);
 }
 
-// Sum of kk <= KMAXB columns over a block, returned to thread j < kk (others: 0): warp shuffles
-// with the columns interleaved, one shared pass.  The caller puts a barrier between the
-// return and the next use of sh.
+// a warp's sums of P columns: lane l returns that of column l mod P.  The columns are halved as
+// the lanes are paired (a lane passes on the half that its partner keeps), P - 1 + log2(32 / P)
+// additions instead of 5 P.
+template <int P, typename T>
+__device__ __forceinline__ T warp_totals(const T (&acc)[KMAXB]) {
+  const int lane = threadIdx.x & 31;
+  T v[P];
+#pragma unroll
+  for (int j = 0; j < P; ++j) v[j] = acc[j];
+#pragma unroll
+  for (int w = P / 2; w > 0; w >>= 1) {
+    const bool up = (lane & w) != 0;
+#pragma unroll
+    for (int j = 0; j < w; ++j) {
+      const T give = up ? v[j] : v[j + w];
+      v[j] = (up ? v[j + w] : v[j]) + __shfl_xor_sync(0xffffffffu, give, w);
+    }
+  }
+#pragma unroll
+  for (int o = P; o < 32; o <<= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  return v[0];
+}
+
+// Sum of kk <= KMAXB columns over a block, returned to thread j < kk (the others' value is
+// unspecified).  The caller puts a barrier between the return and the next use of sh.  Few
+// instructions above all for FP64, where a warp's takes 64 cycles of its scheduler: with a shuffle
+// tree per column and a serial sum over the warps the sums of four columns took 28 additions, 9 now.
 template <typename T>
 __device__ __forceinline__ T block_total(const T (&acc)[KMAXB], int kk, T (&sh)[RED_THREADS / 32][KMAXB]) {
-  T v[KMAXB];
-#pragma unroll
-  for (int j = 0; j < KMAXB; ++j) v[j] = acc[j];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-    for (int j = 0; j < KMAXB; ++j)
-      if (j < kk) v[j] += __shfl_down_sync(0xffffffffu, v[j], o);
-  if ((threadIdx.x & 31) == 0)
-#pragma unroll
-    for (int j = 0; j < KMAXB; ++j)
-      if (j < kk) sh[threadIdx.x >> 5][j] = v[j];
+  static_assert(RED_THREADS == 256 && KMAXB == 8, "a warp adds 8 rows of 8 columns");
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const T v = kk == 1 ? warp_totals<1>(acc) : kk == 2 ? warp_totals<2>(acc) : kk <= 4 ? warp_totals<4>(acc) : warp_totals<8>(acc);
+  if (lane < kk) sh[w][lane] = v;
   __syncthreads();
   T t = T(0);
-  if ((int)threadIdx.x < kk)
-#pragma unroll
-    for (int i = 0; i < RED_THREADS / 32; ++i) t += sh[i][threadIdx.x];
+  if (w == 0) {
+    const int c = lane & 7, r = lane >> 3;
+    if (c < kk) t = sh[r][c] + sh[r + 4][c];
+    t += __shfl_xor_sync(0xffffffffu, t, 8);
+    t += __shfl_xor_sync(0xffffffffu, t, 16);
+  }
   return t;
 }
 
@@ -138,16 +157,19 @@ __device__ __forceinline__ void sum_rows(const T* __restrict__ rows, int nb, int
 // ---------------------------------------------------------------------------
 // GMRES(s) state on the device, in the smoother's precision T (column-major
 // Hessenberg H, leading dim ldh).  The Krylov basis is stored unnormalised:
-// column i holds hn[i] * v_i, where v_i is the orthonormal Arnoldi vector, and
-// Z_i = D^-1 (column i) likewise; their consumers divide by hn[i].  Layout of the state array, in elements of T:
-// H [ldh s] | cs [s] | sn [s] | g [s+1] | y [s] | res | beta | nrm2 | hn [s+1] | yu [2s+1].
+// column i holds hn_i v_i, where v_i is the orthonormal Arnoldi vector, and
+// Z_i = D^-1 (column i) likewise; their consumers multiply by rhn[i] = 1 / hn_i, and rr[i] = 1 / R_ii
+// (both 0 where the divisor is): the divisions are done once, by the bookkeeping block beside
+// the vector work, and none but those of the last step is left for the update.
+// Layout of the state array, in elements of T:
+// H [ldh s] | cs [s] | sn [s] | g [s+1] | y [s] | res | beta | nrm2 | rhn [s+1] | rr [s].
 // ---------------------------------------------------------------------------
 struct GmresLayout {
   int s, ldh;
-  int H, cs, sn, g, y, res, beta, nrm2, hn, yu, total;
+  int H, cs, sn, g, y, res, beta, nrm2, rhn, rr, total;
   __host__ __device__ constexpr explicit GmresLayout(int steps)
       : s(steps), ldh(steps + 1), H(0), cs((steps + 1) * steps), sn(cs + steps), g(sn + steps), y(g + steps + 1),
-        res(y + steps), beta(res + 1), nrm2(beta + 1), hn(nrm2 + 1), yu(hn + steps + 1), total(yu + 2 * steps + 1) {}
+        res(y + steps), beta(res + 1), nrm2(beta + 1), rhn(nrm2 + 1), rr(rhn + steps + 1), total(rr + steps) {}
 };
 
 // host-side handle: the state array (elements of the smoother's precision), s, and the block
@@ -197,17 +219,36 @@ struct GmresView {
   T* sn;
   T* g;       // rotated right-hand side, length s + 1
   T* res;     // |g[k+1]| after step k
-  T* hn;      // stored-column norms, length s + 1
+  T* rhn;     // 1 / norms of the stored columns, length s + 1 (written by the Gram-Schmidt steps)
+  T* rr;      // 1 / R_ii, length s
   T* beta;    // |r0|
   int m;      // s + 1
-  T* yu;      // after the last step: y = R^-1 g (s entries), then u = Q^T (g[s] e_s) / hn (s + 1)
 };
 
 template <typename T>
 __host__ __device__ __forceinline__ GmresView<T> gmres_view(const GmresDev& d) {
   const GmresLayout L(d.s);
   T* b = static_cast<T*>(d.base);
-  return GmresView<T>{b + L.H, L.ldh, b + L.cs, b + L.sn, b + L.g, b + L.res, b + L.hn, b + L.beta, d.s + 1, b + L.yu};
+  return GmresView<T>{b + L.H, L.ldh, b + L.cs, b + L.sn, b + L.g, b + L.res, b + L.rhn, b + L.rr, b + L.beta, d.s + 1};
+}
+
+// 1 / a, or 0 where a is 0 or so small that 1 / a overflows (no direction is left)
+template <typename T>
+__device__ __forceinline__ T recip_or_zero(T a) {
+  const T r = T(1) / a;
+  return isfinite(r) ? r : T(0);
+}
+
+// Givens rotation (c, s) of (a, b), b >= 0, and r = |(a, b)|; the plain sum of squares where
+// it is far from over- and underflow (hypot takes several times the FP64 instructions)
+template <typename T>
+__device__ __forceinline__ void givens(T a, T b, T& c, T& s, T& r) {
+  constexpr T lo = sizeof(T) == 8 ? T(1e-200) : T(1e-20), hi = T(1) / lo;
+  const T q = a * a + b * b;
+  r = q > lo && q < hi ? sqrt(q) : hypot(a, b);
+  c = T(1);
+  s = T(0);
+  if (r > T(0)) { c = a / r; s = b / r; }
 }
 
 // start: beta = |r0|, g = (beta, 0, ...), hn[0] = beta   (one thread)
@@ -215,12 +256,11 @@ template <typename T>
 __device__ __forceinline__ void gmres_start(const GmresView<T>& st, T nrm2) {
   const T b = sqrt(fmax(nrm2, T(0)));
   st.beta[0] = b;
-  st.hn[0] = b;
   st.g[0] = b;
   for (int i = 1; i < st.m; ++i) st.g[i] = T(0);
 }
 
-// step k (k < KMAXB): H[k+1][k] = |w|, hn[k+1] = |w|, then the rotations of
+// step k (k < KMAXB): H[k+1][k] = |w|, then the rotations of
 // column k; all operands are loaded first and every index is a compile-time one (loops
 // unrolled to KMAXB, predicated), so the chain runs in registers (one thread).  With runtime
 // loop bounds the arrays lived in local memory, and this chain, on the serial tail of every
@@ -245,55 +285,73 @@ __device__ __forceinline__ void gmres_step(const GmresView<T>& st, int k, T nrm2
       h[i] = cs[i] * a + sn[i] * b;
       a = -sn[i] * a + cs[i] * b;
     }
-  const T b = hk1;
-  const T r = hypot(a, b);
-  T c = T(1), sv = T(0);
-  if (r > T(0)) { c = a / r; sv = b / r; }
+  T c, sv, r;
+  givens<T>(a, hk1, c, sv, r);
 #pragma unroll
   for (int i = 0; i < KMAXB; ++i)
     if (i <= k) hg[i] = i == k ? r : h[i];
   hg[k + 1] = T(0);
-  st.hn[k + 1] = hk1;
+  st.rr[k] = recip_or_zero<T>(r);
   st.cs[k] = c; st.sn[k] = sv;
   st.g[k + 1] = -sv * gk;
   st.g[k] = c * gk;
   st.res[0] = fabs(sv * gk);
 }
 
-// after step k - 1 (one thread): y = R^-1 g by back substitution on the rotated
-// Hessenberg matrix, and u = Q^T (g[k] e_k) / hn (Q = product of the Givens
-// rotations), so that x + Z y is the GMRES iterate and its residual is
-// sum_i u_i (stored column i) by the Arnoldi relation.  Stored in st.yu.
+// The last step's rotations (k = s - 1, not written back) and, by the warp that calls,
+//   what = 0: lane i < s: y_i / hn_i, y = R^-1 g by back substitution on the rotated matrix;
+//   what = 1: lane i <= s: u_i, u = Q^T (g[s] e_s) / hn (Q = product of the Givens rotations),
+// so that x + sum_i Z_i y_i / hn_i is the GMRES iterate and its residual is
+// sum_i u_i (stored column i) by the Arnoldi relation.  Lane i holds row i: what the rotations
+// and the substitution do to all rows is one instruction each, and the chains are one
+// multiply-add a step.
 template <typename T>
-__device__ __forceinline__ void gmres_coeffs(const GmresView<T>& st, int k) {
-  // (the stores come last: they may alias the state, and would hold the loads back)
-  T ys[KMAXB], us[KMAXB];
+__device__ __forceinline__ T gmres_finish(const GmresView<T>& st, T nrm2, int what) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int s = st.m - 1, k = s - 1, lane = threadIdx.x & 31, i = lane < KMAXB ? lane : 0;
+  const T* hg = st.H + (long long)k * st.ldh;
+  const bool old = lane < k;
+  const T cs = old ? st.cs[i] : T(1), sn = old ? st.sn[i] : T(0);
+  const T b1 = old ? hg[i + 1] : T(0);
+  const T hk1 = sqrt(fmax(nrm2, T(0)));
+  // a_0 = h_0;  a_(i+1) = cs_i h_(i+1) - sn_i a_i;  R_ik = cs_i a_i + sn_i h_(i+1)
+  const T q = cs * b1;
+  T a = hg[0], mine = a;
 #pragma unroll
-  for (int i = KMAXB - 1; i >= 0; --i) {
-    if (i >= k) continue;
-    T a = st.g[i];
-#pragma unroll
-    for (int c = 0; c < KMAXB; ++c)
-      if (c > i && c < k) a -= st.H[(long long)c * st.ldh + i] * ys[c];
-    const T d = st.H[(long long)i * st.ldh + i];
-    ys[i] = d != T(0) ? a / d : T(0);
-  }
-  T b = st.g[k];                    // u_(i+1) before rotation i is undone (u_0..u_i are still 0)
-#pragma unroll
-  for (int i = KMAXB - 1; i >= 0; --i) {
-    if (i >= k) continue;
-    const T hn = st.hn[i + 1];
-    us[i] = hn != T(0) ? (st.cs[i] * b) / hn : T(0);
-    b = -(st.sn[i] * b);
-  }
-  const T h0 = st.hn[0];
-#pragma unroll
-  for (int i = 0; i < KMAXB; ++i)
-    if (i < k) {
-      st.yu[i] = ys[i];
-      st.yu[k + i + 1] = us[i];
+  for (int t = 0; t < KMAXB - 1; ++t)
+    if (t < k) {
+      a = __shfl_sync(FULL, q, t) - __shfl_sync(FULL, sn, t) * a;
+      if (lane == t + 1) mine = a;
     }
-  st.yu[k] = h0 != T(0) ? b / h0 : T(0);
+  T c, sv, r;
+  givens<T>(a, hk1, c, sv, r);
+  const T gk = st.g[k];
+  if (what == 0) {
+    T acc = lane < k ? st.g[i] : lane == k ? c * gk : T(0);
+    const T rik = cs * mine + sn * b1;
+    const T rr = lane < k ? st.rr[i] : lane == k ? recip_or_zero<T>(r) : T(0);
+    T y = T(0);
+#pragma unroll
+    for (int t = KMAXB - 1; t >= 0; --t)
+      if (t < s) {
+        const T yt = __shfl_sync(FULL, acc * rr, t);
+        if (lane == t) y = yt;
+        const T h = t == k ? rik : lane < t ? st.H[(long long)t * st.ldh + i] : T(0);
+        acc -= h * yt;
+      }
+    return lane < s ? y * st.rhn[i] : T(0);
+  }
+  // u_i = cs_(i-1) b_i / hn_i with b_s = g[s], b_(i-1) = -sn_(i-1) b_i; u_0 = b_0 / hn_0
+  T b = -sv * gk, u = b;
+#pragma unroll
+  for (int t = KMAXB - 1; t >= 0; --t)
+    if (t < s) {
+      const T ct = t == k ? c : __shfl_sync(FULL, cs, t), st_ = t == k ? sv : __shfl_sync(FULL, sn, t);
+      if (lane == t + 1) u = ct * b;
+      b = -(st_ * b);
+    }
+  if (lane == 0) u = b;
+  return lane < s ? u * st.rhn[lane] : lane == s ? u * recip_or_zero<T>(hk1) : T(0);
 }
 
 }  // namespace als
