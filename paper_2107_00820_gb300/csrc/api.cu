@@ -201,6 +201,9 @@ als_status alloc_work(als_ctx* c, MGWork& w, int prec) {
     w.b[l] = p; w.x[l] = p + len * w.es; w.t[l] = p + 2 * len * w.es;
     w.t2[l] = p + 3 * len * w.es; w.t3[l] = p + 4 * len * w.es;
     if (l > 0) {
+      // t2 is written by the interior solves alone, at the nodes inside the coarse cells: zeroed
+      // here, it is the sum over coarse cells with 0 on their faces ever after
+      cudaMemsetAsync(w.t2[l], 0, len * w.es, c->stream);
       char* q = nullptr;
       ALS_TRY(dalloc(c, &q, patch_scratch_bytes(c->lev[l], prec)));
       w.scratch[l] = q;
@@ -336,8 +339,8 @@ void smooth(als_ctx* c, MGWork& w, int l, bool x_is_zero = false) {
       vec_axpby(prec, len, 1.0, w.b[l], -1.0, w.t[l], s);                 // t = b - A x
       cudaEvent_t e0 = nullptr, e1 = nullptr;
       if (l == c->L - 1) prof_events(c, t_prof_counter, e0, e1);
-      patch_smooth(Lv, prec, w.t[l], w.t2[l], w.scratch[l], s, e0, e1);  // t2 = D^-1 t
-      vec_axpby(prec, len, c->opt.tau, w.t2[l], 1.0, w.x[l], s);         // x += tau t2
+      patch_smooth(Lv, prec, w.t[l], w.t3[l], w.scratch[l], s, e0, e1);  // t3 = D^-1 t
+      vec_axpby(prec, len, c->opt.tau, w.t3[l], 1.0, w.x[l], s);         // x += tau t3
     }
     return;
   }

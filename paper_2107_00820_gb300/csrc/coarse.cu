@@ -292,42 +292,73 @@ __device__ __forceinline__ int free_dof32(const Geom& g, int f) {
   return c * (int)g.N + i + g.nn[0] * (j + g.nn[1] * k);
 }
 
-// x_free = inv b_free, one warp per row.  STAGE: b at the free dofs is first
-// gathered into shared memory (as double) by every block; otherwise (coarse
+// x_free = inv b_free, x = 0 at Dirichlet nodes; one warp per row.  STAGE: b at the free dofs is
+// first gathered into shared memory (as double) by every block; otherwise (coarse
 // problems too large for shared memory) each term reads b through the index map.
-// Four independent FP64 partial sums per lane (dependent FP64 adds are slow on
-// this GPU), combined in a fixed order.
+// A serial chain of latencies, with the FP64 pipe's 2.2 us (3D, 4^3 cells: 1029^2 products) in it:
+// a lane's part of the row, up to 32 entries, and the staging indices are in registers before
+// the wait on the predecessor.  Four independent FP64 partial sums per lane, combined in a
+// fixed order.  Rows read as they were used and the zeros by a memset before (a node without the
+// early start of a programmatic launch, as one before each interior solve was) made a 16^2 two-level
+// cycle 172 us, 166 now, and a 32^3 four-level cycle 1799, 1783 now.
 template <typename TV, bool STAGE>
-__device__ __forceinline__ void coarse_apply_body(unsigned bx, const Geom& g, int nfree, const double* __restrict__ inv,
-                                                  const TV* __restrict__ b, TV* __restrict__ x) {
+__device__ __forceinline__ void coarse_apply_body(unsigned bx, unsigned nb, const Geom& g, int nfree,
+                                                  const double* __restrict__ inv, const TV* __restrict__ b,
+                                                  TV* __restrict__ x) {
   extern __shared__ double bs[];
-  pdl_wait();
-  if (STAGE) {
-    for (int c = threadIdx.x; c < nfree; c += blockDim.x) bs[c] = (double)b[free_dof32(g, c)];
-    __syncthreads();
-  }
+  constexpr int RP = 32, SP = 8;   // row entries a lane, staged entries a thread held ahead
   const int lane = threadIdx.x & 31;
   const int r = bx * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (r >= nfree) return;
-  const double* row = inv + (long long)r * nfree;
-  auto bv = [&](int c) { return STAGE ? bs[c] : (double)b[free_dof32(g, c)]; };
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-  int c = lane;
-  for (; c + 96 < nfree; c += 128) {
-    a0 += row[c] * bv(c);
-    a1 += row[c + 32] * bv(c + 32);
-    a2 += row[c + 64] * bv(c + 64);
-    a3 += row[c + 96] * bv(c + 96);
+  const double* row = inv + (long long)(r < nfree ? r : 0) * nfree;
+  double rv[RP];
+#pragma unroll
+  for (int p = 0; p < RP; ++p) rv[p] = lane + 32 * p < nfree ? __ldg(row + lane + 32 * p) : 0.0;
+  int at[SP];
+  if (STAGE) {
+#pragma unroll
+    for (int p = 0; p < SP; ++p) {
+      const int c = threadIdx.x + 256 * p;
+      at[p] = c < nfree ? free_dof32(g, c) : -1;
+    }
   }
-  for (; c < nfree; c += 32) a0 += row[c] * bv(c);
-  double acc = (a0 + a1) + (a2 + a3);
+  const int out = lane == 0 && r < nfree ? free_dof32(g, r) : 0;
+  pdl_wait();
+  if (STAGE) {
+    TV v[SP];
+#pragma unroll
+    for (int p = 0; p < SP; ++p) v[p] = at[p] >= 0 ? b[at[p]] : TV(0);
+#pragma unroll
+    for (int p = 0; p < SP; ++p)
+      if ((int)threadIdx.x + 256 * p < ((nfree + 31) & ~31)) bs[threadIdx.x + 256 * p] = (double)v[p];
+    for (int c = threadIdx.x + 256 * SP; c < ((nfree + 31) & ~31); c += 256) bs[c] = c < nfree ? (double)b[free_dof32(g, c)] : 0.0;
+    __syncthreads();
+  }
+  const int len = (int)g.N * g.dim;
+  for (int e = bx * 256 + threadIdx.x; e < len; e += nb * 256) {
+    const int n = e % (int)g.N, q = n / g.nn[0], i = n - q * g.nn[0], k = q / g.nn[1], j = q - k * g.nn[1];
+    if (i == 0 || i == g.nn[0] - 1 || j == 0 || j == g.nn[1] - 1 || (g.dim == 3 && (k == 0 || k == g.nn[2] - 1)))
+      x[e] = TV(0);
+  }
+  if (r >= nfree) return;
+  auto bv = [&](int c) { return STAGE ? bs[c] : c < nfree ? (double)b[free_dof32(g, c)] : 0.0; };
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+  for (int p = 0; p < RP; ++p)
+    if (32 * p < nfree) a[p & 3] += rv[p] * bv(lane + 32 * p);
+  int c = lane + 32 * RP;
+  for (; c + 96 < nfree; c += 128) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) a[u] += row[c + 32 * u] * bv(c + 32 * u);
+  }
+  for (; c < nfree; c += 32) a[0] += row[c] * bv(c);
+  double acc = (a[0] + a[1]) + (a[2] + a[3]);
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if (lane == 0) x[free_dof32(g, r)] = (TV)acc;
+  if (lane == 0) x[out] = (TV)acc;
 }
 template <typename TV, bool STAGE>
 __global__ void __launch_bounds__(256) k_coarse_apply(Geom g, int nfree, const double* __restrict__ inv,
                                                       const TV* __restrict__ b, TV* __restrict__ x) {
-  coarse_apply_body<TV, STAGE>(blockIdx.x, g, nfree, inv, b, x);
+  coarse_apply_body<TV, STAGE>(blockIdx.x, gridDim.x, g, nfree, inv, b, x);
 }
 
 // merged launch (batch.cuh), FP32
@@ -342,14 +373,15 @@ template <bool STAGE>
 __global__ void __launch_bounds__(256) k_coarse_apply_b(const __grid_constant__ BatchTab<CoarseArgs> tb) {
   const int i = batch_slot(tb, blockIdx.x);
   const CoarseArgs& a = tb.a[i];
-  coarse_apply_body<float, STAGE>(blockIdx.x - tb.start[i], a.g, a.nfree, a.inv, a.b, a.x);
+  coarse_apply_body<float, STAGE>(blockIdx.x - tb.start[i], tb.start[i + 1] - tb.start[i], a.g, a.nfree, a.inv, a.b, a.x);
 }
 
 constexpr size_t kCoarseStageMax = 200 * 1024;   // largest staged right-hand side (bytes)
+static size_t coarse_stage_bytes(int nfree) { return (size_t)((nfree + 31) & ~31) * sizeof(double); }
 
 // shared-memory opt-in of the staged apply, set at setup (never while a cycle is captured)
 static void coarse_apply_prepare(int nfree) {
-  const size_t smem = (size_t)nfree * sizeof(double);
+  const size_t smem = coarse_stage_bytes(nfree);
   if (smem > 48 * 1024 && smem <= kCoarseStageMax) {
     cudaFuncSetAttribute(k_coarse_apply<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaFuncSetAttribute(k_coarse_apply<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -359,7 +391,7 @@ static void coarse_apply_prepare(int nfree) {
 template <typename TV>
 static void launch_coarse_apply(const LevelDev& L, const CoarseDev& C, const TV* b, TV* x, cudaStream_t s) {
   const unsigned blocks = (unsigned)((C.nfree + 7) / 8);
-  const size_t smem = (size_t)C.nfree * sizeof(double);
+  const size_t smem = coarse_stage_bytes(C.nfree);
   if (smem <= kCoarseStageMax) {   // opt-in above 48 KB set by coarse_apply_prepare at setup
     launch_pdl(k_coarse_apply<TV, true>, blocks, 256, smem, s, L.g, C.nfree, (const double*)C.inv, b, x);
   } else {
@@ -368,33 +400,28 @@ static void launch_coarse_apply(const LevelDev& L, const CoarseDev& C, const TV*
 }
 
 void coarse_apply(const LevelDev& L, const CoarseDev& C, int prec, const void* b, void* x, cudaStream_t s) {
-  const long long len = L.g.N * L.g.dim;
-  cudaMemsetAsync(x, 0, len * (prec == PREC_F64 ? 8 : 4), s);
   if (prec == PREC_F64) launch_coarse_apply<double>(L, C, (const double*)b, (double*)x, s);
   else launch_coarse_apply<float>(L, C, (const float*)b, (float*)x, s);
   count_launch(1);
 }
 
-// merged: x = 0, then x_free = inv b_free for every item (the staged form when every
+// merged: the same for every item (the staged form when every
 // item's right-hand side fits the staging limit, with room for the largest)
 int batch_coarse_apply(const std::vector<BCoarse>& items, cudaStream_t s) {
-  std::vector<BZero> z;
   std::vector<CoarseArgs> a;
   std::vector<unsigned> nb;
   int maxfree = 0;
   for (const BCoarse& it : items) {
-    z.push_back(BZero{it.x, it.L->g.N * it.L->g.dim});
     a.push_back(CoarseArgs{it.L->g, it.C->nfree, (const double*)it.C->inv, (const float*)it.b, (float*)it.x});
     nb.push_back((unsigned)((it.C->nfree + 7) / 8));
     maxfree = std::max(maxfree, it.C->nfree);
   }
-  const int nz = batch_zero(z, s);
-  const size_t smem = (size_t)maxfree * sizeof(double);
+  const size_t smem = coarse_stage_bytes(maxfree);
   int n = 0;
   if (smem <= kCoarseStageMax) n = launch_batch(k_coarse_apply_b<true>, a, nb, 256, smem, s);
   else n = launch_batch(k_coarse_apply_b<false>, a, nb, 256, 0, s);
   count_launch(n);
-  return nz + n;
+  return n;
 }
 
 // shared-memory opt-in of the merged staged apply (before any capture)

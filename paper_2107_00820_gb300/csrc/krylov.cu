@@ -460,21 +460,6 @@ __global__ void __launch_bounds__(RED_THREADS) k_gm_update_b(const __grid_consta
   gm_update_body<float>(blockIdx.x - tb.start[i], a.n, a.st.s, a.Z, a.V, a.ld, a.st, a.x, a.x_zero, a.t);
 }
 
-struct ZeroArgs {
-  float* x;
-  unsigned n;
-};
-__global__ void __launch_bounds__(256) k_zero_b(const __grid_constant__ BatchTab<ZeroArgs> tb) {
-  const int i = batch_slot(tb, blockIdx.x);
-  const ZeroArgs& a = tb.a[i];
-  pdl_wait();
-  const unsigned e = (blockIdx.x - tb.start[i]) * 1024u + threadIdx.x;
-#pragma unroll
-  for (int q = 0; q < 4; ++q)
-    if (e + 256u * q < a.n) a.x[e + 256u * q] = 0.f;
-  pdl_trigger();
-}
-
 static int batch_gm(void (*k)(BatchTab<GmArgs>), const std::vector<BGmres>& items, int extra, cudaStream_t s) {
   std::vector<GmArgs> a;
   std::vector<unsigned> nb;
@@ -489,18 +474,6 @@ static int batch_gm(void (*k)(BatchTab<GmArgs>), const std::vector<BGmres>& item
 int batch_gm_start(const std::vector<BGmres>& items, cudaStream_t s) { return batch_gm(k_gm_start_b, items, 0, s); }
 int batch_gm_orth(const std::vector<BGmres>& items, cudaStream_t s) { return batch_gm(k_gm_orth_b, items, 1, s); }
 int batch_gm_update(const std::vector<BGmres>& items, cudaStream_t s) { return batch_gm(k_gm_update_b, items, 0, s); }
-
-int batch_zero(const std::vector<BZero>& items, cudaStream_t s) {
-  std::vector<ZeroArgs> a;
-  std::vector<unsigned> nb;
-  for (const BZero& it : items) {
-    a.push_back(ZeroArgs{(float*)it.x, (unsigned)it.n});
-    nb.push_back((unsigned)((it.n + 1023) / 1024));
-  }
-  const int n = launch_batch(k_zero_b, a, nb, 256, 0, s);
-  count_launch(n);
-  return n;
-}
 
 // workspace of the smoother's fused reductions: KMAXB + 2 rows of one value per block (the
 // gathers have at most 0.4 n / 256 + 1 blocks: four nodes a thread, rows of at least five nodes)

@@ -117,7 +117,8 @@ void patch_products(const LevelDev& L, int prec, const void* r, void* scratch, c
 // times the FP32 patch-kernel variants on this level and keeps the fastest (ms_out[3], optional)
 int patch_autotune(LevelDev& L, const void* r, void* scratch, cudaStream_t s, float* ms_out = nullptr);
 // local solves on the coarse-cell interiors (stars of the fine vertices at the
-// coarse-cell centres):  mode 0: out = sum_K E_K A_K^-1 E_K^T in  (out zeroed first)
+// coarse-cell centres):  mode 0: out = sum_K E_K A_K^-1 E_K^T in  at the nodes inside the
+//                                coarse cells; those on their faces are left (0 in the work vector)
 //                        mode 1: out -= sum_K E_K A_K^-1 E_K^T in
 void patch_interior_solve(const LevelDev& fine, int prec, const void* in, void* out, int subtract,
                           cudaStream_t s);
@@ -276,11 +277,6 @@ struct BGmres {            // gm_start (b, V), gm_orth (V, j), gm_update (Z, V, 
 int batch_gm_start(const std::vector<BGmres>& items, cudaStream_t s);
 int batch_gm_orth(const std::vector<BGmres>& items, cudaStream_t s);
 int batch_gm_update(const std::vector<BGmres>& items, cudaStream_t s);
-struct BZero {
-  void* x;
-  long long n;             // floats
-};
-int batch_zero(const std::vector<BZero>& items, cudaStream_t s);
 // resident CTAs per SM of a merged star kernel (variant 0, 1, 2 as above; 3: boundary stars)
 int batch_patch_occupancy(int variant);
 // shared-memory opt-ins of the merged star kernels; call before the first capture

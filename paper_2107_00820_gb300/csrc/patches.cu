@@ -1365,12 +1365,10 @@ void patch_interior_solve(const LevelDev& fine, int prec, const void* in, void* 
   }
   const int md = subtract ? OUT_SUBTRACT : OUT_WRITE;
   if (prec == PREC_F64) {
-    if (!subtract) cudaMemsetAsync(out, 0, sizeof(double) * fine.g.N * fine.g.dim, s);
     if (fine.g.dim == 2) launch_star64<2>(fine, 1, (const double*)in, (double*)out, md, s);
     else launch_star64<3>(fine, 1, (const double*)in, (double*)out, md, s);
   } else {
     const long long nc = (long long)(fine.g.n[0] / 2) * (fine.g.n[1] / 2) * (fine.g.dim == 3 ? fine.g.n[2] / 2 : 1);
-    if (!subtract) cudaMemsetAsync(out, 0, sizeof(float) * fine.g.N * fine.g.dim, s);
     const int v = patch_variant(fine);
     if (fine.g.dim == 2) launch_patch_variant<2>(v, fine, 1, nc, (const float*)in, (float*)out, md, fine.status, s);
     else launch_patch_variant<3>(v, fine, 1, nc, (const float*)in, (float*)out, md, fine.status, s);
@@ -1557,18 +1555,14 @@ int batch_patch_gather(const std::vector<BPatch>& items, cudaStream_t s) {
 
 int batch_interior_solve(int variant, const std::vector<BPatch>& items, int subtract, cudaStream_t s) {
   std::vector<PatchArgs> a;
-  std::vector<BZero> z;
   for (const BPatch& it : items) {
     const Geom& g = it.L->g;
     const long long nc = (long long)(g.n[0] / 2) * (g.n[1] / 2) * (g.dim == 3 ? g.n[2] / 2 : 1);
     a.push_back(patch_args(*it.L, 1, nc, it.r, it.out, subtract ? OUT_SUBTRACT : OUT_WRITE));
-    if (!subtract) z.push_back(BZero{it.out, g.N * g.dim});
   }
-  int n = 0;
-  if (!z.empty()) n += batch_zero(z, s);   // counted there
-  const int m = launch_patch_b(variant, a, s);
-  count_launch(m);
-  return n + m;
+  const int n = launch_patch_b(variant, a, s);
+  count_launch(n);
+  return n;
 }
 
 // Autotuner: times each FP32 patch-kernel variant on this level (one warm-up and

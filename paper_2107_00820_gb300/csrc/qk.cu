@@ -959,8 +959,6 @@ void qk_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* 
 void qk_interior_solve(const LevelDev& fine, int prec, const void* in, void* out, int subtract, cudaStream_t s) {
   if (fine.g.dim == 3) return qk3_interior_solve(fine, prec, in, out, subtract, s);
   const long long nc = (long long)(fine.g.n[0] / 2) * (fine.g.n[1] / 2);
-  const size_t es = prec == PREC_F64 ? 8 : 4;
-  if (!subtract) cudaMemsetAsync(out, 0, es * 2 * fine.g.N, s);
   constexpr int W64 = qk::star_warps<double>(), W32 = qk::star_warps<float>();
   if (prec == PREC_F64)
     qk::k_qk_star_apply<double><<<(unsigned)((nc + W64 - 1) / W64), 32 * W64, 0, s>>>(

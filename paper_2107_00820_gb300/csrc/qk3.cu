@@ -1570,8 +1570,6 @@ void qk3_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void*
 
 void qk3_interior_solve(const LevelDev& fine, int prec, const void* in, void* out, int subtract, cudaStream_t s) {
   const long long nc = (long long)(fine.g.n[0] / 2) * (fine.g.n[1] / 2) * (fine.g.n[2] / 2);
-  const size_t es = prec == PREC_F64 ? 8 : 4;
-  if (!subtract) cudaMemsetAsync(out, 0, es * 3 * fine.g.N, s);
   if (prec == PREC_F64) {
     qk3::k_qk3_star_apply<double><<<(unsigned)nc, qk3::STAR_THREADS, 0, s>>>(
         fine.g, fine.inv64, fine.pstride, 1, subtract ? 2 : 1, (const double*)in, (double*)out);
