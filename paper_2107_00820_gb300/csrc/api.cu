@@ -213,8 +213,8 @@ als_status alloc_work(als_ctx* c, MGWork& w, int prec) {
       ALS_TRY(dalloc(c, &w.small[l], sl.total));
     }
   }
-  const size_t npart = std::max(multidot_partial_doubles(std::max(s + 1, 8)),
-                                 gmres_partial_doubles(c->lev[c->L - 1].g.N * c->dim));
+  size_t npart = multidot_partial_doubles(std::max(s + 1, 8));
+  for (int l = 1; l < L; ++l) npart = std::max(npart, gmres_partial_doubles(c->lev[l]));
   ALS_TRY(dalloc(c, &w.partial, npart));
   cudaMemsetAsync(w.partial, 0, sizeof(double) * npart, c->stream);
   return ALS_OK;
@@ -291,15 +291,39 @@ bool fuse_patch_gather(const als_ctx* c) {
   return v == 1 && c->k == 2;
 }
 
+// levels whose Arnoldi steps are one launch each
+bool tiled_steps(const als_ctx* c, const MGWork& w, int l) {
+  return fuse_patch_gather(c) && arnoldi_tiled(c->lev[l], w.prec);
+}
+
+// step j of a tiled smoothing: w goes through two buffers in the star products' scratch in turn
+// (they hold 2 x 18 / 16 vectors and more), the last one to column `steps`
+ArnoldiStep tiled_step(const MGWork& w, int l, int j, int steps, long long len, bool x_is_zero, const GmresDev& st) {
+  auto buf = [&](int k) { return vptr(w.scratch[l], w.es, (long long)(k & 1) * len); };
+  ArnoldiStep e{};
+  e.j = j;
+  e.store = j > 0 || x_is_zero;
+  e.src = j > 0 ? (const void*)buf(j) : x_is_zero ? w.b[l] : w.V[l];
+  e.wout = j + 1 < steps ? buf(j + 1) : vptr(w.V[l], w.es, (long long)steps * len);
+  e.z = vptr(w.Z[l], w.es, (long long)j * len);
+  e.V = w.V[l];
+  e.ld = len;
+  e.st = st;
+  return e;
+}
+
 void smooth_fused(als_ctx* c, MGWork& w, int l, bool x_is_zero, void* t) {
   const LevelDev& Lv = c->lev[l];
   const int prec = w.prec;
   const long long len = Lv.g.N * c->dim;
   const cudaStream_t s = c->stream;
   const int steps = std::max(1, c->opt.sweeps);
-  const GmresDev st = gmres_dev(Lv, w.small[l], steps, w.partial, x_is_zero);
+  const bool tiled = tiled_steps(c, w, l);
+  const GmresDev st = gmres_dev(Lv, w.small[l], steps, w.partial, x_is_zero, tiled);
   void* V0 = w.V[l];
-  if (x_is_zero) {
+  if (x_is_zero && tiled) {
+    // V0 = b, by the first step
+  } else if (x_is_zero) {
     gm_start(prec, len, w.b[l], V0, st, s);                              // V0 = b
   } else {
     ApplyEpi e{w.b[l], -1.0, 0, nullptr, 0, 1, st};
@@ -311,6 +335,13 @@ void smooth_fused(als_ctx* c, MGWork& w, int l, bool x_is_zero, void* t) {
     void* Zj = vptr(w.Z[l], w.es, (long long)j * len);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (l == c->L - 1) prof_events(c, t_prof_counter, e0, e1);
+    if (tiled) {
+      if (e0) cudaEventRecordWithFlags(e0, s, cudaEventRecordExternal);
+      arnoldi_step(Lv, c->gamma, tiled_step(w, l, j, steps, len, x_is_zero, st), s);
+      if (e1) cudaEventRecordWithFlags(e1, s, cudaEventRecordExternal);
+      if (j == steps - 1) gm_orth(prec, len, j, w.V[l], len, st, s);
+      continue;
+    }
     ApplyEpi e{nullptr, 1.0, j + 1, w.V[l], len, 0, st};
     if (fuse_patch_gather(c)) {
       // patch products only; the cell kernel sums them per node into Z_j = D^-1 V_j
@@ -1010,6 +1041,7 @@ static als_status create_impl(als_ctx* c, const als_mesh* mesh, const als_coeff*
   }
   const LevelDev& F = c->lev[c->L - 1];
   ALS_TRY(dalloc(c, &c->schur, (size_t)F.g.ncells * c->npr * c->npr));
+  if (c->k == 2 && c->dim == 2) arnoldi_prepare();
   ALS_TRY(alloc_work(c, c->w64, PREC_F64));
   ALS_TRY(alloc_work(c, c->w32, PREC_F32));
   return run_setup(c, coeff);
@@ -1749,34 +1781,42 @@ void merged_smooth(MergedCycle& M, int l, bool x_is_zero, bool residual, cudaStr
   const std::vector<als_ctx*> S = at_level(M, l);
   if (S.empty()) return;
   const int steps = std::max(1, S[0]->opt.sweeps);
-  std::vector<BGmres> g;
+  std::vector<BGmres> g, gs;             // all instances; those whose steps are separate kernels
   std::vector<BApply> ap;
   for (als_ctx* c : S) {
     MGWork& w = c->w32;
     const long long len = c->lev[l].g.N * c->dim;
+    const bool tiled = tiled_steps(c, w, l);
     BGmres it{};
     it.n = len;
     it.b = w.b[l];
     it.Z = w.Z[l];
     it.V = w.V[l];
     it.ld = len;
-    it.st = gmres_dev(c->lev[l], w.small[l], steps, w.partial, x_is_zero);
+    it.st = gmres_dev(c->lev[l], w.small[l], steps, w.partial, x_is_zero, tiled);
     it.x = w.x[l];
     it.x_zero = x_is_zero ? 1 : 0;
     it.t = residual ? w.t[l] : nullptr;
     g.push_back(it);
+    if (!tiled) gs.push_back(it);
     ap.push_back(BApply{&c->lev[l], c->gamma, w.x[l], w.V[l],
                         ApplyEpi{w.b[l], -1.0, 0, nullptr, 0, 1, it.st}});
   }
-  if (x_is_zero) batch_gm_start(g, s);     // V0 = b
-  else batch_apply_epi(ap, s);             // V0 = b - A x
+  if (!x_is_zero) batch_apply_epi(ap, s);          // V0 = b - A x
+  else if (!gs.empty()) batch_gm_start(gs, s);     // V0 = b (tiled: by the first step)
   for (int j = 0; j < steps; ++j) {
+    std::vector<BArnoldi> tile;
     std::vector<BPatch> prod, gath;
     std::vector<BApply> az;
     for (size_t i = 0; i < S.size(); ++i) {
       als_ctx* c = S[i];
       MGWork& w = c->w32;
       const long long len = c->lev[l].g.N * c->dim;
+      g[i].j = j;
+      if (tiled_steps(c, w, l)) {
+        tile.push_back(BArnoldi{&c->lev[l], c->gamma, tiled_step(w, l, j, steps, len, x_is_zero, g[i].st)});
+        continue;
+      }
       void* Vj = vptr(w.V[l], w.es, (long long)j * len);
       void* Vn = vptr(w.V[l], w.es, (long long)(j + 1) * len);
       void* Zj = vptr(w.Z[l], w.es, (long long)j * len);
@@ -1788,12 +1828,17 @@ void merged_smooth(MergedCycle& M, int l, bool x_is_zero, bool residual, cudaStr
         gath.push_back(BPatch{&c->lev[l], nullptr, w.scratch[l], Zj});
       }
       az.push_back(BApply{&c->lev[l], c->gamma, Zj, Vn, e});
-      g[i].j = j;
     }
-    batch_star_products(M.var_prod[l], prod, s);    // scratch rows = A_v^-1 V_j|_v
-    if (!gath.empty()) batch_patch_gather(gath, s);  // Z_j = D^-1 v_j (unfused instances)
-    batch_apply_epi(az, s);                          // A Z_j, H[0..j][j]
-    batch_gm_orth(g, s);                             // V_{j+1}, Givens step j
+    for (BGmres& it : gs) it.j = j;
+    if (!tile.empty()) batch_arnoldi_step(tile, s);  // V_j, Z_j, A Z_j, H[0..j][j]
+    if (!prod.empty()) {
+      batch_star_products(M.var_prod[l], prod, s);     // scratch rows = A_v^-1 V_j|_v
+      if (!gath.empty()) batch_patch_gather(gath, s);  // Z_j = D^-1 v_j (unfused instances)
+      batch_apply_epi(az, s);                          // A Z_j, H[0..j][j]
+    }
+    // V_{j+1}, Givens step j; a tiled step takes the one before into itself, all but the last
+    if (j == steps - 1) batch_gm_orth(g, s);
+    else if (!gs.empty()) batch_gm_orth(gs, s);
   }
   batch_gm_update(g, s);
 }

@@ -451,49 +451,21 @@ __device__ __forceinline__ void cell2_from_stars(const Geom& g, const PatchIn<T>
   }
 }
 
-// warp: index of the warp among those of this apply
-template <typename T, bool TENSOR, int MODE, bool STAGED, bool ZP>
-__device__ __forceinline__ void apply_cells2_body(unsigned warp, const Geom& g, const Colour& col,
-                                                  const CellConst<T>& cc, const T* __restrict__ x, T* __restrict__ y,
-                                                  const T* __restrict__ coef, const T* __restrict__ p_in,
-                                                  T* __restrict__ p_out, long long vstride, T* __restrict__ ebuf,
-                                                  const T* __restrict__ winv, const PatchIn<T>& pin) {
-  constexpr bool RAW = (MODE & OP_RAW) != 0;
+// The cell's contribution from its nodal values u (component c; the other lane of the pair holds
+// the other one); store(ay, o) takes the outputs at the nodes (0..2, ay).  Every lane of the warp calls.
+template <typename T, bool TENSOR, int MODE, typename Store>
+__device__ __forceinline__ void cell2_contribution(const CellConst<T>& cc, bool act, int c, int cell, const T (&u)[9],
+                                                   const T* mu, const T* __restrict__ coef,
+                                                   const T* __restrict__ p_in, T* __restrict__ p_out,
+                                                   const T* __restrict__ winv, Store store) {
   constexpr bool VISC = (MODE & OP_VISC) != 0;
   constexpr bool NEED_U = (MODE & (OP_VISC | OP_AL | OP_B)) != 0;
   constexpr bool NEED_FLUX = (MODE & (OP_VISC | OP_AL | OP_BT)) != 0;
-  x += blockIdx.y * vstride;
-  y += blockIdx.y * vstride;
-  const int lane = threadIdx.x & 31, c = lane >> 4;
-  int cx = 0, cy = 0, cz = 0;
-  const bool act = colour_cell(col, (long long)warp * 16 + (lane & 15), cx, cy, cz);
-  const int cell = cx + g.n[0] * cy;
   const DerivTab<T> dx = deriv_tab<T>(cc.s[0]), dy = deriv_tab<T>(cc.s[1]);
-  pdl_wait();
-  // the viscosities (constant) are in flight beside the nodal values
-  T mu[VISC && !TENSOR ? 9 : 1];
-  if constexpr (VISC && !TENSOR) {
-#pragma unroll
-    for (int q = 0; q < 9; ++q) mu[q] = act ? coef[(long long)cell * 9 + q] : T(0);
-  }
   T gd[9], gs[9], od[9];   // d u_c / d x_c; d u_c / d x_(1-c), then the shear sum; the other component's diagonal
 #pragma unroll
   for (int q = 0; q < 9; ++q) gd[q] = gs[q] = od[q] = T(0);
   if constexpr (NEED_U) {
-    T u[9];
-#pragma unroll
-    for (int a = 0; a < 9; ++a) u[a] = T(0);
-    if (act) {
-      if constexpr (ZP) {
-        cell2_from_stars<T>(g, pin, c, cx, cy, u);
-      } else {
-#pragma unroll
-        for (int a = 0; a < 9; ++a) {
-          const int ni = 2 * cx + a % 3, nj = 2 * cy + a / 3;
-          if (RAW || !on_boundary(g, ni, nj, 0)) u[a] = x[c * g.N + (ni + g.nn[0] * nj)];
-        }
-      }
-    }
     T bu[3][3], du[3][3];   // [qx][ay]
 #pragma unroll
     for (int ay = 0; ay < 3; ++ay) {
@@ -604,20 +576,64 @@ __device__ __forceinline__ void apply_cells2_body(unsigned warp, const Geom& g, 
         T o[3];
         line_derivs_t<T, false>(dx, rx[ay][0], rx[ay][1], rx[ay][2], o);
         line_values_t<T, true>(ry[ay][0], ry[ay][1], ry[ay][2], o);
-        if constexpr (STAGED) {
-          T* e = ebuf + (long long)stage_row(g, c, ay, 0, cy, 0) * (3 * g.n[0]) + 3 * cx;
+        store(ay, o);
+      }
+    }
+  }
+}
+
+// warp: index of the warp among those of this apply
+template <typename T, bool TENSOR, int MODE, bool STAGED, bool ZP>
+__device__ __forceinline__ void apply_cells2_body(unsigned warp, const Geom& g, const Colour& col,
+                                                  const CellConst<T>& cc, const T* __restrict__ x, T* __restrict__ y,
+                                                  const T* __restrict__ coef, const T* __restrict__ p_in,
+                                                  T* __restrict__ p_out, long long vstride, T* __restrict__ ebuf,
+                                                  const T* __restrict__ winv, const PatchIn<T>& pin) {
+  constexpr bool RAW = (MODE & OP_RAW) != 0;
+  constexpr bool VISC = (MODE & OP_VISC) != 0;
+  constexpr bool NEED_U = (MODE & (OP_VISC | OP_AL | OP_B)) != 0;
+  x += blockIdx.y * vstride;
+  y += blockIdx.y * vstride;
+  const int lane = threadIdx.x & 31, c = lane >> 4;
+  int cx = 0, cy = 0, cz = 0;
+  const bool act = colour_cell(col, (long long)warp * 16 + (lane & 15), cx, cy, cz);
+  const int cell = cx + g.n[0] * cy;
+  pdl_wait();
+  // the viscosities (constant) are in flight beside the nodal values
+  T mu[VISC && !TENSOR ? 9 : 1];
+  if constexpr (VISC && !TENSOR) {
 #pragma unroll
-          for (int ax = 0; ax < 3; ++ax) e[ax] = o[ax];
-        } else {
+    for (int q = 0; q < 9; ++q) mu[q] = act ? coef[(long long)cell * 9 + q] : T(0);
+  }
+  T u[9];
 #pragma unroll
-          for (int ax = 0; ax < 3; ++ax) {
-            const int ni = 2 * cx + ax, nj = 2 * cy + ay;
-            if (RAW || !on_boundary(g, ni, nj, 0)) y[c * g.N + (ni + g.nn[0] * nj)] += o[ax];
-          }
+  for (int a = 0; a < 9; ++a) u[a] = T(0);
+  if constexpr (NEED_U) {
+    if (act) {
+      if constexpr (ZP) {
+        cell2_from_stars<T>(g, pin, c, cx, cy, u);
+      } else {
+#pragma unroll
+        for (int a = 0; a < 9; ++a) {
+          const int ni = 2 * cx + a % 3, nj = 2 * cy + a / 3;
+          if (RAW || !on_boundary(g, ni, nj, 0)) u[a] = x[c * g.N + (ni + g.nn[0] * nj)];
         }
       }
     }
   }
+  cell2_contribution<T, TENSOR, MODE>(cc, act, c, cell, u, mu, coef, p_in, p_out, winv, [&](int ay, const T(&o)[3]) {
+    if constexpr (STAGED) {
+      T* e = ebuf + (long long)stage_row(g, c, ay, 0, cy, 0) * (3 * g.n[0]) + 3 * cx;
+#pragma unroll
+      for (int ax = 0; ax < 3; ++ax) e[ax] = o[ax];
+    } else {
+#pragma unroll
+      for (int ax = 0; ax < 3; ++ax) {
+        const int ni = 2 * cx + ax, nj = 2 * cy + ay;
+        if (RAW || !on_boundary(g, ni, nj, 0)) y[c * g.N + (ni + g.nn[0] * nj)] += o[ax];
+      }
+    }
+  });
   pdl_trigger();
 }
 constexpr int C2_THREADS = 64, C2_CELLS = C2_THREADS / 2;

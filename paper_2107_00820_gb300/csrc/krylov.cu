@@ -6,6 +6,7 @@
 // single-thread kernels so that no step of a solve needs the host.
 #include <math.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include "batch.cuh"
@@ -256,6 +257,7 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
   T a[GM_PER];
   T vc[GM_PER][KMAXB];
   T rhni = T(0);
+  if (sd.late) pdl_wait();   // column j, its norm and rhn come from the predecessor too
   // columns 0..j, rhn and the norm partials come from earlier kernels of the chain (complete
   // before this launch began): read through L2 before the wait; column j+1 and the dots come
   // from the predecessor
@@ -289,7 +291,7 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
     const unsigned i = base + q * RED_THREADS;
     a[q] = i < n ? w[i] : T(0);
   }
-  sum_rows<T>(dot_rows<T>(sd), sd.nbd, j + 1, acc);
+  sum_rows<T>(dot_rows<T>(sd, j), sd.nbd, j + 1, acc);
   {
     const T v = block_total<T>(acc, j + 1, sh);
     if ((int)threadIdx.x <= j) {
@@ -395,10 +397,12 @@ __global__ void __launch_bounds__(RED_THREADS) k_gm_update(unsigned n, int k, co
   gm_update_body<T>(blockIdx.x, n, k, Z, V, ld, sd, x, x_zero, t);
 }
 
-GmresDev gmres_dev(const LevelDev& L, void* state, int steps, double* partial, bool x_is_zero) {
+GmresDev gmres_dev(const LevelDev& L, void* state, int steps, double* partial, bool x_is_zero, bool tiled) {
   const long long n = L.g.N * L.g.dim;
-  const int nbd = apply_epi_blocks(L), nbv = gm_blocks(n);
-  return GmresDev{state, steps, partial + 1, nbd, x_is_zero ? nbv : nbd, nbd * KMAXB, nbd > nbv ? nbd : nbv};
+  const int nbe = apply_epi_blocks(L), nbv = gm_blocks(n), nbt = tiled ? arnoldi_tiles(L) : 0;
+  const int nbd = tiled ? nbt : nbe, nbn = tiled ? nbt : nbv;
+  return GmresDev{state, steps, partial + 1, nbd, !x_is_zero ? nbe : nbn, nbn, 2 * nbd * KMAXB,
+                  std::max(std::max(nbe, nbv), nbt), tiled ? 1 : 0};
 }
 
 void gm_start(int prec, long long n, const void* b, void* V0, const GmresDev& st, cudaStream_t s) {
@@ -475,10 +479,11 @@ int batch_gm_start(const std::vector<BGmres>& items, cudaStream_t s) { return ba
 int batch_gm_orth(const std::vector<BGmres>& items, cudaStream_t s) { return batch_gm(k_gm_orth_b, items, 1, s); }
 int batch_gm_update(const std::vector<BGmres>& items, cudaStream_t s) { return batch_gm(k_gm_update_b, items, 0, s); }
 
-// workspace of the smoother's fused reductions: KMAXB + 2 rows of one value per block (the
-// gathers have at most 0.4 n / 256 + 1 blocks: four nodes a thread, rows of at least five nodes)
-size_t gmres_partial_doubles(long long n) {
-  return (size_t)((n + 511) / 512 + 1) * (KMAXB + 2) + 1;
+// workspace of a level's fused reductions: two areas of KMAXB rows and two rows, one value per block
+size_t gmres_partial_doubles(const LevelDev& L) {
+  const int nb = std::max(std::max(apply_epi_blocks(L), gm_blocks(L.g.N * L.g.dim)),
+                          L.k == 2 && L.g.dim == 2 ? arnoldi_tiles(L) : 0);
+  return (size_t)nb * (2 * KMAXB + 2) + 1;
 }
 
 // ---------------------------------------------------------------------------

@@ -91,6 +91,21 @@ struct ApplyEpi {
 void op_apply_epi(const LevelDev& L, int prec, double gamma, const void* x, void* y, const ApplyEpi& e,
                   cudaStream_t s, cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr);
 int apply_epi_blocks(const LevelDev& L);   // blocks of its reduction
+// A whole Arnoldi step of a tiled level in one launch (arnoldi2.cuh): V_j from src (j = 0: V_0 itself,
+// or with store what it is a copy of; j > 0: w of the step before), z = D^-1 V_j, wout = A z
+struct ArnoldiStep {
+  int j, store;
+  const void* src;
+  void* wout;
+  void* z;
+  void* V;
+  long long ld;
+  GmresDev st;
+};
+bool arnoldi_tiled(const LevelDev& L, int prec);
+int arnoldi_tiles(const LevelDev& L);   // blocks of its reductions
+void arnoldi_prepare();                 // before any capture
+void arnoldi_step(const LevelDev& L, double gamma, const ArnoldiStep& e, cudaStream_t s);
 void op_load_vector(const LevelDev& L, const double* f_qp, double* F, cudaStream_t s);
 void op_apply_multi(const LevelDev& L, double gamma, const double* X, double* Y, int nvec,
                     long long stride, cudaStream_t s);
@@ -219,9 +234,9 @@ void vec_multiaxpy_norm(int prec, long long n, int k, const void* V, long long l
 // GMRES(s) smoother with an unnormalised stored basis (GmresDev): V0 = b and start;
 // orthogonalise column j+1 and take the Givens step j; x (+)= Z y and, if t, the
 // GMRES residual t = r0 - A Z y from the Arnoldi relation.  s <= KMAXB.
-size_t gmres_partial_doubles(long long n);   // workspace of op_apply_epi and gm_* for n entries
+size_t gmres_partial_doubles(const LevelDev& L);   // workspace of op_apply_epi, arnoldi_step and gm_*
 // a smoothing's state on level L: state array, partials (workspace above), from x = 0 or not
-GmresDev gmres_dev(const LevelDev& L, void* state, int steps, double* partial, bool x_is_zero);
+GmresDev gmres_dev(const LevelDev& L, void* state, int steps, double* partial, bool x_is_zero, bool tiled);
 void gm_start(int prec, long long n, const void* b, void* V0, const GmresDev& st, cudaStream_t s);
 void gm_orth(int prec, long long n, int j, const void* V, long long ld, const GmresDev& st, cudaStream_t s);
 void gm_update(int prec, long long n, int k, const void* Z, const void* V, long long ld, const GmresDev& st,
@@ -274,6 +289,12 @@ struct BGmres {            // gm_start (b, V), gm_orth (V, j), gm_update (Z, V, 
   int x_zero;
   void* t;
 };
+struct BArnoldi {
+  const LevelDev* L;
+  double gamma;
+  ArnoldiStep e;
+};
+int batch_arnoldi_step(const std::vector<BArnoldi>& items, cudaStream_t s);
 int batch_gm_start(const std::vector<BGmres>& items, cudaStream_t s);
 int batch_gm_orth(const std::vector<BGmres>& items, cudaStream_t s);
 int batch_gm_update(const std::vector<BGmres>& items, cudaStream_t s);

@@ -15,6 +15,8 @@
 #include "level.h"
 #include "reduce.cuh"
 #include "pdl.cuh"
+#include "star_blocks.cuh"
+#include "tma.cuh"
 
 #include <type_traits>
 
@@ -581,6 +583,8 @@ int batch_apply_al(const std::vector<BApply>& items, cudaStream_t s) {
   count_launch(n);
   return n;
 }
+
+#include "arnoldi2.cuh"
 
 // Several independent FP64 applies of A_gamma (used to form the coarse matrix
 // column by column from unit vectors): vector v at X + v*stride.

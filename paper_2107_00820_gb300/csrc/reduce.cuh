@@ -177,18 +177,21 @@ struct GmresLayout {
 // every block of the kernel that needs the sums adds them for itself, in one fixed order.
 // (A last-block finish, with its fence, ticket, second fence, reload and one-thread
 // bookkeeping, cost 1 to 2 us at the end of each of the two reductions of a step: a third of a
-// small level's time.)  The dots of a gather: nbd blocks at rows.  |column j|^2: at
-// rows + noff + (j & 1) nstride, written while the other area is still being read; nb0 blocks
-// for column 0 (gather or copy), ceil(n / 1024) for the others.
+// small level's time.)  The dots of step j: nbd blocks in one of two areas from rows, by the parity of
+// j.  |column j|^2: at rows + noff + (j & 1) nstride.  (A kernel that reads one area may write the
+// other.)  nb0 blocks for column 0 (gather or copy), nbn for columns 1 .. s - 1 and ceil(n / 1024) for s.
 struct GmresDev {
   void* base;
   int s;
   void* rows;
-  int nbd, nb0, noff, nstride;
+  int nbd, nb0, nbn, noff, nstride;
+  int late;   // the kernel before the last Gram-Schmidt step writes more than its column (see arnoldi2.cuh)
 };
 
 template <typename T>
-__host__ __device__ __forceinline__ T* dot_rows(const GmresDev& d) { return static_cast<T*>(d.rows); }
+__host__ __device__ __forceinline__ T* dot_rows(const GmresDev& d, int j) {
+  return static_cast<T*>(d.rows) + (j & 1) * (d.nbd * KMAXB);
+}
 template <typename T>
 __host__ __device__ __forceinline__ T* norm_rows(const GmresDev& d, int j) {
   return static_cast<T*>(d.rows) + d.noff + (j & 1) * d.nstride;
@@ -198,7 +201,7 @@ __host__ __device__ __forceinline__ int gm_blocks(long long n) {
   return (int)((n + RED_THREADS * GM_PER - 1) / (RED_THREADS * GM_PER));
 }
 __host__ __device__ __forceinline__ int norm_count(const GmresDev& d, int j, long long n) {
-  return j == 0 ? d.nb0 : gm_blocks(n);
+  return j == 0 ? d.nb0 : j < d.s ? d.nbn : gm_blocks(n);
 }
 
 // the block partials of a gather: |y|^2 of column 0 (start) or the k dots (every thread calls)
@@ -208,7 +211,7 @@ __device__ __forceinline__ void store_partials(const GmresDev& d, int start, int
   __shared__ T sh[RED_THREADS / 32][KMAXB];
   const int kk = start ? 1 : k;
   const T v = block_total<T>(acc, kk, sh);
-  if ((int)threadIdx.x < kk) (start ? norm_rows<T>(d, 0) : dot_rows<T>(d))[threadIdx.x * nb + bx] = v;
+  if ((int)threadIdx.x < kk) (start ? norm_rows<T>(d, 0) : dot_rows<T>(d, k - 1))[threadIdx.x * nb + bx] = v;
 }
 
 template <typename T>
