@@ -296,6 +296,11 @@ bool tiled_steps(const als_ctx* c, const MGWork& w, int l) {
   return fuse_patch_gather(c) && arnoldi_tiled(c->lev[l], w.prec);
 }
 
+// levels whose robust transfers to and from the next coarser level are one launch each
+bool tiled_transfers(const als_ctx* c, const MGWork& w, int l) {
+  return c->opt.transfer == ALS_TRANSFER_ROBUST && fuse_patch_gather(c) && transfer_tiled(c->lev[l], w.prec);
+}
+
 // step j of a tiled smoothing: w goes through two buffers in the star products' scratch in turn
 // (they hold 2 x 18 / 16 vectors and more), the last one to column `steps`
 ArnoldiStep tiled_step(const MGWork& w, int l, int j, int steps, long long len, bool x_is_zero, const GmresDev& st) {
@@ -321,8 +326,9 @@ void smooth_fused(als_ctx* c, MGWork& w, int l, bool x_is_zero, void* t) {
   const bool tiled = tiled_steps(c, w, l);
   const GmresDev st = gmres_dev(Lv, w.small[l], steps, w.partial, x_is_zero, tiled);
   void* V0 = w.V[l];
-  if (x_is_zero && tiled) {
-    // V0 = b, by the first step
+  if (tiled) {
+    // V0 = b by the first step, or V0 = b - A x
+    if (!x_is_zero) tiled_residual(Lv, c->gamma, w.x[l], w.b[l], V0, st, s);
   } else if (x_is_zero) {
     gm_start(prec, len, w.b[l], V0, st, s);                              // V0 = b
   } else {
@@ -411,7 +417,9 @@ void restrict_level(als_ctx* c, MGWork& w, int l, const void* rf, void* rc) {
   const LevelDev& F = c->lev[l];
   const LevelDev& C = c->lev[l - 1];
   const cudaStream_t s = c->stream;
-  if (c->opt.transfer == ALS_TRANSFER_ROBUST) {
+  if (tiled_transfers(c, w, l)) {
+    tiled_restrict(C, F, c->gamma, rf, rc, s);
+  } else if (c->opt.transfer == ALS_TRANSFER_ROBUST) {
     // t2 = sum_K E_K A_K^-1 E_K^T rf ; t3 = G t2 ; rc = P_H^T (rf - t3)
     patch_interior_solve(F, w.prec, rf, w.t2[l], 0, s);
     op_apply(F, w.prec, OP_AL, c->gamma, w.t2[l], w.t3[l], nullptr, nullptr, s);
@@ -426,6 +434,10 @@ void prolong_level(als_ctx* c, MGWork& w, int l, const void* xc, void* t, void* 
   const LevelDev& F = c->lev[l];
   const LevelDev& C = c->lev[l - 1];
   const cudaStream_t s = c->stream;
+  if (tiled_transfers(c, w, l)) {
+    tiled_prolong(C, F, c->gamma, xc, x ? x : t, x ? 1 : 0, s);
+    return;
+  }
   prolong_std(C, F, w.prec, xc, t, s, x);                                     // t = P_H xc, x += t
   if (c->opt.transfer == ALS_TRANSFER_ROBUST) {
     op_apply(F, w.prec, OP_AL, c->gamma, t, w.t3[l], nullptr, nullptr, s);    // t3 = G P_H xc
@@ -1782,7 +1794,7 @@ void merged_smooth(MergedCycle& M, int l, bool x_is_zero, bool residual, cudaStr
   if (S.empty()) return;
   const int steps = std::max(1, S[0]->opt.sweeps);
   std::vector<BGmres> g, gs;             // all instances; those whose steps are separate kernels
-  std::vector<BApply> ap;
+  std::vector<BApply> ap, apt;
   for (als_ctx* c : S) {
     MGWork& w = c->w32;
     const long long len = c->lev[l].g.N * c->dim;
@@ -1799,11 +1811,13 @@ void merged_smooth(MergedCycle& M, int l, bool x_is_zero, bool residual, cudaStr
     it.t = residual ? w.t[l] : nullptr;
     g.push_back(it);
     if (!tiled) gs.push_back(it);
-    ap.push_back(BApply{&c->lev[l], c->gamma, w.x[l], w.V[l],
-                        ApplyEpi{w.b[l], -1.0, 0, nullptr, 0, 1, it.st}});
+    (tiled ? apt : ap).push_back(BApply{&c->lev[l], c->gamma, w.x[l], w.V[l],
+                                        ApplyEpi{w.b[l], -1.0, 0, nullptr, 0, 1, it.st}});
   }
-  if (!x_is_zero) batch_apply_epi(ap, s);          // V0 = b - A x
-  else if (!gs.empty()) batch_gm_start(gs, s);     // V0 = b (tiled: by the first step)
+  if (!x_is_zero) {                                // V0 = b - A x
+    if (!apt.empty()) batch_tiled_residual(apt, s);
+    if (!ap.empty()) batch_apply_epi(ap, s);
+  } else if (!gs.empty()) batch_gm_start(gs, s);     // V0 = b (tiled: by the first step)
   for (int j = 0; j < steps; ++j) {
     std::vector<BArnoldi> tile;
     std::vector<BPatch> prod, gath;
@@ -1848,13 +1862,20 @@ void merged_restrict(MergedCycle& M, int l, cudaStream_t s) {
   std::vector<BPatch> isv;
   std::vector<BApply> ap;
   std::vector<BTransfer> tr;
+  std::vector<BTiledTransfer> tile;
   const bool robust = S[0]->opt.transfer == ALS_TRANSFER_ROBUST;
   for (als_ctx* c : S) {
     MGWork& w = c->w32;
+    if (tiled_transfers(c, w, l)) {
+      tile.push_back(BTiledTransfer{&c->lev[l - 1], &c->lev[l], c->gamma, w.t[l], w.b[l - 1]});
+      continue;
+    }
     isv.push_back(BPatch{&c->lev[l], w.t[l], w.t2[l], nullptr});
     ap.push_back(BApply{&c->lev[l], c->gamma, w.t2[l], w.t3[l], ApplyEpi{}});
     tr.push_back(BTransfer{&c->lev[l - 1], &c->lev[l], w.t[l], w.b[l - 1], robust ? w.t3[l] : nullptr});
   }
+  if (!tile.empty()) batch_tiled_restrict(tile, s);
+  if (tr.empty()) return;
   if (robust) {
     batch_interior_solve(M.var_int[l], isv, 0, s);   // t2 = sum_K E_K A_K^-1 E_K^T t
     batch_apply_al(ap, s);                           // t3 = G t2
@@ -1867,13 +1888,20 @@ void merged_prolong(MergedCycle& M, int l, cudaStream_t s) {
   std::vector<BPatch> isv;
   std::vector<BApply> ap;
   std::vector<BTransfer> tr;
+  std::vector<BTiledTransfer> tile;
   const bool robust = S[0]->opt.transfer == ALS_TRANSFER_ROBUST;
   for (als_ctx* c : S) {
     MGWork& w = c->w32;
+    if (tiled_transfers(c, w, l)) {
+      tile.push_back(BTiledTransfer{&c->lev[l - 1], &c->lev[l], c->gamma, w.x[l - 1], w.x[l]});
+      continue;
+    }
     tr.push_back(BTransfer{&c->lev[l - 1], &c->lev[l], w.x[l - 1], w.t[l], w.x[l]});
     ap.push_back(BApply{&c->lev[l], c->gamma, w.t[l], w.t3[l], ApplyEpi{}});
     isv.push_back(BPatch{&c->lev[l], w.t3[l], w.x[l], nullptr});
   }
+  if (!tile.empty()) batch_tiled_prolong(tile, s);
+  if (tr.empty()) return;
   batch_prolong(tr, s);                              // t = P_H x_{l-1}, x += t
   if (robust) {
     batch_apply_al(ap, s);                           // t3 = G t

@@ -401,7 +401,7 @@ GmresDev gmres_dev(const LevelDev& L, void* state, int steps, double* partial, b
   const long long n = L.g.N * L.g.dim;
   const int nbe = apply_epi_blocks(L), nbv = gm_blocks(n), nbt = tiled ? arnoldi_tiles(L) : 0;
   const int nbd = tiled ? nbt : nbe, nbn = tiled ? nbt : nbv;
-  return GmresDev{state, steps, partial + 1, nbd, !x_is_zero ? nbe : nbn, nbn, 2 * nbd * KMAXB,
+  return GmresDev{state, steps, partial + 1, nbd, tiled ? nbt : x_is_zero ? nbv : nbe, nbn, 2 * nbd * KMAXB,
                   std::max(std::max(nbe, nbv), nbt), tiled ? 1 : 0};
 }
 

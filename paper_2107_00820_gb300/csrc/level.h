@@ -106,6 +106,14 @@ bool arnoldi_tiled(const LevelDev& L, int prec);
 int arnoldi_tiles(const LevelDev& L);   // blocks of its reductions
 void arnoldi_prepare();                 // before any capture
 void arnoldi_step(const LevelDev& L, double gamma, const ArnoldiStep& e, cudaStream_t s);
+// V_0 = b - A x of a tiled level and the partials that start st (tiles2.cuh)
+void tiled_residual(const LevelDev& L, double gamma, const void* x, const void* b, void* y, const GmresDev& st,
+                    cudaStream_t s);
+// the robust transfers, one launch each: rc = P~^T rf;  x = P~ xc, or += with add
+bool transfer_tiled(const LevelDev& fine, int prec);
+void tiled_restrict(const LevelDev& coarse, const LevelDev& fine, double gamma, const void* rf, void* rc, cudaStream_t s);
+void tiled_prolong(const LevelDev& coarse, const LevelDev& fine, double gamma, const void* xc, void* x, int add,
+                   cudaStream_t s);
 void op_load_vector(const LevelDev& L, const double* f_qp, double* F, cudaStream_t s);
 void op_apply_multi(const LevelDev& L, double gamma, const double* X, double* Y, int nvec,
                     long long stride, cudaStream_t s);
@@ -294,6 +302,16 @@ struct BArnoldi {
   double gamma;
   ArnoldiStep e;
 };
+struct BTiledTransfer {
+  const LevelDev* coarse;
+  const LevelDev* fine;
+  double gamma;
+  const void* in;
+  void* out;
+};
+int batch_tiled_residual(const std::vector<BApply>& items, cudaStream_t s);   // x, y, e.b, e.st of the items
+int batch_tiled_restrict(const std::vector<BTiledTransfer>& items, cudaStream_t s);
+int batch_tiled_prolong(const std::vector<BTiledTransfer>& items, cudaStream_t s);   // out +=
 int batch_arnoldi_step(const std::vector<BArnoldi>& items, cudaStream_t s);
 int batch_gm_start(const std::vector<BGmres>& items, cudaStream_t s);
 int batch_gm_orth(const std::vector<BGmres>& items, cudaStream_t s);

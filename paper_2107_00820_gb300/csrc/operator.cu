@@ -585,6 +585,7 @@ int batch_apply_al(const std::vector<BApply>& items, cudaStream_t s) {
 }
 
 #include "arnoldi2.cuh"
+#include "tiles2.cuh"
 
 // Several independent FP64 applies of A_gamma (used to form the coarse matrix
 // column by column from unit vectors): vector v at X + v*stride.
