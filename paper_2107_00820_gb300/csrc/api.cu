@@ -422,8 +422,13 @@ void restrict_level(als_ctx* c, MGWork& w, int l, const void* rf, void* rc) {
   } else if (c->opt.transfer == ALS_TRANSFER_ROBUST) {
     // t2 = sum_K E_K A_K^-1 E_K^T rf ; t3 = G t2 ; rc = P_H^T (rf - t3)
     patch_interior_solve(F, w.prec, rf, w.t2[l], 0, s);
-    op_apply(F, w.prec, OP_AL, c->gamma, w.t2[l], w.t3[l], nullptr, nullptr, s);
-    restrict_std(C, F, w.prec, rf, rc, s, w.t3[l]);                        // P_H^T (rf - t3)
+    if (c->k == 2) {
+      op_residual(F, w.prec, OP_AL, c->gamma, w.t2[l], rf, w.t3[l], s);    // t3 = rf - G t2
+      restrict_std(C, F, w.prec, w.t3[l], rc, s);
+    } else {
+      op_apply(F, w.prec, OP_AL, c->gamma, w.t2[l], w.t3[l], nullptr, nullptr, s);
+      restrict_std(C, F, w.prec, rf, rc, s, w.t3[l]);                      // P_H^T (rf - t3)
+    }
   } else {
     restrict_std(C, F, w.prec, rf, rc, s);
   }
@@ -464,8 +469,12 @@ void cycle_level(als_ctx* c, MGWork& w, int l, bool fcycle, bool zero_guess) {
     // Arnoldi relation; at extreme contrast (gamma / mu_min ~ 1e8) the recurrence drifts
     // from b - A x by far more than the rounding of b - A x itself
     smooth_fused(c, w, l, zero_guess, nullptr);
-    op_apply(Lv, w.prec, OP_VISC | OP_AL, c->gamma, w.x[l], w.t[l], nullptr, nullptr, s);
-    vec_axpby(w.prec, len, 1.0, w.b[l], -1.0, w.t[l], s);                // t = b - A x
+    if (c->k == 2) {
+      op_residual(Lv, w.prec, OP_VISC | OP_AL, c->gamma, w.x[l], w.b[l], w.t[l], s);   // t = b - A x
+    } else {
+      op_apply(Lv, w.prec, OP_VISC | OP_AL, c->gamma, w.x[l], w.t[l], nullptr, nullptr, s);
+      vec_axpby(w.prec, len, 1.0, w.b[l], -1.0, w.t[l], s);
+    }
   } else {
     if (zero_guess) vec_zero(w.prec, len, w.x[l], s);
     smooth(c, w, l, zero_guess && c->opt.smoother == ALS_SMOOTH_GMRES);
@@ -1871,16 +1880,16 @@ void merged_restrict(MergedCycle& M, int l, cudaStream_t s) {
       continue;
     }
     isv.push_back(BPatch{&c->lev[l], w.t[l], w.t2[l], nullptr});
-    ap.push_back(BApply{&c->lev[l], c->gamma, w.t2[l], w.t3[l], ApplyEpi{}});
-    tr.push_back(BTransfer{&c->lev[l - 1], &c->lev[l], w.t[l], w.b[l - 1], robust ? w.t3[l] : nullptr});
+    ap.push_back(BApply{&c->lev[l], c->gamma, w.t2[l], w.t3[l], ApplyEpi{w.t[l]}});
+    tr.push_back(BTransfer{&c->lev[l - 1], &c->lev[l], robust ? w.t3[l] : w.t[l], w.b[l - 1], nullptr});
   }
   if (!tile.empty()) batch_tiled_restrict(tile, s);
   if (tr.empty()) return;
   if (robust) {
     batch_interior_solve(M.var_int[l], isv, 0, s);   // t2 = sum_K E_K A_K^-1 E_K^T t
-    batch_apply_al(ap, s);                           // t3 = G t2
+    batch_apply_al(ap, s);                           // t3 = t - G t2
   }
-  batch_restrict(tr, s);                             // b_{l-1} = P_H^T (t - t3)
+  batch_restrict(tr, s);                             // b_{l-1} = P_H^T t3
 }
 
 void merged_prolong(MergedCycle& M, int l, cudaStream_t s) {

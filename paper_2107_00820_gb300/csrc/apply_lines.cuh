@@ -83,18 +83,25 @@ __device__ __forceinline__ void patch_line(const Geom& g, const PatchIn<T>& pin,
   if (nk & 1) { vz[0] = nk >> 1; oz[0] = 2; vz[1] = vz[0] + 1; oz[1] = 0; okz[0] = okz[1] = true; }
   else { vz[0] = nk >> 1; oz[0] = 1; okz[0] = true; vz[1] = 0; oz[1] = 0; okz[1] = false; }
   const int ncol = 3 * g.nv[0];
+  T v[2][2][4];   // all loads first, predicated (see gather_chunk)
+#pragma unroll
+  for (int tz = 0; tz < 2; ++tz)
+#pragma unroll
+    for (int ty = 0; ty < 2; ++ty) {
+      const bool ok = oky[ty] && okz[tz];
+      const int row = ((c * 3 + oz[tz]) * 3 + oy[ty]) * (g.nv[1] * g.nv[2]) + vz[tz] * g.nv[1] + vy[ty];
+      const T* rp = pin.out + (long long)(ok ? row : 0) * ncol + 3 * cx + 1;   // nodes 2cx | 2cx+1 (two) | 2cx+2
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[tz][ty][k] = ok ? rp[k] : T(0);
+    }
   T acc[3] = {T(0), T(0), T(0)};
 #pragma unroll
   for (int tz = 0; tz < 2; ++tz)
 #pragma unroll
     for (int ty = 0; ty < 2; ++ty) {
-      if (!(oky[ty] && okz[tz])) continue;
-      const int row = ((c * 3 + oz[tz]) * 3 + oy[ty]) * (g.nv[1] * g.nv[2]) + vz[tz] * g.nv[1] + vy[ty];
-      const T* rp = pin.out + (long long)row * ncol + 3 * cx;
-      const T v1 = rp[1], v2 = rp[2], v3 = rp[3], v4 = rp[4];   // nodes 2cx | 2cx+1 (two) | 2cx+2
-      acc[0] += v1;
-      acc[1] += v2 + v3;
-      acc[2] += v4;
+      acc[0] += v[tz][ty][0];
+      acc[1] += v[tz][ty][1] + v[tz][ty][2];
+      acc[2] += v[tz][ty][3];
     }
 #pragma unroll
   for (int a = 0; a < 3; ++a) {

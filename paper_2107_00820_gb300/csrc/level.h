@@ -70,6 +70,9 @@ void count_launch(long long n);
 // ---- operator.cu
 void op_apply(const LevelDev& L, int prec, int mode, double gamma, const void* x, void* y,
               const void* p_in, void* p_out, cudaStream_t s);
+// order 2: y = b - A x in the launches of an apply, mode OP_VISC | OP_AL or OP_AL (L.ebuf set)
+void op_residual(const LevelDev& L, int prec, int mode, double gamma, const void* x, const void* b, void* y,
+                 cudaStream_t s);
 // A_gamma apply (viscous + AL) fused with the reduction that consumes y:
 //   y = b + sigma A x (b NULL: y = sigma A x);
 //   start = 0: block partials of the Arnoldi dots V_j . y, j < k (k <= KMAXB)
@@ -281,7 +284,7 @@ struct BTransfer {
   const LevelDev* fine;
   const void* in;
   void* out;
-  const void* aux;         // prolong: xadd (out added to it, may be NULL); restrict: sub (may be NULL)
+  const void* aux;         // prolong: xadd (out added to it, may be NULL)
 };
 int batch_prolong(const std::vector<BTransfer>& items, cudaStream_t s);     // prolong_std
 int batch_restrict(const std::vector<BTransfer>& items, cudaStream_t s);    // restrict_std

@@ -146,25 +146,33 @@ __device__ __forceinline__ void gather_chunk(const Geom& g, const T* __restrict_
   }
   const int ncol = 3 * g.n[0];
   const int p0 = 6 * rc.j - 1;
+  // all loads first, predicated: a branch per tap pair would make each wait for the one before
+  constexpr int TZ = DIM == 3 ? 2 : 1;
+  T v[TZ][2][6];
+#pragma unroll
+  for (int tz = 0; tz < TZ; ++tz)
+#pragma unroll
+    for (int ty = 0; ty < 2; ++ty) {
+      const bool ok = oky[ty] && (DIM == 2 || okz[tz]);
+      const T* rowp = ebuf + (long long)(ok ? stage_row(g, rc.c, lyv[ty], lzv[tz], cyv[ty], czv[tz]) : 0) * ncol;
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        const int p = p0 + k;
+        v[tz][ty][k] = (ok && p >= 0 && p < ncol) ? rowp[p] : T(0);
+      }
+    }
   T acc[GX];
 #pragma unroll
   for (int q = 0; q < GX; ++q) acc[q] = T(0);
 #pragma unroll
-  for (int tz = 0; tz < (DIM == 3 ? 2 : 1); ++tz)
+  for (int tz = 0; tz < TZ; ++tz)
 #pragma unroll
     for (int ty = 0; ty < 2; ++ty) {
-      if (!(oky[ty] && (DIM == 2 || okz[tz]))) continue;
-      const T* rowp = ebuf + (long long)stage_row(g, rc.c, lyv[ty], lzv[tz], cyv[ty], czv[tz]) * ncol;
-      T v[6];
-#pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        const int p = p0 + k;
-        v[k] = (p >= 0 && p < ncol) ? rowp[p] : T(0);
-      }
-      acc[0] += v[0] + v[1];
-      acc[1] += v[2];
-      acc[2] += v[3] + v[4];
-      acc[3] += v[5];
+      const T* w = v[tz][ty];
+      acc[0] += w[0] + w[1];
+      acc[1] += w[2];
+      acc[2] += w[3] + w[4];
+      acc[3] += w[5];
     }
 #pragma unroll
   for (int q = 0; q < GX; ++q) {
@@ -176,20 +184,26 @@ __device__ __forceinline__ void gather_chunk(const Geom& g, const T* __restrict_
 
 template <typename T, int DIM>
 __device__ __forceinline__ void gather_cells_body(unsigned bx, const Geom& g, const T* __restrict__ ebuf,
-                                                  const T* __restrict__ x, T* __restrict__ y, int keep_bnd, int raw) {
-  pdl_wait();
+                                                  const T* __restrict__ x, T* __restrict__ y, int keep_bnd, int raw,
+                                                  const T* __restrict__ b) {
   RowChunk rc;
-  if (!row_chunk(g, DIM, bx * blockDim.x + threadIdx.x, rc)) return;
-  T out[GX];
-  gather_chunk<T, DIM>(g, ebuf, x, rc, keep_bnd, raw, out);
+  const bool have = row_chunk(g, DIM, bx * blockDim.x + threadIdx.x, rc);
+  pdl_wait();
+  if (have) {
+    T out[GX], bv[GX];
 #pragma unroll
-  for (int q = 0; q < GX; ++q)
-    if (GX * rc.j + q < g.nn[0]) y[rc.t0 + q] = out[q];
+    for (int q = 0; q < GX; ++q) bv[q] = b && GX * rc.j + q < g.nn[0] ? b[rc.t0 + q] : T(0);
+    gather_chunk<T, DIM>(g, ebuf, x, rc, keep_bnd, raw, out);
+#pragma unroll
+    for (int q = 0; q < GX; ++q)
+      if (GX * rc.j + q < g.nn[0]) y[rc.t0 + q] = b ? bv[q] - out[q] : out[q];
+  }
+  pdl_trigger();
 }
 template <typename T, int DIM>
 __global__ void k_gather_cells(Geom g, const T* __restrict__ ebuf, const T* __restrict__ x, T* __restrict__ y,
-                               int keep_bnd, int raw) {
-  gather_cells_body<T, DIM>(blockIdx.x, g, ebuf, x, y, keep_bnd, raw);
+                               int keep_bnd, int raw, const T* __restrict__ b) {
+  gather_cells_body<T, DIM>(blockIdx.x, g, ebuf, x, y, keep_bnd, raw, b);
 }
 
 static unsigned gather_threads(const Geom& g) {
@@ -288,7 +302,7 @@ static void launch_cells(int nvec, cudaStream_t s, const Geom& g, const Colour& 
 
 template <typename T, int DIM, bool TENSOR, int MODE>
 static void launch_apply(const LevelDev& L, double gamma, const void* x, void* y, const void* p_in,
-                         void* p_out, int nvec, long long vstride, cudaStream_t s) {
+                         void* p_out, int nvec, long long vstride, cudaStream_t s, const void* b = nullptr) {
   const Geom& g = L.g;
   constexpr bool NEED_FLUX = (MODE & (OP_VISC | OP_AL | OP_BT)) != 0;
   const T* coef = nullptr;
@@ -304,7 +318,7 @@ static void launch_apply(const LevelDev& L, double gamma, const void* x, void* y
                                              (T*)p_out, 0, (T*)L.ebuf, winv);
     if (NEED_FLUX) {
       launch_pdl(k_gather_cells<T, DIM>, (gather_threads(g) + 255) / 256, 256, 0, s, g, (const T*)L.ebuf,
-                 (const T*)x, (T*)y, keep_bnd, (MODE & OP_RAW) ? 1 : 0);
+                 (const T*)x, (T*)y, keep_bnd, (MODE & OP_RAW) ? 1 : 0, (const T*)b);
     }
     count_launch(NEED_FLUX ? 2 : 1);
     return;
@@ -387,6 +401,24 @@ void op_apply(const LevelDev& L, int prec, int mode, double gamma, const void* x
     return;
   }
   op_dispatch(L, prec, mode, gamma, x, y, p_in, p_out, 1, 0, s);
+}
+
+template <typename T, int DIM>
+static void residual_dim(const LevelDev& L, int mode, double gamma, const void* x, const void* b, void* y,
+                         cudaStream_t s) {
+  if (mode == OP_AL) launch_apply<T, DIM, false, OP_AL>(L, gamma, x, y, nullptr, nullptr, 1, 0, s, b);
+  else if (L.tensor) launch_apply<T, DIM, true, OP_VISC | OP_AL>(L, gamma, x, y, nullptr, nullptr, 1, 0, s, b);
+  else launch_apply<T, DIM, false, OP_VISC | OP_AL>(L, gamma, x, y, nullptr, nullptr, 1, 0, s, b);
+}
+void op_residual(const LevelDev& L, int prec, int mode, double gamma, const void* x, const void* b, void* y,
+                 cudaStream_t s) {
+  if (prec == PREC_F64) {
+    if (L.g.dim == 2) residual_dim<double, 2>(L, mode, gamma, x, b, y, s);
+    else residual_dim<double, 3>(L, mode, gamma, x, b, y, s);
+  } else {
+    if (L.g.dim == 2) residual_dim<float, 2>(L, mode, gamma, x, b, y, s);
+    else residual_dim<float, 3>(L, mode, gamma, x, b, y, s);
+  }
 }
 
 template <typename T, int DIM, bool TENSOR>
@@ -508,8 +540,8 @@ __global__ void __launch_bounds__(256) k_gather_cells_b(const __grid_constant__ 
   const int i = batch_slot(tb, blockIdx.x);
   const GatherArgs& a = tb.a[i];
   const unsigned bx = blockIdx.x - tb.start[i];
-  if (a.g.dim == 3) gather_cells_body<float, 3>(bx, a.g, a.ebuf, a.x, a.y, a.keep_bnd, 0);
-  else gather_cells_body<float, 2>(bx, a.g, a.ebuf, a.x, a.y, a.keep_bnd, 0);
+  if (a.g.dim == 3) gather_cells_body<float, 3>(bx, a.g, a.ebuf, a.x, a.y, a.keep_bnd, 0, a.b);
+  else gather_cells_body<float, 2>(bx, a.g, a.ebuf, a.x, a.y, a.keep_bnd, 0, a.b);
 }
 
 static CellArgs cell_args(const BApply& it, bool zp) {
@@ -575,6 +607,7 @@ int batch_apply_al(const std::vector<BApply>& items, cudaStream_t s) {
     g.ebuf = (const float*)L.ebuf;
     g.x = (const float*)it.x;
     g.y = (float*)it.y;
+    g.b = (const float*)it.e.b;
     g.keep_bnd = 0;   // OP_AL alone: zero Dirichlet rows, as op_apply
     a.push_back(g);
     nb.push_back((gather_threads(L.g) + 255) / 256);

@@ -1146,23 +1146,31 @@ __device__ __forceinline__ void patch_gather_body(unsigned bx, const Geom& g, co
     const int ncol = 3 * g.nv[0];
     const int L = DIM == 3 ? 3 : 1;
     const int p0 = 6 * rc.j + 1;
+    // all loads first, predicated: a branch per tap pair would make each wait for the one before
+    constexpr int TZ = DIM == 3 ? 2 : 1;
+    TV v[TZ][2][6];
 #pragma unroll
-    for (int tz = 0; tz < (DIM == 3 ? 2 : 1); ++tz)
+    for (int tz = 0; tz < TZ; ++tz)
 #pragma unroll
       for (int ty = 0; ty < 2; ++ty) {
-        if (!(oky[ty] && okz[tz])) continue;
+        const bool ok = oky[ty] && okz[tz];
         const int row = ((rc.c * L + ozv[tz]) * 3 + oyv[ty]) * (g.nv[1] * g.nv[2]) + vzv[tz] * g.nv[1] + vyv[ty];
-        const TV* rowp = out + (long long)row * ncol;
-        TV v[6];
+        const TV* rowp = out + (long long)(ok ? row : 0) * ncol;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
           const int p = p0 + k;
-          v[k] = p < ncol ? rowp[p] : TV(0);
+          v[tz][ty][k] = ok && p < ncol ? rowp[p] : TV(0);
         }
-        acc[0] += v[0];
-        acc[1] += v[1] + v[2];
-        acc[2] += v[3];
-        acc[3] += v[4] + v[5];
+      }
+#pragma unroll
+    for (int tz = 0; tz < TZ; ++tz)
+#pragma unroll
+      for (int ty = 0; ty < 2; ++ty) {
+        const TV* w = v[tz][ty];
+        acc[0] += w[0];
+        acc[1] += w[1] + w[2];
+        acc[2] += w[3];
+        acc[3] += w[4] + w[5];
       }
   }
 #pragma unroll
