@@ -280,25 +280,25 @@ bool fused_gmres(const als_ctx* c) {
   return c->opt.smoother == ALS_SMOOTH_GMRES && std::max(1, c->opt.sweeps) <= KMAXB;
 }
 
-// Order-2 cycles form Z_j inside the operator's cell kernel from the patch outputs
+// Order-2 cycles, and those of order 3 in 2D and FP32, form Z_j inside the operator's cell kernel from the patch outputs
 // (one launch less per Arnoldi step); ALS_FUSE_GATHER=0 keeps the separate gather
-bool fuse_patch_gather(const als_ctx* c) {
+bool fuse_patch_gather(const als_ctx* c, int prec) {
   static int v = -1;
   if (v < 0) {
     const char* e = getenv("ALS_FUSE_GATHER");
     v = (e && e[0] == '0') ? 0 : 1;
   }
-  return v == 1 && c->k == 2;
+  return v == 1 && (c->k == 2 || (c->dim == 2 && prec == PREC_F32));
 }
 
 // levels whose Arnoldi steps are one launch each
 bool tiled_steps(const als_ctx* c, const MGWork& w, int l) {
-  return fuse_patch_gather(c) && arnoldi_tiled(c->lev[l], w.prec);
+  return fuse_patch_gather(c, w.prec) && arnoldi_tiled(c->lev[l], w.prec);
 }
 
 // levels whose robust transfers to and from the next coarser level are one launch each
 bool tiled_transfers(const als_ctx* c, const MGWork& w, int l) {
-  return c->opt.transfer == ALS_TRANSFER_ROBUST && fuse_patch_gather(c) && transfer_tiled(c->lev[l], w.prec);
+  return c->opt.transfer == ALS_TRANSFER_ROBUST && fuse_patch_gather(c, w.prec) && transfer_tiled(c->lev[l], w.prec);
 }
 
 // step j of a tiled smoothing: w goes through two buffers in the star products' scratch in turn
@@ -349,7 +349,7 @@ void smooth_fused(als_ctx* c, MGWork& w, int l, bool x_is_zero, void* t) {
       continue;
     }
     ApplyEpi e{nullptr, 1.0, j + 1, w.V[l], len, 0, st};
-    if (fuse_patch_gather(c)) {
+    if (fuse_patch_gather(c, prec)) {
       // patch products only; the cell kernel sums them per node into Z_j = D^-1 V_j
       patch_products(Lv, prec, Vj, w.scratch[l], s, e0, e1);
       e.pout = w.scratch[l];
@@ -1845,7 +1845,7 @@ void merged_smooth(MergedCycle& M, int l, bool x_is_zero, bool residual, cudaStr
       void* Zj = vptr(w.Z[l], w.es, (long long)j * len);
       prod.push_back(BPatch{&c->lev[l], Vj, w.scratch[l], nullptr});
       ApplyEpi e{nullptr, 1.0, j + 1, w.V[l], len, 0, g[i].st};
-      if (fuse_patch_gather(c)) {
+      if (fuse_patch_gather(c, PREC_F32)) {
         e.pout = w.scratch[l];
       } else {
         gath.push_back(BPatch{&c->lev[l], nullptr, w.scratch[l], Zj});

@@ -138,7 +138,7 @@ __device__ __forceinline__ void load_tables(SharedTables<T>& t, T sx, T sy, T wd
 __device__ __forceinline__ double phi(int q, int a) { return cL[q % N1][a % N1] * cL[q / N1][a / N1]; }
 
 // ---------------------------------------------------------------------------
-// operator apply: one warp per cell, lanes 0..15 = Gauss points, then = nodes
+// operator apply (FP64): one warp per cell, lanes 0..15 = Gauss points, then = nodes
 // ---------------------------------------------------------------------------
 template <typename T, int MODE>
 __global__ void __launch_bounds__(256) k_qk_cells(Geom g, CellScal<T> cs, const T* __restrict__ x, const T* __restrict__ mu,
@@ -153,6 +153,8 @@ __global__ void __launch_bounds__(256) k_qk_cells(Geom g, CellScal<T> cs, const 
   load_tables<T>(tb, cs.sx, cs.sy, cs.wdet);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const long long cell = (long long)blockIdx.x * 8 + w;
+  pdl_wait();
+  pdl_trigger();
   if (cell >= g.ncells) return;
   const int cx = (int)(cell % g.n[0]), cy = (int)(cell / g.n[0]);
   if (lane < NB) {
@@ -226,6 +228,227 @@ __global__ void __launch_bounds__(256) k_qk_cells(Geom g, CellScal<T> cs, const 
   }
 }
 
+// ---------------------------------------------------------------------------
+// operator apply, FP32: two lanes per cell (lanes i and i + 16 of a warp: the components of cell i)
+// ---------------------------------------------------------------------------
+// A lane holds its component's 16 nodal values and contracts them axis by axis in registers against
+// the 1D tables (constant operands): 512 FMAs a lane for the two directions, where a warp a cell
+// with the dense 16 x 16 derivative tables takes 128 warp instructions of FMAs and as many shared loads for
+// one cell, half its lanes idle.  The lanes exchange the diagonal gradient and the shear by
+// shuffles and halve the pressure moments.  ZP: u is formed from the star outputs, in the order of
+// k_qk_star_gather, and stored, each node by the cell that owns it (the last cell also the upper
+// ends).  FP64 keeps the form above: a lane's chain of FP64 instructions, 64 cycles each, is longer
+// than a level's time.  One 128^2 five-level cycle, with every kernel of the level now a programmatic
+// launch: 1162 us, 1560 with the other form and the star gather a kernel of its own.
+template <int MODE, bool ZP>
+__global__ void __launch_bounds__(64) k_qk_cells2(Geom g, CellScal<float> cs, const float* __restrict__ x,
+                                                  const float* __restrict__ mu, const float* __restrict__ winv,
+                                                  const float* __restrict__ p_in, float* __restrict__ p_out,
+                                                  float* __restrict__ ebuf, const float* __restrict__ sc,
+                                                  float* __restrict__ z) {
+  constexpr bool RAW = (MODE & OP_RAW) != 0, VISC = (MODE & OP_VISC) != 0, AL = (MODE & OP_AL) != 0;
+  constexpr bool BT = (MODE & OP_BT) != 0, BO = (MODE & OP_B) != 0;
+  constexpr bool NEED_U = VISC || AL || BO, NEED_FLUX = VISC || AL || BT;
+  constexpr unsigned FULL = 0xffffffffu;
+  using TF = Tab<float>;
+  const int lane = threadIdx.x & 31, c = lane >> 4;
+  const int cell = (int)(blockIdx.x * 32 + (threadIdx.x >> 5) * 16 + (lane & 15));
+  const bool act = cell < (int)g.ncells;
+  const int cy = cell / g.n[0], cx = cell - cy * g.n[0];
+  float m[VISC ? NQ : 1], wi[AL ? 3 * NPR : 1];   // constant: ahead of the wait
+  if constexpr (VISC) {
+#pragma unroll
+    for (int k = 0; k < NQ / 4; ++k) {
+      const float4 v = act ? __ldg(reinterpret_cast<const float4*>(mu + (long long)cell * NQ) + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+      m[4 * k] = v.x; m[4 * k + 1] = v.y; m[4 * k + 2] = v.z; m[4 * k + 3] = v.w;
+    }
+  }
+  if constexpr (AL) {
+#pragma unroll
+    for (int k = 0; k < 3 * NPR; ++k) wi[k] = act ? __ldg(winv + (long long)cell * (NPR * NPR) + 3 * c * NPR + k) : 0.f;
+  }
+  pdl_wait();
+  pdl_trigger();
+  float gd[NQ], gs[NQ];   // d u_c / d x_c; d u_c / d x_(1-c), then the shear sum
+  float P[NQ];            // the pressure-like field at the points: gamma pi + p_in
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) gd[q] = gs[q] = P[q] = 0.f;
+  if constexpr (NEED_U) {
+    float u[NB];
+#pragma unroll
+    for (int a = 0; a < NB; ++a) u[a] = 0.f;
+    if (act) {
+      const bool x0 = cx == 0, x1 = cx == g.n[0] - 1, y0 = cy == 0, y1 = cy == g.n[1] - 1;
+      const auto dirichlet = [&](int a, int b) { return (a == 0 && x0) || (a == K && x1) || (b == 0 && y0) || (b == K && y1); };
+      if constexpr (ZP) {
+        const float* s0 = sc + (cx + (g.n[0] + 1) * cy) * NS + c * S1 * S1;
+        const int up = (g.n[0] + 1) * NS;
+#pragma unroll
+        for (int b = 0; b < N1; ++b)
+#pragma unroll
+          for (int a = 0; a < N1; ++a) {
+            // taps: star 0 unless the node is the upper corner, star 1 unless the lower one
+            float t = 0.f;
+#pragma unroll
+            for (int sb = 0; sb < 2; ++sb) {
+              if (sb == 0 ? b == K : b == 0) continue;
+              const int oy = sb == 0 ? b + K - 1 : b - 1;
+#pragma unroll
+              for (int sa = 0; sa < 2; ++sa) {
+                if (sa == 0 ? a == K : a == 0) continue;
+                const int ox = sa == 0 ? a + K - 1 : a - 1;
+                t += s0[sb * up + sa * NS + ox + S1 * oy];
+              }
+            }
+            u[a + N1 * b] = dirichlet(a, b) ? 0.f : t;
+          }
+        float* zc = z + (c * (int)g.N + K * cx + g.nn[0] * (K * cy));
+#pragma unroll
+        for (int b = 0; b < N1; ++b)
+#pragma unroll
+          for (int a = 0; a < N1; ++a)
+            if ((a < K || x1) && (b < K || y1)) zc[a + g.nn[0] * b] = u[a + N1 * b];
+      } else {
+        const float* xc = x + (c * (int)g.N + K * cx + g.nn[0] * (K * cy));
+#pragma unroll
+        for (int b = 0; b < N1; ++b)
+#pragma unroll
+          for (int a = 0; a < N1; ++a) u[a + N1 * b] = RAW || !dirichlet(a, b) ? xc[a + g.nn[0] * b] : 0.f;
+      }
+    }
+#pragma unroll
+    for (int qx = 0; qx < N1; ++qx) {
+      float bx[N1], dx[N1];
+#pragma unroll
+      for (int b = 0; b < N1; ++b) {
+        bx[b] = dx[b] = 0.f;
+#pragma unroll
+        for (int a = 0; a < N1; ++a) {
+          bx[b] += TF::L(qx, a) * u[a + N1 * b];
+          dx[b] += TF::D(qx, a) * u[a + N1 * b];
+        }
+      }
+#pragma unroll
+      for (int qy = 0; qy < N1; ++qy) {
+        float gx = 0.f, gy = 0.f;
+#pragma unroll
+        for (int b = 0; b < N1; ++b) {
+          gx += TF::L(qy, b) * dx[b];
+          gy += TF::D(qy, b) * bx[b];
+        }
+        gx *= cs.sx;
+        gy *= cs.sy;
+        gd[qx + N1 * qy] = c == 0 ? gx : gy;
+        gs[qx + N1 * qy] = c == 0 ? gy : gx;
+      }
+    }
+    if constexpr (AL || BO) {
+      float bu[NPR];   // (B u)_p = -sum_q w |J| psi_p div u, three a lane, then exchanged
+      float mine[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        const float d = cs.wdet * TF::w2(q) * (gd[q] + __shfl_xor_sync(FULL, gd[q], 16));
+#pragma unroll
+        for (int p = 0; p < 3; ++p) mine[p] -= (c == 0 ? TF::psi(q, p) : TF::psi(q, p + 3)) * d;
+      }
+#pragma unroll
+      for (int p = 0; p < 3; ++p) {
+        const float o = __shfl_xor_sync(FULL, mine[p], 16);
+        bu[p] = c == 0 ? mine[p] : o;
+        bu[p + 3] = c == 0 ? o : mine[p];
+      }
+      if constexpr (BO) {
+        if (act) {
+#pragma unroll
+          for (int p = 0; p < 3; ++p) p_out[(long long)cell * NPR + 3 * c + p] = mine[p];
+        }
+      }
+      if constexpr (AL) {
+        float pi[NPR];
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {
+          float s = 0.f;
+#pragma unroll
+          for (int r = 0; r < NPR; ++r) s += wi[p * NPR + r] * bu[r];
+          s *= cs.gamma;
+          const float o = __shfl_xor_sync(FULL, s, 16);
+          pi[p] = c == 0 ? s : o;
+          pi[p + 3] = c == 0 ? o : s;
+        }
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+#pragma unroll
+          for (int p = 0; p < NPR; ++p) P[q] += TF::psi(q, p) * pi[p];
+      }
+    }
+  }
+  if constexpr (NEED_FLUX) {
+    if constexpr (BT) {
+      if (act) {
+#pragma unroll
+        for (int p = 0; p < NPR; ++p) {
+          const float v = p_in[(long long)cell * NPR + p];
+#pragma unroll
+          for (int q = 0; q < NQ; ++q) P[q] += TF::psi(q, p) * v;
+        }
+      }
+    }
+    // fluxes: gd <- w (2 mu d_c u_c - P), gs <- w mu (d_c u_(1-c) + d_(1-c) u_c)
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const float w = cs.wdet * TF::w2(q);
+      if constexpr (VISC) {
+        const float shear = gs[q] + __shfl_xor_sync(FULL, gs[q], 16);
+        gd[q] = w * (2.f * m[q] * gd[q] - P[q]);
+        gs[q] = w * (m[q] * shear);
+      } else {
+        gd[q] = -(w * P[q]);
+      }
+    }
+    float y[NB];
+#pragma unroll
+    for (int a = 0; a < NB; ++a) y[a] = 0.f;
+#pragma unroll
+    for (int qx = 0; qx < N1; ++qx) {
+      float tb[N1], td[N1];
+#pragma unroll
+      for (int b = 0; b < N1; ++b) {
+        tb[b] = td[b] = 0.f;
+#pragma unroll
+        for (int qy = 0; qy < N1; ++qy) {
+          const int q = qx + N1 * qy;
+          const float f = VISC ? gs[q] : 0.f;
+          tb[b] += TF::L(qy, b) * (c == 0 ? gd[q] : f);
+          td[b] += TF::D(qy, b) * (c == 0 ? f : gd[q]);
+        }
+        tb[b] *= cs.sx;
+        td[b] *= cs.sy;
+      }
+#pragma unroll
+      for (int b = 0; b < N1; ++b)
+#pragma unroll
+        for (int a = 0; a < N1; ++a) y[a + N1 * b] += TF::D(qx, a) * tb[b] + TF::L(qx, a) * td[b];
+    }
+    if (act) {
+      float4* e = reinterpret_cast<float4*>(ebuf + ((long long)cell * 2 + c) * NB);
+#pragma unroll
+      for (int k = 0; k < NB / 4; ++k) e[k] = make_float4(y[4 * k], y[4 * k + 1], y[4 * k + 2], y[4 * k + 3]);
+    }
+  }
+}
+// the cell kernel of precision T (FP32 with sc: u formed from the star outputs and stored to z)
+template <typename T, int MODE, bool ZP = false>
+static void launch_cells(const LevelDev& L, double gamma, const void* x, const void* p_in, void* p_out, cudaStream_t s,
+                         const void* sc = nullptr, void* z = nullptr) {
+  if constexpr (std::is_same<T, float>::value)
+    launch_pdl(k_qk_cells2<MODE, ZP>, (unsigned)((L.g.ncells + 31) / 32), 64, 0, s, L.g, cell_scal<float>(L.g, gamma),
+               (const float*)x, (const float*)L.coef32, (const float*)L.winv32, (const float*)p_in, (float*)p_out,
+               (float*)L.ebuf, (const float*)sc, (float*)z);
+  else
+    launch_pdl(k_qk_cells<T, MODE>, (unsigned)((L.g.ncells + 7) / 8), 256, 0, s, L.g, cell_scal<T>(L.g, gamma),
+               (const T*)x, (const T*)L.coef64, (const T*)L.winv64, (const T*)p_in, (T*)p_out, (T*)L.ebuf);
+}
+
 // the cells containing lattice index i along an axis of n cells, two taps in a fixed order:
 // (c - 1, local K) where i is the cell corner between c - 1 and c, then (c, i - K c)
 struct CellTaps {
@@ -266,6 +489,8 @@ template <typename T>
 __global__ void k_qk_gather(Geom g, const T* __restrict__ ebuf, const T* __restrict__ x, T* __restrict__ y, int keep_bnd,
                             int raw) {
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_wait();
+  pdl_trigger();
   if (t >= 2u * (unsigned)g.N) return;
   y[t] = qk_gather_value<T>(g, ebuf, x, t, keep_bnd, raw);
 }
@@ -312,14 +537,11 @@ template <typename T, int MODE>
 static void apply_mode(const LevelDev& L, double gamma, const void* x, void* y, const void* p_in, void* p_out,
                        cudaStream_t s) {
   constexpr bool NEED_FLUX = (MODE & (OP_VISC | OP_AL | OP_BT)) != 0;
-  const T* mu = std::is_same<T, double>::value ? (const T*)L.coef64 : (const T*)L.coef32;
-  const T* winv = std::is_same<T, double>::value ? (const T*)L.winv64 : (const T*)L.winv32;
-  k_qk_cells<T, MODE><<<(unsigned)((L.g.ncells + 7) / 8), 256, 0, s>>>(L.g, cell_scal<T>(L.g, gamma), (const T*)x, mu, winv,
-                                                                      (const T*)p_in, (T*)p_out, (T*)L.ebuf);
+  launch_cells<T, MODE>(L, gamma, x, p_in, p_out, s);
   if (NEED_FLUX) {
     const int keep = ((MODE & OP_VISC) && !(MODE & OP_RAW)) ? 1 : 0;
-    k_qk_gather<T><<<(unsigned)((2 * L.g.N + 255) / 256), 256, 0, s>>>(L.g, (const T*)L.ebuf, (const T*)x, (T*)y,
-                                                                        keep, (MODE & OP_RAW) ? 1 : 0);
+    launch_pdl(k_qk_gather<T>, (unsigned)((2 * L.g.N + 255) / 256), 256, 0, s, L.g, (const T*)L.ebuf, (const T*)x, (T*)y,
+               keep, (MODE & OP_RAW) ? 1 : 0);
   }
   count_launch(NEED_FLUX ? 2 : 1);
 }
@@ -550,6 +772,8 @@ __global__ void __launch_bounds__(32 * star_warps<T>()) k_qk_star_apply(Geom g, 
   const uint4* src = reinterpret_cast<const uint4*>(inv + v * kStarStride);
 #pragma unroll 4
   for (int e = lane; e < NV; e += 32) sbuf[w][e] = __ldg(src + e);
+  pdl_wait();
+  pdl_trigger();
   for (int e = lane; e < NS; e += 32) {
     long long nd;
     rs[w][e] = star_node(g, vx, vy, e, nd) ? r[(e / (S1 * S1)) * g.N + nd] : T(0);
@@ -624,7 +848,7 @@ __global__ void __launch_bounds__(256, kStarWBlocksPerSM) k_qk_star_apply_w(Geom
   // a star's rows and r values into registers (consumed by the next pass's staging)
   float4 pw[PF];
   float pr[R];
-  const auto fetch = [&](long long it) {
+  const auto fetch_rows = [&](long long it) {
     int fx, fy;
     vertex(it, fx, fy);
     const float4* src = reinterpret_cast<const float4*>(inv + ((long long)fx + (long long)(g.n[0] + 1) * fy) * kWStride);
@@ -633,6 +857,10 @@ __global__ void __launch_bounds__(256, kStarWBlocksPerSM) k_qk_star_apply_w(Geom
       const int e = lane + 32 * q;
       if (e < NV) pw[q] = __ldg(src + e);
     }
+  };
+  const auto fetch_r = [&](long long it) {
+    int fx, fy;
+    vertex(it, fx, fy);
 #pragma unroll
     for (int k = 0; k < R; ++k) {
       const int e = lane + 32 * k;
@@ -640,7 +868,10 @@ __global__ void __launch_bounds__(256, kStarWBlocksPerSM) k_qk_star_apply_w(Geom
       pr[k] = (e < NS && star_node(g, fx, fy, e, nd)) ? r[(e / (S1 * S1)) * g.N + nd] : 0.f;
     }
   };
-  fetch(item);
+  fetch_rows(item);
+  pdl_wait();
+  pdl_trigger();
+  fetch_r(item);
   for (;;) {
     int vx, vy;
     vertex(item, vx, vy);
@@ -662,7 +893,10 @@ __global__ void __launch_bounds__(256, kStarWBlocksPerSM) k_qk_star_apply_w(Geom
     }
     __syncwarp();
     const long long next = item + nwarps;
-    if (next < count) fetch(next);   // in flight during this star's products
+    if (next < count) {              // in flight during this star's products
+      fetch_rows(next);
+      fetch_r(next);
+    }
     // lane j < H owns rows j and j + H; row j takes step t while row j + H takes step
     // H - t, which reads the same two r values (r_(j+t) and r_(j-t mod NS)): six shared
     // reads per four FMAs instead of eight
@@ -791,27 +1025,38 @@ __device__ __forceinline__ int owner(int f, int nc, int& fr) {
 }
 
 template <typename T>
-__global__ void k_qk_prolong(Geom gc, Geom gf, const T* __restrict__ xc, T* __restrict__ xf, T* __restrict__ xadd) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 2 * gf.N) return;
-  const int comp = (int)(t / gf.N);
-  const long long nd = t - comp * gf.N;
-  const int i = (int)(nd % gf.nn[0]), j = (int)(nd / gf.nn[0]);
-  T v = T(0);
+__global__ void __launch_bounds__(256) k_qk_prolong(Geom gc, Geom gf, const T* __restrict__ xc, T* __restrict__ xf,
+                                                    T* __restrict__ xadd) {
+  __shared__ T W[2 * K + 1][N1];   // per-lane indices serialise in constant memory
+  for (int e = threadIdx.x; e < (2 * K + 1) * N1; e += blockDim.x) W[e / N1][e % N1] = Tab<T>::pw(e / N1, e % N1);
+  __syncthreads();
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x, N = (unsigned)gf.N, nx = (unsigned)gf.nn[0];
+  pdl_wait();
+  pdl_trigger();
+  if (t >= 2u * N) return;
+  const int comp = (int)(t / N);
+  const unsigned nd = t - comp * N;
+  const int j = (int)(nd / nx), i = (int)(nd - j * nx);
+  T acc = T(0);
   if (!(i == 0 || i == gf.nn[0] - 1 || j == 0 || j == gf.nn[1] - 1)) {
     int fx, fy;
     const int cx = owner(i, gc.n[0], fx), cy = owner(j, gc.n[1], fy);
-    T acc = T(0);
+    T v[N1][N1];
+#pragma unroll
     for (int b = 0; b < N1; ++b)
+#pragma unroll
       for (int a = 0; a < N1; ++a) {
         const int I = K * cx + a, J = K * cy + b;
-        if (I == 0 || I == gc.nn[0] - 1 || J == 0 || J == gc.nn[1] - 1) continue;
-        acc += Tab<T>::pw(fx, a) * Tab<T>::pw(fy, b) * xc[comp * gc.N + I + (long long)gc.nn[0] * J];
+        const bool ok = I > 0 && I < gc.nn[0] - 1 && J > 0 && J < gc.nn[1] - 1;
+        v[b][a] = ok ? xc[comp * (int)gc.N + I + gc.nn[0] * J] : T(0);
       }
-    v = acc;
+#pragma unroll
+    for (int b = 0; b < N1; ++b)
+#pragma unroll
+      for (int a = 0; a < N1; ++a) acc += W[fx][a] * W[fy][b] * v[b][a];
   }
-  xf[t] = v;
-  if (xadd) xadd[t] += v;
+  xf[t] = acc;
+  if (xadd) xadd[t] += acc;
 }
 
 // rc = P_H^T (rf - sub): coarse node J gathers the fine nodes owned by the coarse cells that
@@ -825,6 +1070,8 @@ __global__ void __launch_bounds__(256) k_qk_restrict(Geom gc, Geom gf, const T* 
   for (int e = threadIdx.x; e < (2 * K + 1) * N1; e += blockDim.x) W[e / N1][e % N1] = Tab<T>::pw(e / N1, e % N1);
   __syncthreads();
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x, N = (unsigned)gc.N, nx = (unsigned)gc.nn[0];
+  pdl_wait();
+  pdl_trigger();
   if (t >= 2u * N) return;
   const int comp = (int)(t / N);
   const unsigned nd = t - comp * N;
@@ -887,12 +1134,12 @@ void qk_apply(const LevelDev& L, int prec, int mode, double gamma, const void* x
 template <typename T>
 static void apply_epi_t(const LevelDev& L, double gamma, const void* x, void* y, const ApplyEpi& e, cudaStream_t s,
                         cudaEvent_t e0, cudaEvent_t e1) {
-  const T* mu = std::is_same<T, double>::value ? (const T*)L.coef64 : (const T*)L.coef32;
-  const T* winv = std::is_same<T, double>::value ? (const T*)L.winv64 : (const T*)L.winv32;
   // External records become event-record nodes when the stream is being captured
   if (e0) cudaEventRecordWithFlags(e0, s, cudaEventRecordExternal);
-  qk::k_qk_cells<T, OP_VISC | OP_AL><<<(unsigned)((L.g.ncells + 7) / 8), 256, 0, s>>>(
-      L.g, qk::cell_scal<T>(L.g, gamma), (const T*)x, mu, winv, nullptr, nullptr, (T*)L.ebuf);
+  if (std::is_same<T, float>::value && e.pout)   // x = z formed from the star outputs; z stored on the way
+    qk::launch_cells<float, OP_VISC | OP_AL, true>(L, gamma, nullptr, nullptr, nullptr, s, e.pout, const_cast<void*>(x));
+  else
+    qk::launch_cells<T, OP_VISC | OP_AL>(L, gamma, x, nullptr, nullptr, s);
   if (e1) cudaEventRecordWithFlags(e1, s, cudaEventRecordExternal);
   const auto kernel = qk_epi_per(L) == 1 ? qk::k_qk_gather_epi<T, 1> : qk::k_qk_gather_epi<T, kEpiPer>;
   launch_pdl(kernel, qk_epi_blocks(L), RED_THREADS, 0, s, L.g, (const T*)L.ebuf, (const T*)x, (T*)y, (const T*)e.b,
@@ -940,33 +1187,34 @@ void qk_patch_setup(const LevelDev& L, double gamma, DevStatus* st, cudaStream_t
   count_launch(1);
 }
 
+static void qk2_stars(const LevelDev& L, int prec, int interior, int mode, const void* r, void* out, cudaStream_t s) {
+  const long long count = interior ? (long long)(L.g.n[0] / 2) * (L.g.n[1] / 2) : L.g.nverts;
+  constexpr int W64 = qk::star_warps<double>();
+  if (prec == PREC_F64)
+    launch_pdl(qk::k_qk_star_apply<double>, (unsigned)((count + W64 - 1) / W64), 32 * W64, 0, s, L.g,
+               (const double*)L.inv64, L.pstride, interior, mode, (const double*)r, (double*)out);
+  else
+    launch_pdl(qk::k_qk_star_apply_w, qk::star_w_blocks(count), 256, 0, s, L.g, (const float*)L.inv32, interior, mode,
+               (const float*)r, (float*)out);
+  count_launch(1);
+}
+
+void qk_patch_products(const LevelDev& L, const void* r, void* scratch, cudaStream_t s) {
+  qk2_stars(L, PREC_F32, 0, 0, r, scratch, s);
+}
+
 void qk_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, cudaStream_t s) {
   if (L.g.dim == 3) return qk3_patch_smooth(L, prec, r, z, scratch, s);
   const unsigned b2 = (unsigned)((2 * L.g.N + 255) / 256);
-  constexpr int W64 = qk::star_warps<double>(), W32 = qk::star_warps<float>();
-  if (prec == PREC_F64) {
-    qk::k_qk_star_apply<double><<<(unsigned)((L.g.nverts + W64 - 1) / W64), 32 * W64, 0, s>>>(
-        L.g, L.inv64, L.pstride, 0, 0, (const double*)r, (double*)scratch);
-    launch_pdl(qk::k_qk_star_gather<double>, b2, 256, 0, s, L.g, (const double*)scratch, (double*)z);
-  } else {
-    qk::k_qk_star_apply_w<<<qk::star_w_blocks(L.g.nverts), 256, 0, s>>>(L.g, L.inv32, 0, 0, (const float*)r,
-                                                                      (float*)scratch);
-    launch_pdl(qk::k_qk_star_gather<float>, b2, 256, 0, s, L.g, (const float*)scratch, (float*)z);
-  }
-  count_launch(2);
+  qk2_stars(L, prec, 0, 0, r, scratch, s);
+  if (prec == PREC_F64) launch_pdl(qk::k_qk_star_gather<double>, b2, 256, 0, s, L.g, (const double*)scratch, (double*)z);
+  else launch_pdl(qk::k_qk_star_gather<float>, b2, 256, 0, s, L.g, (const float*)scratch, (float*)z);
+  count_launch(1);
 }
 
 void qk_interior_solve(const LevelDev& fine, int prec, const void* in, void* out, int subtract, cudaStream_t s) {
   if (fine.g.dim == 3) return qk3_interior_solve(fine, prec, in, out, subtract, s);
-  const long long nc = (long long)(fine.g.n[0] / 2) * (fine.g.n[1] / 2);
-  constexpr int W64 = qk::star_warps<double>(), W32 = qk::star_warps<float>();
-  if (prec == PREC_F64)
-    qk::k_qk_star_apply<double><<<(unsigned)((nc + W64 - 1) / W64), 32 * W64, 0, s>>>(
-        fine.g, fine.inv64, fine.pstride, 1, subtract ? 2 : 1, (const double*)in, (double*)out);
-  else
-    qk::k_qk_star_apply_w<<<qk::star_w_blocks(nc), 256, 0, s>>>(fine.g, fine.inv32, 1, subtract ? 2 : 1,
-                                                              (const float*)in, (float*)out);
-  count_launch(1);
+  qk2_stars(fine, prec, 1, subtract ? 2 : 1, in, out, s);
 }
 
 void qk_prolong(const LevelDev& coarse, const LevelDev& fine, int prec, const void* xc, void* xf, cudaStream_t s,
@@ -974,8 +1222,8 @@ void qk_prolong(const LevelDev& coarse, const LevelDev& fine, int prec, const vo
   if (fine.g.dim == 3) return qk3_prolong(coarse, fine, prec, xc, xf, s, xadd);
   const unsigned b = (unsigned)((2 * fine.g.N + 255) / 256);
   if (prec == PREC_F64)
-    qk::k_qk_prolong<double><<<b, 256, 0, s>>>(coarse.g, fine.g, (const double*)xc, (double*)xf, (double*)xadd);
-  else qk::k_qk_prolong<float><<<b, 256, 0, s>>>(coarse.g, fine.g, (const float*)xc, (float*)xf, (float*)xadd);
+    launch_pdl(qk::k_qk_prolong<double>, b, 256, 0, s, coarse.g, fine.g, (const double*)xc, (double*)xf, (double*)xadd);
+  else launch_pdl(qk::k_qk_prolong<float>, b, 256, 0, s, coarse.g, fine.g, (const float*)xc, (float*)xf, (float*)xadd);
   count_launch(1);
 }
 
@@ -984,8 +1232,8 @@ void qk_restrict(const LevelDev& coarse, const LevelDev& fine, int prec, const v
   if (fine.g.dim == 3) return qk3_restrict(coarse, fine, prec, rf, rc, s, sub);
   const unsigned b = (unsigned)((2 * coarse.g.N + 255) / 256);
   if (prec == PREC_F64)
-    qk::k_qk_restrict<double><<<b, 256, 0, s>>>(coarse.g, fine.g, (const double*)rf, (const double*)sub, (double*)rc);
-  else qk::k_qk_restrict<float><<<b, 256, 0, s>>>(coarse.g, fine.g, (const float*)rf, (const float*)sub, (float*)rc);
+    launch_pdl(qk::k_qk_restrict<double>, b, 256, 0, s, coarse.g, fine.g, (const double*)rf, (const double*)sub, (double*)rc);
+  else launch_pdl(qk::k_qk_restrict<float>, b, 256, 0, s, coarse.g, fine.g, (const float*)rf, (const float*)sub, (float*)rc);
   count_launch(1);
 }
 
