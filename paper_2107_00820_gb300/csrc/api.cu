@@ -280,7 +280,7 @@ bool fused_gmres(const als_ctx* c) {
   return c->opt.smoother == ALS_SMOOTH_GMRES && std::max(1, c->opt.sweeps) <= KMAXB;
 }
 
-// Order-2 cycles, and those of order 3 in 2D and FP32, form Z_j inside the operator's cell kernel from the patch outputs
+// Order-2 cycles, and those of order 3 in FP32, form Z_j inside the operator's cell kernel from the patch outputs
 // (one launch less per Arnoldi step); ALS_FUSE_GATHER=0 keeps the separate gather
 bool fuse_patch_gather(const als_ctx* c, int prec) {
   static int v = -1;
@@ -288,7 +288,7 @@ bool fuse_patch_gather(const als_ctx* c, int prec) {
     const char* e = getenv("ALS_FUSE_GATHER");
     v = (e && e[0] == '0') ? 0 : 1;
   }
-  return v == 1 && (c->k == 2 || (c->dim == 2 && prec == PREC_F32));
+  return v == 1 && (c->k == 2 || prec == PREC_F32);
 }
 
 // levels whose Arnoldi steps are one launch each

@@ -85,7 +85,7 @@ struct ApplyEpi {
   long long ld;
   int start;
   GmresDev st;
-  // when pout is set (order 2; order 3 in 2D and FP32), the apply's input x is not read but formed from the
+  // when pout is set (order 2; order 3 in FP32), the apply's input x is not read but formed from the
   // star-patch outputs pout (row layout) and stored into x (the patch gather fused into
   // the cell kernel)
   const void* pout = nullptr;
@@ -153,8 +153,9 @@ void patch_interior_solve(const LevelDev& fine, int prec, const void* in, void* 
 // operator.cu, patches.cu, transfer.cu and coarse.cu call these when L.k == 3, and they
 // pass 3D levels on to qk3.cu's qk3_* functions of the same arguments
 void qk_tables();
-// the star products of 2D FP32 (patch_products)
+// the FP32 star products (patch_products)
 void qk_patch_products(const LevelDev& L, const void* r, void* scratch, cudaStream_t s);
+void qk3_patch_products(const LevelDev& L, const void* r, void* scratch, cudaStream_t s);
 // entries per thread and blocks of the order-3 gathers with a reduction: one entry a thread
 // (latency) until the grid fills the GPU four times over, then kEpiPer
 constexpr int kEpiPer = 4;

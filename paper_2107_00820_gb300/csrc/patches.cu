@@ -1219,7 +1219,7 @@ static void star_products(int v, const LevelDev& L, const float* r, float* scrat
 
 void patch_products(const LevelDev& L, int prec, const void* r, void* scratch, cudaStream_t s, cudaEvent_t e0,
                     cudaEvent_t e1) {
-  if (L.k == 3) {   // 2D FP32
+  if (L.k == 3) {   // FP32
     if (e0) cudaEventRecordWithFlags(e0, s, cudaEventRecordExternal);
     qk_patch_products(L, r, scratch, s);
     if (e1) cudaEventRecordWithFlags(e1, s, cudaEventRecordExternal);

@@ -510,6 +510,13 @@ __global__ void __launch_bounds__(RED_THREADS) k_qk_gather_epi(Geom g, const T* 
 #pragma unroll
   for (int jj = 0; jj < KMAXB; ++jj) acc[jj] = T(0);
   const unsigned n = 2 * (unsigned)g.N, t0 = blockIdx.x * (RED_THREADS * PER) + threadIdx.x;
+  // the basis columns come from kernels before the predecessor: ahead of the wait
+  T vp[PER][KMAXB];
+#pragma unroll
+  for (int q = 0; q < PER; ++q)
+#pragma unroll
+    for (int jj = 0; jj < KMAXB; ++jj)
+      vp[q][jj] = !start && jj < k && t0 + q * RED_THREADS < n ? __ldcg(V + (long long)jj * ld + t0 + q * RED_THREADS) : T(0);
   pdl_wait();
   T v[PER];
 #pragma unroll
@@ -526,7 +533,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_qk_gather_epi(Geom g, const T* 
     } else {
 #pragma unroll
       for (int jj = 0; jj < KMAXB; ++jj)
-        if (jj < k && t < n) acc[jj] += __ldcg(V + (long long)jj * ld + t) * v[q];
+        if (jj < k) acc[jj] += vp[q][jj] * v[q];
     }
   }
   pdl_trigger();
@@ -1200,6 +1207,7 @@ static void qk2_stars(const LevelDev& L, int prec, int interior, int mode, const
 }
 
 void qk_patch_products(const LevelDev& L, const void* r, void* scratch, cudaStream_t s) {
+  if (L.g.dim == 3) return qk3_patch_products(L, r, scratch, s);
   qk2_stars(L, PREC_F32, 0, 0, r, scratch, s);
 }
 

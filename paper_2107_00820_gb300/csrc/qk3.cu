@@ -144,11 +144,68 @@ struct CellShared {
   T sp[CPB][NPR];
 };
 
-template <typename T, int MODE>
+// the vertices whose stars contain lattice index i (|i - 3v| <= 2), two taps: v0 = i / 3, then
+// v0 + 1 unless i = 3 v0; o: offset index in the star, 0 .. S1 - 1
+struct StarTaps {
+  int v[2], o[2];
+  bool two;
+  __device__ __forceinline__ explicit StarTaps(int i) {
+    const int v0 = i / K, r = i - K * v0;
+    v[0] = v0; o[0] = r + K - 1;
+    v[1] = v0 + 1; o[1] = r - 1;
+    two = r != 0;
+  }
+};
+
+// z at node (i, j, k) = sum over the (up to 8) stars containing it, of their outputs sc, fixed order
+template <typename T>
+__device__ __forceinline__ T star_sum(const Geom& g, const T* __restrict__ sc, int comp, int i, int j, int k) {
+  const StarTaps tx(i), ty(j), tz(k);
+  T v[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int a = q & 1, b = (q >> 1) & 1, c = q >> 2;
+    const bool ok = (a == 0 || tx.two) && (b == 0 || ty.two) && (c == 0 || tz.two);
+    const int vid = tx.v[a] + g.nv[0] * (ty.v[b] + g.nv[1] * tz.v[c]);
+    v[q] = ok ? sc[vid * NS + comp * SN + tx.o[a] + S1 * ty.o[b] + S1 * S1 * tz.o[c]] : T(0);
+  }
+  T acc = v[0];
+#pragma unroll
+  for (int q = 1; q < 8; ++q) acc += v[q];
+  return acc;
+}
+
+// a warp's sums of NPR <= 16 values a lane; lane l < NPR returns that of value l (the columns are
+// halved as the lanes are paired: 16 shuffles, where a tree per value takes 5 NPR)
+template <typename T>
+__device__ __forceinline__ T warp_moments(const T (&in)[NPR]) {
+  static_assert(NPR <= 16, "sixteen columns");
+  const int lane = threadIdx.x & 31;
+  T v[16];
+#pragma unroll
+  for (int p = 0; p < 16; ++p) v[p] = p < NPR ? in[p] : T(0);
+#pragma unroll
+  for (int w = 8; w > 0; w >>= 1) {
+    const bool up = (lane & w) != 0;
+#pragma unroll
+    for (int p = 0; p < w; ++p) {
+      const T give = up ? v[p] : v[p + w];
+      v[p] = (up ? v[p + w] : v[p]) + __shfl_xor_sync(0xffffffffu, give, w);
+    }
+  }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 16);
+}
+
+// ZP: u is formed from the star outputs sc and stored to z, each node by the cell that owns it (the
+// last cell also the upper ends).  One 12^3 three-level FP32 cycle: 1478 us, 1550 with a launch of its
+// own for the node sums, plain launches of the cells, gathers and transfers, and a shuffle tree per
+// pressure moment.
+template <typename T, int MODE, bool ZP>
 __global__ void __launch_bounds__(64 * CPB) k_qk3_cells(Geom g, CellScal<T> cs, const T* __restrict__ x,
                                                         const T* __restrict__ mu, const T* __restrict__ winv,
                                                         const T* __restrict__ p_in, T* __restrict__ p_out,
-                                                        T* __restrict__ ebuf) {
+                                                        T* __restrict__ ebuf, const T* __restrict__ sc,
+                                                        T* __restrict__ z) {
   constexpr bool RAW = (MODE & OP_RAW) != 0, VISC = (MODE & OP_VISC) != 0, AL = (MODE & OP_AL) != 0;
   constexpr bool BT = (MODE & OP_BT) != 0, BO = (MODE & OP_B) != 0;
   constexpr bool NEED_U = VISC || AL || BO, NEED_FLUX = VISC || AL || BT;
@@ -169,7 +226,22 @@ __global__ void __launch_bounds__(64 * CPB) k_qk3_cells(Geom g, CellScal<T> cs, 
   const T sx = cs.s[0], sy = cs.s[1], sz = cs.s[2];
   T(*b0)[NB] = sh.b0[w];
   T(*b1)[NB] = sh.b1[w];
-  {
+  const T m2 = (VISC && valid) ? T(2) * mu[cell * NQ + t] : T(0);
+  pdl_wait();
+  pdl_trigger();
+  if constexpr (ZP) {
+    const int i = K * cx + t0, j = K * cy + t1, k = K * cz + t2;
+    const bool in = valid && !bnd_node(g, i, j, k);
+    const bool own = valid && (t0 < K || cx == g.n[0] - 1) && (t1 < K || cy == g.n[1] - 1) && (t2 < K || cz == g.n[2] - 1);
+    T v[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) v[c] = in ? star_sum<T>(g, sc, c, i, j, k) : T(0);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      b0[c][t] = v[c];
+      if (own) z[c * (int)g.N + i + g.nn[0] * (j + g.nn[1] * k)] = v[c];
+    }
+  } else {
     const int i = K * cx + t0, j = K * cy + t1, k = K * cz + t2;
     const bool bnd = bnd_node(g, i, j, k);
     const long long nd = node_id(g, i, j, k);
@@ -235,13 +307,9 @@ __global__ void __launch_bounds__(64 * CPB) k_qk3_cells(Geom g, CellScal<T> cs, 
     // (B u)_p over the cell's 64 points: warp sums, then the two warps in a fixed order
     T bu[NPR];
 #pragma unroll
-    for (int p = 0; p < NPR; ++p) {
-      T v = -sh.wq[q] * sh.psi[q][p] * div;
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      bu[p] = v;
-    }
-    if ((t & 31) == 0)
-      for (int p = 0; p < NPR; ++p) sh.red[w][t >> 5][p] = bu[p];
+    for (int p = 0; p < NPR; ++p) bu[p] = -sh.wq[q] * sh.psi[q][p] * div;
+    const T tot = warp_moments<T>(bu);
+    if ((t & 31) < NPR) sh.red[w][t >> 5][t & 31] = tot;
     __syncthreads();
     for (int p = 0; p < NPR; ++p) bu[p] = sh.red[w][0][p] + sh.red[w][1][p];
     if (BO && valid && t == 0)
@@ -264,7 +332,6 @@ __global__ void __launch_bounds__(64 * CPB) k_qk3_cells(Geom g, CellScal<T> cs, 
     for (int p = 0; p < NPR; ++p) P += sh.psi[q][p] * p_in[cell * NPR + p];
   if (!NEED_FLUX) return;   // uniform over the block
   {
-    const T m2 = (VISC && valid) ? T(2) * mu[cell * NQ + q] : T(0);
     const T wq = sh.wq[q];
     const T sj[3] = {sx, sy, sz};
     for (int c = 0; c < 3; ++c)
@@ -371,6 +438,8 @@ template <typename T>
 __global__ void k_qk3_gather(Geom g, const T* __restrict__ ebuf, const T* __restrict__ x, T* __restrict__ y,
                              int keep_bnd, int raw) {
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_wait();
+  pdl_trigger();
   if (t >= 3u * (unsigned)g.N) return;
   y[t] = gather_value<T>(g, ebuf, x, t, keep_bnd, raw);
 }
@@ -390,6 +459,13 @@ __global__ void __launch_bounds__(RED_THREADS) k_qk3_gather_epi(Geom g, const T*
 #pragma unroll
   for (int jj = 0; jj < KMAXB; ++jj) acc[jj] = T(0);
   const unsigned n = 3 * (unsigned)g.N, t0 = blockIdx.x * (RED_THREADS * PER) + threadIdx.x;
+  // the basis columns come from kernels before the predecessor: ahead of the wait
+  T vp[PER][KMAXB];
+#pragma unroll
+  for (int q = 0; q < PER; ++q)
+#pragma unroll
+    for (int jj = 0; jj < KMAXB; ++jj)
+      vp[q][jj] = !start && jj < k && t0 + q * RED_THREADS < n ? __ldcg(V + (long long)jj * ld + t0 + q * RED_THREADS) : T(0);
   pdl_wait();
   T v[PER];
 #pragma unroll
@@ -406,25 +482,31 @@ __global__ void __launch_bounds__(RED_THREADS) k_qk3_gather_epi(Geom g, const T*
     } else {
 #pragma unroll
       for (int jj = 0; jj < KMAXB; ++jj)
-        if (jj < k && t < n) acc[jj] += __ldcg(V + (long long)jj * ld + t) * v[q];
+        if (jj < k) acc[jj] += vp[q][jj] * v[q];
     }
   }
   pdl_trigger();
   store_partials<T>(sd, start, k, acc, blockIdx.x, gridDim.x);
 }
 
+template <typename T, int MODE, bool ZP = false>
+static void launch_cells(const LevelDev& L, double gamma, const void* x, const void* p_in, void* p_out, cudaStream_t s,
+                         const void* sc = nullptr, void* z = nullptr) {
+  const T* mu = std::is_same<T, double>::value ? (const T*)L.coef64 : (const T*)L.coef32;
+  const T* winv = std::is_same<T, double>::value ? (const T*)L.winv64 : (const T*)L.winv32;
+  launch_pdl(k_qk3_cells<T, MODE, ZP>, (unsigned)((L.g.ncells + CPB - 1) / CPB), 64 * CPB, 0, s, L.g,
+             cell_scal<T>(L.g, gamma), (const T*)x, mu, winv, (const T*)p_in, (T*)p_out, (T*)L.ebuf, (const T*)sc, (T*)z);
+}
+
 template <typename T, int MODE>
 static void apply_mode(const LevelDev& L, double gamma, const void* x, void* y, const void* p_in, void* p_out,
                        cudaStream_t s) {
   constexpr bool NEED_FLUX = (MODE & (OP_VISC | OP_AL | OP_BT)) != 0;
-  const T* mu = std::is_same<T, double>::value ? (const T*)L.coef64 : (const T*)L.coef32;
-  const T* winv = std::is_same<T, double>::value ? (const T*)L.winv64 : (const T*)L.winv32;
-  k_qk3_cells<T, MODE><<<(unsigned)((L.g.ncells + CPB - 1) / CPB), 64 * CPB, 0, s>>>(
-      L.g, cell_scal<T>(L.g, gamma), (const T*)x, mu, winv, (const T*)p_in, (T*)p_out, (T*)L.ebuf);
+  launch_cells<T, MODE>(L, gamma, x, p_in, p_out, s);
   if (NEED_FLUX) {
     const int keep = ((MODE & OP_VISC) && !(MODE & OP_RAW)) ? 1 : 0;
-    k_qk3_gather<T><<<(unsigned)((3 * L.g.N + 255) / 256), 256, 0, s>>>(L.g, (const T*)L.ebuf, (const T*)x, (T*)y,
-                                                                         keep, (MODE & OP_RAW) ? 1 : 0);
+    launch_pdl(k_qk3_gather<T>, (unsigned)((3 * L.g.N + 255) / 256), 256, 0, s, L.g, (const T*)L.ebuf, (const T*)x, (T*)y,
+               keep, (MODE & OP_RAW) ? 1 : 0);
   }
   count_launch(NEED_FLUX ? 2 : 1);
 }
@@ -447,12 +529,12 @@ static void apply_t(const LevelDev& L, int mode, double gamma, const void* x, vo
 template <typename T>
 static void apply_epi_t(const LevelDev& L, double gamma, const void* x, void* y, const ApplyEpi& e, cudaStream_t s,
                         cudaEvent_t e0, cudaEvent_t e1) {
-  const T* mu = std::is_same<T, double>::value ? (const T*)L.coef64 : (const T*)L.coef32;
-  const T* winv = std::is_same<T, double>::value ? (const T*)L.winv64 : (const T*)L.winv32;
   // External records become event-record nodes when the stream is being captured
   if (e0) cudaEventRecordWithFlags(e0, s, cudaEventRecordExternal);
-  k_qk3_cells<T, OP_VISC | OP_AL><<<(unsigned)((L.g.ncells + CPB - 1) / CPB), 64 * CPB, 0, s>>>(
-      L.g, cell_scal<T>(L.g, gamma), (const T*)x, mu, winv, nullptr, nullptr, (T*)L.ebuf);
+  if (std::is_same<T, float>::value && e.pout)   // x = z formed from the star outputs; z stored on the way
+    launch_cells<float, OP_VISC | OP_AL, true>(L, gamma, nullptr, nullptr, nullptr, s, e.pout, const_cast<void*>(x));
+  else
+    launch_cells<T, OP_VISC | OP_AL>(L, gamma, x, nullptr, nullptr, s);
   if (e1) cudaEventRecordWithFlags(e1, s, cudaEventRecordExternal);
   const auto kernel = qk_epi_per(L) == 1 ? k_qk3_gather_epi<T, 1> : k_qk3_gather_epi<T, kEpiPer>;
   launch_pdl(kernel, qk_epi_blocks(L), RED_THREADS, 0, s, L.g, (const T*)L.ebuf, (const T*)x, (T*)y, (const T*)e.b,
@@ -1281,19 +1363,6 @@ __global__ void __launch_bounds__(256) k_qk3_pack(Geom g, int pstride, int nint,
   }
 }
 
-// the vertices whose stars contain lattice index i (|i - 3v| <= 2), two taps: v0 = i / 3, then
-// v0 + 1 unless i = 3 v0; o: offset index in the star, 0 .. S1 - 1
-struct StarTaps {
-  int v[2], o[2];
-  bool two;
-  __device__ __forceinline__ explicit StarTaps(int i) {
-    const int v0 = i / K, r = i - K * v0;
-    v[0] = v0; o[0] = r + K - 1;
-    v[1] = v0 + 1; o[1] = r - 1;
-    two = r != 0;
-  }
-};
-
 // z(node) = sum over the (up to 8) stars containing the node, fixed order; 0 at Dirichlet nodes
 template <typename T>
 __global__ void k_qk3_star_gather(Geom g, const T* __restrict__ sc, T* __restrict__ z) {
@@ -1303,20 +1372,7 @@ __global__ void k_qk3_star_gather(Geom g, const T* __restrict__ sc, T* __restric
     int comp, i, j, k;
     entry_coords(g, t, comp, i, j, k);
     T acc = T(0);
-    if (!bnd_node(g, i, j, k)) {
-      const StarTaps tx(i), ty(j), tz(k);
-      T v[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int a = q & 1, b = (q >> 1) & 1, c = q >> 2;
-        const bool ok = (a == 0 || tx.two) && (b == 0 || ty.two) && (c == 0 || tz.two);
-        const int vid = tx.v[a] + g.nv[0] * (ty.v[b] + g.nv[1] * tz.v[c]);
-        v[q] = ok ? sc[vid * NS + comp * SN + tx.o[a] + S1 * ty.o[b] + S1 * S1 * tz.o[c]] : T(0);
-      }
-      acc = v[0];
-#pragma unroll
-      for (int q = 1; q < 8; ++q) acc += v[q];
-    }
+    if (!bnd_node(g, i, j, k)) acc = star_sum<T>(g, sc, comp, i, j, k);
     z[t] = acc;
   }
   pdl_trigger();
@@ -1345,6 +1401,8 @@ __global__ void __launch_bounds__(128) k_qk3_prolong_cells(Geom gc, Geom gf, con
   const int cx = (int)(cell % gc.n[0]), cy = (int)((cell / gc.n[0]) % gc.n[1]),
             cz = (int)(cell / ((long long)gc.n[0] * gc.n[1]));
   if (tid < NF * N1) pw[tid / N1][tid % N1] = Tab<T>::pw(tid / N1, tid % N1);
+  pdl_wait();
+  pdl_trigger();
   for (int e = tid; e < 3 * NB; e += nt) {
     const int c = e / NB, a = e % NB;
     const int I = K * cx + a % N1, J = K * cy + (a / N1) % N1, Kz = K * cz + a / (N1 * N1);
@@ -1404,6 +1462,8 @@ __global__ void __launch_bounds__(RS_THREADS) k_qk3_restrict_cells(Geom gc, Geom
   const int cx = (int)(cell % gc.n[0]), cy = (int)((cell / gc.n[0]) % gc.n[1]),
             cz = (int)(cell / ((long long)gc.n[0] * gc.n[1]));
   if (tid < NF * N1) pw[tid / N1][tid % N1] = Tab<T>::pw(tid / N1, tid % N1);
+  pdl_wait();
+  pdl_trigger();
   for (int e = tid; e < NF * NF * NF; e += RS_THREADS) {
     const int fx = e % NF, fy = (e / NF) % NF, fz = e / (NF * NF);
     const bool own = (fx < NF - 1 || cx == gc.n[0] - 1) && (fy < NF - 1 || cy == gc.n[1] - 1) &&
@@ -1554,6 +1614,10 @@ void qk3_patch_setup(const LevelDev& L, double gamma, DevStatus* st, cudaStream_
   qk3_derive32(L, s);
 }
 
+void qk3_patch_products(const LevelDev& L, const void* r, void* scratch, cudaStream_t s) {
+  launch_stars32(L, 0, 0, (const float*)r, (float*)scratch, s);
+}
+
 void qk3_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* scratch, cudaStream_t s) {
   const unsigned b3 = (unsigned)((3 * L.g.N + 255) / 256);
   if (prec == PREC_F64) {
@@ -1583,11 +1647,11 @@ void qk3_prolong(const LevelDev& coarse, const LevelDev& fine, int prec, const v
                  void* xadd) {
   const unsigned nc = (unsigned)coarse.g.ncells;
   if (prec == PREC_F64)
-    qk3::k_qk3_prolong_cells<double><<<nc, 128, 0, s>>>(coarse.g, fine.g, (const double*)xc, (double*)xf,
-                                                        (double*)xadd);
+    launch_pdl(qk3::k_qk3_prolong_cells<double>, nc, 128, 0, s, coarse.g, fine.g, (const double*)xc, (double*)xf,
+               (double*)xadd);
   else
-    qk3::k_qk3_prolong_cells<float><<<nc, 128, 0, s>>>(coarse.g, fine.g, (const float*)xc, (float*)xf,
-                                                       (float*)xadd);
+    launch_pdl(qk3::k_qk3_prolong_cells<float>, nc, 128, 0, s, coarse.g, fine.g, (const float*)xc, (float*)xf,
+               (float*)xadd);
   count_launch(1);
 }
 
@@ -1597,13 +1661,15 @@ void qk3_restrict(const LevelDev& coarse, const LevelDev& fine, int prec, const 
                   const void* sub) {
   const unsigned nc = (unsigned)coarse.g.ncells, b = (unsigned)((3 * coarse.g.N + 255) / 256);
   if (prec == PREC_F64) {
-    qk3::k_qk3_restrict_cells<double><<<nc, qk3::RS_THREADS, 0, s>>>(coarse.g, fine.g, (const double*)rf,
-                                                                    (const double*)sub, (double*)coarse.ebuf);
-    qk3::k_qk3_gather<double><<<b, 256, 0, s>>>(coarse.g, (const double*)coarse.ebuf, nullptr, (double*)rc, 0, 0);
+    launch_pdl(qk3::k_qk3_restrict_cells<double>, nc, qk3::RS_THREADS, 0, s, coarse.g, fine.g, (const double*)rf,
+               (const double*)sub, (double*)coarse.ebuf);
+    launch_pdl(qk3::k_qk3_gather<double>, b, 256, 0, s, coarse.g, (const double*)coarse.ebuf, (const double*)nullptr,
+               (double*)rc, 0, 0);
   } else {
-    qk3::k_qk3_restrict_cells<float><<<nc, qk3::RS_THREADS, 0, s>>>(coarse.g, fine.g, (const float*)rf,
-                                                                   (const float*)sub, (float*)coarse.ebuf);
-    qk3::k_qk3_gather<float><<<b, 256, 0, s>>>(coarse.g, (const float*)coarse.ebuf, nullptr, (float*)rc, 0, 0);
+    launch_pdl(qk3::k_qk3_restrict_cells<float>, nc, qk3::RS_THREADS, 0, s, coarse.g, fine.g, (const float*)rf,
+               (const float*)sub, (float*)coarse.ebuf);
+    launch_pdl(qk3::k_qk3_gather<float>, b, 256, 0, s, coarse.g, (const float*)coarse.ebuf, (const float*)nullptr,
+               (float*)rc, 0, 0);
   }
   count_launch(2);
 }
