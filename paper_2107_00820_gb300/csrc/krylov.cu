@@ -243,9 +243,10 @@ __global__ void __launch_bounds__(RED_THREADS) k_gm_start(unsigned n, const T* _
 // Every block adds the partials of the dots (and of |V_j|^2, before the wait: the kernel that
 // wrote them is three launches back) for itself.  The last block is an extra one: it does the
 // one-thread bookkeeping of step j - 1 while the others work.
-template <typename T>
-__device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned n, int j, const T* __restrict__ V,
+template <typename T, int KC>
+__device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned n, const T* __restrict__ V,
                                              long long ld, const GmresDev& sd) {
+  constexpr int j = KC - 1;
   __shared__ T sh[RED_THREADS / 32][KMAXB];
   __shared__ T coef[KMAXB];
   __shared__ T nrm2;
@@ -255,7 +256,7 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
   const unsigned base = bx * (RED_THREADS * GM_PER) + threadIdx.x;
   T* w = const_cast<T*>(V) + (long long)(j + 1) * ld;
   T a[GM_PER];
-  T vc[GM_PER][KMAXB];
+  T vc[GM_PER][KC];
   T rhni = T(0);
   if (sd.late) pdl_wait();   // column j, its norm and rhn come from the predecessor too
   // columns 0..j, rhn and the norm partials come from earlier kernels of the chain (complete
@@ -266,7 +267,7 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
     for (int q = 0; q < GM_PER; ++q) {
       const unsigned i = base + q * RED_THREADS;
 #pragma unroll
-      for (int c = 0; c < KMAXB; ++c) vc[q][c] = (i < n && c <= j) ? __ldcg(V + (long long)c * ld + i) : T(0);
+      for (int c = 0; c < KC; ++c) vc[q][c] = i < n ? __ldcg(V + (long long)c * ld + i) : T(0);
     }
     if ((int)threadIdx.x < j) rhni = __ldcg(st.rhn + threadIdx.x);
   }
@@ -310,8 +311,7 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
     const unsigned i = base + q * RED_THREADS;
     a[q] *= inv;
 #pragma unroll
-    for (int c = 0; c < KMAXB; ++c)
-      if (c <= j) a[q] -= vc[q][c] * coef[c];
+    for (int c = 0; c < KC; ++c) a[q] -= vc[q][c] * coef[c];
     if (i < n) w[i] = a[q];
     acc[0] += a[q] * a[q];
   }
@@ -319,18 +319,18 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
   const T v = block_total<T>(acc, 1, sh);
   if (threadIdx.x == 0) norm_rows<T>(sd, j + 1)[bx] = v;
 }
-template <typename T>
-__global__ void __launch_bounds__(RED_THREADS) k_gm_orth(unsigned n, int j, const T* __restrict__ V, long long ld,
+template <typename T, int KC>
+__global__ void __launch_bounds__(RED_THREADS) k_gm_orth(unsigned n, const T* __restrict__ V, long long ld,
                                                          GmresDev sd) {
-  gm_orth_body<T>(blockIdx.x, gridDim.x, n, j, V, ld, sd);
+  gm_orth_body<T, KC>(blockIdx.x, gridDim.x, n, V, ld, sd);
 }
 
 // x = (x_zero ? 0 : x) + sum_j Z_j y_j / hn_j with y = R^-1 g, and, if t != NULL, the
 // GMRES residual  t = r0 - A Z y = sum_i u_i v_i,  u = Q^T (g[k] e_k)  from the
 // Arnoldi relation (Q = product of the Givens rotations), no operator apply.  Every block
 // finishes the last Givens step and forms y and u for itself, on a copy of the state.
-template <typename T>
-__device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, int k, const T* __restrict__ Z,
+template <typename T, int k>
+__device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, const T* __restrict__ Z,
                                                const T* __restrict__ V, long long ld, const GmresDev& sd,
                                                T* __restrict__ x, int x_zero, T* __restrict__ t) {
   __shared__ T sh[RED_THREADS / 32][KMAXB];
@@ -343,12 +343,12 @@ __device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, int k, c
   // Z, x and V_0..V_{k-1} come from earlier kernels of the chain (complete before this
   // launch began): read through L2 before the wait; V_k, its norm and the last column of H
   // come from the predecessor (the last Gram-Schmidt step)
-  T zc[GM_PER][KMAXB], xa[GM_PER];
+  T zc[GM_PER][k], xa[GM_PER];
 #pragma unroll
   for (int q = 0; q < GM_PER; ++q) {
     const unsigned i = base + q * RED_THREADS;
 #pragma unroll
-    for (int c = 0; c < KMAXB; ++c) zc[q][c] = (i < n && c < k) ? __ldcg(Z + (long long)c * ld + i) : T(0);
+    for (int c = 0; c < k; ++c) zc[q][c] = i < n ? __ldcg(Z + (long long)c * ld + i) : T(0);
     xa[q] = (i < n && !x_zero) ? __ldcg(x + i) : T(0);
   }
   pdl_wait();
@@ -370,8 +370,7 @@ __device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, int k, c
     if (i >= n) break;
     T a = xa[q];
 #pragma unroll
-    for (int c = 0; c < KMAXB; ++c)
-      if (c < k) a += zc[q][c] * y[c];
+    for (int c = 0; c < k; ++c) a += zc[q][c] * y[c];
     x[i] = a;
   }
   if (t) {
@@ -379,22 +378,21 @@ __device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, int k, c
     for (int q = 0; q < GM_PER; ++q) {
       const unsigned i = base + q * RED_THREADS;
       if (i >= n) break;
-      T vc[KMAXB + 1];
+      T vc[k + 1];
 #pragma unroll
-      for (int c = 0; c <= KMAXB; ++c) vc[c] = c <= k ? V[(long long)c * ld + i] : T(0);
+      for (int c = 0; c <= k; ++c) vc[c] = V[(long long)c * ld + i];
       T r = T(0);
 #pragma unroll
-      for (int c = 0; c <= KMAXB; ++c)
-        if (c <= k) r += vc[c] * u[c];
+      for (int c = 0; c <= k; ++c) r += vc[c] * u[c];
       t[i] = r;
     }
   }
 }
-template <typename T>
-__global__ void __launch_bounds__(RED_THREADS) k_gm_update(unsigned n, int k, const T* __restrict__ Z,
+template <typename T, int K>
+__global__ void __launch_bounds__(RED_THREADS) k_gm_update(unsigned n, const T* __restrict__ Z,
                                                            const T* __restrict__ V, long long ld, GmresDev sd,
                                                            T* __restrict__ x, int x_zero, T* __restrict__ t) {
-  gm_update_body<T>(blockIdx.x, n, k, Z, V, ld, sd, x, x_zero, t);
+  gm_update_body<T, K>(blockIdx.x, n, Z, V, ld, sd, x, x_zero, t);
 }
 
 GmresDev gmres_dev(const LevelDev& L, void* state, int steps, double* partial, bool x_is_zero, bool tiled) {
@@ -413,22 +411,38 @@ void gm_start(int prec, long long n, const void* b, void* V0, const GmresDev& st
   count_launch(1);
 }
 
+// The column count is a template parameter: with arrays of KMAXB columns, predicated, a block
+// took 80 registers (three an SM) whatever it needed.
+template <typename T>
+static auto orth_kernel(int j) {
+  static constexpr decltype(&k_gm_orth<T, 1>) f[KMAXB] = {k_gm_orth<T, 1>, k_gm_orth<T, 2>, k_gm_orth<T, 3>, k_gm_orth<T, 4>,
+                                                          k_gm_orth<T, 5>, k_gm_orth<T, 6>, k_gm_orth<T, 7>, k_gm_orth<T, 8>};
+  return f[j];
+}
+template <typename T>
+static auto update_kernel(int k) {
+  static constexpr decltype(&k_gm_update<T, 1>) f[KMAXB] = {
+      k_gm_update<T, 1>, k_gm_update<T, 2>, k_gm_update<T, 3>, k_gm_update<T, 4>,
+      k_gm_update<T, 5>, k_gm_update<T, 6>, k_gm_update<T, 7>, k_gm_update<T, 8>};
+  return f[k - 1];
+}
+
 void gm_orth(int prec, long long n, int j, const void* V, long long ld, const GmresDev& st, cudaStream_t s) {
   if (prec == PREC_F64)
-    launch_pdl(k_gm_orth<double>, gm_blocks(n) + 1, RED_THREADS, 0, s, (unsigned)n, j, (const double*)V, ld, st);
+    launch_pdl(orth_kernel<double>(j), gm_blocks(n) + 1, RED_THREADS, 0, s, (unsigned)n, (const double*)V, ld, st);
   else
-    launch_pdl(k_gm_orth<float>, gm_blocks(n) + 1, RED_THREADS, 0, s, (unsigned)n, j, (const float*)V, ld, st);
+    launch_pdl(orth_kernel<float>(j), gm_blocks(n) + 1, RED_THREADS, 0, s, (unsigned)n, (const float*)V, ld, st);
   count_launch(1);
 }
 
 void gm_update(int prec, long long n, int k, const void* Z, const void* V, long long ld, const GmresDev& st,
                void* x, int x_zero, void* t, cudaStream_t s) {
   if (prec == PREC_F64)
-    launch_pdl(k_gm_update<double>, gm_blocks(n), RED_THREADS, 0, s, (unsigned)n, k, (const double*)Z, (const double*)V, ld,
-                                                               st, (double*)x, x_zero, (double*)t);
+    launch_pdl(update_kernel<double>(k), gm_blocks(n), RED_THREADS, 0, s, (unsigned)n, (const double*)Z,
+               (const double*)V, ld, st, (double*)x, x_zero, (double*)t);
   else
-    launch_pdl(k_gm_update<float>, gm_blocks(n), RED_THREADS, 0, s, (unsigned)n, k, (const float*)Z, (const float*)V, ld,
-                                                              st, (float*)x, x_zero, (float*)t);
+    launch_pdl(update_kernel<float>(k), gm_blocks(n), RED_THREADS, 0, s, (unsigned)n, (const float*)Z, (const float*)V,
+               ld, st, (float*)x, x_zero, (float*)t);
   count_launch(1);
 }
 
@@ -437,7 +451,6 @@ void gm_update(int prec, long long n, int k, const void* Z, const void* V, long 
 // ---------------------------------------------------------------------------
 struct GmArgs {
   unsigned n;
-  int j;
   const float* b;
   const float* Z;
   float* V;
@@ -453,22 +466,24 @@ __global__ void __launch_bounds__(RED_THREADS) k_gm_start_b(const __grid_constan
   const GmArgs& a = tb.a[i];
   gm_start_body<float>(blockIdx.x - tb.start[i], tb.start[i + 1] - tb.start[i], a.n, a.b, a.V, a.st);
 }
+template <int KC>
 __global__ void __launch_bounds__(RED_THREADS) k_gm_orth_b(const __grid_constant__ BatchTab<GmArgs> tb) {
   const int i = batch_slot(tb, blockIdx.x);
   const GmArgs& a = tb.a[i];
-  gm_orth_body<float>(blockIdx.x - tb.start[i], tb.start[i + 1] - tb.start[i], a.n, a.j, a.V, a.ld, a.st);
+  gm_orth_body<float, KC>(blockIdx.x - tb.start[i], tb.start[i + 1] - tb.start[i], a.n, a.V, a.ld, a.st);
 }
+template <int K>
 __global__ void __launch_bounds__(RED_THREADS) k_gm_update_b(const __grid_constant__ BatchTab<GmArgs> tb) {
   const int i = batch_slot(tb, blockIdx.x);
   const GmArgs& a = tb.a[i];
-  gm_update_body<float>(blockIdx.x - tb.start[i], a.n, a.st.s, a.Z, a.V, a.ld, a.st, a.x, a.x_zero, a.t);
+  gm_update_body<float, K>(blockIdx.x - tb.start[i], a.n, a.Z, a.V, a.ld, a.st, a.x, a.x_zero, a.t);
 }
 
 static int batch_gm(void (*k)(BatchTab<GmArgs>), const std::vector<BGmres>& items, int extra, cudaStream_t s) {
   std::vector<GmArgs> a;
   std::vector<unsigned> nb;
   for (const BGmres& it : items) {
-    a.push_back(GmArgs{(unsigned)it.n, it.j, (const float*)it.b, (const float*)it.Z, (float*)it.V, it.ld, it.st, (float*)it.x, it.x_zero, (float*)it.t});
+    a.push_back(GmArgs{(unsigned)it.n, (const float*)it.b, (const float*)it.Z, (float*)it.V, it.ld, it.st, (float*)it.x, it.x_zero, (float*)it.t});
     nb.push_back(gm_blocks(it.n) + extra);
   }
   const int n = launch_batch(k, a, nb, RED_THREADS, 0, s);
@@ -476,8 +491,18 @@ static int batch_gm(void (*k)(BatchTab<GmArgs>), const std::vector<BGmres>& item
   return n;
 }
 int batch_gm_start(const std::vector<BGmres>& items, cudaStream_t s) { return batch_gm(k_gm_start_b, items, 0, s); }
-int batch_gm_orth(const std::vector<BGmres>& items, cudaStream_t s) { return batch_gm(k_gm_orth_b, items, 1, s); }
-int batch_gm_update(const std::vector<BGmres>& items, cudaStream_t s) { return batch_gm(k_gm_update_b, items, 0, s); }
+// (the items of a merged smoothing have the same j and s)
+int batch_gm_orth(const std::vector<BGmres>& items, cudaStream_t s) {
+  static constexpr decltype(&k_gm_orth_b<1>) f[KMAXB] = {k_gm_orth_b<1>, k_gm_orth_b<2>, k_gm_orth_b<3>, k_gm_orth_b<4>,
+                                                         k_gm_orth_b<5>, k_gm_orth_b<6>, k_gm_orth_b<7>, k_gm_orth_b<8>};
+  return batch_gm(f[items[0].j], items, 1, s);
+}
+int batch_gm_update(const std::vector<BGmres>& items, cudaStream_t s) {
+  static constexpr decltype(&k_gm_update_b<1>) f[KMAXB] = {
+      k_gm_update_b<1>, k_gm_update_b<2>, k_gm_update_b<3>, k_gm_update_b<4>,
+      k_gm_update_b<5>, k_gm_update_b<6>, k_gm_update_b<7>, k_gm_update_b<8>};
+  return batch_gm(f[items[0].st.s - 1], items, 0, s);
+}
 
 // workspace of a level's fused reductions: two areas of KMAXB rows and two rows, one value per block
 size_t gmres_partial_doubles(const LevelDev& L) {

@@ -214,11 +214,14 @@ static unsigned gather_threads(const Geom& g) {
 //   y = b + sigma A x (b NULL: y = sigma A x);  block partials of V_j . y, j < k, or, start,
 //   of |y|^2.  Fixed grid and order: reproducible.
 // All sums run in T (in FP32 the GMRES state is float too, see GmresView).
-template <typename T, int DIM>
+// KC = k, or 0 for start (with arrays of KMAXB columns, predicated, a block took 80 registers, three
+// an SM, whatever it needed).
+template <typename T, int DIM, int KC>
 __device__ __forceinline__ void gather_epi_body(unsigned bx, unsigned nb, const Geom& g, const T* __restrict__ ebuf,
                                                 const T* __restrict__ x, T* __restrict__ y, const T* __restrict__ b,
-                                                double sigma, int k, const T* __restrict__ V, long long ld,
-                                                int start, const GmresDev& sd) {
+                                                double sigma, const T* __restrict__ V, long long ld,
+                                                const GmresDev& sd) {
+  constexpr bool start = KC == 0;
   T acc[KMAXB];
 #pragma unroll
   for (int j = 0; j < KMAXB; ++j) acc[j] = T(0);
@@ -227,13 +230,12 @@ __device__ __forceinline__ void gather_epi_body(unsigned bx, unsigned nb, const 
   // The basis columns come from earlier kernels of the chain, which completed before
   // this launch began (every kernel waits on its predecessor before it lets its
   // successor start): they are read through L2 while the preceding kernel finishes.
-  T vp[GX][KMAXB];
+  T vp[GX][start ? 1 : KC];
 #pragma unroll
   for (int q = 0; q < GX; ++q)
 #pragma unroll
-    for (int jj = 0; jj < KMAXB; ++jj)
-      vp[q][jj] = (!start && have && jj < k && GX * rc.j + q < g.nn[0]) ? __ldcg(V + (long long)jj * ld + rc.t0 + q)
-                                                                         : T(0);
+    for (int jj = 0; jj < KC; ++jj)
+      vp[q][jj] = have && GX * rc.j + q < g.nn[0] ? __ldcg(V + (long long)jj * ld + rc.t0 + q) : T(0);
   pdl_wait();
   if (have) {
     T ax[GX];
@@ -244,25 +246,30 @@ __device__ __forceinline__ void gather_epi_body(unsigned bx, unsigned nb, const 
       const long long t = rc.t0 + q;
       const T v = (b ? b[t] : T(0)) + (T)sigma * ax[q];
       y[t] = v;
-      if (start) {
+      if constexpr (start) {
         acc[0] += v * v;
       } else {
 #pragma unroll
-        for (int jj = 0; jj < KMAXB; ++jj)
-          if (jj < k) acc[jj] += vp[q][jj] * v;
+        for (int jj = 0; jj < KC; ++jj) acc[jj] += vp[q][jj] * v;
       }
     }
   }
   pdl_trigger();
-  store_partials<T>(sd, start, k, acc, bx, nb);
+  store_partials<T>(sd, start, KC, acc, bx, nb);
 }
-template <typename T, int DIM>
+template <typename T, int DIM, int KC>
 __global__ void __launch_bounds__(RED_THREADS) k_gather_epi(Geom g, const T* __restrict__ ebuf,
                                                             const T* __restrict__ x, T* __restrict__ y,
-                                                            const T* __restrict__ b, double sigma, int k,
-                                                            const T* __restrict__ V, long long ld, int start,
-                                                            GmresDev sd) {
-  gather_epi_body<T, DIM>(blockIdx.x, gridDim.x, g, ebuf, x, y, b, sigma, k, V, ld, start, sd);
+                                                            const T* __restrict__ b, double sigma,
+                                                            const T* __restrict__ V, long long ld, GmresDev sd) {
+  gather_epi_body<T, DIM, KC>(blockIdx.x, gridDim.x, g, ebuf, x, y, b, sigma, V, ld, sd);
+}
+template <typename T, int DIM>
+static auto gather_epi_kernel(int start, int k) {
+  static constexpr decltype(&k_gather_epi<T, DIM, 0>) f[KMAXB + 1] = {
+      k_gather_epi<T, DIM, 0>, k_gather_epi<T, DIM, 1>, k_gather_epi<T, DIM, 2>, k_gather_epi<T, DIM, 3>, k_gather_epi<T, DIM, 4>,
+      k_gather_epi<T, DIM, 5>, k_gather_epi<T, DIM, 6>, k_gather_epi<T, DIM, 7>, k_gather_epi<T, DIM, 8>};
+  return f[start ? 0 : k];
 }
 
 #include "apply_lines.cuh"
@@ -440,8 +447,8 @@ static void launch_apply_epi(const LevelDev& L, double gamma, const void* x, voi
     launch_cells<T, DIM, TENSOR, OP_VISC | OP_AL, true>(1, s, g, col, cell_const<T>(g, gamma), (const T*)x, (T*)y,
                                                          coef, nullptr, nullptr, 0, (T*)L.ebuf, winv);
   if (e1) cudaEventRecordWithFlags(e1, s, cudaEventRecordExternal);
-  launch_pdl(k_gather_epi<T, DIM>, apply_epi_blocks(L), RED_THREADS, 0, s, g, (const T*)L.ebuf, (const T*)x, (T*)y,
-             (const T*)e.b, e.sigma, e.k, (const T*)e.V, e.ld, e.start, e.st);
+  launch_pdl(gather_epi_kernel<T, DIM>(e.start, e.k), apply_epi_blocks(L), RED_THREADS, 0, s, g, (const T*)L.ebuf,
+             (const T*)x, (T*)y, (const T*)e.b, e.sigma, (const T*)e.V, e.ld, e.st);
   count_launch(2);
 }
 
@@ -522,19 +529,20 @@ struct GatherArgs {
   float* y;
   const float* b;
   double sigma;
-  int k, start, keep_bnd;
+  int keep_bnd;
   const float* V;
   long long ld;
   GmresDev st;
 };
+template <int KC>
 __global__ void __launch_bounds__(RED_THREADS) k_gather_epi_b(const __grid_constant__ BatchTab<GatherArgs> tb) {
   const int i = batch_slot(tb, blockIdx.x);
   const GatherArgs& a = tb.a[i];
   const unsigned bx = blockIdx.x - tb.start[i], nb = tb.start[i + 1] - tb.start[i];
   if (a.g.dim == 3)
-    gather_epi_body<float, 3>(bx, nb, a.g, a.ebuf, a.x, a.y, a.b, a.sigma, a.k, a.V, a.ld, a.start, a.st);
+    gather_epi_body<float, 3, KC>(bx, nb, a.g, a.ebuf, a.x, a.y, a.b, a.sigma, a.V, a.ld, a.st);
   else
-    gather_epi_body<float, 2>(bx, nb, a.g, a.ebuf, a.x, a.y, a.b, a.sigma, a.k, a.V, a.ld, a.start, a.st);
+    gather_epi_body<float, 2, KC>(bx, nb, a.g, a.ebuf, a.x, a.y, a.b, a.sigma, a.V, a.ld, a.st);
 }
 __global__ void __launch_bounds__(256) k_gather_cells_b(const __grid_constant__ BatchTab<GatherArgs> tb) {
   const int i = batch_slot(tb, blockIdx.x);
@@ -588,10 +596,13 @@ int batch_apply_epi(const std::vector<BApply>& items, cudaStream_t s) {
   for (const BApply& it : items) {
     const LevelDev& L = *it.L;
     a.push_back(GatherArgs{L.g, (const float*)L.ebuf, (const float*)it.x, (float*)it.y, (const float*)it.e.b,
-                           it.e.sigma, it.e.k, it.e.start, 1, (const float*)it.e.V, it.e.ld, it.e.st});
+                           it.e.sigma, 1, (const float*)it.e.V, it.e.ld, it.e.st});
     nb.push_back(apply_epi_blocks(L));
   }
-  n += launch_batch(k_gather_epi_b, a, nb, RED_THREADS, 0, s);
+  static constexpr decltype(&k_gather_epi_b<0>) f[KMAXB + 1] = {
+      k_gather_epi_b<0>, k_gather_epi_b<1>, k_gather_epi_b<2>, k_gather_epi_b<3>, k_gather_epi_b<4>,
+      k_gather_epi_b<5>, k_gather_epi_b<6>, k_gather_epi_b<7>, k_gather_epi_b<8>};
+  n += launch_batch(f[items[0].e.start ? 0 : items[0].e.k], a, nb, RED_THREADS, 0, s);   // the items agree in k and start
   count_launch(n);
   return n;
 }
