@@ -1,6 +1,6 @@
 // A whole Arnoldi step of the 2D FP32 smoother in one launch.
 //
-// Included by operator.cu inside namespace als, after apply_cells.cuh.
+// Included by tiles2.cu inside namespace als, after apply_cells.cuh.
 //
 // Step j:  V_j = w / hn - sum_i V_i coef_i  (Gram-Schmidt of the previous step, see k_gm_orth),
 // Z_j = D^-1 V_j (star products and their node sums), w' = A Z_j, and the block partials of
@@ -12,7 +12,8 @@
 // the sums cross blocks, and they go through the partials of the next launch.  The stars'
 // inverses (69 KB) are copied to shared memory before the wait on the predecessor, so their
 // transfer is hidden by it.  Sums within stars, nodes and cells run in the order of the separate
-// kernels.  One cycle, us, separate / tiled: 16^2 two levels 166 / 128, 128^2 five levels 678 / 478.
+// kernels.  One cycle, us, separate / tiled: 16^2 two levels 166 / 128, 128^2 five levels
+// 678 / 478 (112 / 106 and 375 / 351 when the column loops got the length KM, after the other steps).
 //
 // w goes through two buffers in turn (a block reads its neighbours' nodes of w while others write
 // w'), and so do the partials; the last step's w' goes to column s for k_gm_orth.
@@ -58,17 +59,18 @@ struct Tile2 {
 __host__ __device__ __forceinline__ int tiles2_x(const Geom& g) { return (g.n[0] + 7) >> 3; }
 __host__ __device__ __forceinline__ int tiles2(const Geom& g) { return tiles2_x(g) * ((g.n[1] + 7) >> 3); }
 
-template <typename TS, bool TENSOR>
+// KM: the most columns before column j that this instance handles (the column loops are of that length)
+template <typename TS, bool TENSOR, int KM>
 __device__ __forceinline__ void arnoldi2_body(unsigned bx, const ArnoldiArgs& a, unsigned char* smraw) {
   using C = Tile2<TS>;
   constexpr int T = C::T, W = C::W;
   __shared__ float sh[RED_THREADS / 32][KMAXB];
-  __shared__ float coef[KMAXB], s_inv, s_nrm2;
+  __shared__ float coef[KMAXB], s_inv;
   __shared__ int s_fail;
   const Geom& g = a.g;
   const GmresDev& sd = a.st;
   const GmresView<float> st = gmres_view<float>(sd);
-  const int j = a.j, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int j = KM == 0 ? 0 : a.j, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tx = tiles2_x(g), ntiles = tiles2(g);
   float acc[KMAXB];
   if ((int)bx == ntiles) {   // the bookkeeping block
@@ -151,40 +153,41 @@ __device__ __forceinline__ void arnoldi2_body(unsigned bx, const ArnoldiArgs& a,
     in[q] = there && x > 0 && x < g.nn[0] - 1 && y > 0 && y < g.nn[1] - 1;
   }
   // columns 0 .. j-2 come from kernels before the predecessor (complete before this launch began)
-  float vc[4][KMAXB];
+  constexpr int KA = KM > 0 ? KM : 1;
+  float vc[4][KA];
 #pragma unroll
   for (int q = 0; q < 4; ++q)
 #pragma unroll
-    for (int c = 0; c < KMAXB - 1; ++c) vc[q][c] = c < j - 1 && at[q] >= 0 ? __ldcg(a.V + (long long)c * a.ld + at[q]) : 0.f;
+    for (int c = 0; c < KM; ++c) vc[q][c] = c < j - 1 && at[q] >= 0 ? __ldcg(a.V + (long long)c * a.ld + at[q]) : 0.f;
   pdl_wait();
   pdl_trigger();
   // everything that the predecessor wrote is loaded at once: w, V_{j-1}, the partials (the first 256
   // blocks' here), 1 / hn
-  float val[4], d[KMAXB], dn = 0.f, rh = 0.f;
+  float val[4], d[KA], dn = 0.f, rh = 0.f;
 #pragma unroll
   for (int q = 0; q < 4; ++q) val[q] = at[q] >= 0 ? __ldcg(a.src + at[q]) : 0.f;
   if (j > 0) {
     const float *rows = dot_rows<float>(sd, j - 1), *nrows = norm_rows<float>(sd, j - 1);
     const int nbn = norm_count(sd, j - 1, a.ld);
 #pragma unroll
-    for (int c = 0; c < KMAXB - 1; ++c) d[c] = c < j && tid < sd.nbd ? __ldcg(rows + c * sd.nbd + tid) : 0.f;
+    for (int c = 0; c < KM; ++c) d[c] = c < j && tid < sd.nbd ? __ldcg(rows + c * sd.nbd + tid) : 0.f;
     if (tid < nbn) dn = __ldcg(nrows + tid);
     if (lane < j - 1) rh = __ldcg(st.rhn + lane);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const float last = at[q] >= 0 ? __ldcg(a.V + (long long)(j - 1) * a.ld + at[q]) : 0.f;
 #pragma unroll
-      for (int c = 0; c < KMAXB - 1; ++c)
+      for (int c = 0; c < KM; ++c)
         if (c == j - 1) vc[q][c] = last;
     }
     for (int b = tid + RED_THREADS; b < max(sd.nbd, nbn); b += RED_THREADS) {
 #pragma unroll
-      for (int c = 0; c < KMAXB - 1; ++c)
+      for (int c = 0; c < KM; ++c)
         if (c < j && b < sd.nbd) d[c] += __ldcg(rows + c * sd.nbd + b);
       if (b < nbn) dn += __ldcg(nrows + b);
     }
 #pragma unroll
-    for (int c = 0; c < KMAXB; ++c) acc[c] = c == j ? dn : c < KMAXB - 1 ? d[c] : 0.f;
+    for (int c = 0; c < KMAXB; ++c) acc[c] = c == j ? dn : c < KM ? d[c < KM ? c : 0] : 0.f;
     const float v = block_total<float>(acc, j + 1, sh);
     if (warp == 0) {
       const float inv = recip_or_zero<float>(sqrtf(fmaxf(__shfl_sync(0xffffffffu, v, j), 0.f)));
@@ -204,7 +207,7 @@ __device__ __forceinline__ void arnoldi2_body(unsigned bx, const ArnoldiArgs& a,
     for (int q = 0; q < 4; ++q) {
       val[q] *= inv;
 #pragma unroll
-      for (int c = 0; c < KMAXB - 1; ++c)
+      for (int c = 0; c < KM; ++c)
         if (c < j) val[q] -= vc[q][c] * coef[c];
     }
   }
@@ -258,11 +261,11 @@ __device__ __forceinline__ void arnoldi2_body(unsigned bx, const ArnoldiArgs& a,
     }
   }
   // the older columns at the own nodes, for the dots: in flight over the cells
-  float vd[2][KMAXB];
+  float vd[2][KA];
 #pragma unroll
   for (int q = 0; q < 2; ++q)
 #pragma unroll
-    for (int c = 0; c < KMAXB - 1; ++c) vd[q][c] = c < j && own[q] ? __ldcg(a.V + (long long)c * a.ld + at[q]) : 0.f;
+    for (int c = 0; c < KM; ++c) vd[q][c] = c < j && own[q] ? __ldcg(a.V + (long long)c * a.ld + at[q]) : 0.f;
   __syncthreads();
   // cells: 16 a warp, the lanes i and i + 16 hold the components of cell i
   {
@@ -335,8 +338,8 @@ __device__ __forceinline__ void arnoldi2_body(unsigned bx, const ArnoldiArgs& a,
     a.wout[at[q]] = w;
     if (q < 2) {
 #pragma unroll
-      for (int c = 0; c < KMAXB; ++c) {
-        if (c < KMAXB - 1 && c < j) acc[c] += vd[q][c] * w;
+      for (int c = 0; c <= KM; ++c) {
+        if (c < KM && c < j) acc[c] += vd[q][c < KM ? c : 0] * w;
         if (c == j) acc[c] += val[q] * w;
       }
     }
@@ -356,16 +359,30 @@ __device__ __forceinline__ void arnoldi2_body(unsigned bx, const ArnoldiArgs& a,
   }
 }
 
-template <typename TS, bool TENSOR>
+template <typename TS, bool TENSOR, int KM>
 __global__ void __launch_bounds__(RED_THREADS, 2) k_arnoldi2(const __grid_constant__ ArnoldiArgs a) {
   extern __shared__ __align__(128) unsigned char arnoldi_smem[];
-  arnoldi2_body<TS, TENSOR>(blockIdx.x, a, arnoldi_smem);
+  arnoldi2_body<TS, TENSOR, KM>(blockIdx.x, a, arnoldi_smem);
 }
 // merged launch (batch.cuh)
+template <int KM>
 __global__ void __launch_bounds__(RED_THREADS, 2) k_arnoldi2_b(const __grid_constant__ BatchTab<ArnoldiArgs> tb) {
   extern __shared__ __align__(128) unsigned char arnoldi_smem[];
   const int i = batch_slot(tb, blockIdx.x);
-  arnoldi2_body<float, false>(blockIdx.x - tb.start[i], tb.a[i], arnoldi_smem);
+  arnoldi2_body<float, false, KM>(blockIdx.x - tb.start[i], tb.a[i], arnoldi_smem);
+}
+// the instance for step j: KM = 0, 2, 4 or 7
+constexpr int kArnoldiKM = 4;
+static int arnoldi_km(int j) { return j == 0 ? 0 : j <= 2 ? 1 : j <= 4 ? 2 : 3; }
+template <typename TS, bool TENSOR>
+static auto arnoldi_kernel(int i) {
+  static constexpr decltype(&k_arnoldi2<TS, TENSOR, 0>) f[kArnoldiKM] = {
+      k_arnoldi2<TS, TENSOR, 0>, k_arnoldi2<TS, TENSOR, 2>, k_arnoldi2<TS, TENSOR, 4>, k_arnoldi2<TS, TENSOR, 7>};
+  return f[i];
+}
+static auto arnoldi_kernel_b(int i) {
+  static constexpr decltype(&k_arnoldi2_b<0>) f[kArnoldiKM] = {k_arnoldi2_b<0>, k_arnoldi2_b<2>, k_arnoldi2_b<4>, k_arnoldi2_b<7>};
+  return f[i];
 }
 
 // Which levels take their Arnoldi steps tiled: 2D, order 2, FP32, every vertex's inverse in one
@@ -397,23 +414,26 @@ static ArnoldiArgs arnoldi_args(const LevelDev& L, double gamma, const ArnoldiSt
 void arnoldi_prepare() {
   const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
   const int f = (int)Tile2<float>::smem, h = (int)Tile2<__nv_bfloat16>::smem;
-  cudaFuncSetAttribute(k_arnoldi2<float, false>, at, f);
-  cudaFuncSetAttribute(k_arnoldi2<float, true>, at, f);
-  cudaFuncSetAttribute(k_arnoldi2<__nv_bfloat16, false>, at, h);
-  cudaFuncSetAttribute(k_arnoldi2<__nv_bfloat16, true>, at, h);
-  cudaFuncSetAttribute(k_arnoldi2_b, at, f);
+  for (int i = 0; i < kArnoldiKM; ++i) {
+    cudaFuncSetAttribute(arnoldi_kernel<float, false>(i), at, f);
+    cudaFuncSetAttribute(arnoldi_kernel<float, true>(i), at, f);
+    cudaFuncSetAttribute(arnoldi_kernel<__nv_bfloat16, false>(i), at, h);
+    cudaFuncSetAttribute(arnoldi_kernel<__nv_bfloat16, true>(i), at, h);
+    cudaFuncSetAttribute(arnoldi_kernel_b(i), at, f);
+  }
 }
 
 void arnoldi_step(const LevelDev& L, double gamma, const ArnoldiStep& e, cudaStream_t s) {
   const ArnoldiArgs a = arnoldi_args(L, gamma, e);
   const unsigned blocks = (unsigned)(tiles2(L.g) + (e.j > 0 ? 1 : 0));
   const size_t f = Tile2<float>::smem, h = Tile2<__nv_bfloat16>::smem;
+  const int i = arnoldi_km(e.j);
   if (L.inv16) {
-    if (L.tensor) launch_pdl(k_arnoldi2<__nv_bfloat16, true>, blocks, RED_THREADS, h, s, a);
-    else launch_pdl(k_arnoldi2<__nv_bfloat16, false>, blocks, RED_THREADS, h, s, a);
+    if (L.tensor) launch_pdl(arnoldi_kernel<__nv_bfloat16, true>(i), blocks, RED_THREADS, h, s, a);
+    else launch_pdl(arnoldi_kernel<__nv_bfloat16, false>(i), blocks, RED_THREADS, h, s, a);
   } else {
-    if (L.tensor) launch_pdl(k_arnoldi2<float, true>, blocks, RED_THREADS, f, s, a);
-    else launch_pdl(k_arnoldi2<float, false>, blocks, RED_THREADS, f, s, a);
+    if (L.tensor) launch_pdl(arnoldi_kernel<float, true>(i), blocks, RED_THREADS, f, s, a);
+    else launch_pdl(arnoldi_kernel<float, false>(i), blocks, RED_THREADS, f, s, a);
   }
   count_launch(1);
 }
@@ -425,7 +445,7 @@ int batch_arnoldi_step(const std::vector<BArnoldi>& items, cudaStream_t s) {
     a.push_back(arnoldi_args(*it.L, it.gamma, it.e));
     nb.push_back((unsigned)(tiles2(it.L->g) + (it.e.j > 0 ? 1 : 0)));
   }
-  const int n = launch_batch(k_arnoldi2_b, a, nb, RED_THREADS, Tile2<float>::smem, s);
+  const int n = launch_batch(arnoldi_kernel_b(arnoldi_km(items[0].e.j)), a, nb, RED_THREADS, Tile2<float>::smem, s);
   count_launch(n);
   return n;
 }

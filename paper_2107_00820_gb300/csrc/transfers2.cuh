@@ -1,7 +1,7 @@
 // Tiled 2D FP32 operations beside the Arnoldi step (arnoldi2.cuh): the residual that starts a
 // smoothing, and the robust transfers, one launch each.
 //
-// Included by operator.cu inside namespace als, after arnoldi2.cuh.
+// Included by tiles2.cu inside namespace als, after arnoldi2.cuh.
 //
 // As separate kernels a residual is two launches (cells, gather) and a transfer four (interior
 // solves, cells, gather, interpolation), each a chain of latencies with little work.  The
