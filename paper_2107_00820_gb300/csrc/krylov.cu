@@ -46,9 +46,14 @@ __global__ void k_cast(long long n, const S* __restrict__ x, D* __restrict__ y) 
 template <typename T>
 __global__ void k_scale_dev(long long n, const double* __restrict__ num, const double* __restrict__ den,
                             const T* __restrict__ x, T* __restrict__ y, int sqrt_den) {
-  const double dn = den ? (sqrt_den ? sqrt(fmax(den[0], 0.0)) : den[0]) : 1.0;
-  const double f = (num ? num[0] : 1.0);
-  const T s = (T)(dn != 0.0 ? f / dn : 0.0);
+  __shared__ T factor;   // once a block: the square root and the quotient are some 60 FP64 instructions
+  if (threadIdx.x == 0) {
+    const double dn = den ? (sqrt_den ? sqrt(fmax(den[0], 0.0)) : den[0]) : 1.0;
+    const double f = (num ? num[0] : 1.0);
+    factor = (T)(dn != 0.0 ? f / dn : 0.0);
+  }
+  __syncthreads();
+  const T s = factor;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     y[i] = s * x[i];
 }
@@ -65,7 +70,10 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return r;  // valid in thread 0
 }
 
-// out[j] = V_j . w for j < k
+// out[j] = V_j . w for j < k.  Bound by the FP64 pipe (n k / 32 warp FMAs, 60 us for 33 columns of
+// 955 k entries, against 37 us of bytes), so the blocks are few, four an SM: with 933 of them, and a shuffle
+// tree per column in each, the sums of the partials took more FP64 instructions than the
+// products, 165 us; 108 now.
 template <typename T>
 __global__ void __launch_bounds__(RED_THREADS) k_multidot(long long n, int k, const T* __restrict__ V, long long ld,
                                                           const T* __restrict__ w, double* __restrict__ partial,
@@ -155,13 +163,14 @@ void vec_zero(int prec, long long n, void* x, cudaStream_t s) {
 size_t multidot_partial_doubles(int k) { return (size_t)RED_MAX_BLOCKS * (size_t)k + 1; }
 
 static unsigned red_grid(long long n) { return red_blocks(n); }
+static unsigned dot_grid(long long n) { return std::min(red_blocks(n), 4u * 152u); }
 
 void vec_multidot(int prec, long long n, int k, const void* V, long long ld, const void* w, double* out,
                   double* partial, cudaStream_t s) {
   if (prec == PREC_F64)
-    k_multidot<double><<<red_grid(n), RED_THREADS, 0, s>>>(n, k, (const double*)V, ld, (const double*)w, partial, out);
+    k_multidot<double><<<dot_grid(n), RED_THREADS, 0, s>>>(n, k, (const double*)V, ld, (const double*)w, partial, out);
   else
-    k_multidot<float><<<red_grid(n), RED_THREADS, 0, s>>>(n, k, (const float*)V, ld, (const float*)w, partial, out);
+    k_multidot<float><<<dot_grid(n), RED_THREADS, 0, s>>>(n, k, (const float*)V, ld, (const float*)w, partial, out);
   count_launch(1);
 }
 

@@ -24,79 +24,6 @@ inline unsigned red_blocks(long long n, int per_thread = 4) {
   return (unsigned)b;
 }
 
-// block partials of kk <= KMAXB columns: warp shuffles, one shared pass, written to row[0..kk).
-// A is the accumulation type inside the block, R the type of the stored partials
-// (double by default; the FP32 smoother keeps its sums in float throughout: FP64
-// arithmetic runs at a small fraction of the FP32 rate on this GPU, with dependent
-// FP64 latencies of 60-1100 cycles).
-template <typename A, typename R = double>
-__device__ __forceinline__ void block_partials(const A (&acc)[KMAXB], int kk, R* row) {
-  __shared__ A sh[RED_THREADS / 32][KMAXB];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-  for (int j = 0; j < KMAXB; ++j) {
-    if (j >= kk) break;
-    A v = acc[j];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) sh[w][j] = v;
-  }
-  __syncthreads();
-  if ((int)threadIdx.x < kk) {
-    A v = A(0);
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) v += sh[i][threadIdx.x];
-    row[threadIdx.x] = (R)v;
-    __threadfence();   // the writers publish their partial before the block takes its ticket
-  }
-  __syncthreads();
-}
-
-// called right after block_partials (whose writers fenced their partials); nb = the
-// blocks taking part in this reduction (the grid, or an instance's share of a merged launch)
-__device__ __forceinline__ bool last_block(double* ws, unsigned nb) {
-  __shared__ bool is_last;
-  if (threadIdx.x == 0) is_last = atomicAdd(reinterpret_cast<unsigned int*>(ws), 1u) == nb - 1;
-  __syncthreads();
-  return is_last;
-}
-__device__ __forceinline__ bool last_block(double* ws) { return last_block(ws, gridDim.x); }
-
-// Run by every thread of the last block: out[j] = (sum over blocks of column j) / div[j]
-// (div NULL: no division; div[j] == 0 gives 0).  The partials (type R, rows from
-// ws + 1) are read through L2 (other blocks wrote them), each thread over a fixed
-// strided subset, then one fixed block reduction per group of KMAXB columns, in R.
-template <typename R = double>
-__device__ __forceinline__ void finish_sums_n(double* ws, int k, R* out, const R* div, int nb) {
-  if (threadIdx.x == 0) __threadfence();
-  __syncthreads();
-  const R* partial = reinterpret_cast<const R*>(ws + 1);
-  for (int j0 = 0; j0 < k; j0 += KMAXB) {
-    const int kk = (k - j0) < KMAXB ? (k - j0) : KMAXB;
-    R acc[KMAXB];
-#pragma unroll
-    for (int j = 0; j < KMAXB; ++j) acc[j] = R(0);
-#pragma unroll 4
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-#pragma unroll
-      for (int j = 0; j < KMAXB; ++j)
-        if (j < kk) acc[j] += __ldcg(partial + (long long)b * k + j0 + j);
-    }
-    __shared__ R tot[KMAXB];
-    block_partials<R, R>(acc, kk, tot);
-    if ((int)threadIdx.x < kk) {
-      const int j = j0 + threadIdx.x;
-      R v = tot[threadIdx.x];
-      if (div) v = div[j] != R(0) ? v / div[j] : R(0);
-      out[j] = v;
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *reinterpret_cast<unsigned int*>(ws) = 0u;
-}
-template <typename R = double>
-__device__ __forceinline__ void finish_sums(double* ws, int k, R* out, const R* div = nullptr) {
-  finish_sums_n<R>(ws, k, out, div, (int)gridDim.x);
-}
-
 // a warp's sums of P columns: lane l returns that of column l mod P.  The columns are halved as
 // the lanes are paired (a lane passes on the half that its partner keeps), P - 1 + log2(32 / P)
 // additions instead of 5 P.
@@ -139,6 +66,51 @@ __device__ __forceinline__ T block_total(const T (&acc)[KMAXB], int kk, T (&sh)[
     t += __shfl_xor_sync(0xffffffffu, t, 16);
   }
   return t;
+}
+
+// block partials of kk <= KMAXB columns, written to row[0..kk) and fenced
+__device__ __forceinline__ void block_partials(const double (&acc)[KMAXB], int kk, double* row) {
+  __shared__ double sh[RED_THREADS / 32][KMAXB];
+  const double v = block_total<double>(acc, kk, sh);
+  if ((int)threadIdx.x < kk) {
+    row[threadIdx.x] = v;
+    __threadfence();   // the writers publish their partial before the block takes its ticket
+  }
+  __syncthreads();
+}
+
+// called right after block_partials (whose writers fenced their partials)
+__device__ __forceinline__ bool last_block(double* ws) {
+  __shared__ bool is_last;
+  if (threadIdx.x == 0) is_last = atomicAdd(reinterpret_cast<unsigned int*>(ws), 1u) == gridDim.x - 1;
+  __syncthreads();
+  return is_last;
+}
+
+// Run by every thread of the last block: out[j] = sum over blocks of column j.  The partials (rows
+// from ws + 1) are read through L2 (other blocks wrote them), each thread over a fixed
+// strided subset, then one fixed block reduction per group of KMAXB columns.
+__device__ __forceinline__ void finish_sums(double* ws, int k, double* out) {
+  __shared__ double sh[RED_THREADS / 32][KMAXB];
+  if (threadIdx.x == 0) __threadfence();
+  __syncthreads();
+  const double* partial = ws + 1;
+  for (int j0 = 0; j0 < k; j0 += KMAXB) {
+    const int kk = (k - j0) < KMAXB ? (k - j0) : KMAXB;
+    double acc[KMAXB];
+#pragma unroll
+    for (int j = 0; j < KMAXB; ++j) acc[j] = 0.0;
+#pragma unroll 4
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += RED_THREADS) {
+#pragma unroll
+      for (int j = 0; j < KMAXB; ++j)
+        if (j < kk) acc[j] += __ldcg(partial + (long long)b * k + j0 + j);
+    }
+    const double v = block_total<double>(acc, kk, sh);
+    if ((int)threadIdx.x < kk) out[j0 + threadIdx.x] = v;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) *reinterpret_cast<unsigned int*>(ws) = 0u;
 }
 
 // acc[j] += the thread's share (blocks tid, tid + 256, ..) of column j of nb block partials
