@@ -83,6 +83,7 @@ struct als_ctx {
   std::vector<LevelDev> lev;
   CoarseDev coarse{};
   DevStatus* st = nullptr;
+  DevStatus* st_host = nullptr;        // pinned: where check_status brings *st
   double* schur = nullptr;
   MGWork w64, w32;
   // outer solve buffers (FP64), allocated on first solve
@@ -171,11 +172,9 @@ Geom make_geom(int dim, const int n[3], int order = 2) {
   return g;
 }
 
-als_status check_status(als_ctx* c, const char* stage) {
-  DevStatus h{};
-  if (cudaMemcpyAsync(&h, c->st, sizeof(h), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
-      cudaStreamSynchronize(c->stream) != cudaSuccess)
-    return cuda_check(c, stage);
+// the status that a copy on a finished stream brought to c->st_host
+als_status status_result(als_ctx* c, const char* stage) {
+  const DevStatus h = *c->st_host;
   if (h.code != 0) {
     char buf[256];
     snprintf(buf, sizeof(buf), "%s: device reported status %d at index %lld", stage, h.code, h.where);
@@ -183,6 +182,15 @@ als_status check_status(als_ctx* c, const char* stage) {
     return fail(c, (als_status)h.code, buf);
   }
   return ALS_OK;
+}
+
+// The status copy goes to pinned memory, on the stream of the work that it follows, so that one wait covers
+// both (a wait for the work, then a copy to pageable memory and its wait, took about 10 us more a call).
+als_status check_status(als_ctx* c, const char* stage) {
+  if (cudaMemcpyAsync(c->st_host, c->st, sizeof(DevStatus), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
+      cudaStreamSynchronize(c->stream) != cudaSuccess)
+    return cuda_check(c, stage);
+  return status_result(c, stage);
 }
 
 als_status alloc_work(als_ctx* c, MGWork& w, int prec) {
@@ -765,6 +773,7 @@ als_status als_destroy(als_ctx* ctx) try {
   if (ctx->prof.spare1) cudaEventDestroy(ctx->prof.spare1);
   for (void* p : ctx->allocs) cudaFree(p);
   if (ctx->host_res) cudaFreeHost(ctx->host_res);
+  if (ctx->st_host) cudaFreeHost(ctx->st_host);
   if (ctx->order_ev) cudaEventDestroy(ctx->order_ev);
   if (ctx->stream) cudaStreamDestroy(ctx->stream);
   delete ctx;
@@ -993,6 +1002,11 @@ static als_status create_impl(als_ctx* c, const als_mesh* mesh, const als_coeff*
   if (cudaEventCreateWithFlags(&c->order_ev, cudaEventDisableTiming) != cudaSuccess)
     return cuda_check(c, "event create");
   ALS_TRY(dalloc(c, &c->st, 1));
+  if (cudaMallocHost((void**)&c->st_host, sizeof(DevStatus)) != cudaSuccess) {
+    cudaGetLastError();
+    c->st_host = nullptr;
+    return fail(c, ALS_ENOMEM, "pinned status allocation failed");
+  }
   cudaMemsetAsync(c->st, 0, sizeof(DevStatus), c->stream);
   ALS_TRY(dalloc(c, &c->minbits, 1));
   const int NB = c->nq;
@@ -1178,9 +1192,9 @@ static void begin(als_ctx* c) {
 }
 
 static als_status finish(als_ctx* c, const char* what) {
-  if (cudaStreamSynchronize(c->stream) != cudaSuccess) return cuda_check(c, what);
-  ALS_TRY(cuda_check(c, what));
-  return check_status(c, what);
+  const als_status st = check_status(c, what);
+  if (st != ALS_OK) return st;
+  return cuda_check(c, what);   // a launch that was refused
 }
 
 als_status als_apply_agamma(als_ctx* c, int level, int prec, const void* x, void* y) try {
@@ -2398,26 +2412,26 @@ als_status als_batch_vcycle(als_batch* b, int prec, const void* const* bv, void*
     const cudaStream_t s = b->mstream;
     cudaEventRecord(b->ctx[0]->order_ev, b->user_stream);
     cudaStreamWaitEvent(s, b->ctx[0]->order_ev, 0);
+    std::vector<BCopy> in, out;   // every instance's vectors, and its status, in one launch each way
     for (int i = 0; i < n; ++i) {
       als_ctx* c = b->ctx[i];
       const int l = c->L - 1;
-      cudaMemcpyAsync(c->w32.b[l], bv[i], (size_t)(c->lev[l].g.N * c->dim) * 4, cudaMemcpyDeviceToDevice, s);
+      const long long len = c->lev[l].g.N * c->dim;
+      in.push_back(BCopy{bv[i], c->w32.b[l], len, nullptr, nullptr});
+      out.push_back(BCopy{c->w32.x[l], xv[i], len, c->st, c->st_host});
     }
+    batch_copy(in, s);
     const als_status st = batch_plan(b);   // first call: groupings built and timed (the cycle reads b only)
     if (st != ALS_OK) return st;
     if (cudaGraphLaunch(b->plan.exec, s) != cudaSuccess) return batch_fail(b, ALS_ECUDA, "merged cycle launch");
     count_launch(b->plan.kernels);
-    for (int i = 0; i < n; ++i) {
-      als_ctx* c = b->ctx[i];
-      const int l = c->L - 1;
-      cudaMemcpyAsync(xv[i], c->w32.x[l], (size_t)(c->lev[l].g.N * c->dim) * 4, cudaMemcpyDeviceToDevice, s);
-    }
+    batch_copy(out, s);
     if (cudaStreamSynchronize(s) != cudaSuccess) {
       const cudaError_t e = cudaGetLastError();
       return batch_fail(b, ALS_ECUDA, std::string("merged cycle: ") + cudaGetErrorString(e));
     }
     for (int i = 0; i < n; ++i) {
-      const als_status cs = check_status(b->ctx[i], "merged cycle");
+      const als_status cs = status_result(b->ctx[i], "merged cycle");
       if (cs != ALS_OK) return batch_fail(b, cs, "instance " + std::to_string(i) + ": " + b->ctx[i]->err);
     }
     return ALS_OK;
@@ -2468,6 +2482,7 @@ als_status als_batch_vcycle(als_batch* b, int prec, const void* const* bv, void*
     const int l = c->L - 1;
     kernels += w.graph_kernels;
     cudaMemcpyAsync(xv[i], w.x[l], (size_t)(c->lev[l].g.N * c->dim) * w.es, cudaMemcpyDeviceToDevice, s);
+    cudaMemcpyAsync(c->st_host, c->st, sizeof(DevStatus), cudaMemcpyDeviceToHost, s);
   }
   count_launch(kernels);
   if (cudaStreamSynchronize(s) != cudaSuccess) {
@@ -2475,7 +2490,7 @@ als_status als_batch_vcycle(als_batch* b, int prec, const void* const* bv, void*
     return batch_fail(b, ALS_ECUDA, std::string("batch cycle: ") + cudaGetErrorString(e));
   }
   for (int i = 0; i < n; ++i) {
-    const als_status st = check_status(b->ctx[i], "batch cycle");
+    const als_status st = status_result(b->ctx[i], "batch cycle");
     if (st != ALS_OK) return batch_fail(b, st, b->ctx[i]->err);
   }
   return ALS_OK;

@@ -42,10 +42,11 @@ __device__ __forceinline__ int batch_slot(const BatchTab<A>& t, unsigned b) {
 }
 
 // One merged launch per group of at most kBatchMax items: items[i] gets blocks[i]
-// blocks (items with none are left out).  Returns the number of launches.
+// blocks (items with none are left out); pdl: a programmatic launch, for kernels that wait
+// on their predecessor.  Returns the number of launches.
 template <typename A>
 int launch_batch(void (*kernel)(BatchTab<A>), const std::vector<A>& items, const std::vector<unsigned>& blocks,
-                 unsigned threads, size_t smem, cudaStream_t s) {
+                 unsigned threads, size_t smem, cudaStream_t s, bool pdl = true) {
   static_assert(sizeof(BatchTab<A>) <= 32000, "merged-launch table exceeds the kernel parameter space");
   int launches = 0;
   BatchTab<A>* t = new BatchTab<A>();
@@ -62,7 +63,8 @@ int launch_batch(void (*kernel)(BatchTab<A>), const std::vector<A>& items, const
     }
     t->start[t->count] = total;
     if (t->count == 0) continue;
-    launch_pdl(kernel, total, threads, smem, s, *t);
+    if (pdl) launch_pdl(kernel, total, threads, smem, s, *t);
+    else kernel<<<total, threads, smem, s>>>(*t);
     ++launches;
   }
   delete t;

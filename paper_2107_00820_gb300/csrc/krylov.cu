@@ -488,6 +488,36 @@ __global__ void __launch_bounds__(RED_THREADS) k_gm_update_b(const __grid_consta
   gm_update_body<float, K>(blockIdx.x - tb.start[i], a.n, a.Z, a.V, a.ld, a.st, a.x, a.x_zero, a.t);
 }
 
+// Copies of float vectors, and of the instances' statuses to pinned host memory
+struct CopyArgs {
+  const float* src;
+  float* dst;
+  unsigned n;
+  const DevStatus* st;
+  DevStatus* st_host;
+};
+__global__ void __launch_bounds__(256) k_copy_b(const __grid_constant__ BatchTab<CopyArgs> tb) {
+  const int i = batch_slot(tb, blockIdx.x);
+  const CopyArgs& a = tb.a[i];
+  const unsigned b = blockIdx.x - tb.start[i], e = b * 1024u + threadIdx.x;
+  float v[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) v[q] = e + 256u * q < a.n ? a.src[e + 256u * q] : 0.f;
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (e + 256u * q < a.n) a.dst[e + 256u * q] = v[q];
+  if (a.st && b == 0 && threadIdx.x == 0) *a.st_host = *a.st;
+}
+int batch_copy(const std::vector<BCopy>& items, cudaStream_t s) {
+  std::vector<CopyArgs> a;
+  std::vector<unsigned> nb;
+  for (const BCopy& it : items) {
+    a.push_back(CopyArgs{(const float*)it.src, (float*)it.dst, (unsigned)it.n, it.st, it.st_host});
+    nb.push_back((unsigned)((it.n + 1023) / 1024));
+  }
+  return launch_batch(k_copy_b, a, nb, 256, 0, s, false);
+}
+
 static int batch_gm(void (*k)(BatchTab<GmArgs>), const std::vector<BGmres>& items, int extra, cudaStream_t s) {
   std::vector<GmArgs> a;
   std::vector<unsigned> nb;

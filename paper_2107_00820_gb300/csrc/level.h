@@ -303,6 +303,14 @@ struct BGmres {            // gm_start (b, V), gm_orth (V, j), gm_update (Z, V, 
   int x_zero;
   void* t;
 };
+struct BCopy {
+  const void* src;         // n floats
+  void* dst;
+  long long n;
+  const DevStatus* st;     // with it, the instance's status to pinned memory
+  DevStatus* st_host;
+};
+int batch_copy(const std::vector<BCopy>& items, cudaStream_t s);   // launches; not counted as kernels of the work
 struct BArnoldi {
   const LevelDev* L;
   double gamma;
