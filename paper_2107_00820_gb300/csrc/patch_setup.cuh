@@ -29,14 +29,16 @@ struct SetupCfg {
   static constexpr int NP = Sz<DIM>::NP, NB = Sz<DIM>::NB, NPR = Sz<DIM>::NPR;
   static constexpr int NM = Sz<DIM>::NM, NC = Sz<DIM>::NC, NSUB = 1 << DIM;
   static constexpr int NPK = NP * (NP + 1) / 2;
-  // shared doubles: M | pk | qk | gt | bt | wq | wpsi | T, then the row index of every packed entry
-  static constexpr int n_M = NPK, n_pk = NP, n_qk = NP, n_gt = NB * NB * DIM, n_bt = NPR * DIM * NB;
+  // shared doubles: M | gt | bt | wq | wpsi | T
+  static constexpr int n_M = NPK, n_gt = NB * NB * DIM, n_bt = NPR * DIM * NB;
   static constexpr int n_wq = NB * (TENSOR ? NC : 1), n_wpsi = NPR * NB;
   static constexpr int n_T = TENSOR ? NB * NSUB * DIM * NM : 0;
-  static constexpr int n_dbl = n_M + n_pk + n_qk + n_gt + n_bt + n_wq + n_wpsi + n_T;
-  static constexpr size_t smem = sizeof(double) * n_dbl + NPK;   // + uint8 row index per entry
-  static_assert(NP <= 255, "row index stored in 8 bits");
+  static constexpr int n_dbl = n_M + n_gt + n_bt + n_wq + n_wpsi + n_T;
+  static constexpr size_t smem = sizeof(double) * n_dbl;
   static constexpr int THREADS = DIM == 3 ? 256 : 128;
+  // the sweep's register tiles
+  static constexpr int TS = DIM == 3 ? 4 : 2, NBK = (NP + TS - 1) / TS, NT = NBK * (NBK + 1) / 2;
+  static_assert(NT <= THREADS && NP <= THREADS && 3 * NBK * TS <= n_gt, "a tile a thread, the columns in the place of gt");
 };
 
 // patch offset o_k and cell-local index a_k of sub-node bit b_k in a cell on side s_k
@@ -139,14 +141,11 @@ k_patch_setup(Geom g, double gamma_d, SetupGeo sg, const R* __restrict__ tab, co
   __shared__ R s_winv[NPR * NPR];
   R* sm = reinterpret_cast<R*>(sm_raw);
   R* M = sm;                         // packed upper triangle of the patch matrix, swept in place
-  R* pk = M + C::n_M;                // pivot column of the current sweep
-  R* qk = pk + C::n_pk;              // pivot column / pivot
-  R* gt = qk + C::n_qk;              // [q][a][k] physical gradient of phi_a at point q
+  R* gt = M + C::n_M;                // [q][a][k] physical gradient of phi_a at point q
   R* bt = gt + C::n_gt;              // [p][alpha][a]: B_K entries, -(psi_p, d phi_a / d x_alpha)_K
   R* wq = bt + C::n_bt;              // [q] |J| w_q mu_q, or [q][NC] |J| w_q C_q, of the current cell
   R* wpsi = wq + C::n_wq;            // [p][q] |J| w_q psi_p(q)
   R* T = wpsi + C::n_wpsi;           // tensor: [q][j][be][m] = (C_q eps(phi_b(j) e_be))_m
-  unsigned char* rowof = reinterpret_cast<unsigned char*>(sm_raw + C::n_dbl);   // row of every packed entry
   const int tid = threadIdx.x, nt = blockDim.x;
   const long long v = blockIdx.x;
   int vx, vy, vz;
@@ -155,8 +154,6 @@ k_patch_setup(Geom g, double gamma_d, SetupGeo sg, const R* __restrict__ tab, co
   const R gamma = O::from(gamma_d), gvol = O::from(sg.gvol), ir2 = O::from(0.70710678118654752440);
 
   for (int e = tid; e < C::NPK; e += nt) M[e] = zero;
-  for (int i = tid; i < NP; i += nt)
-    for (int j = i; j < NP; ++j) rowof[tri_row(NP, i) + (j - i)] = (unsigned char)i;
   for (int e = tid; e < TB::n_gt; e += nt) gt[e] = tab[e];
   for (int e = tid; e < TB::n_wpsi; e += nt) wpsi[e] = tab[TB::n_gt + e];
   for (int e = tid; e < TB::n_bt; e += nt) bt[e] = tab[TB::n_gt + TB::n_wpsi + e];
@@ -293,55 +290,107 @@ k_patch_setup(Geom g, double gamma_d, SetupGeo sg, const R* __restrict__ tab, co
   }
   __syncthreads();
 
-  // symmetric sweep of every pivot in order: M -> -A_v^-1.  Two phases per pivot:
-  // threads i < NP read the pivot column, form 1/pivot themselves (no wait on one
-  // thread) and the scaled column; then every thread updates its contiguous segment
-  // of the packed entries (row and column tracked incrementally), and threads i < NP
-  // write the pivot row/column (entries the update skips).
-  constexpr int SEG = (C::NPK + C::THREADS - 1) / C::THREADS;
-  const int e0 = tid * SEG < C::NPK ? tid * SEG : C::NPK;
-  const int e1 = e0 + SEG < C::NPK ? e0 + SEG : C::NPK;
-  const int i0 = e0 < C::NPK ? (int)rowof[e0] : NP;
-  const int j0 = e0 < C::NPK ? e0 - tri_row(NP, i0) + i0 : NP;
+  // symmetric sweep of every pivot in order: M -> -A_v^-1.  The packed entries are held in registers over
+  // all pivots, a TS x TS tile of the upper triangle a thread.  Per pivot: the tiles of its row and column
+  // put those entries into shared memory; threads i < NP read the column, form 1/pivot
+  // themselves (no wait on one thread) and the scaled column; then every thread updates its tile from TS
+  // entries of each and sets what belongs to the pivot's row and column.  Coefficient update of 32^3 cells,
+  // double-float: 24.6 ms; with the entries in shared memory, a segment of them a thread, where every update
+  // loaded, indexed and stored its entry, 27.1 ms.
+  constexpr int TS = C::TS, NBK = C::NBK, NT = C::NT;
+  R* col = gt;                 // (the assembly's tables are done with)
+  R* pc = gt + NBK * TS;
+  R* qc = pc + NBK * TS;
+  int I = 0, J = 0;
+  if (tid < NT) {
+    int rem = tid;
+    while (rem >= NBK - I) rem -= NBK - I++;
+    J = I + rem;
+  }
+  R m[TS][TS];
+#pragma unroll
+  for (int a = 0; a < TS; ++a)
+#pragma unroll
+    for (int b = 0; b < TS; ++b) {
+      const int i = I * TS + a, j = J * TS + b;
+      m[a][b] = tid < NT && i <= j && j < NP ? M[tri_row(NP, i) + (j - i)] : zero;
+    }
+  for (int e = tid; e < 3 * NBK * TS; e += nt) col[e] = zero;
+  __syncthreads();
   for (int k = 0; k < NP; ++k) {
-    R dinv = zero;
+    const int kb = k / TS, ko = k - kb * TS;
+    const bool in_col = tid < NT && J == kb, in_row = tid < NT && I == kb;
+    if (in_col) {
+#pragma unroll
+      for (int a = 0; a < TS; ++a) {
+        R v = m[a][0];
+#pragma unroll
+        for (int b = 1; b < TS; ++b)
+          if (b == ko) v = m[a][b];
+        if (I * TS + a <= k) col[I * TS + a] = v;
+      }
+    }
+    if (in_row) {
+#pragma unroll
+      for (int b = 0; b < TS; ++b) {
+        R v = m[0][b];
+#pragma unroll
+        for (int a = 1; a < TS; ++a)
+          if (a == ko) v = m[a][b];
+        if (J * TS + b > k && J * TS + b < NP) col[J * TS + b] = v;
+      }
+    }
+    __syncthreads();
     if (tid < NP) {
-      R d = M[tri_row(NP, k)];
+      R d = col[k];
       if (!(d > 0.f)) {
         if (tid == 0) report(st, 4 /* ALS_ENOTSPD */, v);
         d = one;
       }
-      dinv = one / d;
-      const int i = tid;
-      const R p = (i == k) ? zero : M[i < k ? tri_row(NP, i) + (k - i) : tri_row(NP, k) + (i - k)];
-      pk[i] = p;
-      qk[i] = p * dinv;
+      const R dinv = one / d;
+      const R p = tid == k ? zero : col[tid];
+      pc[tid] = p;
+      qc[tid] = tid == k ? -dinv : p * dinv;   // (q_k itself is 0; its place takes the pivot's new value)
     }
     __syncthreads();
-    {
-      int i = i0, j = j0;
-      R qi = i < NP ? qk[i] : zero;
-      for (int e = e0; e < e1; ++e) {
-        if (i != k && j != k) M[e] = O::sub_prod(M[e], qi, pk[j]);
-        if (++j == NP) {
-          ++i;
-          j = i;
-          if (i < NP) qi = qk[i];
-        }
+    if (tid < NT) {
+      R p[TS];
+#pragma unroll
+      for (int b = 0; b < TS; ++b) p[b] = pc[J * TS + b];
+#pragma unroll
+      for (int a = 0; a < TS; ++a) {
+        const R q = qc[I * TS + a];
+#pragma unroll
+        for (int b = 0; b < TS; ++b) m[a][b] = O::sub_prod(m[a][b], q, p[b]);
+      }
+      // row and column k: q_j, q_i and the pivot's -1 / d (all of them in qc)
+      if (in_row) {
+#pragma unroll
+        for (int a = 0; a < TS; ++a)
+          if (a == ko) {
+#pragma unroll
+            for (int b = 0; b < TS; ++b) m[a][b] = qc[J * TS + b];
+          }
+      }
+      if (in_col) {
+#pragma unroll
+        for (int b = 0; b < TS; ++b)
+          if (b == ko) {
+#pragma unroll
+            for (int a = 0; a < TS; ++a) m[a][b] = qc[I * TS + a];
+          }
       }
     }
-    if (tid < NP) {
-      const int i = tid;
-      if (i == k) M[tri_row(NP, k)] = -dinv;
-      else M[i < k ? tri_row(NP, i) + (k - i) : tri_row(NP, k) + (i - k)] = qk[i];
-    }
-    __syncthreads();
   }
   // A_v^-1 = -M, packed by diagonals in FP64 (the FP32 copies are derived from it)
-  for (int e = tid; e < C::NPK; e += nt) {
-    int t = 0;
-    while (diag_start(NP, t + 1) <= e) ++t;
-    const int i = e - diag_start(NP, t);
-    inv64[v * pstride + e] = O::to_double(-M[tri_row(NP, i) + t]);
-  }
+#pragma unroll
+  for (int a = 0; a < TS; ++a)
+#pragma unroll
+    for (int b = 0; b < TS; ++b) {
+      const int i = I * TS + a, j = J * TS + b;
+      if (tid < NT && i <= j && j < NP) M[tri_row(NP, i) + (j - i)] = m[a][b];
+    }
+  __syncthreads();
+  for (int t = tid >> 5; t < NP; t += nt >> 5)
+    for (int i = tid & 31; i < NP - t; i += 32) inv64[v * pstride + diag_start(NP, t) + i] = O::to_double(-M[tri_row(NP, i) + t]);
 }
