@@ -647,16 +647,23 @@ def ours(args, dist):
     F = pb.n
     nverts = math.prod(v + 1 for v in F)
     # split star storage on levels of >= 32768 vertices at order 2 (interior stars only in the
-    # interior-star kernel); order 3 streams every star's packed inverse in its one star kernel
+    # interior-star kernel); smaller 2D levels take a whole smoother step in one launch, which
+    # is then what is timed
     nint = math.prod(v - 1 for v in F) if (order == 2 and nverts >= 32768) else nverts
     npatch = pb.d * (2 * order - 1) ** pb.d
     packed = npatch * (npatch + 1) // 2
     if order == 2:
         bytes_per_launch = nint * (packed * 4 + npatch * 4) + nu * 4
     else:
-        # order 3 times the star products and their node gather together: packed inverse
-        # read, output rows written and read back, r read, z written
-        bytes_per_launch = nint * (packed * 4 + 2 * npatch * 4) + 2 * nu * 4
+        # order 3 times the star products: packed inverses read (3D: boundary stars hold their free
+        # dofs only, 2 of 5 offsets along an axis), output rows written, r read
+        if pb.d == 3:
+            axes = [[(v - 1, 5), (2, 2)] for v in F]
+            sizes = [(a[0] * b[0] * c[0], 3 * a[1] * b[1] * c[1]) for a in axes[0] for b in axes[1] for c in axes[2]]
+            star_bytes = sum(k * (m * (m + 1) // 2 + m) * 4 for k, m in sizes)
+        else:
+            star_bytes = nint * (packed + npatch) * 4
+        bytes_per_launch = star_bytes + nu * 4
     k4_launch_s = (k4_ms / max(k4_n, 1)) / 1e3
     achieved = bytes_per_launch / k4_launch_s / 1e9 if k4_n else None
     peak, peak_kind = measured_peak_hbm()
@@ -664,15 +671,16 @@ def ours(args, dist):
     ncells = math.prod(F)
     nq = (order + 1) ** pb.d
     ncq = (6 if pb.d == 2 else 21) if tensor else 1
-    fused = pb.d == 3 and order == 2 and os.environ.get("ALS_FUSE_GATHER", "1") != "0"
+    fused = os.environ.get("ALS_FUSE_GATHER", "1") != "0"
+    tiled = fused and pb.d == 2 and order == 2 and nverts < 32768
     if fused:
-        # the 3D smoother's cell kernel also forms Z_j from the star-patch outputs: read the
+        # the smoother's cell kernel also forms Z_j from the star-patch outputs: read the
         # patch outputs, write Z_j and the staged cell outputs, read mu or C (FP32)
         k1_bytes = nverts * npatch * 4 + nu * 4 + ncells * nq * pb.d * 4 + ncells * nq * ncq * 4
     else:
         k1_bytes = nu * 4 * 2 + ncells * nq * ncq * 4      # read x, write y, read mu or C (FP32)
     if order == 3:   # the cell kernel reads x, mu and W^-1 and stages its outputs per cell (FP32)
-        k1_bytes = nu * 4 + ncells * nq * 4 + ncells * pressure_per_cell(pb.d, 3) ** 2 * 4 + \
+        k1_bytes = (nverts * npatch * 4 + nu * 4 if fused else nu * 4) + ncells * nq * 4 + ncells * pressure_per_cell(pb.d, 3) ** 2 * 4 + \
             ncells * nq * pb.d * 4
     k1_flops = ncells * ((APPLY_FLOPS_PER_CELL_Q3 if order == 3 else APPLY_FLOPS_PER_CELL)[pb.d] +
                          (nq * 2 * 2 * ncq if tensor else 0))
@@ -688,9 +696,10 @@ def ours(args, dist):
         roofline_apply = dict(hbm if tensor else alu)
         roofline_apply.update({
             "bound": "hbm" if tensor else "alu",
-            "kernel": ("k_apply_lines (FP32 A_gamma cell kernel%s, finest level)"
-                       % (" with the fused patch gather" if fused else "")) if order == 2 else
-                      "k_qk%s_cells<float> (FP32 order-3 A_gamma cell kernel, finest level)" % ("3" if pb.d == 3 else ""),
+            "kernel": ("%s (FP32 A_gamma cell kernel%s, finest level)"
+                       % ("k_apply_cells%d" % pb.d if pb.d == 2 or (ncells >= 5000 and not tensor) else "k_apply_lines",
+                          " with the fused patch gather" if fused else "")) if order == 2 else
+                      "k_qk%s (FP32 order-3 A_gamma cell kernel, finest level)" % ("3_cells" if pb.d == 3 else "_cells2"),
             ("alu" if tensor else "hbm"): alu if tensor else hbm,
             "us_per_launch": k1_s * 1e6, "launches_timed": k1_n,
             "bytes_per_launch": k1_bytes, "flops_per_launch": k1_flops})
@@ -720,13 +729,14 @@ def ours(args, dist):
         "e2e": {"value": dist.world * dofs / t_e2e, "unit": "DoF/s", "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h},
         "roofline": {"bound": "hbm",
-                     "kernel": ("k_patch_tma<%d> (FP32 interior-star smoother, finest level)" % pb.d) if order == 2
-                     else "k_qk%s_star_apply_w + k_qk%s_star_gather<float> (FP32 order-3 star smoother, finest level)"
-                     % (("3", "3") if pb.d == 3 else ("", "")),
+                     "kernel": "k_arnoldi2 (a whole FP32 smoother step, finest level)" if tiled else
+                     ("k_patch_tma<%d> (FP32 interior-star smoother, finest level)" % pb.d) if order == 2
+                     else "k_qk%s (FP32 order-3 star products, finest level)"
+                     % ("3_stars + k_qk3_stars_bnd" if pb.d == 3 else "_star_apply_w"),
                      "achieved": achieved, "peak": peak, "peak_kind": peak_kind, "unit": "GB/s",
                      "frac": (achieved / peak) if achieved else None,
                      "bytes_per_launch": bytes_per_launch, "launches_timed": k4_n,
-                     "units": {"stars_streamed": nint, "bytes_per_star": packed * 4 + npatch * 4,
+                     "units": {"stars_streamed": nint, "bytes_per_star": (bytes_per_launch - nu * 4) / nint,
                                "r_bytes": nu * 4},
                      "traffic": stored_traffic("k_patch_apply_f32_fine", args.workload)},
         "roofline_apply": roofline_apply,

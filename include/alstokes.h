@@ -135,7 +135,7 @@ typedef struct {
                      zeta^2} in 3D; vertex stars of 5^d nodes (50 / 375 dofs) assembled in
                      FP64 and inverted in FP64, except 3D stars under the setup option's
                      double-float arithmetic (ALS_MODE_MIXED with ALS_SETUP_AUTO); 3D stars
-                     take 564 KB (FP64) + 282 KB (FP32) per vertex and about 57 M
+                     take 564 KB (FP64) + 286 KB (FP32; boundary stars less) per vertex and about 57 M
                      multiply-adds each to set up) */
   int store;      /* storage of the star inverses the FP32 cycle streams: ALS_STORE_FP32
                      (default), or ALS_STORE_BF16: the block-packed stars (every star, or the
@@ -148,7 +148,7 @@ typedef struct {
                      at DR 1e4 (2D and 3D) and, in 2D, up to DR 1e8 at gamma 1e3 (+3), but
                      the 3D 32^3 solve at DR 1e8, gamma 1e4 did not converge; with P1 it
                      costs a few iterations at DR 1e4 and does not converge from DR 1e6.
-                     Order 2, and order 3 in 3D (its wrapped FP32 rows rounded the same way;
+                     Order 2, and order 3 in 3D (its blocked FP32 stars, boundary stars too;
                      the interior solves of the FP32 transfers read them too); refused for
                      order 3 in 2D (ALS_EINVAL). */
 } als_options;
@@ -302,7 +302,9 @@ als_status als_profile_read(als_ctx* ctx, double* total_ms, long long* launches)
 /* As als_profile_read for one kernel class: kind 0 = the finest-level star-patch
  * kernel (same as als_profile_read), kind 1 = the finest-level operator-apply cell
  * kernel of the GMRES smoother steps (its node gather excluded).  Each kind
- * accumulates separately and is reset by its own read.  ALS_EINVAL for another kind. */
+ * accumulates separately and is reset by its own read.  Where a whole smoother step is
+ * one launch (2D FP32 levels below 32,768 vertices) kind 0 is that launch and kind 1
+ * stays empty.  ALS_EINVAL for another kind. */
 als_status als_profile_read_kernel(als_ctx* ctx, int kind, double* total_ms, long long* launches);
 
 /* Factor injection (tests and inspection): replace the setup's inverses by the
@@ -471,7 +473,9 @@ als_status als_batch_merged_tune(const als_batch* batch, int group, int level, i
  * a variant. */
 als_status als_autotune_info(als_ctx* ctx, int level, int* variant, float* ms);
 /* Sets the FP32 patch-kernel variant of a level (0, 1, 2 as above; -1 = tune again
- * before the next capture); the captured cycles are dropped and recaptured. */
+ * before the next capture); the captured cycles are dropped and recaptured.  The
+ * variants serve als_star_smooth and the levels whose smoother steps are separate
+ * kernels; 2D FP32 levels below 32,768 vertices take a step in one launch. */
 als_status als_set_patch_kernel(als_ctx* ctx, int level, int variant);
 
 /* Last error message of the context (never NULL; "" when none).  With ctx NULL:

@@ -1,7 +1,7 @@
 // K1: the cell apply with the 1D contractions in registers.
 //
-// Included by operator.cu inside namespace als, after apply_lines.cuh (whose 1D line functions
-// it uses).  Same arguments and results as k_apply / k_apply_lines up to the order of the sums.
+// Included by operator.cu and tiles2.cu inside namespace als, after apply_lines.cuh.  Same arguments
+// and results as k_apply_lines up to the order of the sums.
 //
 // 3D, scalar viscosity, all cells into the staged rows: one thread per (cell, velocity
 // component), 32 cells a block, a warp per component.  A thread holds its component's 27 nodal

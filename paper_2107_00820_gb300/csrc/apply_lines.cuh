@@ -1,10 +1,8 @@
 // K1, 3D: the cell apply with one lane per (component, 1D line).
 //
-// Included by operator.cu inside namespace als, after CellConst / Colour / colour_cell.  Same
-// arguments and results as k_apply<T, 3, ...>; the difference is the mapping.
-// In the point-per-lane form every lane evaluates one Gauss point and reads
-// each 1D operand from shared memory, with the 1D tables indexed by the lane's
-// runtime coordinates.  Here lane (c, a, b) owns one line of three values of
+// Included by operator.cu and tiles2.cu inside namespace als, after cell_ops.cuh.  Levels of few cells and
+// tensor coefficients take this form, larger ones that of apply_cells.cuh (cells_in_registers).
+// Lane (c, a, b) owns one line of three values of
 // velocity component c along the axis being contracted and applies the 3x3
 // tables to it in registers, so the table entries are compile-time constants
 // (zeros and ones fold away) and three shared-memory values feed six to nine

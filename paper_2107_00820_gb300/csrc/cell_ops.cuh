@@ -27,14 +27,6 @@ inline CellConst<T> cell_const(const Geom& g, double gamma) {
   return c;
 }
 
-template <typename T, int DIM>
-__device__ __forceinline__ void cell_coords(const Geom& g, long long cell, int& cx, int& cy, int& cz) {
-  cx = (int)(cell % g.n[0]);
-  long long r = cell / g.n[0];
-  cy = (int)(r % g.n[1]);
-  cz = (DIM == 3) ? (int)(r / g.n[1]) : 0;
-}
-
 // cells of one colour: index t -> (step i + bx, step j + by, step k + bz);
 // step 2 selects one parity class, step 1 (bits 0) all cells
 struct Colour {

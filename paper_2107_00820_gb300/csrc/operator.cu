@@ -1,7 +1,6 @@
 // K1: matrix-free application of the augmented Stokes operators on one level.
 //
-// One warp per cell (three in 2D) evaluates the cell's contribution with sum
-// factorisation.  The nodal sum is formed without atomics, in a fixed order so
+// The cells' contributions are evaluated with sum factorisation (apply_lines.cuh, apply_cells.cuh).  The nodal sum is formed without atomics, in a fixed order so
 // every result is bitwise reproducible: normally all cells write their local
 // outputs to a per-cell buffer and one gather kernel sums the <= 2^d values of
 // each node (two launches per apply); batched applies (many vectors at once)

@@ -13,8 +13,9 @@
 // The smoother applies z = sum_v I_v A_v^-1 I_v^T r in two deterministic steps:
 // the patch kernel computes y_v = A_v^-1 r|_v into a per-patch buffer (row layout),
 // then the <= 2^d patch values that contain a node are summed in a fixed order (no
-// floating-point atomics) by the patch gather or, in the FP32 3D smoother, by the
-// operator's cell kernel that consumes z.
+// floating-point atomics) by the patch gather or, in the GMRES smoother, by the
+// operator's cell kernel that consumes z.  (2D FP32 levels below kSplitVertices take the whole step
+// in one launch, arnoldi2.cuh.)
 #include <stdint.h>
 #include <stdlib.h>
 
