@@ -223,3 +223,25 @@ def test_q3_3d_star_ring(n):
     z1 = torch.zeros_like(z32)
     ctx.star_smooth(1, dev(r, torch.float32), z1, F32)
     assert torch.equal(z32, z1)
+
+
+# the tiled 2D cycle with tensor coefficients (C = M M^T + I / 2 at every point), and with the P2 pairing's per-cell
+# W^-1, against the FP64 cycle
+@pytest.mark.parametrize("tensor,schur", [(True, A.ALS_SCHUR_P1), (True, A.ALS_SCHUR_P2), (False, A.ALS_SCHUR_P2)])
+def test_tiled_2d_cycle_coefficients(tensor, schur):
+    n, levels = (20, 12), 3
+    if tensor:
+        rng, iu = np.random.default_rng(99), np.triu_indices(3)
+        Cs = []
+        for l in range(levels):
+            m = rng.standard_normal((n[0] * n[1] // 4 ** (levels - 1 - l), 9, 3, 3))
+            Cs.append(np.einsum("cqij,cqkj->cqik", m, m) + 0.5 * np.eye(3))
+        ctx = Context(2, n, levels, [np.ascontiguousarray(C[:, :, iu[0], iu[1]]) for C in Cs], 1.0,
+                      mu_eff=[np.ascontiguousarray(C[:, :, 0, 0] / 2) for C in Cs], schur=schur, sweeps=3)
+    else:
+        ctx = context(sinker(2, n, levels, 1.0, dr=1e2, seed=99), schur=schur, sweeps=3)
+    b = np.random.default_rng(100).standard_normal(ctx.nu()).astype(np.float32).astype(np.float64)
+    x32, x64 = _zeros(b.shape[0], F32), _zeros(b.shape[0], F64)
+    ctx.vcycle(dev(b, torch.float32), x32, F32)
+    ctx.vcycle(dev(b), x64)
+    assert rel(host(x32), host(x64)) <= 1e-4
