@@ -323,6 +323,7 @@ __device__ __forceinline__ void coarse_apply_body(unsigned bx, unsigned nb, cons
   }
   const int out = lane == 0 && r < nfree ? free_dof32(g, r) : 0;
   pdl_wait();
+  pdl_trigger();
   if (STAGE) {
     TV v[SP];
 #pragma unroll

@@ -267,7 +267,10 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
   T a[GM_PER];
   T vc[GM_PER][KC];
   T rhni = T(0);
-  if (sd.late) pdl_wait();   // column j, its norm and rhn come from the predecessor too
+  if (sd.late) {   // column j, its norm and rhn come from the predecessor too
+    pdl_wait();
+    pdl_trigger();   // (tiled levels: short blocks, few of them; 128^2 cycle 345 -> 332 us with the update's)
+  }
   // columns 0..j, rhn and the norm partials come from earlier kernels of the chain (complete
   // before this launch began): read through L2 before the wait; column j+1 and the dots come
   // from the predecessor
@@ -324,7 +327,7 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
     if (i < n) w[i] = a[q];
     acc[0] += a[q] * a[q];
   }
-  pdl_trigger();
+  if (!sd.late) pdl_trigger();
   const T v = block_total<T>(acc, 1, sh);
   if (threadIdx.x == 0) norm_rows<T>(sd, j + 1)[bx] = v;
 }
@@ -361,6 +364,7 @@ __device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, const T*
     xa[q] = (i < n && !x_zero) ? __ldcg(x + i) : T(0);
   }
   pdl_wait();
+  if (sd.late) pdl_trigger();
   if ((int)threadIdx.x < GmresLayout(k).total) state[threadIdx.x] = __ldcg(static_cast<const T*>(sd.base) + threadIdx.x);
   T acc[KMAXB];
   sum_rows<T>(norm_rows<T>(sd, k), norm_count(sd, k, n), 1, acc);
