@@ -299,6 +299,7 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
   const T inv = recip_or_zero<T>(sqrt(fmax(nrm2, T(0))));
   if ((int)threadIdx.x == j) rhni = inv;
   pdl_wait();
+  if (sd.early) pdl_trigger();
 #pragma unroll
   for (int q = 0; q < GM_PER; ++q) {
     const unsigned i = base + q * RED_THREADS;
@@ -327,7 +328,7 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
     if (i < n) w[i] = a[q];
     acc[0] += a[q] * a[q];
   }
-  if (!sd.late) pdl_trigger();
+  if (!sd.early) pdl_trigger();
   const T v = block_total<T>(acc, 1, sh);
   if (threadIdx.x == 0) norm_rows<T>(sd, j + 1)[bx] = v;
 }
@@ -364,7 +365,7 @@ __device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, const T*
     xa[q] = (i < n && !x_zero) ? __ldcg(x + i) : T(0);
   }
   pdl_wait();
-  if (sd.late) pdl_trigger();
+  if (sd.early) pdl_trigger();
   if ((int)threadIdx.x < GmresLayout(k).total) state[threadIdx.x] = __ldcg(static_cast<const T*>(sd.base) + threadIdx.x);
   T acc[KMAXB];
   sum_rows<T>(norm_rows<T>(sd, k), norm_count(sd, k, n), 1, acc);
@@ -413,7 +414,7 @@ GmresDev gmres_dev(const LevelDev& L, void* state, int steps, double* partial, b
   const int nbe = apply_epi_blocks(L), nbv = gm_blocks(n), nbt = tiled ? arnoldi_tiles(L) : 0;
   const int nbd = tiled ? nbt : nbe, nbn = tiled ? nbt : nbv;
   return GmresDev{state, steps, partial + 1, nbd, tiled ? nbt : x_is_zero ? nbv : nbe, nbn, 2 * nbd * KMAXB,
-                  std::max(std::max(nbe, nbv), nbt), tiled ? 1 : 0};
+                  std::max(std::max(nbe, nbv), nbt), tiled ? 1 : 0, tiled || (L.k == 3 && L.g.dim == 2) ? 1 : 0};
 }
 
 void gm_start(int prec, long long n, const void* b, void* V0, const GmresDev& st, cudaStream_t s) {
