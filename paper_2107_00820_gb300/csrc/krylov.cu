@@ -414,7 +414,7 @@ GmresDev gmres_dev(const LevelDev& L, void* state, int steps, double* partial, b
   const int nbe = apply_epi_blocks(L), nbv = gm_blocks(n), nbt = tiled ? arnoldi_tiles(L) : 0;
   const int nbd = tiled ? nbt : nbe, nbn = tiled ? nbt : nbv;
   return GmresDev{state, steps, partial + 1, nbd, tiled ? nbt : x_is_zero ? nbv : nbe, nbn, 2 * nbd * KMAXB,
-                  std::max(std::max(nbe, nbv), nbt), tiled ? 1 : 0, tiled || (L.k == 3 && L.g.dim == 2) ? 1 : 0};
+                  std::max(std::max(nbe, nbv), nbt), tiled ? 1 : 0, tiled || L.k == 3 ? 1 : 0};
 }
 
 void gm_start(int prec, long long n, const void* b, void* V0, const GmresDev& st, cudaStream_t s) {

@@ -467,6 +467,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_qk3_gather_epi(Geom g, const T*
     for (int jj = 0; jj < KMAXB; ++jj)
       vp[q][jj] = !start && jj < k && t0 + q * RED_THREADS < n ? __ldcg(V + (long long)jj * ld + t0 + q * RED_THREADS) : T(0);
   pdl_wait();
+  pdl_trigger();
   T v[PER];
 #pragma unroll
   for (int q = 0; q < PER; ++q) {
@@ -485,7 +486,6 @@ __global__ void __launch_bounds__(RED_THREADS) k_qk3_gather_epi(Geom g, const T*
         if (jj < k) acc[jj] += vp[q][jj] * v[q];
     }
   }
-  pdl_trigger();
   store_partials<T>(sd, start, k, acc, blockIdx.x, gridDim.x);
 }
 

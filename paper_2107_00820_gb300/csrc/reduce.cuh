@@ -158,7 +158,7 @@ struct GmresDev {
   void* rows;
   int nbd, nb0, nbn, noff, nstride;
   int late;   // the kernel before the last Gram-Schmidt step writes more than its column (see arnoldi2.cuh)
-  int early;  // short blocks (tiled levels, order 3 in 2D): trigger the successor right after the wait
+  int early;  // short blocks (tiled levels, order 3): trigger the successor right after the wait
 };
 
 template <typename T>
