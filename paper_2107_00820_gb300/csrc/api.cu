@@ -332,7 +332,7 @@ void smooth_fused(als_ctx* c, MGWork& w, int l, bool x_is_zero, void* t) {
   const cudaStream_t s = c->stream;
   const int steps = std::max(1, c->opt.sweeps);
   const bool tiled = tiled_steps(c, w, l);
-  const GmresDev st = gmres_dev(Lv, w.small[l], steps, w.partial, x_is_zero, tiled);
+  const GmresDev st = gmres_dev(Lv, prec, w.small[l], steps, w.partial, x_is_zero, tiled);
   void* V0 = w.V[l];
   if (tiled) {
     // V0 = b by the first step, or V0 = b - A x
@@ -1828,7 +1828,7 @@ void merged_smooth(MergedCycle& M, int l, bool x_is_zero, bool residual, cudaStr
     it.Z = w.Z[l];
     it.V = w.V[l];
     it.ld = len;
-    it.st = gmres_dev(c->lev[l], w.small[l], steps, w.partial, x_is_zero, tiled);
+    it.st = gmres_dev(c->lev[l], PREC_F32, w.small[l], steps, w.partial, x_is_zero, tiled);
     it.x = w.x[l];
     it.x_zero = x_is_zero ? 1 : 0;
     it.t = residual ? w.t[l] : nullptr;

@@ -269,7 +269,7 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
   T rhni = T(0);
   if (sd.late) {   // column j, its norm and rhn come from the predecessor too
     pdl_wait();
-    pdl_trigger();   // (tiled levels: short blocks, few of them; 128^2 cycle 345 -> 332 us with the update's)
+    pdl_trigger();
   }
   // columns 0..j, rhn and the norm partials come from earlier kernels of the chain (complete
   // before this launch began): read through L2 before the wait; column j+1 and the dots come
@@ -409,12 +409,12 @@ __global__ void __launch_bounds__(RED_THREADS) k_gm_update(unsigned n, const T* 
   gm_update_body<T, K>(blockIdx.x, n, Z, V, ld, sd, x, x_zero, t);
 }
 
-GmresDev gmres_dev(const LevelDev& L, void* state, int steps, double* partial, bool x_is_zero, bool tiled) {
+GmresDev gmres_dev(const LevelDev& L, int prec, void* state, int steps, double* partial, bool x_is_zero, bool tiled) {
   const long long n = L.g.N * L.g.dim;
   const int nbe = apply_epi_blocks(L), nbv = gm_blocks(n), nbt = tiled ? arnoldi_tiles(L) : 0;
   const int nbd = tiled ? nbt : nbe, nbn = tiled ? nbt : nbv;
   return GmresDev{state, steps, partial + 1, nbd, tiled ? nbt : x_is_zero ? nbv : nbe, nbn, 2 * nbd * KMAXB,
-                  std::max(std::max(nbe, nbv), nbt), tiled ? 1 : 0, tiled || L.k == 3 ? 1 : 0};
+                  std::max(std::max(nbe, nbv), nbt), tiled ? 1 : 0, prec == PREC_F32 || L.g.dim == 2 ? 1 : 0};
 }
 
 void gm_start(int prec, long long n, const void* b, void* V0, const GmresDev& st, cudaStream_t s) {

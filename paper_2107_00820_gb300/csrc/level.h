@@ -250,7 +250,7 @@ void vec_multiaxpy_norm(int prec, long long n, int k, const void* V, long long l
 // GMRES residual t = r0 - A Z y from the Arnoldi relation.  s <= KMAXB.
 size_t gmres_partial_doubles(const LevelDev& L);   // workspace of op_apply_epi, arnoldi_step and gm_*
 // a smoothing's state on level L: state array, partials (workspace above), from x = 0 or not
-GmresDev gmres_dev(const LevelDev& L, void* state, int steps, double* partial, bool x_is_zero, bool tiled);
+GmresDev gmres_dev(const LevelDev& L, int prec, void* state, int steps, double* partial, bool x_is_zero, bool tiled);
 void gm_start(int prec, long long n, const void* b, void* V0, const GmresDev& st, cudaStream_t s);
 void gm_orth(int prec, long long n, int j, const void* V, long long ld, const GmresDev& st, cudaStream_t s);
 void gm_update(int prec, long long n, int k, const void* Z, const void* V, long long ld, const GmresDev& st,
