@@ -17,7 +17,7 @@ namespace als {
 //
 // Prolongation: a thread takes four consecutive fine nodes x = 4j .. 4j+3 of a row, which are
 // combinations of the three coarse nodes 2j .. 2j+2 of the 1 or 3 x 1 or 3 coarse rows around it: all of
-// those are loaded at once, predicated, summed over the rows, then combined along x.  A tap counts
+// those are loaded at once, predicated.  A tap counts
 // only if it lies off the Dirichlet ends of its axis: the boundary of the box is exactly the set of
 // nodes with some coordinate at an end.  A thread per node, 27 taps each, took 18 us on 32^3 cells; with
 // both directions as they are now, and the coarse correction's residual formed by the gather before the
@@ -67,17 +67,23 @@ __device__ __forceinline__ void prolong_body(unsigned bx, const Geom& gc, const 
       }
 #pragma unroll
     for (int q = 0; q < GX; ++q) old[q] = xadd && GX * rc.j + q < gf.nn[0] ? xadd[rc.t0 + q] : T(0);
-    T a[3] = {T(0), T(0), T(0)};
+    // the taps in one order (z, y, x) for every node: the robust correction that follows amplifies
+    // a change of rounding here by gamma / mu
+    T out[GX] = {T(0), T(0), T(0), T(0)};
 #pragma unroll
     for (int cz = 0; cz < NZ; ++cz)
 #pragma unroll
       for (int cy = 0; cy < 3; ++cy) {
-        const T w = wy[cy] * wz[cz];
-#pragma unroll
-        for (int cx = 0; cx < 3; ++cx) a[cx] += w * v[cz][cy][cx];
+        const T w = wy[cy] * wz[cz], *u = v[cz][cy];   // dyadic: every product of weights is exact
+        out[0] += w * u[0];
+        out[1] += (T(0.375) * w) * u[0];
+        out[1] += (T(0.75) * w) * u[1];
+        out[1] += (T(-0.125) * w) * u[2];
+        out[2] += w * u[1];
+        out[3] += (T(-0.125) * w) * u[0];
+        out[3] += (T(0.75) * w) * u[1];
+        out[3] += (T(0.375) * w) * u[2];
       }
-    const T out[GX] = {a[0], T(0.375) * a[0] + T(0.75) * a[1] - T(0.125) * a[2], a[1],
-                       T(0.75) * a[1] + T(0.375) * a[2] - T(0.125) * a[0]};
 #pragma unroll
     for (int q = 0; q < GX; ++q) {
       const int x = GX * rc.j + q;
