@@ -451,10 +451,10 @@ __device__ __forceinline__ void cell2_from_stars(const Geom& g, const PatchIn<T>
   }
 }
 
-// The cell's contribution from its nodal values u (component c; the other lane of the pair holds
+// The cell's contribution from its nodal values un (component c; the other lane of the pair holds
 // the other one); store(ay, o) takes the outputs at the nodes (0..2, ay).  Every lane of the warp calls.
 template <typename T, bool TENSOR, int MODE, typename Store>
-__device__ __forceinline__ void cell2_contribution(const CellConst<T>& cc, bool act, int c, int cell, const T (&u)[9],
+__device__ __forceinline__ void cell2_contribution(const CellConst<T>& cc, bool act, int c, int cell, const T (&un)[9],
                                                    const T* mu, const T* __restrict__ coef,
                                                    const T* __restrict__ p_in, T* __restrict__ p_out,
                                                    const T* __restrict__ winv, Store store) {
@@ -462,6 +462,11 @@ __device__ __forceinline__ void cell2_contribution(const CellConst<T>& cc, bool 
   constexpr bool NEED_U = (MODE & (OP_VISC | OP_AL | OP_B)) != 0;
   constexpr bool NEED_FLUX = (MODE & (OP_VISC | OP_AL | OP_BT)) != 0;
   const DerivTab<T> dx = deriv_tab<T>(cc.s[0]), dy = deriv_tab<T>(cc.s[1]);
+  // Only differences of u count: in FP32 those to the cell's middle node are taken first, so that what
+  // follows rounds relative to them and not to u.
+  T u[9];
+#pragma unroll
+  for (int a = 0; a < 9; ++a) u[a] = sizeof(T) == 4 ? un[a] - un[4] : un[a];
   T gd[9], gs[9], od[9];   // d u_c / d x_c; d u_c / d x_(1-c), then the shear sum; the other component's diagonal
 #pragma unroll
   for (int q = 0; q < 9; ++q) gd[q] = gs[q] = od[q] = T(0);

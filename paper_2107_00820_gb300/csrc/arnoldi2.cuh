@@ -59,17 +59,29 @@ struct Tile2 {
 __host__ __device__ __forceinline__ int tiles2_x(const Geom& g) { return (g.n[0] + 7) >> 3; }
 __host__ __device__ __forceinline__ int tiles2(const Geom& g) { return tiles2_x(g) * ((g.n[1] + 7) >> 3); }
 
+// the sum, rounded once, of the outputs [3 ay + ax][cell] (CN cells a row, CP apart) of the one, two or four cells
+// of a node, e at the first of them; odd_x, odd_y: the node is in the middle of its cell along the axis
+template <int CN, int CP>
+__device__ __forceinline__ float node_sum2(const float* e, bool odd_x, bool odd_y) {
+  const float* f = e + ((odd_y ? 3 : 6) + (odd_x ? 1 : 2)) * CP;
+  const DF64 a = df_two_sum(f[0], odd_x ? 0.f : e[(odd_y ? 3 : 6) * CP + 1]);
+  if (odd_y) return a.hi;   // (a sum of two is rounded once as it is)
+  const DF64 b = df_two_sum(e[CN + (odd_x ? 1 : 2) * CP], odd_x ? 0.f : e[CN + 1]);
+  const DF64 c = df_two_sum(a.hi, b.hi);
+  return __fadd_rn(c.hi, __fadd_rn(__fadd_rn(a.lo, b.lo), c.lo));
+}
+
 // KM: the most columns before column j that this instance handles (the column loops are of that length)
 template <typename TS, bool TENSOR, int KM>
 __device__ __forceinline__ void arnoldi2_body(unsigned bx, const ArnoldiArgs& a, unsigned char* smraw) {
   using C = Tile2<TS>;
   constexpr int T = C::T, W = C::W;
   __shared__ float sh[RED_THREADS / 32][KMAXB];
-  __shared__ float coef[KMAXB], s_inv;
+  __shared__ DF64 coef[KMAXB], s_inv;
   __shared__ int s_fail;
   const Geom& g = a.g;
   const GmresDev& sd = a.st;
-  const GmresView<float> st = gmres_view<float>(sd);
+  const GmresView<DF64> st = gmres_view<float>(sd);
   const int j = KM == 0 ? 0 : a.j, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tx = tiles2_x(g), ntiles = tiles2(g);
   float acc[KMAXB];
@@ -79,8 +91,8 @@ __device__ __forceinline__ void arnoldi2_body(unsigned bx, const ArnoldiArgs& a,
     sum_rows<float>(norm_rows<float>(sd, j - 1), norm_count(sd, j - 1, a.ld), 1, acc);
     const float v = block_total<float>(acc, 1, sh);
     if (tid == 0) {
-      if (j == 1) gmres_start(st, v);
-      else gmres_step(st, j - 2, v);
+      if (j == 1) gmres_start(st, to_small(v));
+      else gmres_step(st, j - 2, to_small(v));
     }
     return;
   }
@@ -163,7 +175,8 @@ __device__ __forceinline__ void arnoldi2_body(unsigned bx, const ArnoldiArgs& a,
   pdl_trigger();
   // everything that the predecessor wrote is loaded at once: w, V_{j-1}, the partials (the first 256
   // blocks' here), 1 / hn
-  float val[4], d[KA], dn = 0.f, rh = 0.f;
+  float val[4], d[KA], dn = 0.f;
+  DF64 rh{};
 #pragma unroll
   for (int q = 0; q < 4; ++q) val[q] = at[q] >= 0 ? __ldcg(a.src + at[q]) : 0.f;
   if (j > 0) {
@@ -172,7 +185,7 @@ __device__ __forceinline__ void arnoldi2_body(unsigned bx, const ArnoldiArgs& a,
 #pragma unroll
     for (int c = 0; c < KM; ++c) d[c] = c < j && tid < sd.nbd ? __ldcg(rows + c * sd.nbd + tid) : 0.f;
     if (tid < nbn) dn = __ldcg(nrows + tid);
-    if (lane < j - 1) rh = __ldcg(st.rhn + lane);
+    if (lane < j - 1) rh = load_small(st.rhn + lane);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const float last = at[q] >= 0 ? __ldcg(a.V + (long long)(j - 1) * a.ld + at[q]) : 0.f;
@@ -190,9 +203,10 @@ __device__ __forceinline__ void arnoldi2_body(unsigned bx, const ArnoldiArgs& a,
     for (int c = 0; c < KMAXB; ++c) acc[c] = c == j ? dn : c < KM ? d[c < KM ? c : 0] : 0.f;
     const float v = block_total<float>(acc, j + 1, sh);
     if (warp == 0) {
-      const float inv = recip_or_zero<float>(sqrtf(fmaxf(__shfl_sync(0xffffffffu, v, j), 0.f)));
+      DF64 nrm, inv;
+      sqrt_recip(to_small(__shfl_sync(0xffffffffu, v, j)), nrm, inv);
       if (lane < j) {
-        const float rhni = lane == j - 1 ? inv : rh, h = v * rhni * inv;
+        const DF64 rhni = lane == j - 1 ? inv : rh, h = to_small(v) * rhni * inv;
         coef[lane] = h * rhni;
         if (bx == 0) {
           st.H[(long long)(j - 1) * st.ldh + lane] = h;
@@ -202,13 +216,15 @@ __device__ __forceinline__ void arnoldi2_body(unsigned bx, const ArnoldiArgs& a,
       if (lane == 0) s_inv = inv;
     }
     __syncthreads();
-    const float inv = s_inv;
+    const DF64 inv = s_inv;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      val[q] *= inv;
+      LinComb<float> sum(val[q]);
+      sum.scale(inv);
 #pragma unroll
       for (int c = 0; c < KM; ++c)
-        if (c < j) val[q] -= vc[q][c] * coef[c];
+        if (c < j) sum.sub(vc[q][c], coef[c]);
+      val[q] = sum.value();
     }
   }
   float nrm = 0.f;
@@ -317,7 +333,7 @@ __device__ __forceinline__ void arnoldi2_body(unsigned bx, const ArnoldiArgs& a,
     }
   }
   __syncthreads();
-  // node sums (the order of gather_chunk), the dots and the norm
+  // node sums, the dots and the norm
 #pragma unroll
   for (int c = 0; c < KMAXB; ++c) acc[c] = 0.f;
 #pragma unroll
@@ -326,14 +342,7 @@ __device__ __forceinline__ void arnoldi2_body(unsigned bx, const ArnoldiArgs& a,
     float w = 0.f;
     if (q < 2 && in[q]) {
       const int lx = tid & (2 * T - 1), ly = tid / (2 * T);
-      const float* e = se + q * 9 * C::CP + (ly >> 1) * C::C + (lx >> 1);   // cells (cx - 1, cy - 1) of the node's own
-      const bool ox = lx & 1, oy = ly & 1;
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        if (oy && k == 1) continue;
-        const float* p = e + (oy ? C::C : k * C::C) + (oy ? 3 : 6 - 6 * k) * C::CP;
-        w += ox ? p[1 + C::CP] : p[2 * C::CP] + p[1];
-      }
+      w = node_sum2<C::C, C::CP>(se + q * 9 * C::CP + ((ly + 1) >> 1) * C::C + ((lx + 1) >> 1), lx & 1, ly & 1);
     }
     a.wout[at[q]] = w;
     if (q < 2) {

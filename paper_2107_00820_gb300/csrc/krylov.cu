@@ -213,9 +213,9 @@ void vec_scale_dev(int prec, long long n, const double* num, const double* den, 
 // Each thread handles GM_PER entries spaced RED_THREADS apart, with all loads of
 // its entries issued before any arithmetic; the grid then has about n / 1024
 // blocks, which keeps the partials that every consumer block adds few.
-// Column loops are unrolled to KMAXB with predicates.  In FP32 the arithmetic
-// and all sums run in float, and so does the small GMRES bookkeeping (the state
-// array holds elements of the smoother's precision).
+// Column loops are unrolled to KMAXB with predicates.  In FP32 the reductions
+// run in float; the small GMRES bookkeeping and the combinations of columns keep the
+// low parts (see GmresView, LinComb).
 
 // V0 = b, |b|^2 partials
 // (bx, nb: the block's index and the blocks of this reduction, see batch.cuh)
@@ -257,16 +257,17 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
                                              long long ld, const GmresDev& sd) {
   constexpr int j = KC - 1;
   __shared__ T sh[RED_THREADS / 32][KMAXB];
-  __shared__ T coef[KMAXB];
+  __shared__ small_t<T> coef[KMAXB];
   __shared__ T nrm2;
-  const GmresView<T> st = gmres_view<T>(sd);
+  using S = small_t<T>;
+  const GmresView<S> st = gmres_view<T>(sd);
   T acc[KMAXB];
   const bool extra = bx == nb - 1;
   const unsigned base = bx * (RED_THREADS * GM_PER) + threadIdx.x;
   T* w = const_cast<T*>(V) + (long long)(j + 1) * ld;
   T a[GM_PER];
   T vc[GM_PER][KC];
-  T rhni = T(0);
+  S rhni = S{};
   if (sd.late) {   // column j, its norm and rhn come from the predecessor too
     pdl_wait();
     pdl_trigger();
@@ -281,7 +282,7 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
 #pragma unroll
       for (int c = 0; c < KC; ++c) vc[q][c] = i < n ? __ldcg(V + (long long)c * ld + i) : T(0);
     }
-    if ((int)threadIdx.x < j) rhni = __ldcg(st.rhn + threadIdx.x);
+    if ((int)threadIdx.x < j) rhni = load_small(st.rhn + threadIdx.x);
   }
   sum_rows<T>(norm_rows<T>(sd, j), norm_count(sd, j, n), 1, acc);
   {
@@ -291,12 +292,13 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
   __syncthreads();
   if (extra) {
     if (threadIdx.x == 0) {
-      if (j == 0) gmres_start(st, nrm2);
-      else gmres_step(st, j - 1, nrm2);
+      if (j == 0) gmres_start(st, to_small(nrm2));
+      else gmres_step(st, j - 1, to_small(nrm2));
     }
     return;
   }
-  const T inv = recip_or_zero<T>(sqrt(fmax(nrm2, T(0))));
+  S nrm, inv;
+  sqrt_recip(to_small(nrm2), nrm, inv);
   if ((int)threadIdx.x == j) rhni = inv;
   pdl_wait();
   if (sd.early) pdl_trigger();
@@ -309,7 +311,7 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
   {
     const T v = block_total<T>(acc, j + 1, sh);
     if ((int)threadIdx.x <= j) {
-      const T h = v * rhni * inv;
+      const S h = to_small(v) * rhni * inv;
       coef[threadIdx.x] = h * rhni;
       if (bx == 0) {
         st.H[(long long)j * st.ldh + threadIdx.x] = h;
@@ -322,9 +324,11 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
 #pragma unroll
   for (int q = 0; q < GM_PER; ++q) {
     const unsigned i = base + q * RED_THREADS;
-    a[q] *= inv;
+    LinComb<T> sum(a[q]);
+    sum.scale(inv);
 #pragma unroll
-    for (int c = 0; c < KC; ++c) a[q] -= vc[q][c] * coef[c];
+    for (int c = 0; c < KC; ++c) sum.sub(vc[q][c], coef[c]);
+    a[q] = sum.value();
     if (i < n) w[i] = a[q];
     acc[0] += a[q] * a[q];
   }
@@ -347,11 +351,12 @@ __device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, const T*
                                                const T* __restrict__ V, long long ld, const GmresDev& sd,
                                                T* __restrict__ x, int x_zero, T* __restrict__ t) {
   __shared__ T sh[RED_THREADS / 32][KMAXB];
-  __shared__ T state[GmresLayout(KMAXB).total];
-  __shared__ T y[KMAXB], u[KMAXB + 1];
+  using S = small_t<T>;
+  __shared__ S state[GmresLayout(KMAXB).total];
+  __shared__ S y[KMAXB], u[KMAXB + 1];
   __shared__ T nrm2;
   static_assert(GmresLayout(KMAXB).total <= RED_THREADS, "one state entry a thread");
-  const GmresView<T> st = gmres_view<T>(GmresDev{state, k});
+  const GmresView<S> st = gmres_view<T>(GmresDev{state, k});
   const unsigned base = bx * (RED_THREADS * GM_PER) + threadIdx.x;
   // Z, x and V_0..V_{k-1} come from earlier kernels of the chain (complete before this
   // launch began): read through L2 before the wait; V_k, its norm and the last column of H
@@ -366,7 +371,7 @@ __device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, const T*
   }
   pdl_wait();
   if (sd.early) pdl_trigger();
-  if ((int)threadIdx.x < GmresLayout(k).total) state[threadIdx.x] = __ldcg(static_cast<const T*>(sd.base) + threadIdx.x);
+  if ((int)threadIdx.x < GmresLayout(k).total) state[threadIdx.x] = load_small(static_cast<const S*>(sd.base) + threadIdx.x);
   T acc[KMAXB];
   sum_rows<T>(norm_rows<T>(sd, k), norm_count(sd, k, n), 1, acc);
   const T tot = block_total<T>(acc, 1, sh);   // (its barrier also publishes the state)
@@ -374,7 +379,7 @@ __device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, const T*
   __syncthreads();
   if (threadIdx.x < 64) {   // y and u in a warp each
     const int what = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const T v = gmres_finish<T>(st, nrm2, what);
+    const S v = gmres_finish(st, to_small(nrm2), what);
     if (lane < k + what) (what ? u : y)[lane] = v;
   }
   __syncthreads();
@@ -382,10 +387,10 @@ __device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, const T*
   for (int q = 0; q < GM_PER; ++q) {
     const unsigned i = base + q * RED_THREADS;
     if (i >= n) break;
-    T a = xa[q];
+    LinComb<T> a(xa[q]);
 #pragma unroll
-    for (int c = 0; c < k; ++c) a += zc[q][c] * y[c];
-    x[i] = a;
+    for (int c = 0; c < k; ++c) a.add(zc[q][c], y[c]);
+    x[i] = a.value();
   }
   if (t) {
 #pragma unroll
@@ -395,10 +400,10 @@ __device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, const T*
       T vc[k + 1];
 #pragma unroll
       for (int c = 0; c <= k; ++c) vc[c] = V[(long long)c * ld + i];
-      T r = T(0);
+      LinComb<T> r(T(0));
 #pragma unroll
-      for (int c = 0; c <= k; ++c) r += vc[c] * u[c];
-      t[i] = r;
+      for (int c = 0; c <= k; ++c) r.add(vc[c], u[c]);
+      t[i] = r.value();
     }
   }
 }

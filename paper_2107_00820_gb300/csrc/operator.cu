@@ -138,7 +138,7 @@ static unsigned gather_threads(const Geom& g) {
 // Gather fused with the reduction that consumes the result:
 //   y = b + sigma A x (b NULL: y = sigma A x);  block partials of V_j . y, j < k, or, start,
 //   of |y|^2.  Fixed grid and order: reproducible.
-// All sums run in T (in FP32 the GMRES state is float too, see GmresView).
+// All sums run in T.
 // KC = k, or 0 for start (with arrays of KMAXB columns, predicated, a block took 80 registers, three
 // an SM, whatever it needed).
 template <typename T, int DIM, int KC>

@@ -10,6 +10,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "df64.cuh"
+
 namespace als {
 
 constexpr int RED_THREADS = 256;
@@ -127,15 +129,95 @@ __device__ __forceinline__ void sum_rows(const T* __restrict__ rows, int nb, int
 }
 
 // ---------------------------------------------------------------------------
-// GMRES(s) state on the device, in the smoother's precision T (column-major
-// Hessenberg H, leading dim ldh).  The Krylov basis is stored unnormalised:
+// GMRES(s) state on the device, in S = small_t<T> for a smoother of precision T (column-major
+// Hessenberg H, leading dim ldh): FP64, or, for an FP32 smoother, double-float.  The least-squares
+// problem of a smoothing amplifies a change of its small numbers into the iterate, as it does the roundings
+// of the vectors.  Relative error of one FP32 96^2 five-level cycle (gamma 100, contrast 1e6, P2) against FP64
+// over 240 problems, median and 90th percentile: 3.1e-7 and 5.8e-7 with the state, the coefficients and the
+// combinations of columns in plain FP32, 2.2e-7 and 3.1e-7 so (with the cells' differences to their middle
+// node and the node sums of the tiles, apply_cells.cuh and arnoldi2.cuh, which are part of that).  One
+// cycle, us, plain / so: 2D 16^2 96 / 105, 128^2 333 / 354, order 3 1013 / 1028, 3D 32^3 1643 / 1657.
+// The Krylov basis is stored unnormalised:
 // column i holds hn_i v_i, where v_i is the orthonormal Arnoldi vector, and
 // Z_i = D^-1 (column i) likewise; their consumers multiply by rhn[i] = 1 / hn_i, and rr[i] = 1 / R_ii
 // (both 0 where the divisor is): the divisions are done once, by the bookkeeping block beside
 // the vector work, and none but those of the last step is left for the update.
-// Layout of the state array, in elements of T:
+// Layout of the state array, in elements of S (eight bytes either way):
 // H [ldh s] | cs [s] | sn [s] | g [s+1] | y [s] | res | beta | nrm2 | rhn [s+1] | rr [s].
 // ---------------------------------------------------------------------------
+template <typename T> struct SmallReal { using S = double; };
+template <> struct SmallReal<float> { using S = DF64; };
+template <typename T> using small_t = typename SmallReal<T>::S;
+
+__device__ __forceinline__ double to_small(double v) { return v; }
+__device__ __forceinline__ DF64 to_small(float v) { return DF64{v, 0.f}; }
+__device__ __forceinline__ double load_small(const double* p) { return __ldcg(p); }
+__device__ __forceinline__ DF64 load_small(const DF64* p) {
+  const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
+  return DF64{v.x, v.y};
+}
+__device__ __forceinline__ double shfl_small(double v, int l) { return __shfl_sync(0xffffffffu, v, l); }
+__device__ __forceinline__ DF64 shfl_small(DF64 v, int l) {
+  return DF64{__shfl_sync(0xffffffffu, v.hi, l), __shfl_sync(0xffffffffu, v.lo, l)};
+}
+// 1 / a, or 0 where a is 0 or so small that 1 / a overflows (no direction is left)
+__device__ __forceinline__ double recip_or_zero(double a) {
+  const double r = 1.0 / a;
+  return isfinite(r) ? r : 0.0;
+}
+__device__ __forceinline__ DF64 recip_or_zero(DF64 a) {
+  const float r = __frcp_rn(a.hi);
+  if (!isfinite(r) || r == 0.f) return DF64{0.f, 0.f};
+  const float e = __fmaf_rn(-r, a.lo, __fmaf_rn(-r, a.hi, 1.f));   // 1 - r a
+  return df_quick_two_sum(r, __fmul_rn(r, e));
+}
+// r = sqrt(a) and 1 / r, 0 where a <= 0 (1 / r: or so small that it overflows).  Double-float: one Newton step from the
+// FP32 reciprocal root, no division.
+__device__ __forceinline__ void sqrt_recip(double a, double& r, double& inv) {
+  r = sqrt(fmax(a, 0.0));
+  inv = recip_or_zero(r);
+}
+__device__ __forceinline__ void sqrt_recip(DF64 a, DF64& r, DF64& inv) {
+  const float y = rsqrtf(fmaxf(a.hi, 0.f));
+  r = inv = DF64{0.f, 0.f};
+  if (!isfinite(y)) return;
+  if (y == 0.f) { r = a; return; }   // a = inf
+  const float t = __fmul_rn(a.hi, y);
+  const float tl = __fmaf_rn(a.lo, y, __fmaf_rn(a.hi, y, -t));     // a y = t + tl
+  const float e = __fmul_rn(0.5f, __fmaf_rn(-tl, y, __fmaf_rn(-t, y, 1.f)));   // (1 - a y^2) / 2
+  r = df_quick_two_sum(t, __fmaf_rn(t, e, tl));
+  inv = df_quick_two_sum(y, __fmul_rn(y, e));
+}
+
+// start + sum_i v_i c_i for entries v_i of precision T and coefficients c_i of small_t<T>.  T = float: the low parts
+// of the coefficients and the roundings of the sum (all but a bit of them) are kept beside it and added at
+// the end, five instructions a term (the exact error of every product and sum takes eleven).
+template <typename T> struct LinComb;
+template <> struct LinComb<double> {
+  double s;
+  __device__ __forceinline__ explicit LinComb(double v) : s(v) {}
+  __device__ __forceinline__ void add(double v, double c) { s += v * c; }
+  __device__ __forceinline__ void sub(double v, double c) { s -= v * c; }
+  __device__ __forceinline__ void scale(double c) { s *= c; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <> struct LinComb<float> {
+  float hi, lo;
+  __device__ __forceinline__ explicit LinComb(float v) : hi(v), lo(0.f) {}
+  __device__ __forceinline__ void add(float v, DF64 c) {
+    const float t = __fmaf_rn(v, c.hi, hi);
+    lo = __fmaf_rn(v, c.lo, __fadd_rn(lo, __fmaf_rn(v, c.hi, __fsub_rn(hi, t))));
+    hi = t;
+  }
+  __device__ __forceinline__ void sub(float v, DF64 c) { add(v, -c); }
+  __device__ __forceinline__ void scale(DF64 c) {   // before any term
+    const float v = hi;
+    hi = __fmul_rn(v, c.hi);
+    lo = __fmaf_rn(v, c.lo, __fmaf_rn(v, c.hi, -hi));
+  }
+  __device__ __forceinline__ float value() const { return __fadd_rn(hi, lo); }
+};
+
 struct GmresLayout {
   int s, ldh;
   int H, cs, sn, g, y, res, beta, nrm2, rhn, rr, total;
@@ -144,7 +226,7 @@ struct GmresLayout {
         res(y + steps), beta(res + 1), nrm2(beta + 1), rhn(nrm2 + 1), rr(rhn + steps + 1), total(rr + steps) {}
 };
 
-// host-side handle: the state array (elements of the smoother's precision), s, and the block
+// host-side handle: the state array (elements of small_t), s, and the block
 // partials of the reductions.  A reduction kernel only writes its partials, [column][block];
 // every block of the kernel that needs the sums adds them for itself, in one fixed order.
 // (A last-block finish, with its fence, ticket, second fence, reload and one-thread
@@ -191,53 +273,60 @@ __device__ __forceinline__ void store_partials(const GmresDev& d, int start, int
   if ((int)threadIdx.x < kk) (start ? norm_rows<T>(d, 0) : dot_rows<T>(d, k - 1))[threadIdx.x * nb + bx] = v;
 }
 
-template <typename T>
+template <typename S>
 struct GmresView {
-  T* H;
+  S* H;
   int ldh;
-  T* cs;
-  T* sn;
-  T* g;       // rotated right-hand side, length s + 1
-  T* res;     // |g[k+1]| after step k
-  T* rhn;     // 1 / norms of the stored columns, length s + 1 (written by the Gram-Schmidt steps)
-  T* rr;      // 1 / R_ii, length s
-  T* beta;    // |r0|
+  S* cs;
+  S* sn;
+  S* g;       // rotated right-hand side, length s + 1
+  S* rhn;     // 1 / norms of the stored columns, length s + 1 (written by the Gram-Schmidt steps)
+  S* rr;      // 1 / R_ii, length s
+  S* beta;    // |r0|
   int m;      // s + 1
 };
 
+// T: the smoother's precision
 template <typename T>
-__host__ __device__ __forceinline__ GmresView<T> gmres_view(const GmresDev& d) {
+__host__ __device__ __forceinline__ GmresView<small_t<T>> gmres_view(const GmresDev& d) {
   const GmresLayout L(d.s);
-  T* b = static_cast<T*>(d.base);
-  return GmresView<T>{b + L.H, L.ldh, b + L.cs, b + L.sn, b + L.g, b + L.res, b + L.rhn, b + L.rr, b + L.beta, d.s + 1};
+  small_t<T>* b = static_cast<small_t<T>*>(d.base);
+  return GmresView<small_t<T>>{b + L.H, L.ldh, b + L.cs, b + L.sn, b + L.g, b + L.rhn, b + L.rr, b + L.beta, d.s + 1};
 }
 
-// 1 / a, or 0 where a is 0 or so small that 1 / a overflows (no direction is left)
-template <typename T>
-__device__ __forceinline__ T recip_or_zero(T a) {
-  const T r = T(1) / a;
-  return isfinite(r) ? r : T(0);
+// Givens rotation (c, s) of (a, b), b >= 0, r = |(a, b)| and rr = 1 / r (0 where that overflows); the plain
+// sum of squares where it is far from over- and underflow (hypot takes several times the FP64 instructions)
+__device__ __forceinline__ void givens(double a, double b, double& c, double& s, double& r, double& rr) {
+  const double q = a * a + b * b;
+  r = q > 1e-200 && q < 1e200 ? sqrt(q) : hypot(a, b);
+  c = 1.0;
+  s = 0.0;
+  if (r > 0.0) { c = a / r; s = b / r; }
+  rr = recip_or_zero(r);
+}
+__device__ __forceinline__ void givens(DF64 a, DF64 b, DF64& c, DF64& s, DF64& r, DF64& rr) {
+  const DF64 q = a * a + b * b;
+  c = DF64{1.f, 0.f};
+  s = DF64{0.f, 0.f};
+  if (q.hi > 1e-20f && q.hi < 1e20f) {
+    sqrt_recip(q, r, rr);
+    c = a * rr;
+    s = b * rr;
+  } else {
+    r = DF64{hypotf(a.hi, b.hi), 0.f};
+    rr = recip_or_zero(r);
+    if (r.hi > 0.f) { c = a / r; s = b / r; }
+  }
 }
 
-// Givens rotation (c, s) of (a, b), b >= 0, and r = |(a, b)|; the plain sum of squares where
-// it is far from over- and underflow (hypot takes several times the FP64 instructions)
-template <typename T>
-__device__ __forceinline__ void givens(T a, T b, T& c, T& s, T& r) {
-  constexpr T lo = sizeof(T) == 8 ? T(1e-200) : T(1e-20), hi = T(1) / lo;
-  const T q = a * a + b * b;
-  r = q > lo && q < hi ? sqrt(q) : hypot(a, b);
-  c = T(1);
-  s = T(0);
-  if (r > T(0)) { c = a / r; s = b / r; }
-}
-
-// start: beta = |r0|, g = (beta, 0, ...), hn[0] = beta   (one thread)
-template <typename T>
-__device__ __forceinline__ void gmres_start(const GmresView<T>& st, T nrm2) {
-  const T b = sqrt(fmax(nrm2, T(0)));
+// start: beta = |r0|, g = (beta, 0, ...)   (one thread)
+template <typename S>
+__device__ __forceinline__ void gmres_start(const GmresView<S>& st, S nrm2) {
+  S b, inv;
+  sqrt_recip(nrm2, b, inv);
   st.beta[0] = b;
   st.g[0] = b;
-  for (int i = 1; i < st.m; ++i) st.g[i] = T(0);
+  for (int i = 1; i < st.m; ++i) st.g[i] = S{};
 }
 
 // step k (k < KMAXB): H[k+1][k] = |w|, then the rotations of
@@ -245,37 +334,37 @@ __device__ __forceinline__ void gmres_start(const GmresView<T>& st, T nrm2) {
 // unrolled to KMAXB, predicated), so the chain runs in registers (one thread).  With runtime
 // loop bounds the arrays lived in local memory, and this chain, on the serial tail of every
 // Gram-Schmidt step, took about three times as long.
-template <typename T>
-__device__ __forceinline__ void gmres_step(const GmresView<T>& st, int k, T nrm2) {
-  T* hg = st.H + (long long)k * st.ldh;
-  T h[KMAXB], cs[KMAXB], sn[KMAXB];
+template <typename S>
+__device__ __forceinline__ void gmres_step(const GmresView<S>& st, int k, S nrm2) {
+  S* hg = st.H + (long long)k * st.ldh;
+  S h[KMAXB], cs[KMAXB], sn[KMAXB];
 #pragma unroll
   for (int i = 0; i < KMAXB; ++i) {
-    h[i] = i <= k ? hg[i] : T(0);
-    cs[i] = i < k ? st.cs[i] : T(1);
-    sn[i] = i < k ? st.sn[i] : T(0);
+    h[i] = i <= k ? hg[i] : S{};
+    cs[i] = i < k ? st.cs[i] : S{1};
+    sn[i] = i < k ? st.sn[i] : S{};
   }
-  const T gk = st.g[k];
-  const T hk1 = sqrt(fmax(nrm2, T(0)));
-  T a = h[0];                       // the entry the next rotation starts from
+  const S gk = st.g[k];
+  S hk1, unused;
+  sqrt_recip(nrm2, hk1, unused);
+  S a = h[0];                       // the entry the next rotation starts from
 #pragma unroll
   for (int i = 0; i < KMAXB - 1; ++i)
     if (i < k) {
-      const T b = h[i + 1];
+      const S b = h[i + 1];
       h[i] = cs[i] * a + sn[i] * b;
       a = -sn[i] * a + cs[i] * b;
     }
-  T c, sv, r;
-  givens<T>(a, hk1, c, sv, r);
+  S c, sv, r, rr;
+  givens(a, hk1, c, sv, r, rr);
 #pragma unroll
   for (int i = 0; i < KMAXB; ++i)
     if (i <= k) hg[i] = i == k ? r : h[i];
-  hg[k + 1] = T(0);
-  st.rr[k] = recip_or_zero<T>(r);
+  hg[k + 1] = S{};
+  st.rr[k] = rr;
   st.cs[k] = c; st.sn[k] = sv;
   st.g[k + 1] = -sv * gk;
   st.g[k] = c * gk;
-  st.res[0] = fabs(sv * gk);
 }
 
 // The last step's rotations (k = s - 1, not written back) and, by the warp that calls,
@@ -285,53 +374,53 @@ __device__ __forceinline__ void gmres_step(const GmresView<T>& st, int k, T nrm2
 // sum_i u_i (stored column i) by the Arnoldi relation.  Lane i holds row i: what the rotations
 // and the substitution do to all rows is one instruction each, and the chains are one
 // multiply-add a step.
-template <typename T>
-__device__ __forceinline__ T gmres_finish(const GmresView<T>& st, T nrm2, int what) {
-  constexpr unsigned FULL = 0xffffffffu;
+template <typename S>
+__device__ __forceinline__ S gmres_finish(const GmresView<S>& st, S nrm2, int what) {
   const int s = st.m - 1, k = s - 1, lane = threadIdx.x & 31, i = lane < KMAXB ? lane : 0;
-  const T* hg = st.H + (long long)k * st.ldh;
+  const S* hg = st.H + (long long)k * st.ldh;
   const bool old = lane < k;
-  const T cs = old ? st.cs[i] : T(1), sn = old ? st.sn[i] : T(0);
-  const T b1 = old ? hg[i + 1] : T(0);
-  const T hk1 = sqrt(fmax(nrm2, T(0)));
+  const S cs = old ? st.cs[i] : S{1}, sn = old ? st.sn[i] : S{};
+  const S b1 = old ? hg[i + 1] : S{};
+  S hk1, inv;
+  sqrt_recip(nrm2, hk1, inv);
   // a_0 = h_0;  a_(i+1) = cs_i h_(i+1) - sn_i a_i;  R_ik = cs_i a_i + sn_i h_(i+1)
-  const T q = cs * b1;
-  T a = hg[0], mine = a;
+  const S q = cs * b1;
+  S a = hg[0], mine = a;
 #pragma unroll
   for (int t = 0; t < KMAXB - 1; ++t)
     if (t < k) {
-      a = __shfl_sync(FULL, q, t) - __shfl_sync(FULL, sn, t) * a;
+      a = RealOps<S>::sub_prod(shfl_small(q, t), shfl_small(sn, t), a);
       if (lane == t + 1) mine = a;
     }
-  T c, sv, r;
-  givens<T>(a, hk1, c, sv, r);
-  const T gk = st.g[k];
+  S c, sv, r, rk;
+  givens(a, hk1, c, sv, r, rk);
+  const S gk = st.g[k];
   if (what == 0) {
-    T acc = lane < k ? st.g[i] : lane == k ? c * gk : T(0);
-    const T rik = cs * mine + sn * b1;
-    const T rr = lane < k ? st.rr[i] : lane == k ? recip_or_zero<T>(r) : T(0);
-    T y = T(0);
+    S acc = lane < k ? st.g[i] : lane == k ? c * gk : S{};
+    const S rik = cs * mine + sn * b1;
+    const S rr = lane < k ? st.rr[i] : lane == k ? rk : S{};
+    S y = S{};
 #pragma unroll
     for (int t = KMAXB - 1; t >= 0; --t)
       if (t < s) {
-        const T yt = __shfl_sync(FULL, acc * rr, t);
+        const S yt = shfl_small(acc * rr, t);
         if (lane == t) y = yt;
-        const T h = t == k ? rik : lane < t ? st.H[(long long)t * st.ldh + i] : T(0);
-        acc -= h * yt;
+        const S h = t == k ? rik : lane < t ? st.H[(long long)t * st.ldh + i] : S{};
+        acc = RealOps<S>::sub_prod(acc, h, yt);
       }
-    return lane < s ? y * st.rhn[i] : T(0);
+    return lane < s ? y * st.rhn[i] : S{};
   }
   // u_i = cs_(i-1) b_i / hn_i with b_s = g[s], b_(i-1) = -sn_(i-1) b_i; u_0 = b_0 / hn_0
-  T b = -sv * gk, u = b;
+  S b = -sv * gk, u = b;
 #pragma unroll
   for (int t = KMAXB - 1; t >= 0; --t)
     if (t < s) {
-      const T ct = t == k ? c : __shfl_sync(FULL, cs, t), st_ = t == k ? sv : __shfl_sync(FULL, sn, t);
+      const S ct = t == k ? c : shfl_small(cs, t), st_ = t == k ? sv : shfl_small(sn, t);
       if (lane == t + 1) u = ct * b;
       b = -(st_ * b);
     }
   if (lane == 0) u = b;
-  return lane < s ? u * st.rhn[lane] : lane == s ? u * recip_or_zero<T>(hk1) : T(0);
+  return lane < s ? u * st.rhn[lane] : lane == s ? u * inv : S{};
 }
 
 }  // namespace als

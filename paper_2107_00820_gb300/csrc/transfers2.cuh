@@ -39,18 +39,11 @@ __device__ __forceinline__ void cells2_tile(const Geom& g, const CellConst<float
                                             });
   }
 }
-// the sum of those outputs at node (px, py) of the tile, not on its rim; e: the component's outputs
+// their sum at node (px, py) of the tile, not on its rim; e: the component's outputs
 template <int CN, int CP>
-__device__ __forceinline__ float node_sum2(const float* e, int px, int py) {
-  const bool ox = px & 1, oy = py & 1;
-  float s = 0.f;
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    if (oy && k == 1) continue;
-    const float* p = e + (oy ? 3 : 6 - 6 * k) * CP + ((py >> 1) - (oy ? 0 : 1 - k)) * CN + (px >> 1);
-    s += ox ? p[CP] : p[2 * CP - 1] + p[0];
-  }
-  return s;
+__device__ __forceinline__ float tile_sum2(const float* e, int px, int py) {
+  const int cx = (px >> 1) - (px & 1 ? 0 : 1), cy = (py >> 1) - (py & 1 ? 0 : 1);   // the first of its cells
+  return node_sum2<CN, CP>(e + cy * CN + cx, px & 1, py & 1);
 }
 
 // V_0 = b - A x (b - x at Dirichlet nodes) and the partials of its norm
@@ -109,7 +102,7 @@ __device__ __forceinline__ void residual2_body(unsigned bx, const Residual2Args&
   for (int q = 0; q < NQ; ++q) {
     if (!(flag[q] & 1)) continue;
     const int e = tid + q * RED_THREADS, c = e >= W * W ? 1 : 0, f = e - c * W * W, py = f / W, px = f - W * py;
-    const float v = bv[q] - (flag[q] & 2 ? node_sum2<CN, CP>(se + c * 9 * CP, px, py) : xv[q]);
+    const float v = bv[q] - (flag[q] & 2 ? tile_sum2<CN, CP>(se + c * 9 * CP, px, py) : xv[q]);
     a.y[at[q]] = v;
     acc[0] += v * v;
   }
@@ -240,7 +233,7 @@ __device__ __forceinline__ void restrict2_body(unsigned bx, const Transfer2Args&
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
     const int e = tid + q * RED_THREADS, c = e >= W * W ? 1 : 0, f = e - c * W * W, py = f / W, px = f - W * py;
-    if (at[q] >= 0 && px > 0 && px < W - 1 && py > 0 && py < W - 1) fr[e] = v[q] - node_sum2<CN, CP>(se + c * 9 * CP, px, py);
+    if (at[q] >= 0 && px > 0 && px < W - 1 && py > 0 && py < W - 1) fr[e] = v[q] - tile_sum2<CN, CP>(se + c * 9 * CP, px, py);
   }
   __syncthreads();
   // coarse node (i, j) of the block's 8 x 8, and the last column and row of the level (Dirichlet)
@@ -335,7 +328,7 @@ __device__ __forceinline__ void prolong2_body(unsigned bx, const Transfer2Args& 
   __syncthreads();
   for (int e = tid; e < KN * KN * 18; e += RED_THREADS) {
     const int k = e & (KN * KN - 1), i = e / (KN * KN), c = i / 9, o = i - 9 * c;
-    rs[i * KP + k] = node_sum2<CN, CP>(se + c * 9 * CP, 4 * (k % KN) + 1 + o % 3, 4 * (k / KN) + 1 + o / 3);
+    rs[i * KP + k] = tile_sum2<CN, CP>(se + c * 9 * CP, 4 * (k % KN) + 1 + o % 3, 4 * (k / KN) + 1 + o / 3);
   }
   __syncthreads();
   if (warp < 2) I2::products(a, kx0, ky0, mats, [&](int c, int o, int k) { return rs[(c * 9 + o) * KP + k]; }, part);
