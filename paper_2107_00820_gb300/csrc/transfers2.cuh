@@ -314,12 +314,27 @@ __device__ __forceinline__ void prolong2_body(unsigned bx, const Transfer2Args& 
     const int e = tid + q * RED_THREADS, c = e >= W * W ? 1 : 0, f = e - c * W * W, py = f / W, px = f - W * py;
     tv[q] = 0.f;
     if (at[q] >= 0 && !on_boundary(gf, 4 * kx0 + px, 4 * ky0 + py, 0)) {
+      // the taps one after another (y, then x) as in prolong_body of transfer.cu, with its products: the correction
+      // that follows amplifies a change of rounding here by gamma / mu
       const int ix = px & 1 ? 2 * (px >> 2) : px >> 1, iy = py & 1 ? 2 * (py >> 2) : py >> 1;
       const float ax = (px & 3) == 1 ? 0.375f : -0.125f, bx2 = (px & 3) == 1 ? -0.125f : 0.375f;
       const float ay = (py & 3) == 1 ? 0.375f : -0.125f, by2 = (py & 3) == 1 ? -0.125f : 0.375f;
       const float* p = cs + (c * WC + iy) * WC + ix;
-      auto row = [&](const float* r) { return px & 1 ? ax * r[0] + 0.75f * r[1] + bx2 * r[2] : r[0]; };
-      tv[q] = py & 1 ? ay * row(p) + 0.75f * row(p + WC) + by2 * row(p + 2 * WC) : row(p);
+      float t = 0.f;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        if (k > 0 && !(py & 1)) continue;
+        const float w = !(py & 1) ? 1.f : k == 0 ? ay : k == 1 ? 0.75f : by2;   // dyadic: every product of weights is exact
+        const float* r = p + k * WC;
+        if (px & 1) {
+          t += (ax * w) * r[0];
+          t += (0.75f * w) * r[1];
+          t += (bx2 * w) * r[2];
+        } else {
+          t += w * r[0];
+        }
+      }
+      tv[q] = t;
     }
     if (e < NN) nt[e] = tv[q];
   }

@@ -39,3 +39,19 @@ def test_2d_cycle_error_over_many_problems():
         ctx.close()
     assert np.median(errs) <= 2.6e-7
     assert np.quantile(errs, 0.9) <= 4.2e-7
+
+
+# ragged tiles; sizes of one tile and less
+@pytest.mark.parametrize("n", [(4, 4), (20, 12), (16, 34)])
+def test_robust_prolongation_interpolates_as_the_standard_one(n):
+    """With the stars' inverses set to 0 the robust prolongation is the interpolation alone, and that has the
+    standard prolongation's bits: the robust correction amplifies a change of its rounding by gamma / mu."""
+    pb = sinker(2, n, 2, 100.0, 1e4, 7)
+    robust, standard = context(pb), context(pb, transfer=A.ALS_TRANSFER_STANDARD)
+    stride = (18 * 19 // 2 + 3) // 4 * 4
+    robust.load_patch_inverses(1, np.zeros((n[0] + 1) * (n[1] + 1) * stride))
+    xc = dev(_free((n[0] // 2, n[1] // 2), 8), torch.float32)
+    out = [torch.zeros(robust.nu(), dtype=torch.float32, device="cuda") for _ in range(2)]
+    robust.prolong(1, xc, out[0], F32)
+    standard.prolong(1, xc, out[1], F32)
+    assert torch.equal(out[0], out[1])
