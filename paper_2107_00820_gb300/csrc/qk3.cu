@@ -1026,6 +1026,17 @@ __global__ void __launch_bounds__(STAR_THREADS) k_qk3_star_apply(Geom g, const T
 // storing, waits (at the default limit) for the copies in flight and returns.
 constexpr int STARS_WARPS = 11, STARS_THREADS = 32 * (STARS_WARPS + 1);
 
+// named barrier 1 of the consumer warps, and whether any of their threads brought a flag
+__device__ __forceinline__ bool consumers_vote(int flag) {
+  int any;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n bar.red.or.pred q, 1, %2, p;\n selp.s32 %0, 1, 0, q;\n}\n"
+      : "=r"(any)
+      : "r"(flag), "n"(32 * STARS_WARPS)
+      : "memory");
+  return any != 0;
+}
+
 __device__ __forceinline__ float4 star_quad(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ float4 star_quad(const __nv_bfloat16* p) {
   const uint2 u = *reinterpret_cast<const uint2*>(p);
@@ -1231,8 +1242,9 @@ __global__ void __launch_bounds__(STARS_THREADS, 1) k_qk3_stars(Geom g, const TS
           for (int q = 0; q < SB; ++q) part[(SB * J + q) * kFullRows + I] = yJ[q];
         }
       }
-      asm volatile("bar.sync 1, %0;" ::"n"(32 * STARS_WARPS) : "memory");
-      if (*(volatile int*)&s_fail) break;
+      // The producer may set s_fail at any time: the consumers vote, so that all of them leave or none (one that left
+      // alone would be missing at the others' next barrier).
+      if (consumers_vote(*(volatile int*)&s_fail)) break;
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         const int i = tid + 32 * STARS_WARPS * q;
