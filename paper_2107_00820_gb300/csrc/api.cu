@@ -343,6 +343,7 @@ void smooth_fused(als_ctx* c, MGWork& w, int l, bool x_is_zero, void* t) {
     ApplyEpi e{w.b[l], -1.0, 0, nullptr, 0, 1, st};
     op_apply_epi(Lv, prec, c->gamma, w.x[l], V0, e, s);                  // V0 = b - A x
   }
+  gm_fold(prec, st, 1, 0, len, s);
   for (int j = 0; j < steps; ++j) {
     void* Vj = vptr(w.V[l], w.es, (long long)j * len);
     void* Vn = vptr(w.V[l], w.es, (long long)(j + 1) * len);
@@ -367,7 +368,9 @@ void smooth_fused(als_ctx* c, MGWork& w, int l, bool x_is_zero, void* t) {
     cudaEvent_t a0 = nullptr, a1 = nullptr;
     if (l == c->L - 1) prof_events(c, t_prof_counter, a0, a1, 1);
     op_apply_epi(Lv, prec, c->gamma, Zj, Vn, e, s, a0, a1);            // A Z_j and its dots
+    gm_fold(prec, st, 0, j, len, s);
     gm_orth(prec, len, j, w.V[l], len, st, s);                            // V_{j+1}, H[0..j][j]
+    gm_fold(prec, st, 1, j + 1, len, s);
   }
   gm_update(prec, len, steps, w.Z[l], w.V[l], len, st, w.x[l], x_is_zero ? 1 : 0, t, s);
 }
@@ -1841,6 +1844,7 @@ void merged_smooth(MergedCycle& M, int l, bool x_is_zero, bool residual, cudaStr
     if (!apt.empty()) batch_tiled_residual(apt, s);
     if (!ap.empty()) batch_apply_epi(ap, s);
   } else if (!gs.empty()) batch_gm_start(gs, s);     // V0 = b (tiled: by the first step)
+  batch_gm_fold(gs, 1, 0, s);
   for (int j = 0; j < steps; ++j) {
     std::vector<BArnoldi> tile;
     std::vector<BPatch> prod, gath;
@@ -1871,11 +1875,13 @@ void merged_smooth(MergedCycle& M, int l, bool x_is_zero, bool residual, cudaStr
     if (!prod.empty()) {
       batch_star_products(M.var_prod[l], prod, s);     // scratch rows = A_v^-1 V_j|_v
       if (!gath.empty()) batch_patch_gather(gath, s);  // Z_j = D^-1 v_j (unfused instances)
-      batch_apply_epi(az, s);                          // A Z_j, H[0..j][j]
+      batch_apply_epi(az, s);                          // A Z_j and its dots
+      batch_gm_fold(gs, 0, j, s);
     }
     // V_{j+1}, Givens step j; a tiled step takes the one before into itself, all but the last
     if (j == steps - 1) batch_gm_orth(g, s);
     else if (!gs.empty()) batch_gm_orth(gs, s);
+    batch_gm_fold(gs, 1, j + 1, s);
   }
   batch_gm_update(g, s);
 }

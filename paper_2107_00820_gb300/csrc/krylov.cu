@@ -284,7 +284,7 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
     }
     if ((int)threadIdx.x < j) rhni = load_small(st.rhn + threadIdx.x);
   }
-  sum_rows<T>(norm_rows<T>(sd, j), norm_count(sd, j, n), 1, acc);
+  sum_rows<T>(norm_sums<T>(sd, j), norm_parts(sd, j, n), 1, acc);
   {
     const T v = block_total<T>(acc, 1, sh);
     if (threadIdx.x == 0) nrm2 = v;
@@ -307,7 +307,7 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
     const unsigned i = base + q * RED_THREADS;
     a[q] = i < n ? w[i] : T(0);
   }
-  sum_rows<T>(dot_rows<T>(sd, j), sd.nbd, j + 1, acc);
+  sum_rows<T>(dot_sums<T>(sd, j), dot_parts(sd), j + 1, acc);
   {
     const T v = block_total<T>(acc, j + 1, sh);
     if ((int)threadIdx.x <= j) {
@@ -373,7 +373,7 @@ __device__ __forceinline__ void gm_update_body(unsigned bx, unsigned n, const T*
   if (sd.early) pdl_trigger();
   if ((int)threadIdx.x < GmresLayout(k).total) state[threadIdx.x] = load_small(static_cast<const S*>(sd.base) + threadIdx.x);
   T acc[KMAXB];
-  sum_rows<T>(norm_rows<T>(sd, k), norm_count(sd, k, n), 1, acc);
+  sum_rows<T>(norm_sums<T>(sd, k), norm_parts(sd, k, n), 1, acc);
   const T tot = block_total<T>(acc, 1, sh);   // (its barrier also publishes the state)
   if (threadIdx.x == 0) nrm2 = tot;
   __syncthreads();
@@ -414,12 +414,53 @@ __global__ void __launch_bounds__(RED_THREADS) k_gm_update(unsigned n, const T* 
   gm_update_body<T, K>(blockIdx.x, n, Z, V, ld, sd, x, x_zero, t);
 }
 
+// dst[c][p] = the sum of every kFold-th chunk of 256 of column c's nb partials, from chunk p on (block c kFold + p)
+template <typename T>
+struct FoldArgs {
+  const T* src;
+  T* dst;
+  int nb;
+};
+template <typename T>
+__device__ __forceinline__ void gm_fold_body(unsigned bx, const FoldArgs<T>& a) {
+  __shared__ T sh[RED_THREADS / 32][KMAXB];
+  const int c = bx / kFold, p = bx - c * kFold;
+  pdl_wait();
+  pdl_trigger();
+  T acc[KMAXB] = {T(0)};
+#pragma unroll 4
+  for (int i = p * RED_THREADS + threadIdx.x; i < a.nb; i += kFold * RED_THREADS) acc[0] += __ldcg(a.src + (long long)c * a.nb + i);
+  const T v = block_total<T>(acc, 1, sh);
+  if (threadIdx.x == 0) a.dst[bx] = v;
+}
+template <typename T>
+__global__ void __launch_bounds__(RED_THREADS) k_gm_fold(const FoldArgs<T> a) {
+  gm_fold_body<T>(blockIdx.x, a);
+}
+// the dots of step j (norm = 0) or |column j|^2 (norm = 1) of n entries
+template <typename T>
+static FoldArgs<T> fold_args(const GmresDev& st, int norm, int j, long long n) {
+  return norm ? FoldArgs<T>{norm_rows<T>(st, j), fold_norm<T>(st, j), norm_count(st, j, n)}
+              : FoldArgs<T>{dot_rows<T>(st, j), fold_dots<T>(st, j), st.nbd};
+}
+void gm_fold(int prec, const GmresDev& st, int norm, int j, long long n, cudaStream_t s) {
+  if (!st.foff) return;
+  const unsigned blocks = kFold * (norm ? 1 : j + 1);
+  if (prec == PREC_F64) launch_pdl(k_gm_fold<double>, blocks, RED_THREADS, 0, s, fold_args<double>(st, norm, j, n));
+  else launch_pdl(k_gm_fold<float>, blocks, RED_THREADS, 0, s, fold_args<float>(st, norm, j, n));
+  count_launch(1);
+}
+
+static int gmres_blocks(const LevelDev& L) { return std::max(apply_epi_blocks(L), gm_blocks(L.g.N * L.g.dim)); }
+
 GmresDev gmres_dev(const LevelDev& L, int prec, void* state, int steps, double* partial, bool x_is_zero, bool tiled) {
   const long long n = L.g.N * L.g.dim;
   const int nbe = apply_epi_blocks(L), nbv = gm_blocks(n), nbt = tiled ? arnoldi_tiles(L) : 0;
   const int nbd = tiled ? nbt : nbe, nbn = tiled ? nbt : nbv;
-  return GmresDev{state, steps, partial + 1, nbd, tiled ? nbt : x_is_zero ? nbv : nbe, nbn, 2 * nbd * KMAXB,
-                  std::max(std::max(nbe, nbv), nbt), tiled ? 1 : 0, prec == PREC_F32 || L.g.dim == 2 ? 1 : 0};
+  const int noff = 2 * nbd * KMAXB, nstride = std::max(gmres_blocks(L), nbt);
+  return GmresDev{state, steps, partial + 1, nbd, tiled ? nbt : x_is_zero ? nbv : nbe, nbn, noff, nstride,
+                  !tiled && gmres_blocks(L) > kFoldFrom ? noff + 2 * nstride : 0, tiled ? 1 : 0,
+                  prec == PREC_F32 || L.g.dim == 2 ? 1 : 0};
 }
 
 void gm_start(int prec, long long n, const void* b, void* V0, const GmresDev& st, cudaStream_t s) {
@@ -553,11 +594,30 @@ int batch_gm_update(const std::vector<BGmres>& items, cudaStream_t s) {
   return batch_gm(f[items[0].st.s - 1], items, 0, s);
 }
 
-// workspace of a level's fused reductions: two areas of KMAXB rows and two rows, one value per block
+// the folds of a merged operation's items: their dots of step j, or |column j|^2
+__global__ void __launch_bounds__(RED_THREADS) k_gm_fold_b(const __grid_constant__ BatchTab<FoldArgs<float>> tb) {
+  const int i = batch_slot(tb, blockIdx.x);
+  gm_fold_body<float>(blockIdx.x - tb.start[i], tb.a[i]);
+}
+int batch_gm_fold(const std::vector<BGmres>& items, int norm, int j, cudaStream_t s) {
+  std::vector<FoldArgs<float>> a;
+  std::vector<unsigned> nb;
+  for (const BGmres& it : items) {
+    if (!it.st.foff) continue;
+    a.push_back(fold_args<float>(it.st, norm, j, it.n));
+    nb.push_back(kFold * (norm ? 1 : j + 1));
+  }
+  if (a.empty()) return 0;
+  const int n = launch_batch(k_gm_fold_b, a, nb, RED_THREADS, 0, s);
+  count_launch(n);
+  return n;
+}
+
+// workspace of a level's fused reductions: two areas of KMAXB rows and two rows, one value per block, and the
+// same folded
 size_t gmres_partial_doubles(const LevelDev& L) {
-  const int nb = std::max(std::max(apply_epi_blocks(L), gm_blocks(L.g.N * L.g.dim)),
-                          L.k == 2 && L.g.dim == 2 ? arnoldi_tiles(L) : 0);
-  return (size_t)nb * (2 * KMAXB + 2) + 1;
+  const int nb = std::max(gmres_blocks(L), L.k == 2 && L.g.dim == 2 ? arnoldi_tiles(L) : 0);
+  return (size_t)(nb + kFold) * (2 * KMAXB + 2) + 1;
 }
 
 // ---------------------------------------------------------------------------

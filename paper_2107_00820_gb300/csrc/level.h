@@ -253,6 +253,8 @@ size_t gmres_partial_doubles(const LevelDev& L);   // workspace of op_apply_epi,
 GmresDev gmres_dev(const LevelDev& L, int prec, void* state, int steps, double* partial, bool x_is_zero, bool tiled);
 void gm_start(int prec, long long n, const void* b, void* V0, const GmresDev& st, cudaStream_t s);
 void gm_orth(int prec, long long n, int j, const void* V, long long ld, const GmresDev& st, cudaStream_t s);
+// levels of many blocks only: the partials of the dots of step j, or (norm) of |column j|^2, folded for their consumers
+void gm_fold(int prec, const GmresDev& st, int norm, int j, long long n, cudaStream_t s);
 void gm_update(int prec, long long n, int k, const void* Z, const void* V, long long ld, const GmresDev& st,
                void* x, int x_zero, void* t, cudaStream_t s);
 size_t multidot_partial_doubles(int k);
@@ -329,6 +331,7 @@ int batch_tiled_prolong(const std::vector<BTiledTransfer>& items, cudaStream_t s
 int batch_arnoldi_step(const std::vector<BArnoldi>& items, cudaStream_t s);
 int batch_gm_start(const std::vector<BGmres>& items, cudaStream_t s);
 int batch_gm_orth(const std::vector<BGmres>& items, cudaStream_t s);
+int batch_gm_fold(const std::vector<BGmres>& items, int norm, int j, cudaStream_t s);
 int batch_gm_update(const std::vector<BGmres>& items, cudaStream_t s);
 // resident CTAs per SM of a merged star kernel (variant 0, 1, 2 as above; 3: boundary stars)
 int batch_patch_occupancy(int variant);

@@ -228,7 +228,8 @@ struct GmresLayout {
 
 // host-side handle: the state array (elements of small_t), s, and the block
 // partials of the reductions.  A reduction kernel only writes its partials, [column][block];
-// every block of the kernel that needs the sums adds them for itself, in one fixed order.
+// every block of the kernel that needs the sums adds them for itself, in one fixed order (on large levels
+// after a kernel has folded them, see kFoldFrom).
 // (A last-block finish, with its fence, ticket, second fence, reload and one-thread
 // bookkeeping, cost 1 to 2 us at the end of each of the two reductions of a step: a third of a
 // small level's time.)  The dots of step j: nbd blocks in one of two areas from rows, by the parity of
@@ -239,6 +240,7 @@ struct GmresDev {
   int s;
   void* rows;
   int nbd, nb0, nbn, noff, nstride;
+  int foff;   // where the folded partials lie, beyond the others; 0: a level that does not fold
   int late;   // the kernel before the last Gram-Schmidt step writes more than its column (see arnoldi2.cuh)
   // The Gram-Schmidt and update kernels trigger their successor right after the wait, not at their end: all
   // but FP64 in 3D, whose successors take the registers that the predecessors' long blocks
@@ -262,6 +264,27 @@ __host__ __device__ __forceinline__ int gm_blocks(long long n) {
 __host__ __device__ __forceinline__ int norm_count(const GmresDev& d, int j, long long n) {
   return j == 0 ? d.nb0 : j < d.s ? d.nbn : gm_blocks(n);
 }
+
+// Every consumer block reads every partial, which grows with the square of the level.  Levels whose kernels have more than
+// kFoldFrom blocks put a kernel between (k_gm_fold) that leaves kFold sums a column.  One cycle, us, without / with it
+// on every level: 3D FP32 32^3 (804 blocks on the finest) 1651 / 1683, 36^3 (1,140) 2927 / 2935, 40^3 (1,615) 2855 / 2838;
+// FP64 40^3 17198 / 17039; beyond: FP32 96^3 35400 / 29600, 2D 2048^2 31200 / 16700, FP64 256800 / 220100, 234700 / 143400.
+constexpr int kFoldFrom = 1400, kFold = 32;
+template <typename T>
+__host__ __device__ __forceinline__ T* fold_dots(const GmresDev& d, int j) {
+  return static_cast<T*>(d.rows) + d.foff + (j & 1) * (KMAXB * kFold);
+}
+template <typename T>
+__host__ __device__ __forceinline__ T* fold_norm(const GmresDev& d, int j) {
+  return static_cast<T*>(d.rows) + d.foff + (2 * KMAXB + (j & 1)) * kFold;
+}
+// what the consumers add: the dots of step j (columns dot_parts apart), |column j|^2
+template <typename T>
+__device__ __forceinline__ const T* dot_sums(const GmresDev& d, int j) { return d.foff ? fold_dots<T>(d, j) : dot_rows<T>(d, j); }
+__device__ __forceinline__ int dot_parts(const GmresDev& d) { return d.foff ? kFold : d.nbd; }
+template <typename T>
+__device__ __forceinline__ const T* norm_sums(const GmresDev& d, int j) { return d.foff ? fold_norm<T>(d, j) : norm_rows<T>(d, j); }
+__device__ __forceinline__ int norm_parts(const GmresDev& d, int j, long long n) { return d.foff ? kFold : norm_count(d, j, n); }
 
 // the block partials of a gather: |y|^2 of column 0 (start) or the k dots (every thread calls)
 template <typename T>

@@ -1,0 +1,86 @@
+"""Levels whose reductions have more blocks than every consumer adds up for itself (a kernel folds the partials in
+between): at order 2 on the finest one or two of 512^2 cells, the finest of 48^3."""
+import numpy as np
+import pytest
+
+from gpu_helpers import context, dev, host, rel, sinker, torch
+
+from paper_2107_00820_gb300 import Batch, alstokes as A
+
+pytestmark = pytest.mark.gpu
+
+F32, F64 = A.ALS_PREC_FP32, A.ALS_PREC_FP64
+
+
+def _composed_cycle(ctx, b, sweeps):
+    """The V-cycle from the context's own single steps, with GMRES(s) and its sums formed by torch in 64 bits."""
+    def zeros(l):
+        return torch.zeros(ctx.nu(l), dtype=torch.float64, device="cuda")
+
+    def apply(l, x):
+        y = zeros(l)
+        ctx.apply_agamma(x, y, l)
+        return y
+
+    def smooth(l, x, b):
+        V, Z, H = [b - apply(l, x)], [], torch.zeros(sweeps + 1, sweeps, dtype=torch.float64)
+        beta = V[0].norm()
+        V[0] = V[0] / beta
+        for j in range(sweeps):
+            Z.append(zeros(l))
+            ctx.star_smooth(l, V[j], Z[j])
+            w = apply(l, Z[j])
+            h = torch.stack(V) @ w
+            w = w - h @ torch.stack(V)
+            H[:j + 1, j], H[j + 1, j] = h.cpu(), float(w.norm())
+            V.append(w / w.norm())
+        e = torch.zeros(sweeps + 1, 1, dtype=torch.float64)
+        e[0] = float(beta)
+        y = torch.linalg.lstsq(H, e).solution[:, 0]
+        return x + y.cuda() @ torch.stack(Z)
+
+    def cycle(l, b):
+        x = zeros(l)
+        if l == 0:
+            ctx.coarse_solve(b, x)
+            return x
+        x = smooth(l, x, b)
+        rc, xf = zeros(l - 1), zeros(l)
+        ctx.restrict(l, b - apply(l, x), rc)
+        ctx.prolong(l, cycle(l - 1, rc), xf)
+        return smooth(l, x + xf, b)
+
+    return cycle(ctx.levels - 1, b)
+
+
+# tolerances of the parity tests for cycles at mild contrast
+@pytest.mark.parametrize("d,n,levels", [(2, 512, 7), (3, 48, 5)])
+def test_cycle_on_a_folding_level(d, n, levels):
+    pb = sinker(d, n, levels, 1.0, 1e2, 21)
+    ctx = context(pb, sweeps=3)
+    b = torch.randn(ctx.nu(), dtype=torch.float32, device="cuda", generator=torch.Generator("cuda").manual_seed(22))
+    x32, x64 = torch.zeros_like(b), torch.zeros_like(b, dtype=torch.float64)
+    ctx.vcycle(b, x32, F32)
+    ctx.vcycle(b.double(), x64)
+    ref = host(_composed_cycle(ctx, b.double(), 3))
+    assert rel(host(x64), ref) <= 1e-12
+    assert rel(host(x32), ref) <= 1e-4
+
+
+def test_merged_cycle_with_a_folding_level():
+    """A large instance beside small ones: the merged launches give the single cycles' bits."""
+    pbs = [sinker(2, 512, 7, 1.0, 1e2, 23), sinker(2, 16, 2, 1.0, 1e2, 24), sinker(3, 8, 2, 1.0, 1e2, 25)]
+    opts = {"mode": A.ALS_MODE_MIXED, "schur": A.ALS_SCHUR_P2, "sweeps": 3}
+    batch = Batch([{"dim": p.d, "n": p.n, "levels": p.levels, "coeffs": p.mu, "gamma": p.gamma, "options": opts}
+                   for p in pbs])
+    rng = np.random.default_rng(26)
+    bs = [dev(rng.standard_normal(s[0]), torch.float32) for s in batch.shapes]
+    xs = [torch.zeros_like(b) for b in bs]
+    batch.vcycle(bs, xs, F32)
+    for pb, b, xm in zip(pbs, bs, xs):
+        ctx = context(pb, **opts)
+        x = torch.zeros_like(b)
+        ctx.vcycle(b, x, F32)
+        assert torch.equal(x, xm)
+        ctx.close()
+    batch.close()
