@@ -395,8 +395,13 @@ static auto arnoldi_kernel_b(int i) {
 }
 
 // Which levels take their Arnoldi steps tiled: 2D, order 2, FP32, every vertex's inverse in one
-// array (below kSplitVertices vertices; both sides measured above).
-bool arnoldi_tiled(const LevelDev& L, int prec) { return L.k == 2 && L.g.dim == 2 && prec == PREC_F32 && !L.split; }
+// array, fewer than kTiledVertices vertices.  The repeated stars and cells cost more than the launches from about
+// there on: one FP32 cycle, us, whose finest level takes tiles / separate kernels: 192^2 542 / 560, 256^2 740 / 666,
+// 384^2 1652 / 1169 (16^2 and 128^2 above).
+constexpr long long kTiledVertices = 32768;
+bool arnoldi_tiled(const LevelDev& L, int prec) {
+  return L.k == 2 && L.g.dim == 2 && prec == PREC_F32 && !L.split && L.g.nverts < kTiledVertices;
+}
 int arnoldi_tiles(const LevelDev& L) { return tiles2(L.g); }
 
 static ArnoldiArgs arnoldi_args(const LevelDev& L, double gamma, const ArnoldiStep& e) {

@@ -1,5 +1,9 @@
 """Levels whose reductions have more blocks than every consumer adds up for itself (a kernel folds the partials in
 between): at order 2 on the finest one or two of 512^2 cells, the finest of 48^3."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -10,6 +14,7 @@ from paper_2107_00820_gb300 import Batch, alstokes as A
 pytestmark = pytest.mark.gpu
 
 F32, F64 = A.ALS_PREC_FP32, A.ALS_PREC_FP64
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def _composed_cycle(ctx, b, sweeps):
@@ -84,3 +89,28 @@ def test_merged_cycle_with_a_folding_level():
         assert torch.equal(x, xm)
         ctx.close()
     batch.close()
+
+
+def test_large_levels_in_one_piece_take_separate_kernels():
+    """A 2D level of 32,768 vertices and more whose stars are stored whole (a switch) takes its smoother steps as
+    separate kernels like one with split stars: the operator's cell kernel is timed there, and is not where a step is
+    one launch."""
+    code = """if True:
+        import sys
+        import numpy as np
+        import torch
+        sys.path.insert(0, "tests")
+        from gpu_helpers import context, sinker
+        from paper_2107_00820_gb300 import alstokes as A
+        for n, separate in ((128, False), (192, True)):
+            ctx = context(sinker(2, n, 6, 1.0, 1e2, 27), mode=A.ALS_MODE_MIXED, sweeps=2)
+            ctx.profile(True)
+            b = torch.randn(ctx.nu(), dtype=torch.float32, device="cuda")
+            x = torch.zeros_like(b)
+            ctx.vcycle(b, x, A.ALS_PREC_FP32)
+            assert (ctx.profile_read_kernel(1)[1] > 0) == separate, n
+            ctx.close()
+    """
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, ALS_SPLIT_STARS="0"),
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
