@@ -453,7 +453,8 @@ als_status als_batch_get_mode(const als_batch* batch, int* mode);
  * whole batch.  als_batch_merged_tune: for group `group` and level index `level`
  * (0 = coarsest, 1 <= level < the group's largest level count), the variants chosen
  * for the merged star products and interior solves, ms[6] (optional) the time per
- * launch of each variant (products, then interior solves), and instances (optional,
+ * launch of each variant (products, then interior solves; 0 where no instance of the level takes
+ * such launches, as 2D FP32 levels below 32,768 vertices do not), and instances (optional,
  * room for count entries) the batch indices of the group's instances in order.
  * ALS_EINVAL: NULL batch or required output, index out of range, or no plan yet. */
 als_status als_batch_merged_plan(const als_batch* batch, int* grouping, int* groups, float* ms, long long* kernels);

@@ -1955,7 +1955,8 @@ void merged_cycle(MergedCycle& M, cudaStream_t s) {
 
 // Autotuner of the merged cycle: for every level index, time the three patch-kernel
 // variants of the merged star products and of the merged interior solves (one warm-up
-// and three timed launches each, CUDA events) and keep the fastest.  Inputs: the
+// and three timed launches each, CUDA events) and keep the fastest.  Instances whose steps or transfers are
+// tiled launch neither and are left out (a level of such instances alone keeps variant 0, times 0).  Inputs: the
 // instances' zeroed V_0 of that level; outputs go to scratch the cycle overwrites.
 void merged_tune(MergedCycle& M, cudaStream_t s) {
   const long long launches0 = launch_count();
@@ -1971,10 +1972,11 @@ void merged_tune(MergedCycle& M, cudaStream_t s) {
     for (als_ctx* c : at_level(M, l)) {
       MGWork& w = c->w32;
       vec_zero(PREC_F32, c->lev[l].g.N * c->dim, w.V[l], s);
-      prod.push_back(BPatch{&c->lev[l], w.V[l], w.scratch[l], nullptr});
-      isv.push_back(BPatch{&c->lev[l], w.V[l], w.t2[l], nullptr});
+      if (!tiled_steps(c, w, l)) prod.push_back(BPatch{&c->lev[l], w.V[l], w.scratch[l], nullptr});
+      if (!tiled_transfers(c, w, l)) isv.push_back(BPatch{&c->lev[l], w.V[l], w.t2[l], nullptr});
     }
     for (int kind = 0; kind < 2; ++kind) {
+      if ((kind == 0 ? prod : isv).empty()) continue;
       float best = 1e30f;
       for (int v = 0; v < 3; ++v) {
         for (int rep = 0; rep < 4; ++rep) {

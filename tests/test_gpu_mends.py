@@ -1,0 +1,30 @@
+"""Calls about the edges of the binding: what the autotuners time, how a call is ordered after the caller's stream,
+which buffers it takes."""
+import numpy as np
+import pytest
+
+from gpu_helpers import dev, sinker, torch
+
+from paper_2107_00820_gb300 import Batch, alstokes as A
+
+pytestmark = pytest.mark.gpu
+
+F32, F64 = A.ALS_PREC_FP32, A.ALS_PREC_FP64
+
+
+def _batch(pbs, **opts):
+    opts = {"mode": A.ALS_MODE_MIXED, "schur": A.ALS_SCHUR_P2, "sweeps": 3, **opts}
+    return Batch([{"dim": p.d, "n": p.n, "levels": p.levels, "coeffs": p.mu, "gamma": p.gamma, "options": opts}
+                  for p in pbs])
+
+
+def test_merged_tuner_times_the_launches_that_run():
+    """Tiled 2D levels launch neither star products nor interior solves of their own: beside a 3D instance the tuner
+    leaves them out, and a level that has only those is not timed."""
+    batch = _batch([sinker(2, (20, 12), 3, 10.0, 1e2, 31), sinker(2, (16, 16), 2, 10.0, 1e2, 32), sinker(3, 4, 2, 10.0, 1e2, 33)])
+    batch.set_grouping(0)
+    bs = [dev(np.random.default_rng(34).standard_normal(s[0]), torch.float32) for s in batch.shapes]
+    batch.vcycle(bs, [torch.zeros_like(b) for b in bs], F32)
+    assert min(batch.merged_tune(0, 1)[2]) > 0          # the 3D instance's
+    assert batch.merged_tune(0, 2)[:3] == (0, 0, [0.0] * 6)
+    batch.close()
