@@ -438,7 +438,7 @@ void restrict_level(als_ctx* c, MGWork& w, int l, const void* rf, void* rc) {
       restrict_std(C, F, w.prec, w.t3[l], rc, s);
     } else {
       op_apply(F, w.prec, OP_AL, c->gamma, w.t2[l], w.t3[l], nullptr, nullptr, s);
-      restrict_std(C, F, w.prec, rf, rc, s, w.t3[l]);                      // P_H^T (rf - t3)
+      qk_restrict(C, F, w.prec, rf, rc, s, w.t3[l]);                       // P_H^T (rf - t3)
     }
   } else {
     restrict_std(C, F, w.prec, rf, rc, s);

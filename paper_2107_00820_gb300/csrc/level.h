@@ -184,6 +184,7 @@ void qk_patch_smooth(const LevelDev& L, int prec, const void* r, void* z, void* 
 void qk_interior_solve(const LevelDev& fine, int prec, const void* in, void* out, int subtract, cudaStream_t s);
 void qk_prolong(const LevelDev& coarse, const LevelDev& fine, int prec, const void* xc, void* xf, cudaStream_t s,
                 void* xadd);
+// rc = P_H^T rf, or P_H^T (rf - sub) when sub is given
 void qk_restrict(const LevelDev& coarse, const LevelDev& fine, int prec, const void* rf, void* rc, cudaStream_t s,
                  const void* sub);
 // ---- qk3.cu: [Q3]^3 x P2disc
@@ -223,9 +224,8 @@ void newton_coeffs(const Geom& fine, const Geom& level, const double* u, double 
 // xf = P_H xc; if xadd, also xadd += P_H xc
 void prolong_std(const LevelDev& coarse, const LevelDev& fine, int prec, const void* xc, void* xf,
                  cudaStream_t s, void* xadd = nullptr);
-// rc = P_H^T rf, or P_H^T (rf - sub) when sub is given
-void restrict_std(const LevelDev& coarse, const LevelDev& fine, int prec, const void* rf, void* rc,
-                  cudaStream_t s, const void* sub = nullptr);
+// rc = P_H^T rf
+void restrict_std(const LevelDev& coarse, const LevelDev& fine, int prec, const void* rf, void* rc, cudaStream_t s);
 
 // ---- krylov.cu (vector kernels)
 void vec_axpby(int prec, long long n, double a, const void* x, double b, void* y, cudaStream_t s);

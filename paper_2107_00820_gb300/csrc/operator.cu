@@ -16,6 +16,7 @@
 #include "reduce.cuh"
 #include "pdl.cuh"
 
+#include <stdexcept>
 #include <type_traits>
 
 namespace als {
@@ -344,6 +345,7 @@ static void residual_dim(const LevelDev& L, int mode, double gamma, const void* 
 }
 void op_residual(const LevelDev& L, int prec, int mode, double gamma, const void* x, const void* b, void* y,
                  cudaStream_t s) {
+  if (!L.ebuf) throw std::logic_error("op_residual: a level without the staging buffer");   // the coloured form takes no b
   if (prec == PREC_F64) {
     if (L.g.dim == 2) residual_dim<double, 2>(L, mode, gamma, x, b, y, s);
     else residual_dim<double, 3>(L, mode, gamma, x, b, y, s);

@@ -193,7 +193,7 @@ struct TransferArgs {
   Geom gc, gf;
   const float* in;
   float* out;
-  float* aux;
+  float* aux;   // prolongation: xadd (may be NULL)
 };
 __global__ void __launch_bounds__(256) k_prolong_b(const __grid_constant__ BatchTab<TransferArgs> tb) {
   const int i = batch_slot(tb, blockIdx.x);
@@ -231,10 +231,9 @@ void prolong_std(const LevelDev& coarse, const LevelDev& fine, int prec, const v
   count_launch(1);
 }
 
-void restrict_std(const LevelDev& coarse, const LevelDev& fine, int prec, const void* rf, void* rc, cudaStream_t s,
-                  const void* sub) {
+void restrict_std(const LevelDev& coarse, const LevelDev& fine, int prec, const void* rf, void* rc, cudaStream_t s) {
   if (fine.k == 3) {
-    qk_restrict(coarse, fine, prec, rf, rc, s, sub);
+    qk_restrict(coarse, fine, prec, rf, rc, s, nullptr);
     return;
   }
   const unsigned b = restrict_blocks(coarse.g);
@@ -264,7 +263,7 @@ int batch_restrict(const std::vector<BTransfer>& items, cudaStream_t s) {
   std::vector<TransferArgs> a;
   std::vector<unsigned> nb;
   for (const BTransfer& it : items) {
-    a.push_back(TransferArgs{it.coarse->g, it.fine->g, (const float*)it.in, (float*)it.out, (float*)it.aux});
+    a.push_back(TransferArgs{it.coarse->g, it.fine->g, (const float*)it.in, (float*)it.out, nullptr});
     nb.push_back(restrict_blocks(it.coarse->g));
   }
   const int n = launch_batch(k_restrict_b, a, nb, 256, 0, s);
