@@ -41,8 +41,12 @@
  * depend on them unless stated): ALS_NO_GRAPH=1 issues every cycle kernel by
  * kernel instead of replaying a captured CUDA graph; ALS_PDL=0 launches without
  * programmatic dependent launch; ALS_PATCH_KERNEL=tma2|tma3|direct forces one FP32
- * star-patch kernel variant on every level; ALS_FUSE_GATHER=0 keeps the separate
- * patch-gather kernel in the order-2 smoother (bitwise the same results);
+ * star-patch kernel variant on every level (it serves what als_set_patch_kernel's does: not the
+ * cycle on 2D levels whose smoother steps and transfers are one launch each);
+ * ALS_FUSE_GATHER=0 sums the star outputs per node in a kernel of their own (order 2, and order 3
+ * in FP32, where the operator's cell kernel does it otherwise: bitwise the same results) and, with
+ * it, takes every operation of the 2D FP32 order-2 cycle as separate kernels, which sum in another
+ * order than the tiled ones (the results differ in their rounding);
  * ALS_SPLIT_STARS=1 / 0 makes every smoothed level store its FP32 star inverses split
  * (interior stars block-packed, boundary stars restricted to their free dofs, applied by a
  * second kernel) or whole (every star padded to d 3^d dofs); by default levels with at
