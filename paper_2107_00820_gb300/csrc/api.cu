@@ -1095,7 +1095,7 @@ als_status als_create(const als_mesh* mesh, const als_coeff* coeff, double gamma
   *out = nullptr;
   als_ctx* c = new als_ctx();
   c->user_stream = (cudaStream_t)stream;
-  if (stream) cudaStreamSynchronize((cudaStream_t)stream);
+  cudaStreamSynchronize((cudaStream_t)stream);   // the coefficients may be on their way there (NULL: the default stream)
   als_status st = create_impl(c, mesh, coeff, gamma, opt);
   if (st != ALS_OK) {
     t_create_err = c->err;   // read back with als_last_error(NULL): the context is gone

@@ -5,7 +5,7 @@ import pytest
 
 from gpu_helpers import dev, sinker, torch
 
-from paper_2107_00820_gb300 import Batch, alstokes as A
+from paper_2107_00820_gb300 import Batch, Context, alstokes as A
 
 pytestmark = pytest.mark.gpu
 
@@ -28,3 +28,20 @@ def test_merged_tuner_times_the_launches_that_run():
     assert min(batch.merged_tune(0, 1)[2]) > 0          # the 3D instance's
     assert batch.merged_tune(0, 2)[:3] == (0, 0, [0.0] * 6)
     batch.close()
+
+
+@pytest.mark.parametrize("batch", [False, True])
+def test_create_waits_for_the_default_stream(batch):
+    """Coefficients that are still being written on the caller's stream, the default one included, are waited for."""
+    pb = sinker(2, (16, 16), 2, 10.0, 1e2, 35)
+    made = [dev(m) for m in pb.mu]
+    late = [torch.zeros_like(m) for m in made]
+    torch.cuda.synchronize()
+    torch.cuda._sleep(200_000_000)          # about a tenth of a second
+    for m, v in zip(late, made):
+        m.copy_(v)
+    if batch:
+        ctx = Batch([{"dim": 2, "n": pb.n, "levels": 2, "coeffs": late, "gamma": pb.gamma, "options": {}}])
+    else:
+        ctx = Context(2, pb.n, 2, late, pb.gamma)
+    ctx.close()
