@@ -2406,6 +2406,20 @@ als_status als_batch_solve(als_batch* b, const double* const* f_qp, const double
   return caught_exception();
 }
 
+// the copies of a merged cycle: one kernel, or, where a caller's vector is not aligned as floats are, copy calls
+static void copy_all(const std::vector<BCopy>& items, cudaStream_t s) {
+  bool aligned = true;
+  for (const BCopy& it : items) aligned = aligned && ((uintptr_t)it.src | (uintptr_t)it.dst) % sizeof(float) == 0;
+  if (aligned) {
+    batch_copy(items, s);
+    return;
+  }
+  for (const BCopy& it : items) {
+    cudaMemcpyAsync(it.dst, it.src, (size_t)it.n * sizeof(float), cudaMemcpyDeviceToDevice, s);
+    if (it.st) cudaMemcpyAsync(it.st_host, it.st, sizeof(DevStatus), cudaMemcpyDeviceToHost, s);
+  }
+}
+
 als_status als_batch_vcycle(als_batch* b, int prec, const void* const* bv, void* const* xv) try {
   if (!b || !bv || !xv) return ALS_EINVAL;
   if (prec != PREC_F64 && prec != PREC_F32) return batch_fail(b, ALS_EINVAL, "prec must be FP64 or FP32");
@@ -2428,12 +2442,12 @@ als_status als_batch_vcycle(als_batch* b, int prec, const void* const* bv, void*
       in.push_back(BCopy{bv[i], c->w32.b[l], len, nullptr, nullptr});
       out.push_back(BCopy{c->w32.x[l], xv[i], len, c->st, c->st_host});
     }
-    batch_copy(in, s);
+    copy_all(in, s);
     const als_status st = batch_plan(b);   // first call: groupings built and timed (the cycle reads b only)
     if (st != ALS_OK) return st;
     if (cudaGraphLaunch(b->plan.exec, s) != cudaSuccess) return batch_fail(b, ALS_ECUDA, "merged cycle launch");
     count_launch(b->plan.kernels);
-    batch_copy(out, s);
+    copy_all(out, s);
     if (cudaStreamSynchronize(s) != cudaSuccess) {
       const cudaError_t e = cudaGetLastError();
       return batch_fail(b, ALS_ECUDA, std::string("merged cycle: ") + cudaGetErrorString(e));

@@ -1,5 +1,7 @@
 """Calls about the edges of the binding: what the autotuners time, how a call is ordered after the caller's stream,
 which buffers it takes."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -45,3 +47,24 @@ def test_create_waits_for_the_default_stream(batch):
     else:
         ctx = Context(2, pb.n, 2, late, pb.gamma)
     ctx.close()
+
+
+def test_merged_cycle_takes_vectors_of_any_alignment():
+    """Vectors that do not start on a float's boundary are copied in and out like others."""
+    batch = _batch([sinker(2, (20, 12), 2, 10.0, 1e2, 36), sinker(3, 4, 2, 10.0, 1e2, 37)])
+    bs = [dev(np.random.default_rng(38).standard_normal(s[0]), torch.float32) for s in batch.shapes]
+    xs = [torch.zeros_like(b) for b in bs]
+    batch.vcycle(bs, xs, F32)
+
+    def odd(t):
+        raw = torch.zeros(4 * t.numel() + 1, dtype=torch.uint8, device="cuda")
+        raw[1:] = t.view(torch.uint8)
+        return raw
+
+    b1, x1 = [odd(b) for b in bs], [odd(torch.zeros_like(b)) for b in bs]
+    torch.cuda.synchronize()
+    arrays = [(ctypes.c_void_p * 2)(*[t.data_ptr() + 1 for t in ts]) for ts in (b1, x1)]
+    assert A.load().als_batch_vcycle(batch._b, F32, *arrays) == A.ALS_OK
+    for x, raw in zip(xs, x1):
+        assert torch.equal(x.view(torch.uint8), raw[1:])
+    batch.close()
