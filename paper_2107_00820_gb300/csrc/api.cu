@@ -1195,9 +1195,10 @@ static void begin(als_ctx* c) {
 }
 
 static als_status finish(als_ctx* c, const char* what) {
-  const als_status st = check_status(c, what);
-  if (st != ALS_OK) return st;
-  return cuda_check(c, what);   // a launch that was refused
+  // a launch that was refused goes first, and is taken off the runtime's record in any case: left there, it
+  // would be reported by a later call
+  const als_status st = check_status(c, what), refused = cuda_check(c, what);
+  return refused != ALS_OK ? refused : st;
 }
 
 als_status als_apply_agamma(als_ctx* c, int level, int prec, const void* x, void* y) try {
