@@ -13,7 +13,8 @@
 // inverses (69 KB) are copied to shared memory before the wait on the predecessor, so their
 // transfer is hidden by it.  Sums within stars, nodes and cells run in the order of the separate
 // kernels.  One cycle, us, separate / tiled: 16^2 two levels 166 / 128, 128^2 five levels
-// 678 / 478 (112 / 106 and 375 / 351 when the column loops got the length KM, after the other steps).
+// 678 / 478 (112 / 106 and 375 / 351 when the column loops got the length KM, after the other steps; 105 and
+// 354 with the state and the combinations of columns in double-float, see reduce.cuh).
 //
 // w goes through two buffers in turn (a block reads its neighbours' nodes of w while others write
 // w'), and so do the partials; the last step's w' goes to column s for k_gm_orth.

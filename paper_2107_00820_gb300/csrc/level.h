@@ -109,7 +109,7 @@ bool arnoldi_tiled(const LevelDev& L, int prec);
 int arnoldi_tiles(const LevelDev& L);   // blocks of its reductions
 void arnoldi_prepare();                 // before any capture
 void arnoldi_step(const LevelDev& L, double gamma, const ArnoldiStep& e, cudaStream_t s);
-// V_0 = b - A x of a tiled level and the partials that start st (tiles2.cuh)
+// V_0 = b - A x of a tiled level and the partials that start st (transfers2.cuh)
 void tiled_residual(const LevelDev& L, double gamma, const void* x, const void* b, void* y, const GmresDev& st,
                     cudaStream_t s);
 // the robust transfers, one launch each: rc = P~^T rf;  x = P~ xc, or += with add

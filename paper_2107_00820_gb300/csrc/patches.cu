@@ -930,7 +930,7 @@ __global__ void __launch_bounds__(256) k_derive32_bnd(Geom g, int pstride, const
 }
 
 void patch_derive32(const LevelDev& L, cudaStream_t s) {
-  if (L.k == 3) {   // the FP32 wrapped rows of the order-3 stars
+  if (L.k == 3) {   // the FP32 form of the order-3 stars: wrapped rows (2D), blocks (3D)
     qk_derive32(L, s);
     return;
   }

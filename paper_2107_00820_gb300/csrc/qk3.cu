@@ -1001,13 +1001,6 @@ __global__ void __launch_bounds__(STAR_THREADS) k_qk3_star_apply(Geom g, const T
   }
 }
 
-// FP32 star storage, "wrapped rows": for odd NS every unordered pair {i, j}, i != j, has a
-// circular distance t = (j - i) mod NS or NS - t in 1..(NS - 1) / 2, so the symmetric
-// matrix is the WT = (NS + 1) / 2 rows W_t[i] = A(i, (i + t) mod NS), t = 0..WT - 1, each
-// padded to WLD = 376 entries (16-byte rows) -- 70,688 floats per star against 70,500 for
-// the packed triangle.  The product y_i = sum_t W_t[i] r_(i+t) + sum_(t>0) W_t[i-t] r_(i-t)
-// (indices mod NS) then reads each row once, coalesced, 16 bytes a thread.
-
 // y_v = A_v^-1 r|_v in FP32 from the blocked storage; every entry of a block is used for both
 // y_I += S r_J and y_J += S^T r_I from registers, the partial sums of a row (one per block
 // column) meet in shared memory and are added in a fixed order.  TS: float, or bfloat16

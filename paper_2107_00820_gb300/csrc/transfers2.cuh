@@ -10,7 +10,7 @@
 // prolongation needs nothing from outside its coarse cells, and a restriction the coarse cells
 // around its coarse nodes.  A block takes 8 x 8 fine cells (4 x 4 coarse ones); a restriction
 // repeats a ring on two sides, 5 x 5 coarse cells.  One cycle, us, separate / tiled: 16^2 two levels
-// 128 / 116, 128^2 five levels 478 / 397.
+// 128 / 116, 128^2 five levels 478 / 397 (105 and 354 with what came after).
 #pragma once
 
 // u on a tile of nodes [component][node], W nodes a row, first node at a cell's corner -> the outputs of
