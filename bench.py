@@ -220,11 +220,13 @@ def stored_traffic(kernel, workload):
         parts = line.split()
         if len(parts) != 5 or line.startswith("#") or parts[0] != kernel or parts[1] != workload:
             continue
+        src = hashlib.sha256()
         try:
-            src = open(os.path.join(ROOT, parts[2]), "rb").read()
+            for f in parts[2].split(","):   # every file that makes up the kernel
+                src.update(open(os.path.join(ROOT, f), "rb").read())
         except OSError:
             return None
-        if hashlib.sha256(src).hexdigest()[:16] != parts[3]:
+        if src.hexdigest()[:16] != parts[3]:
             return None
         return float(parts[4])
     return None
@@ -405,6 +407,8 @@ def ours(args, dist):
     launches = A.als_kernel_launches() - launches0
     clk = clocks.stop()
     k4_ms, k4_n = ctx.profile_read()
+    # the variant that the autotuner kept for the finest level (0, 1: bulk copies, 2: direct loads)
+    star_variant = "direct" if order == 2 and ctx.autotune_info(pb.levels - 1)[0] == 2 else "tma"
     k1_ms, k1_n = ctx.profile_read_kernel(1)
     ctx.profile(False)
 
@@ -730,7 +734,7 @@ def ours(args, dist):
                 "d2h_bytes_per_step": d2h},
         "roofline": {"bound": "hbm",
                      "kernel": "k_arnoldi2 (a whole FP32 smoother step, finest level)" if tiled else
-                     ("k_patch_tma<%d> (FP32 interior-star smoother, finest level)" % pb.d) if order == 2
+                     ("k_patch_%s<%d> (FP32 interior-star smoother, finest level)" % (star_variant, pb.d)) if order == 2
                      else "k_qk%s (FP32 order-3 star products, finest level)"
                      % ("3_stars + k_qk3_stars_bnd" if pb.d == 3 else "_star_apply_w"),
                      "achieved": achieved, "peak": peak, "peak_kind": peak_kind, "unit": "GB/s",
