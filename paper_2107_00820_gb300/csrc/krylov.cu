@@ -299,6 +299,7 @@ __device__ __forceinline__ void gm_orth_body(unsigned bx, unsigned nb, unsigned 
   }
   S nrm, inv;
   sqrt_recip(to_small(nrm2), nrm, inv);
+  inv = recip_of(nrm, inv);
   if ((int)threadIdx.x == j) rhni = inv;
   pdl_wait();
   if (sd.early) pdl_trigger();

@@ -172,11 +172,13 @@ __device__ __forceinline__ DF64 recip_or_zero(DF64 a) {
   return df_quick_two_sum(r, __fmul_rn(r, e));
 }
 // r = sqrt(a) and 1 / r, 0 where a <= 0 (1 / r: or so small that it overflows).  Double-float: one Newton step from the
-// FP32 reciprocal root, no division.
+// FP32 reciprocal root, no division.  FP64: 1 / r is left to recip_of, on the path that needs it.
 __device__ __forceinline__ void sqrt_recip(double a, double& r, double& inv) {
   r = sqrt(fmax(a, 0.0));
-  inv = recip_or_zero(r);
+  inv = 0.0;
 }
+__device__ __forceinline__ double recip_of(double r, double) { return recip_or_zero(r); }
+__device__ __forceinline__ DF64 recip_of(DF64, DF64 inv) { return inv; }
 __device__ __forceinline__ void sqrt_recip(DF64 a, DF64& r, DF64& inv) {
   const float y = rsqrtf(fmaxf(a.hi, 0.f));
   r = inv = DF64{0.f, 0.f};
@@ -317,7 +319,7 @@ __host__ __device__ __forceinline__ GmresView<small_t<T>> gmres_view(const Gmres
   return GmresView<small_t<T>>{b + L.H, L.ldh, b + L.cs, b + L.sn, b + L.g, b + L.rhn, b + L.rr, b + L.beta, d.s + 1};
 }
 
-// Givens rotation (c, s) of (a, b), b >= 0, r = |(a, b)| and rr = 1 / r (0 where that overflows); the plain
+// Givens rotation (c, s) of (a, b), b >= 0, r = |(a, b)| and 1 / r for recip_of; the plain
 // sum of squares where it is far from over- and underflow (hypot takes several times the FP64 instructions)
 __device__ __forceinline__ void givens(double a, double b, double& c, double& s, double& r, double& rr) {
   const double q = a * a + b * b;
@@ -325,7 +327,7 @@ __device__ __forceinline__ void givens(double a, double b, double& c, double& s,
   c = 1.0;
   s = 0.0;
   if (r > 0.0) { c = a / r; s = b / r; }
-  rr = recip_or_zero(r);
+  rr = 0.0;
 }
 __device__ __forceinline__ void givens(DF64 a, DF64 b, DF64& c, DF64& s, DF64& r, DF64& rr) {
   const DF64 q = a * a + b * b;
@@ -384,7 +386,7 @@ __device__ __forceinline__ void gmres_step(const GmresView<S>& st, int k, S nrm2
   for (int i = 0; i < KMAXB; ++i)
     if (i <= k) hg[i] = i == k ? r : h[i];
   hg[k + 1] = S{};
-  st.rr[k] = rr;
+  st.rr[k] = recip_of(r, rr);
   st.cs[k] = c; st.sn[k] = sv;
   st.g[k + 1] = -sv * gk;
   st.g[k] = c * gk;
@@ -421,7 +423,7 @@ __device__ __forceinline__ S gmres_finish(const GmresView<S>& st, S nrm2, int wh
   if (what == 0) {
     S acc = lane < k ? st.g[i] : lane == k ? c * gk : S{};
     const S rik = cs * mine + sn * b1;
-    const S rr = lane < k ? st.rr[i] : lane == k ? rk : S{};
+    const S rr = lane < k ? st.rr[i] : lane == k ? recip_of(r, rk) : S{};
     S y = S{};
 #pragma unroll
     for (int t = KMAXB - 1; t >= 0; --t)
@@ -443,7 +445,7 @@ __device__ __forceinline__ S gmres_finish(const GmresView<S>& st, S nrm2, int wh
       b = -(st_ * b);
     }
   if (lane == 0) u = b;
-  return lane < s ? u * st.rhn[lane] : lane == s ? u * inv : S{};
+  return lane < s ? u * st.rhn[lane] : lane == s ? u * recip_of(hk1, inv) : S{};
 }
 
 }  // namespace als

@@ -1,5 +1,5 @@
 """Levels whose reductions have more blocks than every consumer adds up for itself (a kernel folds the partials in
-between): at order 2 on the finest one or two of 512^2 cells, the finest of 48^3."""
+between): the finest of 512^2, 48^3 and, at order 3, 288^2 cells."""
 import os
 import subprocess
 import sys
@@ -8,6 +8,7 @@ import numpy as np
 import pytest
 
 from gpu_helpers import context, dev, host, rel, sinker, torch
+from synthetic import problems as P
 
 from paper_2107_00820_gb300 import Batch, alstokes as A
 
@@ -59,10 +60,13 @@ def _composed_cycle(ctx, b, sweeps):
 
 
 # tolerances of the parity tests for cycles at mild contrast
-@pytest.mark.parametrize("d,n,levels", [(2, 512, 7), (3, 48, 5)])
-def test_cycle_on_a_folding_level(d, n, levels):
-    pb = sinker(d, n, levels, 1.0, 1e2, 21)
-    ctx = context(pb, sweeps=3)
+@pytest.mark.parametrize("d,n,levels,order", [(2, 512, 7, 2), (3, 48, 5, 2), (2, 288, 6, 3)])
+def test_cycle_on_a_folding_level(d, n, levels, order):
+    if order == 2:
+        pb = sinker(d, n, levels, 1.0, 1e2, 21)
+    else:
+        pb = P.sinker_problem_k((n,) * d, levels, order, 8, 0.1, 200.0, 1e2, 10.0, 1.0, 21, d=d)
+    ctx = context(pb, sweeps=3, order=order)
     b = torch.randn(ctx.nu(), dtype=torch.float32, device="cuda", generator=torch.Generator("cuda").manual_seed(22))
     x32, x64 = torch.zeros_like(b), torch.zeros_like(b, dtype=torch.float64)
     ctx.vcycle(b, x32, F32)
